@@ -4,6 +4,8 @@
 
 #include <cuda.h>
 
+#include <algorithm>
+#include <cstring>
 #include <mutex>
 #include <vector>
 
@@ -208,16 +210,31 @@ inline EncodeFn get_encode() {
   return fn;
 }
 
-struct TmapEntry {
+struct TmapKey {
   const void* base;
   uint64_t dims[5];
   uint64_t strides[4];
   uint32_t box[5];
+  uint32_t pad;  // zero: the key is hashed and compared as bytes
+};
+struct TmapEntry {
+  TmapKey key;
   CUtensorMap map;
 };
 
+// A decoding loop names a few maps per layer on every call (hundreds for a deep model): an
+// open-addressed table, so that a look-up does not grow with the number of layers.
 struct TmapCache {
+  static constexpr uint32_t kSlots = 8192, kMaxUsed = 4096;
+  std::vector<int32_t> slot = std::vector<int32_t>(kSlots, -1);  // index into entries, -1 = empty
   std::vector<TmapEntry> entries;
+
+  static uint32_t hash(const TmapKey& k) {
+    uint64_t h = reinterpret_cast<uintptr_t>(k.base);
+    h = (h ^ k.dims[1] ^ (k.dims[3] << 20) ^ (static_cast<uint64_t>(k.box[1]) << 40)) * 0x9E3779B97F4A7C15ull;
+    h = (h ^ k.strides[0] ^ (k.strides[2] << 24)) * 0xD6E8FEB86659FD93ull;
+    return static_cast<uint32_t>(h >> 40);
+  }
 };
 
 // 5-D bf16 tensor map with 128-byte swizzle, cached per (base, shape, strides, box) in the context.
@@ -226,31 +243,33 @@ inline bool get_tmap(falcon_ctx* ctx, const void* base, const uint64_t dims[5], 
                      const uint32_t box[5], CUtensorMap* out) {
   if (!ctx->tmap_cache) ctx->tmap_cache = new TmapCache();
   TmapCache* cache = static_cast<TmapCache*>(ctx->tmap_cache);
-  for (const TmapEntry& e : cache->entries) {
-    if (e.base != base) continue;
-    bool same = true;
-    for (int i = 0; i < 5; ++i) same = same && e.dims[i] == dims[i] && e.box[i] == box[i];
-    for (int i = 0; i < 4; ++i) same = same && e.strides[i] == strides[i];
-    if (same) {
+  TmapKey key = {};
+  key.base = base;
+  for (int i = 0; i < 5; ++i) { key.dims[i] = dims[i]; key.box[i] = box[i]; }
+  for (int i = 0; i < 4; ++i) key.strides[i] = strides[i];
+  uint32_t at = TmapCache::hash(key) % TmapCache::kSlots;
+  for (; cache->slot[at] >= 0; at = (at + 1) % TmapCache::kSlots) {
+    const TmapEntry& e = cache->entries[cache->slot[at]];
+    if (std::memcmp(&e.key, &key, sizeof(key)) == 0) {
       *out = e.map;
       return true;
     }
   }
   EncodeFn enc = get_encode();
   if (!enc) return false;
-  if (cache->entries.size() >= 4096) cache->entries.clear();
-  TmapEntry e;
-  e.base = base;
-  for (int i = 0; i < 5; ++i) { e.dims[i] = dims[i]; e.box[i] = box[i]; }
-  for (int i = 0; i < 4; ++i) e.strides[i] = strides[i];
   const cuuint32_t elem[5] = {1, 1, 1, 1, 1};
   alignas(64) CUtensorMap m;
   CUresult r = enc(&m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(base), dims, strides, box, elem,
                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return false;
-  e.map = m;
-  cache->entries.push_back(e);
+  if (cache->entries.size() >= TmapCache::kMaxUsed) {  // start over (at most half full: probes stay short)
+    cache->entries.clear();
+    std::fill(cache->slot.begin(), cache->slot.end(), -1);
+    at = TmapCache::hash(key) % TmapCache::kSlots;
+  }
+  cache->slot[at] = static_cast<int32_t>(cache->entries.size());
+  cache->entries.push_back(TmapEntry{key, m});
   *out = m;
   return true;
 }
