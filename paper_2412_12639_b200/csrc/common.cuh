@@ -29,9 +29,9 @@ struct falcon_ctx {
   void* tmap_cache = nullptr;
   // Per-context launch state of the tensor-core attention kernels: whether the dynamic shared
   // memory limit has been raised on this device, and how many clusters of each size fit at once
-  // (0 = not asked yet, -1 = none).  Index 0: rows-on-lanes kernel; 1-3: the keys-on-lanes kernel's
-  // three variants.
-  bool attn_attr_set[4] = {false, false, false, false};
+  // (0 = not asked yet, -1 = none).  Index 0: rows-on-lanes kernel; from 1: the keys-on-lanes kernel's
+  // three variants (times head dimension and place of the tree's K/V for the limit).
+  bool attn_attr_set[13] = {};
   bool lm_attr_set = false;  // the same for the LM-head kernel
   int attn_resident[4][9] = {};
 };
@@ -61,6 +61,7 @@ bool tree_attn_tck_supports(const falcon_ctx* ctx, const falcon_attn_args& a);
 bool tree_attn_tck_preferred(const falcon_ctx* ctx, const falcon_attn_args& a);
 int launch_tree_attn_warp(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s);
 bool tree_attn_warp_supports(const falcon_ctx* ctx, const falcon_attn_args& a);
+bool tree_attn_warp_preferred(const falcon_attn_args& a);
 void tree_attn_tc_release(falcon_ctx* ctx);
 
 #ifdef __CUDACC__

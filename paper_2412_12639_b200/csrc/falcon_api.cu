@@ -153,9 +153,11 @@ static int attn_plan(falcon_ctx* ctx, const falcon_attn_args* a, int* kernel) {
       *kernel = FALCON_ATTN_WARP;
       return FALCON_OK;
     case FALCON_ATTN_AUTO:
-      // tensor cores where a kernel takes the shape (which of the two: by shape, measured); else one
-      // warp per query row while the scores of a row fit its shared memory; else the tiled kernel
-      if (tree_attn_tck_supports(ctx, *a) && (tree_attn_tck_preferred(ctx, *a) || !tree_attn_tc_supports(ctx, *a)))
+      // the small-problem kernel where it is the fastest; else tensor cores where a kernel takes the
+      // shape (which of the two: by shape, measured); else (Hq / Hkv no power of two) CUDA cores
+      if (tree_attn_warp_supports(ctx, *a) && tree_attn_warp_preferred(*a))
+        *kernel = FALCON_ATTN_WARP;
+      else if (tree_attn_tck_supports(ctx, *a) && (tree_attn_tck_preferred(ctx, *a) || !tree_attn_tc_supports(ctx, *a)))
         *kernel = FALCON_ATTN_TCK;
       else if (tree_attn_tc_supports(ctx, *a))
         *kernel = FALCON_ATTN_TC;

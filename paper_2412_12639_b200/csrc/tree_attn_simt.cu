@@ -1,6 +1,6 @@
 // falcon_tree_attn, CUDA-core kernel: the path for shapes the tensor-core
-// kernel does not take (head_dim 64, separate tree buffers, odd strides) and the
-// on-GPU cross-check of that kernel.
+// kernels do not take (a head grouping that is no power of two, more than 8 splits)
+// and the on-GPU cross-check of those kernels.
 //
 // One CTA handles one (sequence, query head, KV split): it keeps the head's
 // T x D queries in shared memory, walks its key range in tiles of 32 keys

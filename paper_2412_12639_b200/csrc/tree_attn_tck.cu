@@ -1,5 +1,5 @@
-// falcon_tree_attn, tensor-core kernel with the KEYS on the tensor-memory lanes (head_dim 128, tree
-// K/V in the cache).
+// falcon_tree_attn, tensor-core kernel with the KEYS on the tensor-memory lanes (head_dim 64 or 128,
+// the tree's K/V in the cache or in buffers of its own).
 //
 // A verification tree has few query rows (60-80 nodes x the query heads of one KV head) and many
 // keys, so the score tile is computed transposed: S^T = K_tile . Q^T with the 128 keys of a tile on
@@ -54,7 +54,6 @@ namespace falcon {
 namespace {
 using namespace tc;
 
-constexpr int kD = 128;
 constexpr int kBKMax = 128;                     // keys per tile at most = TMEM lanes (the launcher picks the tile height)
 // Three variants by the number of query rows N of a unit.  A softmax thread works on chunks of kCW
 // query columns; chunk c belongs to column group c % kGroups, and a lane quadrant has one warp per
@@ -118,12 +117,26 @@ struct Cfg {
   static constexpr uint32_t kSmallBytes = kOffMisc + 16;
 };
 
+// The K/V ring's stage for a head dimension and a block of at most n_max query rows.  A tile's matrix is
+// kHalves blocks of 64 head-dim columns; P^T (64 query rows a block) lies over the K tile, which
+// for 64-wide heads and more than 64 rows is given the room of two blocks.  The P.V MMA always has
+// 128 output lanes: with 64-wide heads its A operand's upper 64 rows are whatever follows the V
+// tile, so there the V tile comes first and K / P^T (always inside the stage) after it; the lanes
+// 64-127 of that accumulator are never read.
+template <int kHD>
+struct Stage {
+  static constexpr uint32_t kHalves = kHD / 64;
+  static __host__ __device__ constexpr uint32_t k_halves(int n_max) { return kHD == 128 || n_max > 64 ? 2u : 1u; }
+  static __host__ __device__ constexpr uint32_t halves(int n_max) { return k_halves(n_max) + kHalves; }
+  static __host__ __device__ constexpr uint32_t k_first(void) { return kHD == 128; }
+};
+
 // bytes between the rows of a partial result of n query columns: an odd number of 16-byte units, so
 // that 16-byte accesses of consecutive rows fall into different banks
 __host__ __device__ constexpr uint32_t part_pitch(int n) { return static_cast<uint32_t>(n) * 2u + 16u; }
 
 struct TckParams {
-  int32_t Hq, Hkv, G, g_shift, s_cap, total_nodes;
+  int32_t Hq, Hkv, G, g_shift, s_cap;
   int32_t n_rows;          // query rows per unit (multiple of 16, at most Cfg::kN)
   int32_t tile_keys;       // keys per K/V tile (multiple of 16, at most 128)
   int32_t n_stages;        // ring depth, 2 or 3
@@ -139,6 +152,8 @@ struct TckParams {
   const __nv_bfloat16* q;
   const __nv_bfloat16* k;
   const __nv_bfloat16* v;
+  const __nv_bfloat16* k_tree;  // the tree's own buffers [N, Hkv, D] (null: its rows follow the prefix in the cache)
+  const __nv_bfloat16* v_tree;
   int64_t kv_stride_b, kv_stride_h, kv_stride_s;
   __nv_bfloat16* out;
   int32_t have_host;
@@ -285,8 +300,10 @@ __device__ __forceinline__ float bf16hi(uint32_t x) { return __uint_as_float(x &
 
 // One query row recomputed exactly by a warp from global memory (running maximum in fp32): the
 // fallback for rows whose scores lie too far from the reference for the fast path.
+template <int kHD>
 __device__ void rescue_row(const TckParams& p, int b, int kvh, int node_base, int T, int Lc, int S_valid, int mg,
                            int lane) {
+  constexpr int kW = kHD / 64;  // 32-bit words (pairs of head dimensions) per lane
   const int node = mg >> p.g_shift, head = kvh * p.G + (mg & (p.G - 1));
   uint64_t lo = 0, hi = 0;
   if (p.tree_mask) {
@@ -295,41 +312,59 @@ __device__ void rescue_row(const TckParams& p, int b, int kvh, int node_base, in
   } else {
     ancestor_mask(p.parent + node_base, T, node, lo, hi);
   }
-  const uint2 qv = *reinterpret_cast<const uint2*>(p.q + (static_cast<int64_t>(node_base + node) * p.Hq + head) * kD + 4 * lane);
-  const float q0 = bf16lo(qv.x), q1 = bf16hi(qv.x), q2 = bf16lo(qv.y), q3 = bf16hi(qv.y);
-  const __nv_bfloat16* kb = p.k + b * p.kv_stride_b + kvh * p.kv_stride_h + 4 * lane;
-  const __nv_bfloat16* vb = p.v + b * p.kv_stride_b + kvh * p.kv_stride_h + 4 * lane;
-  float m = -INFINITY, l = 0.f, a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+  auto load = [&](const __nv_bfloat16* row, float (&x)[2 * kW]) {
+    uint32_t w[kW];
+    if constexpr (kW == 2) {
+      const uint2 t = *reinterpret_cast<const uint2*>(row + 4 * lane);
+      w[0] = t.x;
+      w[1] = t.y;
+    } else {
+      w[0] = *reinterpret_cast<const uint32_t*>(row + 2 * lane);
+    }
+#pragma unroll
+    for (int i = 0; i < kW; ++i) {
+      x[2 * i] = bf16lo(w[i]);
+      x[2 * i + 1] = bf16hi(w[i]);
+    }
+  };
+  const int64_t at = (static_cast<int64_t>(node_base + node) * p.Hq + head) * kHD;
+  float q[2 * kW], acc[2 * kW];
+  load(p.q + at, q);
+#pragma unroll
+  for (int i = 0; i < 2 * kW; ++i) acc[i] = 0.f;
+  const int64_t cache = b * p.kv_stride_b + kvh * p.kv_stride_h;
+  float m = -INFINITY, l = 0.f;
   for (int key = 0; key < S_valid; ++key) {
     if (key >= Lc && !bit128(lo, hi, key - Lc)) continue;
-    const uint2 kk = *reinterpret_cast<const uint2*>(kb + key * p.kv_stride_s);
-    float s = q0 * bf16lo(kk.x);
-    s = fmaf(q1, bf16hi(kk.x), s);
-    s = fmaf(q2, bf16lo(kk.y), s);
-    s = fmaf(q3, bf16hi(kk.y), s);
+    const bool own = p.k_tree && key >= Lc;
+    const int64_t row = own ? (static_cast<int64_t>(node_base + key - Lc) * p.Hkv + kvh) * kHD : cache + key * p.kv_stride_s;
+    float k[2 * kW], v[2 * kW];
+    load((own ? p.k_tree : p.k) + row, k);
+    float s = q[0] * k[0];
+#pragma unroll
+    for (int i = 1; i < 2 * kW; ++i) s = fmaf(q[i], k[i], s);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     s *= p.scale_log2;
     const float mn = fmaxf(m, s);
     const float alpha = ex2(m - mn), pw = ex2(s - mn);
-    const uint2 vv = *reinterpret_cast<const uint2*>(vb + key * p.kv_stride_s);
+    load((own ? p.v_tree : p.v) + row, v);
     l = fmaf(l, alpha, pw);
-    a0 = fmaf(a0, alpha, pw * bf16lo(vv.x));
-    a1 = fmaf(a1, alpha, pw * bf16hi(vv.x));
-    a2 = fmaf(a2, alpha, pw * bf16lo(vv.y));
-    a3 = fmaf(a3, alpha, pw * bf16hi(vv.y));
+#pragma unroll
+    for (int i = 0; i < 2 * kW; ++i) acc[i] = fmaf(acc[i], alpha, pw * v[i]);
     m = mn;
   }
   const float inv = l > 0.f ? 1.f / l : 0.f;
-  const __nv_bfloat162 h0 = __floats2bfloat162_rn(a0 * inv, a1 * inv), h1 = __floats2bfloat162_rn(a2 * inv, a3 * inv);
-  uint2 o;
-  o.x = *reinterpret_cast<const uint32_t*>(&h0);
-  o.y = *reinterpret_cast<const uint32_t*>(&h1);
-  *reinterpret_cast<uint2*>(p.out + (static_cast<int64_t>(node_base + node) * p.Hq + head) * kD + 4 * lane) = o;
+#pragma unroll
+  for (int i = 0; i < kW; ++i)
+    *reinterpret_cast<__nv_bfloat162*>(p.out + at + 2 * kW * lane + 2 * i) =
+        __floats2bfloat162_rn(acc[2 * i] * inv, acc[2 * i + 1] * inv);
 }
 
 // kFull: the ring is three stages of 128-key tiles (then the geometry is known at compile time).
-template <int kVar, bool kFull>
+// kSep: the tree's K/V rows are in buffers of their own; its keys then start a tile of their own
+// (the prefix's last tile is cut at the prefix length) and tm_nk / tm_nv describe those buffers.
+template <int kVar, bool kFull, int kHD, bool kSep>
 __global__ void __launch_bounds__(Var<kVar>::kThreads, 1)
 tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                      const __grid_constant__ CUtensorMap tm_nk, const __grid_constant__ CUtensorMap tm_nv,
@@ -350,8 +385,12 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
   // K/V ring geometry
   const int BK = kFull ? kBKMax : p.tile_keys, kStages = kFull ? 3 : p.n_stages;
   const uint32_t kHalfTile = static_cast<uint32_t>(BK) * 128u;   // one 64-column half of a K or V tile
-  const uint32_t kTileBytes = 2u * kHalfTile, kStageBytes = 2u * kTileBytes;
-  const uint32_t off_q = 0, off_kv = static_cast<uint32_t>(p.n_rows) * 256u, off_mrg = p.off_mrg, off_stage = 0;
+  using SG = Stage<kHD>;
+  constexpr uint32_t kHalves = SG::kHalves;
+  const uint32_t kStageBytes = SG::halves(VT::kNMax) * kHalfTile;
+  const uint32_t kOffK = SG::k_first() ? 0u : kHalves * kHalfTile;               // within a stage
+  const uint32_t kOffV = SG::k_first() ? SG::k_halves(VT::kNMax) * kHalfTile : 0u;
+  const uint32_t off_q = 0, off_kv = static_cast<uint32_t>(p.n_rows) * (2u * kHD), off_mrg = p.off_mrg, off_stage = 0;
   const uint32_t tmem_cols = (kVar == 0 || p.n_rows <= 64) ? 256u : 512u, col_stride = tmem_cols / 4;  // S^T(0), S^T(1), O^T
   auto bar = [&](int i) { return bars + 8u * static_cast<uint32_t>(i); };
 
@@ -388,21 +427,33 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
 
   // Geometry of this CTA's share, from the sequence's node range and prefix length.
   int node_base = 0, T_real = 0, L_raw = 0;
-  int T = 0, rows_total, n_valid = 0, L = 0, Lc = 0, S_valid = 0, tile_begin, tile_end = 0, n_my = 0, key_begin = 0;
+  int T = 0, rows_total, n_valid = 0, L = 0, Lc = 0, S_valid = 0, tile_begin = 0, tile_end = 0, n_my = 0, key_begin = 0;
+  int n_pre = 0;  // kSep: tiles that hold prefix keys
   auto geometry = [&]() {
     T = min(T_real, FALCON_T_MAX);
     rows_total = T * G;
     n_valid = min(N, rows_total - mtile * N);
     L = max(L_raw, 0);
     Lc = min(L, p.s_cap);
-    S_valid = min(L + T, p.s_cap);  // keys that exist below the cache capacity
+    S_valid = kSep ? Lc + T : min(L + T, p.s_cap);  // keys that exist (in the cache: below its capacity)
     // Whole tiles per split, boundaries rounded up: a longer run goes to an early split; the last
     // one has the tree's tiles and the longest set-up (the tree's visibility sets).
-    const int n_tiles = (S_valid + BK - 1) / BK;
+    if (kSep) n_pre = (Lc + BK - 1) / BK;
+    const int n_tiles = kSep ? n_pre + (T + BK - 1) / BK : (S_valid + BK - 1) / BK;
     tile_begin = (split * n_tiles + n_splits - 1) / n_splits;
     tile_end = ((split + 1) * n_tiles + n_splits - 1) / n_splits;
     n_my = tile_end - tile_begin;
     key_begin = tile_begin * BK;
+  };
+  // tile j of this CTA: its first key (prefix keys 0 .. Lc-1, then the tree's) and how many keys it holds
+  auto tile_key0 = [&](int j) {
+    if (!kSep) return key_begin + j * BK;
+    const int g = tile_begin + j;
+    return g < n_pre ? g * BK : Lc + (g - n_pre) * BK;
+  };
+  auto tile_keys_in = [&](int j, int k0) {
+    const int end = kSep && tile_begin + j < n_pre ? Lc : S_valid;
+    return min(BK, end - k0);
   };
   auto device_scalars = [&]() {
     node_base = p.node_off[b];
@@ -415,16 +466,23 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
     if (j == 0 && p.stall_first) return;
     const int st = j % kStages;
     const uint32_t dst = smem_base + off_kv + st * kStageBytes;
-    mbar_expect_tx(bar(kBarKVFull + st), kStageBytes);
-    tma_load_5d_hint(dst, &tm_k, bar(kBarKVFull + st), 0, key_begin + j * BK, 0, kvh, b, kv_policy);
-    tma_load_5d_hint(dst + kTileBytes, &tm_v, bar(kBarKVFull + st), 0, key_begin + j * BK, 0, kvh, b, kv_policy);
+    mbar_expect_tx(bar(kBarKVFull + st), 2u * kHalves * kHalfTile);
+    if (kSep && tile_begin + j >= n_pre) {
+      const int row = node_base + (tile_begin + j - n_pre) * BK;
+      tma_load_5d_hint(dst + kOffK, &tm_nk, bar(kBarKVFull + st), 0, row, 0, kvh, 0, kv_policy);
+      tma_load_5d_hint(dst + kOffV, &tm_nv, bar(kBarKVFull + st), 0, row, 0, kvh, 0, kv_policy);
+      return;
+    }
+    const int k0 = tile_key0(j);
+    tma_load_5d_hint(dst + kOffK, &tm_k, bar(kBarKVFull + st), 0, k0, 0, kvh, b, kv_policy);
+    tma_load_5d_hint(dst + kOffV, &tm_v, bar(kBarKVFull + st), 0, k0, 0, kvh, b, kv_policy);
   };
-  // This thread's piece of the Q block (softmax threads): 16 head-dim columns of one or two rows.
+  // This thread's piece of the Q block (softmax threads): an eighth of the head dimension of one or two rows.
   const int st_id = tid - 32 * kWarpSm0;
   const int q_part = st_id & 7;
   auto q_piece = [&](int r) -> const __nv_bfloat16* {
     const int mg = mtile * N + r;
-    return p.q + (static_cast<int64_t>(node_base + (mg >> p.g_shift)) * p.Hq + kvh * G + (mg & (G - 1))) * kD + q_part * 16;
+    return p.q + (static_cast<int64_t>(node_base + (mg >> p.g_shift)) * p.Hq + kvh * G + (mg & (G - 1))) * kHD + q_part * (kHD / 8);
   };
   if (p.have_host) {  // the caller's host copies of the per-sequence scalars: no round trip to global memory
     node_base = p.h_node_off[b];
@@ -439,7 +497,8 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
   // where it must: the softmax warps at once, because the loads everything waits for (Q, the
   // reference key, the tree) are theirs and their set-up can run under those loads; the producer
   // and the MMA warp after set-up that touches no global memory.
-  uint4 qreg[VT::kQPasses][2], kref[2];
+  constexpr int kQV = kHalves;  // 16-byte pieces
+  uint4 qreg[VT::kQPasses][kQV], kref[kQV];
   int par_raw = -1;
   int n_early = 0;  // K/V tiles requested before the producer's wait
   if (warp >= kWarpSm0) {
@@ -452,16 +511,17 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
 #pragma unroll
       for (int pass = 0; pass < VT::kQPasses; ++pass) {
         const int r = (st_id >> 3) + VT::kRowsPerPass * pass;
-        qreg[pass][0] = qreg[pass][1] = make_uint4(0u, 0u, 0u, 0u);
-        if (r < n_valid) {
-          qreg[pass][0] = reinterpret_cast<const uint4*>(q_piece(r))[0];
-          qreg[pass][1] = reinterpret_cast<const uint4*>(q_piece(r))[1];
+#pragma unroll
+        for (int i = 0; i < kQV; ++i) {
+          qreg[pass][i] = make_uint4(0u, 0u, 0u, 0u);
+          if (r < n_valid) qreg[pass][i] = reinterpret_cast<const uint4*>(q_piece(r))[i];
         }
       }
-      const __nv_bfloat16* k0p = p.k + b * p.kv_stride_b + kvh * p.kv_stride_h + q_part * 16;
-      kref[0] = reinterpret_cast<const uint4*>(k0p)[0];
-      kref[1] = reinterpret_cast<const uint4*>(k0p)[1];
-      const bool tree_here = tile_end * BK > Lc || (split == 0 && kvh == 0);
+      const __nv_bfloat16* k0p = (kSep && Lc == 0) ? p.k_tree + (static_cast<int64_t>(node_base) * p.Hkv + kvh) * kHD
+                                                   : p.k + b * p.kv_stride_b + kvh * p.kv_stride_h;
+#pragma unroll
+      for (int i = 0; i < kQV; ++i) kref[i] = reinterpret_cast<const uint4*>(k0p + q_part * (kHD / 8))[i];
+      const bool tree_here = (kSep ? tile_end > n_pre : tile_end * BK > Lc) || (split == 0 && kvh == 0);
       if (tree_here && !p.tree_mask && st_id < T) par_raw = p.parent[node_base + st_id];
     }
     for (int i = st_id; i < 128 * static_cast<int>(C::kDescWords); i += kSmThreads) s_desc[i] = 0u;
@@ -474,7 +534,7 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
       // one in the stream started) may be requested while that kernel is still finishing.
       // (One tile: more would only delay the Q block, which queues behind them in the memory system.)
       const int n_ask = min(n_my, kEarlyTiles);
-      for (int j = 0; j < n_ask && key_begin + (j + 1) * BK <= Lc; ++j) {
+      for (int j = 0; j < n_ask && tile_key0(j) + BK <= Lc; ++j) {
         load_tile(j);
         ++n_early;
       }
@@ -503,21 +563,21 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
     }
     return;
   }
-  const bool has_tree_keys = tile_end * BK > Lc;
+  const bool has_tree_keys = kSep ? tile_end > n_pre : tile_end * BK > Lc;
   const bool need_tree = has_tree_keys || (split == 0 && kvh == 0);  // the latter reports malformed trees
 
   // merge geometry: CTA `rank` owns head-dim rows [rank * d_per, ...) of the unit's result
   const uint32_t pitch = part_pitch(N);
-  const int d_per = (kD + n_splits - 1) / n_splits;
+  const int d_per = (kHD + n_splits - 1) / n_splits;
   const int d0 = split * d_per;
-  const int d_mine = max(0, min(kD, d0 + d_per) - d0);
+  const int d_mine = max(0, min(kHD, d0 + d_per) - d0);
   const uint32_t slot_bytes = static_cast<uint32_t>(d_per + 2) * pitch;
 
   if (warp == kWarpProducer && lane == 0) {
     // every split (this one included) delivers its share of this CTA's head-dim rows and the row sums
     mbar_expect_tx(bar(kBarMrg), static_cast<uint32_t>(n_splits * (d_mine + 2) * N * 2));
     for (int j = n_early; j < min(n_my, kStages); ++j) load_tile(j);
-    if (split == 0 && mtile == 0 && kvh == 0 && (L + T > p.s_cap || T_real > FALCON_T_MAX))
+    if (split == 0 && mtile == 0 && kvh == 0 && (L + (kSep ? 0 : T) > p.s_cap || T_real > FALCON_T_MAX))
       dev_status_or(p.status, b, FALCON_DEV_CAPACITY);
     FALCON_TRACE(true, 3);
   }
@@ -547,7 +607,7 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
         for (int j = max(0, issued - kStages); j < issued; ++j)
           if (!(j == 0 && p.stall_first)) mbar_wait_drain(bar(kBarKVFull + j % kStages), (j / kStages) & 1);
       }
-      if (p.prefetch_next && ok && n_my > 0 && n_my <= kStages) {
+      if (!kSep && p.prefetch_next && ok && n_my > 0 && n_my <= kStages) {
         // The caller named the caches of the next call.  Where a CTA's whole key range fits the ring
         // (short prefixes: the loads are over early and memory idles during the rest of the
         // launch), once its last tile has landed it asks for the same tiles of those caches, as far
@@ -574,10 +634,10 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
         if (!mbar_wait_warp(bar(kBarKVFull + st), (j / kStages) & 1, abort_flag)) return false;
         FALCON_TRACE(elected && j < 4, 10 + 4 * j);
         tc_fence_after();
-        const uint32_t kbase = smem_base + off_kv + st * kStageBytes;
+        const uint32_t kbase = smem_base + off_kv + st * kStageBytes + kOffK;
         if (elected) {
 #pragma unroll
-          for (int kk = 0; kk < kD / 16; ++kk) {
+          for (int kk = 0; kk < kHD / 16; ++kk) {
             // K tile (A) and Q block (B): K-major, 16 head-dim columns = 32 bytes inside the 128-byte swizzle row
             const uint64_t ad = smem_desc(kbase + (kk >> 2) * kHalfTile + (kk & 3) * 32, 16, 1024);
             const uint64_t bd = smem_desc(smem_base + off_q + (kk >> 2) * q_half_bytes + (kk & 3) * 32, 16, 1024);
@@ -591,10 +651,10 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
       };
       auto issue_pv = [&](int t) {
         const int st = t % kStages;
-        const uint32_t pbase = smem_base + off_kv + st * kStageBytes;   // P^T lies over the K tile
-        const uint32_t vbase = pbase + kTileBytes;
+        const uint32_t pbase = smem_base + off_kv + st * kStageBytes + kOffK;   // P^T lies over the K tile
+        const uint32_t vbase = smem_base + off_kv + st * kStageBytes + kOffV;
         // keys of the tile that exist, in MMA steps of 16 (rows above them hold zeros in P^T and V)
-        const int nk = (min(BK, S_valid - (key_begin + t * BK)) + 15) >> 4;
+        const int nk = (tile_keys_in(t, tile_key0(t)) + 15) >> 4;
         if (elected) {
           for (int kk = 0; kk < nk; ++kk) {
             // V^T (A) and P^T (B): both with the M / N index contiguous; 16 keys = 2 KB, the 64-column
@@ -640,30 +700,31 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
       for (int pass = 0; pass < VT::kQPasses; ++pass) {
         const int r = (st_id >> 3) + VT::kRowsPerPass * pass;
         if (r < N) {
-          unsigned char* qrow = smem_gen + off_q + (q_part >> 2) * q_half_bytes + r * 128;
-          const int u0 = 2 * (q_part & 3);
-          *reinterpret_cast<uint4*>(qrow + ((u0 ^ (r & 7)) << 4)) = qreg[pass][0];
-          *reinterpret_cast<uint4*>(qrow + (((u0 + 1) ^ (r & 7)) << 4)) = qreg[pass][1];
+          const int u_all = kQV * q_part;  // 16-byte unit of the row; 8 units are a 64-column half
+          unsigned char* qrow = smem_gen + off_q + (u_all >> 3) * q_half_bytes + r * 128;
+#pragma unroll
+          for (int i = 0; i < kQV; ++i) *reinterpret_cast<uint4*>(qrow + ((((u_all & 7) + i) ^ (r & 7)) << 4)) = qreg[pass][i];
         }
       }
       fence_async_smem();  // the MMA reads Q through the async proxy
       __syncwarp();
       if (lane == 0) mbar_arrive(bar(kBarQ));
       FALCON_TRACE(tid == 64, 9);
-      // the reference of every query row: its scaled score against cache row 0 (8 threads per row,
-      // 16 columns each)
-      const uint32_t kw[8] = {kref[0].x, kref[0].y, kref[0].z, kref[0].w, kref[1].x, kref[1].y, kref[1].z, kref[1].w};
+      // the reference of every query row: its scaled score against cache row 0 (8 threads per row)
 #pragma unroll
       for (int pass = 0; pass < VT::kQPasses; ++pass) {
         const int r = (st_id >> 3) + VT::kRowsPerPass * pass;
         if (r < N) {
-          const uint32_t qw[8] = {qreg[pass][0].x, qreg[pass][0].y, qreg[pass][0].z, qreg[pass][0].w,
-                                  qreg[pass][1].x, qreg[pass][1].y, qreg[pass][1].z, qreg[pass][1].w};
           float d = 0.f;
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            d = fmaf(bf16lo(qw[i]), bf16lo(kw[i]), d);
-            d = fmaf(bf16hi(qw[i]), bf16hi(kw[i]), d);
+          for (int i = 0; i < kQV; ++i) {
+            const uint32_t qw[4] = {qreg[pass][i].x, qreg[pass][i].y, qreg[pass][i].z, qreg[pass][i].w};
+            const uint32_t kw[4] = {kref[i].x, kref[i].y, kref[i].z, kref[i].w};
+#pragma unroll
+            for (int w = 0; w < 4; ++w) {
+              d = fmaf(bf16lo(qw[w]), bf16lo(kw[w]), d);
+              d = fmaf(bf16hi(qw[w]), bf16hi(kw[w]), d);
+            }
           }
           d += __shfl_xor_sync(0xffffffffu, d, 1);
           d += __shfl_xor_sync(0xffffffffu, d, 2);
@@ -732,7 +793,7 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
 
     for (int j = 0; live && j < n_my; ++j) {
       const int sb = j & 1, st = j % kStages;
-      const int k0 = key_begin + j * BK, key = k0 + kr;
+      const int k0 = tile_key0(j), key = k0 + kr, nv = tile_keys_in(j, k0);
       if (!mbar_wait_warp(bar(kBarSFull + sb), (j >> 1) & 1, abort_flag)) { live = false; break; }
       FALCON_TRACE(tid == 64 && j < 4, 32 + 3 * j);
       tc_fence_after();
@@ -750,18 +811,18 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
 
       // all of this warp's keys lie in the prefix: every one exists and is visible to every row
       const bool full = k0 + BK <= Lc && q4 * 32 + 32 <= BK;
-      unsigned char* ptile = smem_gen + off_kv + st * kStageBytes;
-      if (!full && k0 + BK > S_valid && grp == 0) {
-        // The sequence's last tile: V rows past the last key may hold anything (0 x NaN = NaN in the
+      unsigned char* ptile = smem_gen + off_kv + st * kStageBytes + kOffK;
+      unsigned char* vtile = smem_gen + off_kv + st * kStageBytes + kOffV;
+      if (!full && nv < BK && grp == 0) {
+        // The sequence's last tile (or the prefix's, before a tree kept elsewhere): V rows past the last key may hold anything (0 x NaN = NaN in the
         // MMA).  The rows up to the next multiple of 16 are read by the last MMA step: clear them.
         if (!mbar_wait_warp(bar(kBarKVFull + st), (j / kStages) & 1, abort_flag)) { live = false; break; }
-        const int nv = S_valid - k0;
         if (kr >= nv && kr < ((nv + 15) & ~15)) {
 #pragma unroll
-          for (int h = 0; h < 2; ++h)
+          for (int h = 0; h < static_cast<int>(kHalves); ++h)
 #pragma unroll
             for (int u = 0; u < 8; ++u)
-              *reinterpret_cast<uint4*>(ptile + kTileBytes + h * kHalfTile + kr * 128 + u * 16) = make_uint4(0, 0, 0, 0);
+              *reinterpret_cast<uint4*>(vtile + h * kHalfTile + kr * 128 + u * 16) = make_uint4(0, 0, 0, 0);
         }
       }
 #pragma unroll
@@ -770,7 +831,7 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
         if (ch < n_chunks) {
           uint32_t vis = (1u << kCW) - 1u;
           if (!full) {
-            if (key >= S_valid || kr >= BK) vis = 0u;
+            if (kr >= nv) vis = 0u;
             else if (key >= Lc) vis &= s_desc[(key - Lc) * C::kDescWords + ((ch * kCW) >> 5)] >> ((ch * kCW) & 31);
           }
           constexpr int kSel = kRefInRegs ? 1 : 0;
@@ -881,12 +942,13 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
     if (st_id * 4 < N)
       st_async_v4(slot_addr(split) + static_cast<uint32_t>(d_per) * pitch + st_id * 16, own_l[0], own_l[1], own_l[2], own_l[3],
                   map_to_rank(bar(kBarMrg), static_cast<uint32_t>(split)));
-    const uint32_t row_dst = slot_addr(o_me) + static_cast<uint32_t>(dl_me) * pitch;
-    const uint32_t row_bar = map_to_rank(bar(kBarMrg), static_cast<uint32_t>(o_me));
+    const bool o_lane = kHD == 128 || kr < kHD;  // this lane holds a head-dim row (whole warps do or do not)
+    const uint32_t row_dst = slot_addr(o_lane ? o_me : split) + static_cast<uint32_t>(dl_me) * pitch;
+    const uint32_t row_bar = map_to_rank(bar(kBarMrg), static_cast<uint32_t>(o_lane ? o_me : split));
 #pragma unroll
     for (int ci = 0; ci < kPer; ++ci) {
       const int ch = grp + kColGroups * ci;
-      if (ch < n_chunks) {
+      if (o_lane && ch < n_chunks) {
         uint32_t o[kCW];
 #pragma unroll
         for (int c = 0; c < kCW; ++c) o[c] = have ? 0x7fc00000u : 0u;
@@ -922,7 +984,7 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
   // timing), normalised and stored.  An item is one head-dim row and 4 query rows; consecutive
   // threads take consecutive head-dim rows (adjacent bf16 in `out`).  A row whose sum is too far
   // from the reference's scale (or not finite) is left to the exact path below.
-  __nv_bfloat16* out_base = p.out + (static_cast<int64_t>(node_base) * p.Hq + kvh * G) * kD + d0;
+  __nv_bfloat16* out_base = p.out + (static_cast<int64_t>(node_base) * p.Hq + kvh * G) * kHD + d0;
   const int n_q4 = (n_valid + 3) >> 2;
   FALCON_TRACE(tid == 0, 56);
   for (int item = tid; item < d_mine * n_q4; item += kThreads) {
@@ -948,7 +1010,7 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
       if (r < n_valid) {
         if (got && ls[c] >= kLMin && ls[c] <= kLMax && acc[c] == acc[c]) {
           const int mg = mtile * N + r;
-          out_base[((mg >> p.g_shift) * p.Hq + (mg & (G - 1))) * kD + dl] = __float2bfloat16_rn(__fdividef(acc[c], ls[c]));
+          out_base[((mg >> p.g_shift) * p.Hq + (mg & (G - 1))) * kHD + dl] = __float2bfloat16_rn(__fdividef(acc[c], ls[c]));
         } else if (dl == 0) {
           s_rescue[r] = 1;
         }
@@ -959,7 +1021,7 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
   __syncthreads();
   // exact path for the rows that need it, shared out over the cluster's CTAs and this CTA's warps
   for (int r = split + n_splits * warp; r < n_valid; r += n_splits * (kThreads / 32))
-    if (s_rescue[r]) rescue_row(p, b, kvh, node_base, T, Lc, S_valid, mtile * N + r, lane);
+    if (s_rescue[r]) rescue_row<kHD>(p, b, kvh, node_base, T, Lc, S_valid, mtile * N + r, lane);
   FALCON_TRACE(tid == 0, 54);
   if (warp == kWarpMma) {
     // (after a wait that gave up, MMAs may still be running: the last commit covers them all)
@@ -971,6 +1033,7 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
 
 bool is_pow2(int x) { return x > 0 && (x & (x - 1)) == 0; }
 
+// (every instantiation of a variant has the same footprint: one CTA per SM)
 template <int kVar>
 int pick_splits(falcon_ctx* ctx, int units, int max_tiles) {
   int* resident = ctx->attn_resident[1 + kVar];
@@ -990,7 +1053,7 @@ int pick_splits(falcon_ctx* ctx, int units, int max_tiles) {
       cfg.attrs = &attr;
       cfg.numAttrs = 1;
       int n = 0;
-      if (cudaOccupancyMaxActiveClusters(&n, tree_attn_tck_kernel<kVar, true>, &cfg) != cudaSuccess) n = -1;
+      if (cudaOccupancyMaxActiveClusters(&n, tree_attn_tck_kernel<kVar, true, 128, false>, &cfg) != cudaSuccess) n = -1;
       resident[s] = n > 0 ? n : -1;
       cudaGetLastError();
     }
@@ -999,7 +1062,7 @@ int pick_splits(falcon_ctx* ctx, int units, int max_tiles) {
   return best;
 }
 
-template <int kVar>
+template <int kVar, int kHD, bool kSep>
 int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s, int q_nodes) {
   using C = Cfg<Var<kVar>::kCfg>;
   const int B = a.tree.batch, Hq = a.n_q_heads, Hkv = a.n_kv_heads, G = Hq / Hkv;
@@ -1007,17 +1070,23 @@ int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s, int 
   const int n_units = (a.tree.max_tree + q_nodes - 1) / q_nodes;
   if (static_cast<int64_t>(Hkv) * n_units > 65535) return FALCON_ERR_CAPACITY;
 
-  bool& attr_set = ctx->attn_attr_set[1 + kVar];
+  // 64-wide heads: three stages of 128 keys always fit
+  constexpr bool kMayBeLow = kHD == 128;
+  bool& attr_set = ctx->attn_attr_set[1 + 4 * kVar + 2 * (kHD == 64) + kSep];
   if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(tree_attn_tck_kernel<kVar, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(kSmemMax));
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(tree_attn_tck_kernel<kVar, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(tree_attn_tck_kernel<kVar, true, kHD, kSep>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSmemMax));
+    if (e == cudaSuccess && !(kHD == 128 && !kSep))  // (the occupancy query below is made with this one)
+      e = cudaFuncSetAttribute(tree_attn_tck_kernel<kVar, true, 128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                static_cast<int>(kSmemMax));
+    if (e == cudaSuccess && kMayBeLow)
+      e = cudaFuncSetAttribute(tree_attn_tck_kernel<kVar, !kMayBeLow, kHD, kSep>,
+                               cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSmemMax));
     if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute(tree_attn_tck_kernel)");
     attr_set = true;
   }
-  const int max_tiles = (a.tree.max_prefix_len + a.tree.max_tree + kBKMax - 1) / kBKMax;
+  const int max_tiles = kSep ? (a.tree.max_prefix_len + kBKMax - 1) / kBKMax + 1
+                             : (a.tree.max_prefix_len + a.tree.max_tree + kBKMax - 1) / kBKMax;
   int splits = a.n_splits;
   if (splits == 0) splits = pick_splits<kVar>(ctx, Hkv * n_units * B, max_tiles > 0 ? max_tiles : 1);
   if (splits < 1) splits = 1;
@@ -1025,39 +1094,50 @@ int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s, int 
   // sums) and the small arrays are fixed by the shape; the K/V ring takes the rest, as three stages
   // of the highest tile that fits (two if three would be lower than 64 keys).  A split count whose
   // merge area would leave less than two 64-key stages is reduced.
-  const uint32_t q_bytes = static_cast<uint32_t>(N) * 256u;
+  const uint32_t q_bytes = static_cast<uint32_t>(N) * 2u * kHD;
+  const int row_bytes = static_cast<int>(Stage<kHD>::halves(Var<kVar>::kNMax)) * 128;  // of the ring, per key
   auto merge_bytes = [&](int ns) {
-    return ns > 1 ? static_cast<uint32_t>(ns - 1) * ((kD + ns - 1) / ns + 2) * part_pitch(N) : 0u;
+    return ns > 1 ? static_cast<uint32_t>(ns - 1) * ((kHD + ns - 1) / ns + 2) * part_pitch(N) : 0u;
   };
   auto ring_room = [&](int ns) { return static_cast<int>(kSmemMax) - static_cast<int>(q_bytes + merge_bytes(ns) + C::kSmallBytes); };
-  while (splits > 1 && ring_room(splits) < 2 * 64 * 512) --splits;
+  while (splits > 1 && ring_room(splits) < 2 * 64 * row_bytes) --splits;
   const int room = ring_room(splits);
-  int n_stages = 3, tile_keys = room / (3 * 512) / 16 * 16;
+  int n_stages = 3, tile_keys = room / (3 * row_bytes) / 16 * 16;
   if (tile_keys < 64) {
     n_stages = 2;
-    tile_keys = room / (2 * 512) / 16 * 16;
+    tile_keys = room / (2 * row_bytes) / 16 * 16;
   }
   if (tile_keys > kBKMax) tile_keys = kBKMax;
-  const uint32_t off_mrg = q_bytes + static_cast<uint32_t>(n_stages * tile_keys) * 512u;
+  const uint32_t off_mrg = q_bytes + static_cast<uint32_t>(n_stages * tile_keys * row_bytes);
   const uint32_t off_small = off_mrg + merge_bytes(splits);
   const uint32_t smem_bytes = off_small + C::kSmallBytes;
 
   // Tensor maps.  The head dimension is split into (64 columns, 2 halves) so that one box covers both
   // 128-byte-swizzled half tiles.  K/V cache: [64, s_cap, 2, Hkv, B], box 64 x tile_keys x 2.
-  uint64_t kv_dims[5] = {64, static_cast<uint64_t>(a.s_cap), 2, static_cast<uint64_t>(Hkv), static_cast<uint64_t>(B)};
+  uint64_t kv_dims[5] = {64, static_cast<uint64_t>(a.s_cap), Stage<kHD>::kHalves, static_cast<uint64_t>(Hkv), static_cast<uint64_t>(B)};
   uint64_t kv_strides[4] = {static_cast<uint64_t>(a.kv_stride_s) * 2, 128, static_cast<uint64_t>(a.kv_stride_h) * 2,
                             static_cast<uint64_t>(a.kv_stride_b) * 2};
   if (Hkv == 1 && kv_strides[2] == 0) kv_strides[2] = kv_strides[0] * a.s_cap;  // a size-1 dimension never strides
   if (B == 1 && kv_strides[3] == 0) kv_strides[3] = kv_strides[2] * Hkv;
-  const uint32_t kv_box[5] = {64, static_cast<uint32_t>(tile_keys), 2, 1, 1};
+  const uint32_t kv_box[5] = {64, static_cast<uint32_t>(tile_keys), Stage<kHD>::kHalves, 1, 1};
   CUtensorMap mk, mv;
   if (!get_tmap(ctx, a.k_cache, kv_dims, kv_strides, kv_box, &mk) || !get_tmap(ctx, a.v_cache, kv_dims, kv_strides, kv_box, &mv)) {
     ctx->last_error = "cuTensorMapEncodeTiled failed";
     return FALCON_ERR_CUDA;
   }
-  // the next call's caches (a prefetch hint): same geometry, only with the stable-prefix promise
+  // the next call's caches (a prefetch hint): same geometry, only with the stable-prefix promise; or,
+  // in their place, the tree's own buffers [N, Hkv, D]
   CUtensorMap mnk = mk, mnv = mv;
-  const bool prefetch_next = a.next_k_cache && a.next_v_cache && (a.flags & FALCON_ATTN_PREFIX_STABLE) &&
+  if (kSep) {
+    const uint64_t n_all = static_cast<uint64_t>(a.tree.total_nodes), row = static_cast<uint64_t>(Hkv) * kHD * 2;
+    const uint64_t t_dims[5] = {64, n_all, Stage<kHD>::kHalves, static_cast<uint64_t>(Hkv), 1};
+    const uint64_t t_strides[4] = {row, 128, static_cast<uint64_t>(kHD) * 2, row * n_all};
+    if (!get_tmap(ctx, a.k_tree, t_dims, t_strides, kv_box, &mnk) || !get_tmap(ctx, a.v_tree, t_dims, t_strides, kv_box, &mnv)) {
+      ctx->last_error = "cuTensorMapEncodeTiled failed";
+      return FALCON_ERR_CUDA;
+    }
+  }
+  const bool prefetch_next = !kSep && a.next_k_cache && a.next_v_cache && (a.flags & FALCON_ATTN_PREFIX_STABLE) &&
                              !((reinterpret_cast<uintptr_t>(a.next_k_cache) | reinterpret_cast<uintptr_t>(a.next_v_cache)) & 15) &&
                              get_tmap(ctx, a.next_k_cache, kv_dims, kv_strides, kv_box, &mnk) &&
                              get_tmap(ctx, a.next_v_cache, kv_dims, kv_strides, kv_box, &mnv);
@@ -1069,14 +1149,13 @@ int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s, int 
   p.g_shift = 0;
   while ((1 << p.g_shift) < G) ++p.g_shift;
   p.s_cap = a.s_cap;
-  p.total_nodes = a.tree.total_nodes;
   p.n_rows = N;
   p.tile_keys = tile_keys;
   p.n_stages = n_stages;
   p.off_mrg = off_mrg;
   p.off_small = off_small;
   p.idesc_qk = make_idesc(128, N, false, false);
-  p.idesc_pv = make_idesc(kD, N, true, true);
+  p.idesc_pv = make_idesc(128, N, true, true);
   p.scale_log2 = a.sm_scale * kLog2e;
   p.node_off = a.tree.node_off;
   p.parent = a.tree.parent;
@@ -1086,6 +1165,8 @@ int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s, int 
   p.q = static_cast<const __nv_bfloat16*>(a.q);
   p.k = static_cast<const __nv_bfloat16*>(a.k_cache);
   p.v = static_cast<const __nv_bfloat16*>(a.v_cache);
+  p.k_tree = static_cast<const __nv_bfloat16*>(a.k_tree);
+  p.v_tree = static_cast<const __nv_bfloat16*>(a.v_tree);
   p.kv_stride_b = a.kv_stride_b;
   p.kv_stride_h = a.kv_stride_h;
   p.kv_stride_s = a.kv_stride_s;
@@ -1121,8 +1202,8 @@ int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s, int 
   cfg.attrs = attr;
   cfg.numAttrs = 2;
   cudaError_t e = (tile_keys == kBKMax && n_stages == 3)
-                      ? cudaLaunchKernelEx(&cfg, tree_attn_tck_kernel<kVar, true>, mk, mv, mnk, mnv, p)
-                      : cudaLaunchKernelEx(&cfg, tree_attn_tck_kernel<kVar, false>, mk, mv, mnk, mnv, p);
+                      ? cudaLaunchKernelEx(&cfg, tree_attn_tck_kernel<kVar, true, kHD, kSep>, mk, mv, mnk, mnv, p)
+                      : cudaLaunchKernelEx(&cfg, tree_attn_tck_kernel<kVar, !kMayBeLow, kHD, kSep>, mk, mv, mnk, mnv, p);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "tree_attn_tck_kernel launch");
   return FALCON_OK;
 }
@@ -1131,8 +1212,7 @@ int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s, int 
 
 bool tree_attn_tck_supports(const falcon_ctx* ctx, const falcon_attn_args& a) {
   (void)ctx;
-  if (a.head_dim != kD) return false;
-  if (a.k_tree != nullptr) return false;
+  if (a.head_dim != 64 && a.head_dim != 128) return false;
   const int G = a.n_q_heads / a.n_kv_heads;
   if (!is_pow2(G) || G > 128) return false;
   if (a.n_splits > kMaxSplits) return false;
@@ -1161,12 +1241,21 @@ bool tree_attn_tck_preferred(const falcon_ctx* ctx, const falcon_attn_args& a) {
   return q_nodes * G <= 64 || units >= ctx->sm_count;
 }
 
+namespace {
+template <int kVar>
+int launch_variant(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s, int q_nodes) {
+  if (a.head_dim == 128)
+    return a.k_tree ? launch_impl<kVar, 128, true>(ctx, a, s, q_nodes) : launch_impl<kVar, 128, false>(ctx, a, s, q_nodes);
+  return a.k_tree ? launch_impl<kVar, 64, true>(ctx, a, s, q_nodes) : launch_impl<kVar, 64, false>(ctx, a, s, q_nodes);
+}
+}  // namespace
+
 int launch_tree_attn_tck(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s) {
-  const int G = a.n_q_heads / a.n_kv_heads, q_nodes = nodes_per_unit(a);
-  const int rows = q_nodes * G;
-  if (rows <= 64) return launch_impl<0>(ctx, a, s, q_nodes);
-  if (rows <= 80) return launch_impl<1>(ctx, a, s, q_nodes);
-  return launch_impl<2>(ctx, a, s, q_nodes);
+  const int q_nodes = nodes_per_unit(a);
+  const int rows = q_nodes * (a.n_q_heads / a.n_kv_heads);
+  if (rows <= 64) return launch_variant<0>(ctx, a, s, q_nodes);
+  if (rows <= 80) return launch_variant<1>(ctx, a, s, q_nodes);
+  return launch_variant<2>(ctx, a, s, q_nodes);
 }
 
 }  // namespace falcon

@@ -504,6 +504,36 @@ def test_attn_tc_row_arrangements(T, G, L, splits, tck):
     H.assert_attn_close(out, ref, tb.node_off)
 
 
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("separate", [False, True])
+@pytest.mark.parametrize("T,G,L,splits", [(1, 1, 0, 1), (60, 1, 0, 1), (60, 1, 1024, 4), (33, 1, 127, 2), (80, 1, 129, 1), (64, 2, 256, 3),
+                                           (128, 1, 250, 8), (17, 8, 640, 0), (72, 4, 1, 1)])
+def test_attn_tck_head_sizes_and_separate_tree_buffers(T, G, L, splits, separate, D):
+    """The keys-on-lanes kernel with 64- and 128-wide heads and with the tree's K/V in buffers of its own (whose keys
+    start a tile of their own), two sequences of different sizes; what lies past the prefix in the cache is NaN then."""
+    rng = np.random.default_rng(1000 * T + 10 * G + splits + D)
+    Hkv = 2
+    sizes, prefs = [T, max(1, T // 3)], [L, L // 2]
+    tb, q, k, v = random_case(rng, sizes, prefs, Hkv * G, Hkv, D, slack=1)
+    ref = oracle_attn(tb, Hkv * G, Hkv, D, q, k, v)
+    kw = {}
+    if separate:
+        kt = np.empty((tb.total_nodes, Hkv, D), np.uint16)
+        vt = np.empty_like(kt)
+        for b in range(2):
+            Lb, Tb, o = prefs[b], sizes[b], tb.node_off[b]
+            kt[o:o + Tb] = k[b, :, Lb:Lb + Tb].transpose(1, 0, 2)
+            vt[o:o + Tb] = v[b, :, Lb:Lb + Tb].transpose(1, 0, 2)
+            k[b, :, Lb:] = 0x7FC0
+            v[b, :, Lb:] = 0x7FC0
+        kw = dict(k_tree=kt, v_tree=vt)
+    for hc in (False, True):
+        dt = H.DevTrees(tb)
+        out, rc = H.run_attn(dt, Hkv * G, Hkv, D, q, k, v, kernel=binding.ATTN_TCK, n_splits=splits, host_copies=hc, **kw)
+        H.assert_attn_close(out, ref, tb.node_off)
+        assert not dt.status.cpu().numpy().any()
+
+
 @pytest.mark.parametrize("tck", TC_KERNELS)
 @pytest.mark.parametrize("T,G,L,splits", [(60, 1, 1024, 0), (60, 1, 700, 4), (80, 1, 500, 3), (16, 8, 1000, 5),
                                            (20, 1, 10, 2), (33, 2, 0, 1)])
