@@ -120,9 +120,8 @@ typedef struct {
  *             per query row (at most 1024 keys per sequence; the small-problem kernel), _TC tensor
  *             cores with the query rows on the tensor-memory lanes, _TCK tensor cores with the
  *             keys on the lanes.
- *             The tensor-core kernels need Hq/Hkv a power of two, and _TC also head_dim 128 and
- *             the tree's K/V in the cache; a forced kernel that cannot take the shape
- *             returns FALCON_ERR_UNSUPPORTED.  _SIMT and _WARP keep the softmax weights in fp32,
+ *             The tensor-core kernels need Hq/Hkv a power of two (_TC also sm_scale > 0); a forced
+ *             kernel that cannot take the shape returns FALCON_ERR_UNSUPPORTED.  _SIMT and _WARP keep the softmax weights in fp32,
  *             the tensor-core kernels give them to the MMA as bf16.
  * n_splits    0 = automatic; else the number of KV splits per head (1..8 for
  *             the tensor-core kernels, an upper bound: _TCK lowers it when the other

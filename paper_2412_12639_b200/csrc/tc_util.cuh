@@ -66,10 +66,6 @@ __device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap* map
       "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4)
       : "memory");
 }
-// One K or V tile: 64 keys x (2 halves of 64 head-dim columns), landing as two 128-byte-swizzled half tiles.
-__device__ __forceinline__ void load_kv_tile(uint32_t dst, const CUtensorMap* map, uint32_t bar, int k0, int kvh, int b) {
-  tma_load_5d(dst, map, bar, 0, k0, 0, kvh, b);
-}
 __device__ __forceinline__ void prefetch_tmap(const CUtensorMap* map) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
 }
@@ -106,7 +102,7 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo_bytes,
 
 // Instruction descriptor of tcgen05.mma kind::f16: bf16 x bf16 -> fp32, M x N tile; an operand is
 // K-major unless its flag says that the M (or N) index is the contiguous one.
-constexpr uint32_t make_idesc(uint32_t m, uint32_t n, bool a_mn_major, bool b_mn_major) {
+__host__ __device__ constexpr uint32_t make_idesc(uint32_t m, uint32_t n, bool a_mn_major, bool b_mn_major) {
   return (1u << 4) | (1u << 7) | (1u << 10) | (a_mn_major ? (1u << 15) : 0u) | (b_mn_major ? (1u << 16) : 0u) |
          ((n >> 3) << 17) | ((m >> 4) << 24);
 }
@@ -160,25 +156,114 @@ __device__ __forceinline__ float ex2(float x) {
 // Phase-1 arrival: orders nothing itself (the barrier initialisation it announces was released to the
 // cluster by fence.mbarrier_init), so it does not wait for this thread's loads in flight.
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
-// Arrival that orders nothing: used where the barrier only keeps CTAs alive, so that it does not
-// have to wait for this thread's outstanding global stores.
-__device__ __forceinline__ void cluster_arrive_relaxed() {
-  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
-}
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// Cluster barrier that also makes what its threads wrote before visible to those that pass it.
+__device__ __forceinline__ void cluster_sync_release() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
 __device__ __forceinline__ uint32_t map_to_rank(uint32_t local_addr, uint32_t rank) {
   uint32_t r;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local_addr), "r"(rank));
   return r;
 }
-// Asynchronous copy of `bytes` (multiple of 16) from this CTA's shared memory into a cluster peer's;
-// completion is counted on the peer's mbarrier.
-__device__ __forceinline__ void bulk_copy_to_peer(uint32_t dst_cluster, uint32_t src_cta, uint32_t bytes,
-                                                  uint32_t bar_cluster) {
-  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                   dst_cluster),
-               "r"(src_cta), "r"(bytes), "r"(bar_cluster)
+// (d0, d1) = (a0, a1) * (b0, b1) + (c0, c1) in one instruction
+__device__ __forceinline__ void fma2(float a0, float a1, float b0, float b1, float c0, float c1, float& d0, float& d1) {
+  asm("{ .reg .b64 ra, rb, rc, rd; mov.b64 ra, {%2, %3}; mov.b64 rb, {%4, %5}; mov.b64 rc, {%6, %7}; "
+      "fma.rn.f32x2 rd, ra, rb, rc; mov.b64 {%0, %1}, rd; }"
+      : "=f"(d0), "=f"(d1)
+      : "f"(a0), "f"(a1), "f"(b0), "f"(b1), "f"(c0), "f"(c1));
+}
+// (x0, x1) += (y0, y1) in one instruction
+__device__ __forceinline__ void add2(float& x0, float& x1, float y0, float y1) {
+  asm("{ .reg .b64 ra, rb, rd; mov.b64 ra, {%0, %1}; mov.b64 rb, {%2, %3}; add.rn.f32x2 rd, ra, rb; mov.b64 {%0, %1}, rd; }"
+      : "+f"(x0), "+f"(x1)
+      : "f"(y0), "f"(y1));
+}
+// 16 bytes into the shared memory of a CTA of the cluster (this one included); the store counts 16
+// bytes on the mbarrier `bar`, which must live in the same CTA as the destination.
+__device__ __forceinline__ void st_async_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d, uint32_t bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(addr),
+               "r"(a), "r"(b), "r"(c), "r"(d), "r"(bar)
                : "memory");
+}
+// Bounded wait of one thread that does not look at the CTA's abort flag: for draining what is in
+// flight after another wait has given up, and for what peers deliver whatever happened.
+__device__ __forceinline__ bool mbar_wait_drain(uint32_t bar, uint32_t parity) {
+  for (uint32_t it = 0; it < (1u << 20); ++it) {
+    uint32_t ok;
+    asm volatile("{ .reg .pred p; mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
+                 : "=r"(ok)
+                 : "r"(bar), "r"(parity)
+                 : "memory");
+    if (ok) return true;
+  }
+  return false;
+}
+__device__ __forceinline__ float bf16lo(uint32_t x) { return __uint_as_float(x << 16); }
+__device__ __forceinline__ float bf16hi(uint32_t x) { return __uint_as_float(x & 0xffff0000u); }
+
+// One query row recomputed exactly by a warp from global memory (running maximum in fp32): the
+// fallback for rows whose scores lie too far from the reference for the fast path.
+// (P: the parameter struct of either tensor-core kernel.)
+template <int kHD, class P>
+__device__ __forceinline__ void rescue_row(const P& p, int b, int kvh, int node_base, int T, int Lc, int S_valid, int mg,
+                           int lane) {
+  constexpr int kW = kHD / 64;  // 32-bit words (pairs of head dimensions) per lane
+  const int node = mg >> p.g_shift, head = kvh * p.G + (mg & (p.G - 1));
+  uint64_t lo = 0, hi = 0;
+  if (p.tree_mask) {
+    lo = p.tree_mask[2 * static_cast<int64_t>(node_base + node)];
+    hi = p.tree_mask[2 * static_cast<int64_t>(node_base + node) + 1];
+  } else {
+    ancestor_mask(p.parent + node_base, T, node, lo, hi);
+  }
+  auto load = [&](const __nv_bfloat16* row, float (&x)[2 * kW]) {
+    uint32_t w[kW];
+    if constexpr (kW == 2) {
+      const uint2 t = *reinterpret_cast<const uint2*>(row + 4 * lane);
+      w[0] = t.x;
+      w[1] = t.y;
+    } else {
+      w[0] = *reinterpret_cast<const uint32_t*>(row + 2 * lane);
+    }
+#pragma unroll
+    for (int i = 0; i < kW; ++i) {
+      x[2 * i] = bf16lo(w[i]);
+      x[2 * i + 1] = bf16hi(w[i]);
+    }
+  };
+  const int64_t at = (static_cast<int64_t>(node_base + node) * p.Hq + head) * kHD;
+  float q[2 * kW], acc[2 * kW];
+  load(p.q + at, q);
+#pragma unroll
+  for (int i = 0; i < 2 * kW; ++i) acc[i] = 0.f;
+  const int64_t cache = b * p.kv_stride_b + kvh * p.kv_stride_h;
+  float m = -INFINITY, l = 0.f;
+  for (int key = 0; key < S_valid; ++key) {
+    if (key >= Lc && !bit128(lo, hi, key - Lc)) continue;
+    const bool own = p.k_tree && key >= Lc;
+    const int64_t row = own ? (static_cast<int64_t>(node_base + key - Lc) * p.Hkv + kvh) * kHD : cache + key * p.kv_stride_s;
+    float k[2 * kW], v[2 * kW];
+    load((own ? p.k_tree : p.k) + row, k);
+    float s = q[0] * k[0];
+#pragma unroll
+    for (int i = 1; i < 2 * kW; ++i) s = fmaf(q[i], k[i], s);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    s *= p.scale_log2;
+    const float mn = fmaxf(m, s);
+    const float alpha = ex2(m - mn), pw = ex2(s - mn);
+    load((own ? p.v_tree : p.v) + row, v);
+    l = fmaf(l, alpha, pw);
+#pragma unroll
+    for (int i = 0; i < 2 * kW; ++i) acc[i] = fmaf(acc[i], alpha, pw * v[i]);
+    m = mn;
+  }
+  const float inv = l > 0.f ? 1.f / l : 0.f;
+#pragma unroll
+  for (int i = 0; i < kW; ++i)
+    *reinterpret_cast<__nv_bfloat162*>(p.out + at + 2 * kW * lane + 2 * i) =
+        __floats2bfloat162_rn(acc[2 * i] * inv, acc[2 * i + 1] * inv);
 }
 
 // 64 visibility bits for tree indices off .. off+63 of a 128-bit set; negative indices (prefix keys) are visible.

@@ -190,19 +190,6 @@ __device__ __forceinline__ void prefetch_tile_l2(const CUtensorMap* map, int key
                : "memory");
 }
 
-// (d0, d1) = (a0, a1) * (b0, b1) + (c0, c1) in one instruction
-__device__ __forceinline__ void fma2(float a0, float a1, float b0, float b1, float c0, float c1, float& d0, float& d1) {
-  asm("{ .reg .b64 ra, rb, rc, rd; mov.b64 ra, {%2, %3}; mov.b64 rb, {%4, %5}; mov.b64 rc, {%6, %7}; "
-      "fma.rn.f32x2 rd, ra, rb, rc; mov.b64 {%0, %1}, rd; }"
-      : "=f"(d0), "=f"(d1)
-      : "f"(a0), "f"(a1), "f"(b0), "f"(b1), "f"(c0), "f"(c1));
-}
-// (x0, x1) += (y0, y1) in one instruction
-__device__ __forceinline__ void add2(float& x0, float& x1, float y0, float y1) {
-  asm("{ .reg .b64 ra, rb, rd; mov.b64 ra, {%0, %1}; mov.b64 rb, {%2, %3}; add.rn.f32x2 rd, ra, rb; mov.b64 {%0, %1}, rd; }"
-      : "+f"(x0), "+f"(x1)
-      : "f"(y0), "f"(y1));
-}
 template <int kW>
 __device__ __forceinline__ void tmem_ld_chunk(uint32_t taddr, uint32_t (&r)[kW]) {
   if constexpr (kW == 16) {
@@ -216,26 +203,6 @@ __device__ __forceinline__ void tmem_ld_chunk(uint32_t taddr, uint32_t (&r)[kW])
   }
 }
 
-// 16 bytes into the shared memory of a CTA of the cluster (this one included); the store counts 16
-// bytes on the mbarrier `bar`, which must live in the same CTA as the destination.
-__device__ __forceinline__ void st_async_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d, uint32_t bar) {
-  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(addr),
-               "r"(a), "r"(b), "r"(c), "r"(d), "r"(bar)
-               : "memory");
-}
-// Bounded wait of one thread that does not look at the CTA's abort flag: for draining what is in
-// flight after another wait has given up.
-__device__ __forceinline__ bool mbar_wait_drain(uint32_t bar, uint32_t parity) {
-  for (uint32_t it = 0; it < (1u << 20); ++it) {
-    uint32_t ok;
-    asm volatile("{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
-                 : "=r"(ok)
-                 : "r"(bar), "r"(parity)
-                 : "memory");
-    if (ok) return true;
-  }
-  return false;
-}
 // Bounded wait with cluster-scope acquire, for a whole warp.
 __device__ __forceinline__ bool mbar_wait_cluster_warp(uint32_t bar, uint32_t parity) {
   bool done = false;
@@ -293,72 +260,6 @@ __device__ __forceinline__ float warp_col_sums(const float (&v)[kW], int lane) {
 template <int kW>
 __device__ __forceinline__ int col_of_lane(int lane) {
   return (kW == 16 ? ((lane >> 4) & 1) * 8 : 0) + ((lane >> 3) & 1) * 4 + ((lane >> 2) & 1) * 2 + ((lane >> 1) & 1);
-}
-
-__device__ __forceinline__ float bf16lo(uint32_t x) { return __uint_as_float(x << 16); }
-__device__ __forceinline__ float bf16hi(uint32_t x) { return __uint_as_float(x & 0xffff0000u); }
-
-// One query row recomputed exactly by a warp from global memory (running maximum in fp32): the
-// fallback for rows whose scores lie too far from the reference for the fast path.
-template <int kHD>
-__device__ void rescue_row(const TckParams& p, int b, int kvh, int node_base, int T, int Lc, int S_valid, int mg,
-                           int lane) {
-  constexpr int kW = kHD / 64;  // 32-bit words (pairs of head dimensions) per lane
-  const int node = mg >> p.g_shift, head = kvh * p.G + (mg & (p.G - 1));
-  uint64_t lo = 0, hi = 0;
-  if (p.tree_mask) {
-    lo = p.tree_mask[2 * static_cast<int64_t>(node_base + node)];
-    hi = p.tree_mask[2 * static_cast<int64_t>(node_base + node) + 1];
-  } else {
-    ancestor_mask(p.parent + node_base, T, node, lo, hi);
-  }
-  auto load = [&](const __nv_bfloat16* row, float (&x)[2 * kW]) {
-    uint32_t w[kW];
-    if constexpr (kW == 2) {
-      const uint2 t = *reinterpret_cast<const uint2*>(row + 4 * lane);
-      w[0] = t.x;
-      w[1] = t.y;
-    } else {
-      w[0] = *reinterpret_cast<const uint32_t*>(row + 2 * lane);
-    }
-#pragma unroll
-    for (int i = 0; i < kW; ++i) {
-      x[2 * i] = bf16lo(w[i]);
-      x[2 * i + 1] = bf16hi(w[i]);
-    }
-  };
-  const int64_t at = (static_cast<int64_t>(node_base + node) * p.Hq + head) * kHD;
-  float q[2 * kW], acc[2 * kW];
-  load(p.q + at, q);
-#pragma unroll
-  for (int i = 0; i < 2 * kW; ++i) acc[i] = 0.f;
-  const int64_t cache = b * p.kv_stride_b + kvh * p.kv_stride_h;
-  float m = -INFINITY, l = 0.f;
-  for (int key = 0; key < S_valid; ++key) {
-    if (key >= Lc && !bit128(lo, hi, key - Lc)) continue;
-    const bool own = p.k_tree && key >= Lc;
-    const int64_t row = own ? (static_cast<int64_t>(node_base + key - Lc) * p.Hkv + kvh) * kHD : cache + key * p.kv_stride_s;
-    float k[2 * kW], v[2 * kW];
-    load((own ? p.k_tree : p.k) + row, k);
-    float s = q[0] * k[0];
-#pragma unroll
-    for (int i = 1; i < 2 * kW; ++i) s = fmaf(q[i], k[i], s);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    s *= p.scale_log2;
-    const float mn = fmaxf(m, s);
-    const float alpha = ex2(m - mn), pw = ex2(s - mn);
-    load((own ? p.v_tree : p.v) + row, v);
-    l = fmaf(l, alpha, pw);
-#pragma unroll
-    for (int i = 0; i < 2 * kW; ++i) acc[i] = fmaf(acc[i], alpha, pw * v[i]);
-    m = mn;
-  }
-  const float inv = l > 0.f ? 1.f / l : 0.f;
-#pragma unroll
-  for (int i = 0; i < kW; ++i)
-    *reinterpret_cast<__nv_bfloat162*>(p.out + at + 2 * kW * lane + 2 * i) =
-        __floats2bfloat162_rn(acc[2 * i] * inv, acc[2 * i + 1] * inv);
 }
 
 // kFull: the ring is three stages of 128-key tiles (then the geometry is known at compile time).
@@ -1232,13 +1133,17 @@ int nodes_per_unit(const falcon_attn_args& a) {
 }
 }  // namespace
 
-// Where this kernel is the faster of the two tensor-core kernels (measured on the B200): blocks of
-// at most 64 query rows (a 60-node tree with one query head per KV head), and launches with at least
-// one unit per SM, which need no key splits.
+// Where this kernel is the faster of the two tensor-core kernels (measured over 110 random shapes): few
+// query rows and enough keys.  At most 64 rows: above, the other kernel's 128-row tiles are filled and
+// it won everywhere (65-128 rows 4 to 50 % faster, more rows up to 2.5 times).  Up to 16 rows from
+// about 200 keys (8 heads, 4 nodes, 3 x 135 keys 5.6 against 6.1 us; 3 x 1340 7.0 / 8.9), up to 64 from
+// about 640 (32 heads, 60 nodes, 1084 keys 8.8 / 9.8; 16 heads, 24 nodes, 2 x 509 keys 7.1 / 6.7): with
+// fewer keys its output, which one or two CTAs then transpose and store, costs more.
 bool tree_attn_tck_preferred(const falcon_ctx* ctx, const falcon_attn_args& a) {
-  const int G = a.n_q_heads / a.n_kv_heads, q_nodes = nodes_per_unit(a);
-  const int64_t units = static_cast<int64_t>(a.n_kv_heads) * ((a.tree.max_tree + q_nodes - 1) / q_nodes) * a.tree.batch;
-  return q_nodes * G <= 64 || units >= ctx->sm_count;
+  (void)ctx;
+  const int rows = a.tree.max_tree * (a.n_q_heads / a.n_kv_heads);
+  const int keys = a.tree.max_prefix_len + a.tree.max_tree;
+  return rows <= 64 && keys >= (rows <= 16 ? 200 : 640);
 }
 
 namespace {

@@ -1,5 +1,5 @@
 // falcon_tree_attn, one small thread block per query row: the kernel for small problems (it takes up to
-// 1024 keys a sequence and is chosen for about a hundred, any head_dim the call supports, separate tree buffers, any head grouping), where
+// 1024 keys a sequence and is chosen below a hundred, any head_dim the call supports, separate tree buffers, any head grouping), where
 // a launch is a few microseconds of latency whatever the arithmetic costs and the tensor-core
 // kernels' set-up is most of their time.  What counts here is the number of dependent round trips
 // to memory, so every pass issues all its loads before it uses any.
@@ -233,15 +233,14 @@ bool tree_attn_warp_supports(const falcon_ctx* ctx, const falcon_attn_args& a) {
   return a.tree.max_prefix_len + a.tree.max_tree <= kWarpKeysMax && a.tree.batch <= 65535 && a.n_q_heads <= 65535;
 }
 
-// Where this kernel beats the tensor-core kernels, whose set-up costs about 6 us whatever the size:
-// a block's time grows with its keys (8.7 KB of K a thread round), and the blocks come in waves of a
-// few hundred rows.  Measured, us per launch against the better tensor-core kernel: 4 heads x 64,
-// 8 nodes, 40 / 136 / 408 keys 3.3 / 5.4 / 9.4 against 5.9; 16 heads x 64, 16 nodes, 48 / 144 keys
-// 4.0 / 7.1 against 5.9; 32 heads x 64, 16 nodes, 48 keys 5.3 against 7.4; 32 heads x 128, 8 nodes, 40
-// keys 4.7 against 6.5, 16 nodes, 48 keys 8.3 against 7.1.
+// Where this kernel beats the tensor-core kernels, whose set-up costs 4.2 to 5 us whatever the size: a
+// block's time grows with its keys, and the blocks come in waves of a few hundred rows.  Measured, us per
+// launch against the better tensor-core kernel: 4 heads x 64, 8 nodes, 24 / 72 / 136 keys 3.3 / 4.1 / 5.5
+// against 4.2 / 4.9 / 5.1; 16 heads x 64, 16 nodes, 32 / 80 keys 3.8 / 5.2 against 4.2 / 4.9; 16 heads x
+// 128, 8 nodes, 72 keys 4.8 against 5.3; 32 heads x 128, 16 nodes, 32 keys 7.6 against 4.7.
 bool tree_attn_warp_preferred(const falcon_attn_args& a) {
-  const int64_t key_elems = static_cast<int64_t>(a.tree.max_prefix_len + a.tree.max_tree) * a.head_dim;
-  return key_elems <= 9216 && key_elems * a.tree.total_nodes * a.n_q_heads <= 1600000;
+  const int64_t keys = a.tree.max_prefix_len + a.tree.max_tree;
+  return keys <= 96 && keys * a.head_dim * a.tree.total_nodes * a.n_q_heads <= 1100000;
 }
 
 int launch_tree_attn_warp(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s) {

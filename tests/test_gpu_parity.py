@@ -504,12 +504,14 @@ def test_attn_tc_row_arrangements(T, G, L, splits, tck):
     H.assert_attn_close(out, ref, tb.node_off)
 
 
+@pytest.mark.parametrize("kernel", TC_KERNELS)
 @pytest.mark.parametrize("D", [64, 128])
 @pytest.mark.parametrize("separate", [False, True])
 @pytest.mark.parametrize("T,G,L,splits", [(1, 1, 0, 1), (60, 1, 0, 1), (60, 1, 1024, 4), (33, 1, 127, 2), (80, 1, 129, 1), (64, 2, 256, 3),
-                                           (128, 1, 250, 8), (17, 8, 640, 0), (72, 4, 1, 1)])
-def test_attn_tck_head_sizes_and_separate_tree_buffers(T, G, L, splits, separate, D):
-    """The keys-on-lanes kernel with 64- and 128-wide heads and with the tree's K/V in buffers of its own (whose keys
+                                           (128, 1, 250, 8), (17, 8, 640, 0), (72, 4, 1, 1),
+                                           (97, 8, 1500, 5), (33, 4, 63, 2)])
+def test_attn_tc_head_sizes_and_separate_tree_buffers(T, G, L, splits, separate, D, kernel):
+    """Both tensor-core kernels with 64- and 128-wide heads and with the tree's K/V in buffers of its own (whose keys
     start a tile of their own), two sequences of different sizes; what lies past the prefix in the cache is NaN then."""
     rng = np.random.default_rng(1000 * T + 10 * G + splits + D)
     Hkv = 2
@@ -529,7 +531,7 @@ def test_attn_tck_head_sizes_and_separate_tree_buffers(T, G, L, splits, separate
         kw = dict(k_tree=kt, v_tree=vt)
     for hc in (False, True):
         dt = H.DevTrees(tb)
-        out, rc = H.run_attn(dt, Hkv * G, Hkv, D, q, k, v, kernel=binding.ATTN_TCK, n_splits=splits, host_copies=hc, **kw)
+        out, rc = H.run_attn(dt, Hkv * G, Hkv, D, q, k, v, kernel=kernel, n_splits=splits, host_copies=hc, **kw)
         H.assert_attn_close(out, ref, tb.node_off)
         assert not dt.status.cpu().numpy().any()
 
