@@ -32,7 +32,8 @@ struct falcon_ctx {
   // (0 = not asked yet, -1 = none).  Index 0: rows-on-lanes kernel; from 1: the keys-on-lanes kernel's
   // three variants (times head dimension and place of the tree's K/V for the limit).
   bool attn_attr_set[13] = {};
-  bool lm_attr_set = false;  // the same for the LM-head kernel
+  bool lm_attr_set = false;    // the same for the LM-head kernel
+  bool topm_attr_set = false;  // and for the streaming top-m kernel
   int attn_resident[4][9] = {};
 };
 

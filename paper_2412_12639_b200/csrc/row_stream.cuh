@@ -1,0 +1,111 @@
+// A stretch of one fp32 logits row streamed through shared memory by bulk copies: the loop of the
+// kernels that scan [rows, vocab] matrices (top-m, acceptance, non-greedy acceptance) where there is
+// more data than fits the registers of the CTAs that run at once.  Internal to the library.
+//
+// What bounds such a scan is bytes in flight: an SM draws about 45 GB/s with 64 KB outstanding, which
+// register loads reach only with most of the register file, and every address, predicate and
+// register move of the loads is issued by the warps that should be comparing.  Here one thread of an extra
+// warp asks for 32 KB at a time and the eight working warps read 16 bytes per lane from shared memory.
+//
+// Rows start anywhere (4-byte aligned): the copies cover the whole 16-byte units inside the stretch, and
+// the up to three entries before and after them are `edge` entries, for the caller to read.
+#pragma once
+
+#include "tc_util.cuh"
+
+namespace falcon {
+
+constexpr int kStreamWarps = 8;
+constexpr int kStreamThreads = 32 * kStreamWarps;           // working threads; one more warp issues the copies
+constexpr int kStreamLane = 32;                             // entries a lane takes per stage
+constexpr int kStreamStage = kStreamThreads * kStreamLane;  // 8192 entries, 32 KB
+constexpr int kStreamStages = 2;
+constexpr uint32_t kStreamBytes = kStreamStages * kStreamStage * 4;
+
+struct StreamBars {
+  uint64_t full[kStreamStages], empty[kStreamStages];
+  int abort;
+};
+
+struct RowStream {
+  const float* base;  // first entry of the 16-byte aligned part
+  int head, body, tail;  // entries before it, in it (a multiple of 4), after it
+  uint32_t buf, bars;    // shared-memory addresses
+  volatile int* abort;
+
+  __device__ __forceinline__ int stages() const { return (body + kStreamStage - 1) / kStreamStage; }
+  // Entries [0, n) of `row`.  Threads 0 .. of any warp call this; one thread calls init().
+  __device__ __forceinline__ RowStream(const float* row, int n, void* smem, StreamBars* b) {
+    const int mis = static_cast<int>((4 - ((reinterpret_cast<uintptr_t>(row) >> 2) & 3)) & 3);
+    head = min(n, mis);
+    body = (n - head) & ~3;
+    tail = n - head - body;
+    base = row + head;
+    buf = tc::smem_u32(smem);
+    bars = tc::smem_u32(b);
+    abort = &b->abort;
+  }
+  __device__ __forceinline__ static void init(StreamBars* b) {
+    for (int i = 0; i < kStreamStages; ++i) {
+      tc::mbar_init(tc::smem_u32(&b->full[i]), 1);
+      tc::mbar_init(tc::smem_u32(&b->empty[i]), kStreamWarps);
+    }
+    b->abort = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  // The copying thread: stages [i0, i1), in order.
+  __device__ __forceinline__ void produce(int i0, int i1) const {
+    for (int i = i0; i < i1; ++i) {
+      const int st = i % kStreamStages;
+      const uint32_t full = bars + 8u * st;
+      if (i >= kStreamStages && !tc::mbar_wait(bars + 8u * (kStreamStages + st), (i / kStreamStages - 1) & 1, abort)) {
+        for (int k = i - kStreamStages; k < i; ++k) tc::mbar_wait_drain(bars + 8u * (k % kStreamStages), (k / kStreamStages) & 1);
+        return;
+      }
+      const uint32_t bytes = static_cast<uint32_t>(min(kStreamStage, body - i * kStreamStage)) * 4u;
+      tc::mbar_expect_tx(full, bytes);
+      asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(buf + st * kStreamStage * 4u),
+                   "l"(base + static_cast<int64_t>(i) * kStreamStage), "r"(bytes), "r"(full)
+                   : "memory");
+    }
+    // (until the last copies have landed: none may be in flight when the CTA leaves, whatever became of its waits)
+    if (i1 == stages())
+      for (int k = max(0, i1 - kStreamStages); k < i1; ++k) tc::mbar_wait_drain(bars + 8u * (k % kStreamStages), (k / kStreamStages) & 1);
+  }
+  // Entry e (0 .. 3) of the lane's j-th 16-byte piece of stage i, counted from `base`.
+  __device__ __forceinline__ int index(int i, int j, int e) const {
+    return i * kStreamStage + (((threadIdx.x >> 5) * (kStreamLane / 4) + j) * 32 + (threadIdx.x & 31)) * 4 + e;
+  }
+  // The lane's 32 entries of stage i into registers (beyond the end: -inf).  False when the wait gave up.
+  __device__ __forceinline__ bool take(int i, float (&x)[kStreamLane]) const {
+    const int st = i % kStreamStages;
+    if (!tc::mbar_wait_warp(bars + 8u * st, (i / kStreamStages) & 1, abort)) return false;
+    const uint32_t at = buf + st * kStreamStage * 4u + (((threadIdx.x >> 5) * (kStreamLane / 4)) * 32 + (threadIdx.x & 31)) * 16u;
+#pragma unroll
+    for (int j = 0; j < kStreamLane / 4; ++j)
+      asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x[4 * j]), "=f"(x[4 * j + 1]), "=f"(x[4 * j + 2]), "=f"(x[4 * j + 3]) : "r"(at + j * 512) : "memory");
+    if (body - i * kStreamStage < kStreamStage) {
+#pragma unroll
+      for (int j = 0; j < kStreamLane / 4; ++j)
+        if (index(i, j, 0) >= body) x[4 * j] = x[4 * j + 1] = x[4 * j + 2] = x[4 * j + 3] = -INFINITY;
+    }
+    return true;
+  }
+  // Which of them exist, and one of them (k = 4 j + e) again, until the stage is handed back.
+  __device__ __forceinline__ uint32_t live(int i) const {
+    const int pieces = min(kStreamStage, body - i * kStreamStage) >> 2, mine = (threadIdx.x >> 5) * (kStreamLane / 4) * 32 + (threadIdx.x & 31);
+    const int nj = max(0, min(kStreamLane / 4, (pieces - mine + 31) >> 5));
+    return nj >= 8 ? 0xffffffffu : (1u << (4 * nj)) - 1u;
+  }
+  __device__ __forceinline__ float value(int i, int k) const {
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(buf + (i % kStreamStages) * kStreamStage * 4u + (index(i, k >> 2, k & 3) - i * kStreamStage) * 4u));
+    return v;
+  }
+  __device__ __forceinline__ void give_back(int i) const {
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) tc::mbar_arrive(bars + 8u * (kStreamStages + i % kStreamStages));
+  }
+};
+
+}  // namespace falcon

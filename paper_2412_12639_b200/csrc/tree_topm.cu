@@ -2,55 +2,73 @@
 // node gets when the decoding tree is grown, Appendix A).
 //
 // Order: larger value first, the lower index among equal values; a NaN counts as -inf.
-// One launch, no block-wide rounds.  The building block is a warp that thins the entries it holds
-// in registers to at most 64 that contain its m best: the m-th largest of the 32 lanes' maxima
-// (every lane ranks its maximum against the others) is a threshold that at least m entries reach, so everything
-// below it can go whichever way ties are broken.  Only when more than 64 entries reach the
-// threshold (many equal values, or m close to 32) does the warp take the exact m best instead: the
-// m-th largest key by bisection over its bits, ties by bisection over the index bits (a warp-wide
-// count per bit).  Values are compared as floats where they are read (maximum, threshold test: two
-// or three instructions an entry) and become 32-bit keys whose unsigned order is the selection
-// order (key 0 = "no entry") only once they have survived.
-//   A  grid (chunks, rows), 8 warps per CTA: each warp loads its share of the CTA's chunk (up to
-//      16 or 32 entries per lane) straight into registers and leaves its survivors in shared memory;
-//   B  the survivors go to scratch as they are (a second threshold over the whole CTA, from the
-//      warps' four largest lane maxima, keeps them to a few dozen), or thinned by warp 0 if more than 64;
-//   C  the last CTA of a row to finish (arrival counter) spreads the chunks' survivors over
-//      its 8 warps (eight chunks each);  D  its warp 0 thins the warps' survivors once more if more
-//      than one warp had any, ranks the at most 64 that remain and writes the first m.
-// The row is read from HBM once (4 V bytes).
+// One thread-block cluster of up to eight CTAs per row (8 warps each); the row is read once (4 V bytes)
+// and no intermediate result touches global memory.  A call is a chain of latencies, so it has as few
+// hops as the selection allows (one row of 32000: 4.6 us; through scratch lists and an arrival counter
+// in global memory it took 7.8):
+//   1  every CTA loads the first step of its share into registers (up to 32 entries per lane) and finds
+//      the maxima of its groups of lanes, 64 groups in the whole cluster, which go to the shared memory
+//      of every CTA; cluster barrier.
+//   2  the m-th largest of the 64 group maxima is a threshold that at least m entries of the row reach:
+//      everything below it can go, whichever way ties are broken.  On continuous data it leaves little
+//      more than m entries of the first steps (about -64 ln(1 - m/64)).
+//   3  the survivors go to a list.  Where the share is longer than a step the loads of the next step run
+//      under the filtering of this one (two instructions an entry), and after steps 2, 4, 8, ... the
+//      threshold is taken afresh from the list, so that each doubling of what has been seen adds
+//      about as many survivors as the first step did.
+//   4  CTA 0 has or is sent all lists; cluster barrier; it ranks the survivors, a thread each, and
+//      writes the first m.
+// When a list overflows (many equal values, e.g. a row that is mostly -inf) the cluster takes the exact
+// route instead: every warp cuts its entries to at most 64 that contain its m best (threshold from the
+// lanes' maxima, or bisection over key and index bits), every CTA its warps', CTA 0 the CTAs'.  Values are
+// compared as floats where they are read and become 32-bit keys whose unsigned order is the
+// selection order (key 0 = "no entry") only once they have survived.
 
 #include <climits>
 
-#include "common.cuh"
+#include "row_stream.cuh"
 
 namespace falcon {
 namespace {
 
 constexpr int kTopmThreads = 256;
 constexpr int kTopmWarps = kTopmThreads / 32;
+constexpr int kTopmMaxCluster = 8;
+constexpr int kTopmGroups = 64;                                   // group maxima of a row
 constexpr int kTopmPerLane = 16;                                  // entries a lane holds in the passes over lists
 constexpr int kTopmRowsMax = 32;                                  // entries a lane holds at most in the first pass
-constexpr int kTopmChunkMax = kTopmWarps * 32 * kTopmRowsMax;     // 8192 entries per CTA
 constexpr int kTopmCap = 64;                                      // entries a thinning pass leaves at most
-static_assert(64 * kTopmCap <= kTopmWarps * 32 * kTopmPerLane, "the last CTA's warps hold the survivors of 64 chunks");
+constexpr int kList = 512;                                        // survivors a list holds at most
+constexpr int kRankMax = 128;                                     // more than these are thinned before they are ranked
+static_assert(kTopmMaxCluster * kTopmCap <= 32 * kTopmPerLane, "one warp holds all CTAs' survivors");
 static_assert(kTopmWarps * kTopmCap <= 32 * kTopmPerLane, "one warp holds all warps' survivors");
+static_assert(kList <= 2 * kTopmThreads, "a thread holds two list entries at most");
 static_assert(FALCON_TOPM_MAX <= 32, "the threshold is the m-th largest of 32 lane maxima");
 static_assert(FALCON_TOPM_MAX <= kTopmCap, "the exact selection's m entries fit where the survivors go");
 
 struct TopmParams {
-  int32_t n_rows, vocab, m, chunks, chunk_len;
-  int32_t warp_span;   // entries of a chunk that one warp takes (a multiple of 32, at most 32 * kTopmRowsMax)
-  int32_t cta_thresh;  // pass A also uses a threshold over the whole CTA (see warp_thin_first)
+  int32_t vocab, m;
+  int32_t chunk_len;   // entries per CTA of the cluster
+  int32_t steps;       // in which the exact route takes a CTA's share: of 256 x (entries per lane)
   int64_t logits_stride;
   const float* logits;
   float* top_val;
   int32_t* top_idx;
-  uint32_t* part_key;  // [rows, chunks, kTopmCap]
-  int32_t* part_idx;   // [rows, chunks, kTopmCap]
-  int32_t* part_cnt;   // [rows, chunks] entries in use
-  int32_t* tickets;    // [rows], zero between calls
 };
+
+struct TopmShared {
+  uint32_t max[kTopmGroups];            // group maxima (keys; 0 = empty group)
+  uint64_t list[kList];                 // survivors
+  int cnt;                              // how many there are (also beyond kList)
+  uint32_t tau;
+  // exact route
+  uint32_t key[kTopmWarps * kTopmCap];
+  int id[kTopmWarps * kTopmCap];
+  uint32_t acc_key[2 * kTopmCap];
+  int acc_id[2 * kTopmCap];
+  int fill, acc;
+};
+static_assert(kTopmMaxCluster * kTopmCap <= kList, "CTA 0's list takes every CTA's exact entries");
 
 // float -> key: unsigned order of the keys = order of the values; NaN -> -inf, -0 -> +0; never 0
 __device__ __forceinline__ uint32_t to_key(float x) {
@@ -133,49 +151,58 @@ __device__ __forceinline__ int warp_reserve(int* fill, int total, int lane) {
   return __shfl_sync(0xffffffffu, base, 0);
 }
 
-// First pass.  The warp's share of a row's chunk is rowp[0 .. n_w): lane l takes entries l, l + 32,
-// ... (kRows at most) as floats, and the survivors (at most kTopmCap) are appended to the list
-// out_val / out_id, whose fill count is *fill, as raw values and vocabulary indices (id0 = index
-// of rowp[0]).  A NaN is skipped by the maxima and passes the threshold test (it counts as -inf:
-// only the later passes, which work on keys, can tell whether it belongs).
+
+// Barrier of the 256 working threads of a CTA (the streaming kernel has a warp more).
+__device__ __forceinline__ void worker_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kTopmThreads) : "memory"); }
+
+// Address of this CTA's shared variable in CTA `rank` of the cluster, and accesses to it.
+__device__ __forceinline__ uint32_t peer_addr(const void* p, int rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(p))), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void peer_store(uint32_t addr, uint32_t v) {
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+__device__ __forceinline__ void peer_store64(uint32_t addr, uint64_t v) {
+  asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(addr), "l"(v) : "memory");
+}
+__device__ __forceinline__ int peer_add(uint32_t addr, int v) {
+  int old;
+  asm volatile("atom.add.shared::cluster.u32 %0, [%1], %2;" : "=r"(old) : "r"(addr), "r"(v) : "memory");
+  return old;
+}
+__device__ __forceinline__ int peer_load(uint32_t addr) {
+  int v;
+  asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+  return v;
+}
+// Barrier of the row's CTAs (its stores to peers' shared memory are visible behind it).
+__device__ __forceinline__ void row_arrive(int n_ctas) {
+  if (n_ctas > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void row_wait(int n_ctas) {
+  if (n_ctas > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  else worker_sync();
+}
+
+// Exact route, first pass: the warp's share rowp[0 .. n_w) (lane l: l, l + 32, ..., read again from L2) is
+// cut to at most kTopmCap entries that contain its m best, which are appended to the CTA's list.
 template <int kRows>
-__device__ __forceinline__ int warp_thin_first(const float* rowp, int n_w, int id0, int m, int lane, float* out_val, int* out_id,
-                                               int* fill, uint32_t* cta_top, bool use_cta_top) {
+__device__ __noinline__ void warp_cut(const float* rowp, int n_w, int id0, int m, int lane, uint32_t* out_key, int* out_id, int* fill) {
   float x[kRows];
 #pragma unroll
   for (int k = 0; k < kRows; ++k) x[k] = (k * 32 + lane < n_w) ? rowp[k * 32 + lane] : -INFINITY;
-  // the lane's entries are a prefix of its kRows slots
   const int n_lane = max(0, min(kRows, (n_w - lane + 31) >> 5));
   const uint32_t valid = n_lane >= 32 ? 0xffffffffu : ((1u << n_lane) - 1u);
-  float lm = x[0];
+  float lm = -INFINITY;
 #pragma unroll
-  for (int k = 1; k < kRows; ++k) lm = fmaxf(lm, x[k]);
-  // The warp's threshold and, if asked for, a tighter one for the whole CTA (every warp of the CTA is here
-  // then): the four largest lane maxima of each of its 8 warps are 32 different entries, so their m-th
-  // largest is reached by at least m entries of the chunk.  With it the CTA's survivors are mostly few enough
-  // to go to the row as they are, without a pass of their own: fewer instructions, but a block-wide barrier in
-  // the middle of the pass.  The launcher asks for it when the grid is more than one wave (throughput counts);
-  // in a single wave the warps are better left to run ahead of one another (60 x 32000: 11.3 against 12.5 us).
-  const uint32_t lk = to_key(lm);
-  int rank = 0;
-#pragma unroll 4
-  for (int j = 0; j < 32; ++j) {
-    const uint32_t o = __shfl_sync(0xffffffffu, lk, j);
-    rank += (o > lk || (o == lk && j < lane)) ? 1 : 0;
-  }
-  if (rank < 4) cta_top[4 * (threadIdx.x >> 5) + rank] = lk;
-  const unsigned hit = __ballot_sync(0xffffffffu, rank == m - 1);
-  const uint32_t tau_w = __shfl_sync(0xffffffffu, lk, __ffs(static_cast<int>(hit)) - 1);
-  uint32_t tau_c = 0u;
-  if (use_cta_top) {
-    __syncthreads();
-    tau_c = warp_kth_largest(cta_top[lane], m - 1, lane);
-  }
-  const float tau = from_key(max(tau_w, tau_c));
+  for (int k = 0; k < kRows; ++k) lm = fmaxf(lm, x[k]);
+  const float tau = from_key(max(1u, warp_kth_largest(valid ? to_key(lm) : 0u, m - 1, lane)));
   uint32_t mask = 0u;
 #pragma unroll
   for (int k = 0; k < kRows; ++k)
-    if (!(x[k] < tau)) mask |= 1u << k;
+    if (!(x[k] < tau)) mask |= 1u << k;  // (a NaN passes: whether it belongs is decided on keys)
   mask &= valid;
   if (warp_sum(__popc(mask)) > kTopmCap) {
     uint32_t key[kRows];
@@ -194,19 +221,18 @@ __device__ __forceinline__ int warp_thin_first(const float* rowp, int n_w, int i
       if (key[k] > t || (key[k] == t && id[k] <= u)) mask |= 1u << k;
   }
   int total;
-  int off = warp_offsets(__popc(mask), lane, total) + warp_reserve(fill, total, lane);
-  while (mask) {  // one or two entries in most lanes: read them again (L1) instead of indexing registers
-    const int k = __ffs(static_cast<int>(mask)) - 1;
-    mask &= mask - 1u;
-    out_val[off] = rowp[k * 32 + lane];
-    out_id[off] = id0 + k * 32 + lane;
-    ++off;
-  }
-  return total;
+  int off = warp_offsets(__popc(mask), lane, total);
+  off += warp_reserve(fill, total, lane);
+#pragma unroll
+  for (int k = 0; k < kRows; ++k)
+    if ((mask >> k) & 1u) {
+      out_key[off] = to_key(x[k]);
+      out_id[off] = id0 + k * 32 + lane;
+      ++off;
+    }
 }
 
-// Later passes: the same on entries that are (key, id) pairs in registers (16 per lane: key 0 =
-// none).  The survivors go to out_key / out_id in no particular order: appended to a list shared
+// The same on entries that are (key, id) pairs in registers (16 per lane: key 0 = none).  The survivors go to out_key / out_id in no particular order: appended to a list shared
 // with other warps when `fill` is its fill count, from position 0 when `fill` is null; returns
 // their number (the same in every lane).
 __device__ __forceinline__ int warp_thin(const uint32_t (&key)[kTopmPerLane], const int (&id)[kTopmPerLane], int m, int lane,
@@ -227,7 +253,8 @@ __device__ __forceinline__ int warp_thin(const uint32_t (&key)[kTopmPerLane], co
     for (int k = 0; k < kTopmPerLane; ++k) cnt += (key[k] > tau || (key[k] == tau && id[k] <= id_max)) ? 1 : 0;
   }
   int total;
-  int off = warp_offsets(cnt, lane, total) + (fill ? warp_reserve(fill, total, lane) : 0);
+  int off = warp_offsets(cnt, lane, total);
+  if (fill) off += warp_reserve(fill, total, lane);
 #pragma unroll
   for (int k = 0; k < kTopmPerLane; ++k) {
     if (key[k] > tau || (key[k] == tau && id[k] <= id_max)) {
@@ -239,141 +266,320 @@ __device__ __forceinline__ int warp_thin(const uint32_t (&key)[kTopmPerLane], co
   return total;
 }
 
-template <int kRows>
-__global__ void __launch_bounds__(kTopmThreads, kRows <= 16 ? 4 : 3) tree_topm_kernel(const TopmParams p) {
-  // the CTA's list of survivors: pass A appends raw float bits and indices, pass C keys and indices
-  __shared__ uint32_t s_key[kTopmWarps * kTopmCap];
-  __shared__ int s_id[kTopmWarps * kTopmCap];
-  __shared__ uint32_t s_fin_key[kTopmCap];
-  __shared__ int s_fin_id[kTopmCap];
-  __shared__ uint32_t s_top[4 * kTopmWarps];  // the four largest lane maxima of every warp (pass A)
-  __shared__ int s_fill;
-  __shared__ int s_last;
 
-  // Under programmatic dependent launch the grid may start while the previous kernel of the stream
-  // drains: nothing is read or written before that kernel has completed.
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  const int row = blockIdx.y, chunk = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int c0 = chunk * p.chunk_len;
-  const int n = min(p.vocab, c0 + p.chunk_len) - c0;  // >= 1 by construction of the grid
-  const float* rowp = p.logits + static_cast<int64_t>(row) * p.logits_stride + c0;
-  const int m = p.m;
-
-  if (tid == 0) s_fill = 0;
-  __syncthreads();
-
-  // ---- A: each warp thins its share of the chunk (coalesced 128-byte loads, all in flight at once) ----
-  {
-    const int w0 = warp * p.warp_span;
-    const int n_w = max(0, min(p.warp_span, n - w0));
-    warp_thin_first<kRows>(rowp + w0, n_w, c0 + w0, m, lane, reinterpret_cast<float*>(s_key), s_id, &s_fill, s_top, p.cta_thresh != 0);
+// The m-th largest of the 64 group maxima: the smallest of those that fewer than m exceed.  sh.tau must
+// read 0xffffffff before; every thread of the CTA calls this and finds it there afterwards.
+__device__ __forceinline__ void find_tau(TopmShared& sh, int m, int warp, int lane) {
+  const uint32_t mine = sh.max[warp * 8 + (lane & 7)];
+  const uint4* seg = reinterpret_cast<const uint4*>(sh.max + (lane >> 3) * 16);
+  int above = 0;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const uint4 v = seg[i];
+    above += (v.x > mine) + (v.y > mine) + (v.z > mine) + (v.w > mine);
   }
-  __syncthreads();
+  above += __shfl_xor_sync(0xffffffffu, above, 8);
+  above += __shfl_xor_sync(0xffffffffu, above, 16);
+  const uint32_t t = __reduce_min_sync(0xffffffffu, above < m ? mine : 0xffffffffu);
+  if (lane == 0) atomicMin(&sh.tau, t);
+  worker_sync();
+}
 
-  // The CTA's list, 16 entries per lane of one warp (raw: it holds raw values, which become keys here).
-  auto from_list = [&](uint32_t (&key)[kTopmPerLane], int (&id)[kTopmPerLane], bool raw) {
-    const int fill = s_fill;
+// The CTA's list thinned in place by a threshold of its own (64 groups of its entries, dealt out evenly):
+// at least m of them stay.  Every thread of the CTA calls this.  Returns the threshold.
+__device__ __forceinline__ uint32_t thin_list(TopmShared& sh, int m, int tid) {
+  const int warp = tid >> 5, lane = tid & 31, n = sh.cnt;
+  const uint64_t e0 = tid < n ? sh.list[tid] : 0ull, e1 = tid + kTopmThreads < n ? sh.list[tid + kTopmThreads] : 0ull;
+  if (tid < kTopmGroups) sh.max[tid] = 0u;
+  if (tid == 0) sh.tau = 0xffffffffu;
+  worker_sync();
+  if (e0 | e1) atomicMax(&sh.max[tid % kTopmGroups], static_cast<uint32_t>(max(e0, e1) >> 32));
+  worker_sync();
+  if (tid == 0) sh.cnt = 0;
+  find_tau(sh, m, warp, lane);
+  const uint32_t tau = max(1u, sh.tau);
+  const bool k0 = static_cast<uint32_t>(e0 >> 32) >= tau, k1 = static_cast<uint32_t>(e1 >> 32) >= tau;
+  int total;
+  int off = warp_offsets((k0 ? 1 : 0) + (k1 ? 1 : 0), lane, total);
+  off += warp_reserve(&sh.cnt, total, lane);
+  if (k0) sh.list[off++] = e0;
+  if (k1) sh.list[off] = e1;
+  worker_sync();
+  return tau;
+}
+
+// Exact route: every CTA leaves its at most kTopmCap entries, key 0 beyond them, in CTA 0's list (64 places
+// each).  Every thread of the cluster calls this, with CTA 0's shared memory still there.
+template <int kRows>
+__device__ __noinline__ void exact_entries(const TopmParams& p, TopmShared& sh, const float* rowp, int n, int c0, int rank) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, m = p.m;
+  auto from_list = [&](const uint32_t* lk, const int* li, int fill, uint32_t (&key)[kTopmPerLane], int (&id)[kTopmPerLane]) {
 #pragma unroll
     for (int k = 0; k < kTopmPerLane; ++k) {
       const int j = k * 32 + lane;
-      const bool in = j < fill;
-      const uint32_t v = in ? s_key[j] : 0u;
-      key[k] = in ? (raw ? to_key(__uint_as_float(v)) : v) : 0u;
-      id[k] = in ? s_id[j] : 0;
+      key[k] = j < fill ? lk[j] : 0u;
+      id[k] = j < fill ? li[j] : 0;
     }
   };
-
-  // ---- B: the CTA's survivors go to the row: as they are when they are few enough, else thinned by warp 0 ----
-  const int64_t po = static_cast<int64_t>(row) * p.chunks + chunk;
-  const int fill_a = s_fill;
-  if (fill_a <= kTopmCap) {
-    if (tid < fill_a) {
-      p.part_key[po * kTopmCap + tid] = to_key(__uint_as_float(s_key[tid]));
-      p.part_idx[po * kTopmCap + tid] = s_id[tid];
-    }
-    __syncthreads();  // every thread's entries before thread 0's fence
-    if (tid == 0) {
-      p.part_cnt[po] = fill_a;
-      s_fill = 0;
-      __threadfence();
-      s_last = (atomicAdd(&p.tickets[row], 1) == p.chunks - 1);
-    }
-  } else if (warp == 0) {
-    uint32_t key[kTopmPerLane];
-    int id[kTopmPerLane];
-    from_list(key, id, true);
-    const int cnt = warp_thin(key, id, m, lane, p.part_key + po * kTopmCap, p.part_idx + po * kTopmCap, nullptr);
-    __syncwarp();  // every lane's entries before lane 0's fence
-    if (lane == 0) {
-      p.part_cnt[po] = cnt;
-      s_fill = 0;  // (the list is in registers: pass C may refill it)
-      __threadfence();
-      s_last = (atomicAdd(&p.tickets[row], 1) == p.chunks - 1);
-    }
+  if (threadIdx.x == 0) {
+    sh.fill = 0;
+    sh.acc = 0;
   }
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-
-  // ---- C: last CTA of the row: the chunks' survivors, eight chunks per warp ----
-  {
-    const int64_t ro = static_cast<int64_t>(row) * p.chunks;
-    uint32_t key[kTopmPerLane];
-    int id[kTopmPerLane];
-    int cn[kTopmPerLane / 2];
-#pragma unroll
-    for (int c = 0; c < kTopmPerLane / 2; ++c) {
-      const int ch = warp * (kTopmPerLane / 2) + c;
-      cn[c] = ch < p.chunks ? __ldcg(p.part_cnt + ro + ch) : 0;
-    }
-#pragma unroll
-    for (int k = 0; k < kTopmPerLane; ++k) {
-      // entry k * 32 + lane of this warp: chunk k / 2 of its eight, slot (k & 1) * 32 + lane
-      const int slot = (k & 1) * 32 + lane;
-      const bool in = slot < cn[k >> 1];
-      const int64_t at = (ro + warp * (kTopmPerLane / 2) + (k >> 1)) * kTopmCap + slot;
-      key[k] = in ? __ldcg(p.part_key + at) : 0u;
-      id[k] = in ? __ldcg(p.part_idx + at) : 0;
-    }
-    if (warp * (kTopmPerLane / 2) < p.chunks) warp_thin(key, id, m, lane, s_key, s_id, &s_fill);
-  }
-  __syncthreads();
-
-  // ---- D: warp 0 thins once more (when several warps had chunks), ranks what is left and writes
-  // the row's result ----
-  if (warp == 0) {
-    const uint32_t* fin_key = s_key;
-    const int* fin_id = s_id;
-    int cnt = s_fill;
-    if (p.chunks > kTopmPerLane / 2) {
+  worker_sync();
+  for (int step = 0; step < p.steps; ++step) {
+    const int v0 = (step * kTopmWarps + warp) * 32 * kRows;
+    warp_cut<kRows>(rowp + v0, max(0, min(32 * kRows, n - v0)), c0 + v0, m, lane, sh.key, sh.id, &sh.fill);
+    worker_sync();
+    if (warp == 0) {  // the best so far and this step's
       uint32_t key[kTopmPerLane];
       int id[kTopmPerLane];
-      from_list(key, id, false);
-      cnt = warp_thin(key, id, m, lane, s_fin_key, s_fin_id, nullptr);
-      fin_key = s_fin_key;
-      fin_id = s_fin_id;
+      from_list(sh.key, sh.id, sh.fill, key, id);
+      const int got = warp_thin(key, id, m, lane, sh.acc_key + sh.acc, sh.acc_id + sh.acc, nullptr);
+      __syncwarp();
+      if (sh.acc > 0) {
+        from_list(sh.acc_key, sh.acc_id, sh.acc + got, key, id);
+        __syncwarp();
+        const int both = warp_thin(key, id, m, lane, sh.acc_key, sh.acc_id, nullptr);
+        __syncwarp();
+        if (lane == 0) sh.acc = both;
+      } else if (lane == 0) {
+        sh.acc = got;
+      }
+      if (lane == 0) sh.fill = 0;
     }
-    __syncwarp();
-    // At most 64 entries, two per lane: an entry's place in the result is the number of entries that
-    // come before it (the entries are distinct, so the places are too).
-    const uint64_t e0 = lane < cnt ? entry(fin_key[lane], fin_id[lane]) : 0ull;
-    const uint64_t e1 = lane + 32 < cnt ? entry(fin_key[lane + 32], fin_id[lane + 32]) : 0ull;
-    int r0 = 0, r1 = 0;
-    for (int j = 0; j < cnt; ++j) {
-      const uint64_t o = entry(fin_key[j], fin_id[j]);
-      r0 += o > e0 ? 1 : 0;
-      r1 += o > e1 ? 1 : 0;
-    }
-    if (e0 != 0ull && r0 < m) {
-      p.top_val[static_cast<int64_t>(row) * m + r0] = from_key(static_cast<uint32_t>(e0 >> 32));
-      p.top_idx[static_cast<int64_t>(row) * m + r0] = static_cast<int>(~static_cast<uint32_t>(e0));
-    }
-    if (e1 != 0ull && r1 < m) {
-      p.top_val[static_cast<int64_t>(row) * m + r1] = from_key(static_cast<uint32_t>(e1 >> 32));
-      p.top_idx[static_cast<int64_t>(row) * m + r1] = static_cast<int>(~static_cast<uint32_t>(e1));
-    }
-    if (lane == 0) p.tickets[row] = 0;  // ready for the next call
+    worker_sync();
   }
+  if (warp == 0)
+    for (int j = lane; j < kTopmCap; j += 32)
+      peer_store64(peer_addr(&sh.list[rank * kTopmCap + j], 0), j < sh.acc ? entry(sh.acc_key[j], sh.acc_id[j]) : 0ull);
+}
+// ... and CTA 0 cuts them to at most kTopmCap at the head of its list.
+__device__ __noinline__ void exact_finish(TopmShared& sh, int n_ctas, int m) {
+  const int lane = threadIdx.x & 31;
+  if (threadIdx.x < 32) {
+    uint32_t key[kTopmPerLane];
+    int id[kTopmPerLane];
+#pragma unroll
+    for (int k = 0; k < kTopmPerLane; ++k) {
+      const int j = k * 32 + lane;
+      const uint64_t e = j < n_ctas * kTopmCap ? sh.list[j] : 0ull;
+      key[k] = static_cast<uint32_t>(e >> 32);
+      id[k] = static_cast<int>(~static_cast<uint32_t>(e));
+    }
+    const int got = warp_thin(key, id, m, lane, sh.key, sh.id, nullptr);
+    __syncwarp();
+    for (int j = lane; j < got; j += 32) sh.list[j] = entry(sh.key[j], sh.id[j]);
+    if (lane == 0) sh.cnt = got;
+  }
+  worker_sync();
+}
+
+// Appends the entries of one batch of registers that reach the threshold to a list (the CTA's own, or with
+// `remote` CTA 0's).  live: which of x[0 .. kN) are entries; index(k), value(k): vocabulary index and value of
+// the lane's entry k, asked for the few survivors only.  A compact loop over them: written out entry by
+// entry this was 13 KB of instructions, and fetching those for the first time in a launch took 7000 cycles.
+template <int kN, class Index, class Value>
+__device__ __forceinline__ void append(TopmShared& sh, const float (&x)[kN], uint32_t tau_key, uint32_t live, bool remote, int lane,
+                                       Index index, Value value) {
+  const float tau = from_key(tau_key);
+  uint32_t mask = 0u;
+#pragma unroll
+  for (int k = 0; k < kN; ++k) mask |= x[k] >= tau ? 1u << k : 0u;
+  if (tau_key <= to_key(-INFINITY)) mask = live;
+  const int total = warp_sum(__popc(mask));
+  if (total == 0) return;
+  int base = 0;
+  if (lane == 0) base = remote ? peer_add(peer_addr(&sh.cnt, 0), total) : atomicAdd(&sh.cnt, total);
+  base = __shfl_sync(0xffffffffu, base, 0);
+  if (base + total > kList) return;  // (the count says so)
+#pragma unroll 1
+  for (uint32_t left = __ballot_sync(0xffffffffu, mask != 0u); left; left = __ballot_sync(0xffffffffu, mask != 0u)) {
+    if (mask) {
+      const int k = __ffs(static_cast<int>(mask)) - 1;
+      mask &= mask - 1u;
+      const int at = base + __popc(left & ((1u << lane) - 1u));
+      const uint64_t e = entry(to_key(value(k)), index(k));
+      if (remote) peer_store64(peer_addr(&sh.list[at], 0), e);
+      else sh.list[at] = e;
+    }
+    base += __popc(left);
+  }
+}
+
+// Group maxima to every CTA of the row, and the threshold.  lk: the largest key of this lane's entries (0: it
+// has none).  Every working thread calls this.
+__device__ __forceinline__ uint32_t first_tau(TopmShared& sh, uint32_t lk, int m, int rank, int n_ctas, int warp, int lane) {
+  // 64 groups in the cluster: 8 / n_ctas per warp; lane l sends group l % per to CTA l / per
+  const int per = kTopmMaxCluster / n_ctas, width = 32 / per;
+  for (int o = width >> 1; o > 0; o >>= 1) lk = max(lk, __shfl_xor_sync(0xffffffffu, lk, o));
+  const uint32_t gmax = __shfl_sync(0xffffffffu, lk, (lane % per) * width);
+  row_wait(n_ctas);
+  if (lane < kTopmMaxCluster) peer_store(peer_addr(&sh.max[(rank * kTopmWarps + warp) * per + lane % per], lane / per), gmax);
+  row_arrive(n_ctas);
+  row_wait(n_ctas);
+  find_tau(sh, m, warp, lane);
+  return max(1u, sh.tau);  // (fewer than m groups hold anything: every entry passes)
+}
+
+// The end of both kernels: all survivors are in CTA 0's list, or its count says that they are too many.
+template <int kRows>
+__device__ __forceinline__ void finish_row(const TopmParams& p, TopmShared& sh, const float* rowp, int n, int c0, int rank, int n_ctas, int row) {
+  const int tid = threadIdx.x, m = p.m;
+  row_arrive(n_ctas);
+  row_wait(n_ctas);
+  const int cnt = rank == 0 ? sh.cnt : peer_load(peer_addr(&sh.cnt, 0));
+  row_arrive(n_ctas);  // CTA 0's shared memory is needed until every CTA has read the count
+  if (cnt > kList) {
+    row_wait(n_ctas);
+    exact_entries<kRows>(p, sh, rowp, n, c0, rank);
+    row_arrive(n_ctas);
+    row_wait(n_ctas);
+    if (rank != 0) return;
+    exact_finish(sh, n_ctas, m);
+  } else {
+    if (rank != 0) return;
+    if (n_ctas > 1) row_wait(n_ctas);
+    if (cnt > kRankMax) thin_list(sh, m, tid);
+  }
+  // An entry's place is the number of entries that come before it (they are distinct).
+  const int got = sh.cnt;
+  for (int t = tid; t < got; t += kTopmThreads) {
+    const uint64_t e = sh.list[t];
+    int r = 0;
+    for (int j = 0; j < got; ++j) r += sh.list[j] > e ? 1 : 0;
+    if (r < m) {
+      p.top_val[static_cast<int64_t>(row) * m + r] = from_key(static_cast<uint32_t>(e >> 32));
+      p.top_idx[static_cast<int64_t>(row) * m + r] = static_cast<int>(~static_cast<uint32_t>(e));
+    }
+  }
+}
+
+// The row in the cluster's registers: kRows entries per lane.
+template <int kRows>
+__global__ void __launch_bounds__(kTopmThreads, kRows <= 8 ? 6 : (kRows <= 16 ? 4 : 3)) tree_topm_kernel(const __grid_constant__ TopmParams p) {
+  __shared__ __align__(16) TopmShared sh;
+  const int row = blockIdx.y, rank = blockIdx.x, n_ctas = gridDim.x;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int c0 = rank * p.chunk_len;
+  const int n = max(0, min(p.vocab, c0 + p.chunk_len) - c0);
+  const float* rowp = p.logits + static_cast<int64_t>(row) * p.logits_stride + c0;
+  if (tid == 0) {
+    sh.cnt = 0;
+    sh.tau = 0xffffffffu;
+  }
+  row_arrive(n_ctas);  // waited for before the first store to a peer: by then it runs
+  // Under programmatic dependent launch the grid may start while the previous kernel of the stream
+  // drains: nothing is read or written before that kernel has completed.
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // Lane l of a warp holds entries l, l + 32, ... of its share: coalesced 128-byte loads, all in flight at once.
+  const int w0 = warp * 32 * kRows + lane;
+  float x[kRows];
+#pragma unroll
+  for (int k = 0; k < kRows; ++k) x[k] = w0 + k * 32 < n ? __ldcs(rowp + w0 + k * 32) : -INFINITY;
+  float lm = -INFINITY;
+#pragma unroll
+  for (int k = 0; k < kRows; ++k) lm = fmaxf(lm, x[k]);
+  const uint32_t tau = first_tau(sh, w0 < n ? to_key(lm) : 0u, p.m, rank, n_ctas, warp, lane);
+  const int n_lane = max(0, min(kRows, (n - w0 + 31) >> 5));  // the lane's entries are a prefix of its slots
+  append<kRows>(sh, x, tau, n_lane >= 32 ? 0xffffffffu : (1u << n_lane) - 1u, n_ctas > 1, lane, [&](int k) { return c0 + w0 + k * 32; },
+                [&](int k) {
+                  float v = x[0];
+#pragma unroll
+                  for (int i = 1; i < kRows; ++i) v = k == i ? x[i] : v;
+                  return v;
+                });
+  finish_row<kRows>(p, sh, rowp, n, c0, rank, n_ctas, row);
+}
+
+// The row streamed through shared memory, 8192 entries of a CTA at a time.
+__global__ void __launch_bounds__(kStreamThreads + 32, 3) tree_topm_stream_kernel(const __grid_constant__ TopmParams p) {
+  extern __shared__ __align__(128) unsigned char stream_buf[];
+  __shared__ __align__(16) TopmShared sh;
+  __shared__ __align__(8) StreamBars bars;
+  static_assert(kStreamThreads == kTopmThreads, "the list passes count on 256 working threads");
+  const int row = blockIdx.y, rank = blockIdx.x, n_ctas = gridDim.x;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int m = p.m, c0 = rank * p.chunk_len;
+  const int n = max(0, min(p.vocab, c0 + p.chunk_len) - c0);
+  const float* rowp = p.logits + static_cast<int64_t>(row) * p.logits_stride + c0;
+  const RowStream rs(rowp, n, stream_buf, &bars);
+  if (tid == kStreamThreads) {
+    sh.cnt = 0;
+    sh.tau = 0xffffffffu;
+    RowStream::init(&bars);
+  }
+  __syncthreads();
+  row_arrive(n_ctas);
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int n_st = rs.stages();
+  if (warp == kStreamWarps) {
+    // The cluster barriers of first_tau() count this warp too: it goes through them once the ring is full, and
+    // has left before the next one (all stages are issued by the time the last is taken).
+    if (lane == 0) rs.produce(0, min(n_st, kStreamStages));
+    __syncwarp();
+    if (n_ctas > 1) {
+      row_wait(n_ctas);
+      row_arrive(n_ctas);
+      row_wait(n_ctas);
+    }
+    if (lane == 0) rs.produce(min(n_st, kStreamStages), n_st);
+    return;
+  }
+  {
+    float x[kStreamLane];
+    bool ok = n_st == 0 || rs.take(0, x);
+    float lm = -INFINITY;
+    if (n_st > 0 && ok) {
+#pragma unroll
+      for (int k = 0; k < kStreamLane; ++k) lm = fmaxf(lm, x[k]);
+    }
+    uint32_t tau = first_tau(sh, n_st > 0 && ok && rs.index(0, 0, 0) < rs.body ? to_key(lm) : 0u, m, rank, n_ctas, warp, lane);
+    // the up to six entries outside the copies
+    if (warp == 0) {
+      const bool in = lane < rs.head + rs.tail;
+      const int i = lane < rs.head ? lane : lane + rs.body;
+      const float xe[1] = {in ? __ldcs(rowp + i) : -INFINITY};
+      append<1>(sh, xe, tau, in ? 1u : 0u, false, lane, [&](int) { return c0 + i; }, [&](int) { return xe[0]; });
+    }
+    for (int st = 0; ok && st < n_st; ++st) {
+      if (st > 0) {
+        ok = rs.take(st, x);
+        if (!ok) break;
+        lm = -INFINITY;
+#pragma unroll
+        for (int k = 0; k < kStreamLane; ++k) lm = fmaxf(lm, x[k]);
+      }
+      if (tau <= to_key(-INFINITY) || __any_sync(0xffffffffu, to_key(lm) >= tau))
+        append<kStreamLane>(sh, x, tau, rs.live(st), false, lane, [&](int k) { return c0 + rs.head + rs.index(st, k >> 2, k & 3); },
+                            [&](int k) { return rs.value(st, k); });
+      rs.give_back(st);
+      if (((st + 1) & st) == 0 && st > 0 && st + 1 < n_st) {  // 2, 4, 8, ... stages seen
+        worker_sync();
+        if (sh.cnt <= kList) tau = max(tau, thin_list(sh, m, tid));  // (beyond: the exact route)
+      }
+    }
+    if (!ok && lane == 0) atomicAdd(&sh.cnt, kList + 1);  // a wait gave up: the exact route reads the row itself
+  }
+  worker_sync();
+  if (n_ctas > 1) {  // the CTA's own survivors to CTA 0 (which keeps its own where they are)
+    const int mine = sh.cnt;
+    row_arrive(n_ctas);       // every list is complete: CTA 0's may be appended to
+    row_wait(n_ctas);
+    if (rank != 0) {
+      const uint32_t cnt0 = peer_addr(&sh.cnt, 0), list0 = peer_addr(&sh.list[0], 0);
+      for (int j0 = warp * 32; j0 < min(mine, kList); j0 += kStreamThreads) {
+        const int some = min(32, mine - j0);
+        int base = 0;
+        if (lane == 0) base = peer_add(cnt0, some);
+        base = __shfl_sync(0xffffffffu, base, 0);
+        if (lane < some && base + lane < kList) peer_store64(list0 + 8 * (base + lane), sh.list[j0 + lane]);
+      }
+      if (mine > kList && tid == 0) peer_add(cnt0, kList + 1);  // overflowed: so does the sum
+    }
+  }
+  finish_row<kStreamLane>(p, sh, rowp, n, c0, rank, n_ctas, row);
 }
 
 }  // namespace
@@ -381,57 +587,70 @@ __global__ void __launch_bounds__(kTopmThreads, kRows <= 16 ? 4 : 3) tree_topm_k
 int launch_tree_topm(falcon_ctx* ctx, const falcon_topm_args& a, cudaStream_t s) {
   const int N = a.n_rows;
   if (N > 65535) return FALCON_ERR_CAPACITY;
-  // As many CTAs as are resident at once (four per SM) where the vocabulary allows; a chunk is at
-  // most what a CTA holds in registers, split evenly over its warps in units of 32 entries.
-  int chunks = 4 * ctx->sm_count / N;
-  if (chunks < 1) chunks = 1;
-  const int max_chunks = (a.vocab + 2047) / 2048;
-  if (chunks > max_chunks) chunks = max_chunks;
-  if (chunks > kTopmPerLane / 2) chunks = kTopmPerLane / 2;  // one warp of the row's last CTA then holds all survivors
-  const int min_chunks = (a.vocab + kTopmChunkMax - 1) / kTopmChunkMax;
-  if (chunks < min_chunks) chunks = min_chunks;
-  if (chunks > 64) return FALCON_ERR_CAPACITY;  // vocabulary beyond 64 x 8192 entries
-  int chunk_len = (a.vocab + chunks - 1) / chunks;
-  int warp_span = ((chunk_len + kTopmWarps - 1) / kTopmWarps + 31) & ~31;
-  if (warp_span > 32 * kTopmRowsMax) warp_span = 32 * kTopmRowsMax;
-  chunk_len = kTopmWarps * warp_span;  // (the last chunk of a row may be shorter or, rounded up, missing)
-  chunks = (a.vocab + chunk_len - 1) / chunk_len;
-
-  const size_t part = static_cast<size_t>(N) * chunks * kTopmCap;
-  int rc = ensure_workspace(ctx, part * 8 + static_cast<size_t>(N) * chunks * 4 + 256);
-  if (rc) return rc;
-  rc = ensure_tickets(ctx, N, s);
-  if (rc) return rc;
-
   TopmParams p;
-  p.n_rows = N;
   p.vocab = a.vocab;
   p.m = a.m;
-  p.chunks = chunks;
-  p.chunk_len = chunk_len;
-  p.warp_span = warp_span;
-  // (CTAs resident per SM: 4 with 16 entries per lane, 3 with 32: the kernel's launch bounds)
-  p.cta_thresh = static_cast<int64_t>(N) * chunks > static_cast<int64_t>(warp_span <= 16 * 32 ? 4 : 3) * ctx->sm_count ? 1 : 0;
   p.logits_stride = a.logits_stride;
   p.logits = a.logits;
   p.top_val = a.top_val;
   p.top_idx = a.top_idx;
-  p.part_key = static_cast<uint32_t*>(ctx->ws);
-  p.part_idx = reinterpret_cast<int32_t*>(static_cast<uint32_t*>(ctx->ws) + part);
-  p.part_cnt = p.part_idx + part;
-  p.tickets = ctx->tickets;
+
+  // Rows in registers while the whole grid is resident at once (six CTAs per SM with 8 entries per
+  // lane, four with 16, three with 32): the shortest chain.  As many CTAs per row as leave a lane 8 entries.  Else
+  // streamed, three CTAs per SM: a second wave of the register kernel starts its loads only when a
+  // first one has gone through its barriers.
+  int ctas = 1, per_lane = 0, chunk = 0;
+  auto split = [&](int c) {
+    ctas = c;
+    chunk = ((a.vocab + c - 1) / c + 3) & ~3;
+    per_lane = (chunk + kTopmThreads - 1) / kTopmThreads;
+  };
+  auto fits = [&]() { return static_cast<int64_t>(N) * ctas <= (per_lane <= 8 ? 6 : per_lane <= 16 ? 4 : 3) * ctx->sm_count; };
+  int c = 1;
+  while (c < kTopmMaxCluster && a.vocab > c * kTopmThreads * 8) c *= 2;
+  bool in_regs = false;
+  for (; c >= 1 && !in_regs; c /= 2) {
+    split(c);
+    if (per_lane > kTopmRowsMax) break;
+    in_regs = fits();
+  }
+  if (!in_regs) {
+    c = 1;
+    while (c < kTopmMaxCluster && static_cast<int64_t>(N) * 2 * c <= 3 * ctx->sm_count && a.vocab >= 2 * c * kStreamStage) c *= 2;
+    split(c);
+  }
+  p.chunk_len = chunk;
 
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(chunks, N);
+  cfg.gridDim = dim3(ctas, N);
   cfg.blockDim = dim3(kTopmThreads);
   cfg.stream = s;
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
-  cudaError_t e = warp_span <= 16 * 32 ? cudaLaunchKernelEx(&cfg, tree_topm_kernel<16>, p)
-                                       : cudaLaunchKernelEx(&cfg, tree_topm_kernel<kTopmRowsMax>, p);
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = ctas;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = ctas > 1 ? 2 : 1;
+  cudaError_t e;
+  if (in_regs) {
+    p.steps = 1;
+    e = per_lane <= 8    ? cudaLaunchKernelEx(&cfg, tree_topm_kernel<8>, p)
+        : per_lane <= 16 ? cudaLaunchKernelEx(&cfg, tree_topm_kernel<16>, p)
+                         : cudaLaunchKernelEx(&cfg, tree_topm_kernel<kTopmRowsMax>, p);
+  } else {
+    if (!ctx->topm_attr_set) {
+      e = cudaFuncSetAttribute(tree_topm_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kStreamBytes));
+      if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute(tree_topm_stream_kernel)");
+      ctx->topm_attr_set = true;
+    }
+    p.steps = (chunk + kTopmThreads * kStreamLane - 1) / (kTopmThreads * kStreamLane);
+    cfg.blockDim = dim3(kStreamThreads + 32);
+    cfg.dynamicSmemBytes = kStreamBytes;
+    e = cudaLaunchKernelEx(&cfg, tree_topm_stream_kernel, p);
+  }
   if (e != cudaSuccess) return cuda_fail(ctx, e, "tree_topm_kernel launch");
   return FALCON_OK;
 }

@@ -633,6 +633,25 @@ def test_topm_bit_exact(N, V, stride, m):
         np.testing.assert_array_equal(gv, rv)
 
 
+@pytest.mark.parametrize("N,V,stride,m", [(160, 8191, 8191, 20), (150, 24577, 24580, 8), (450, 8200, 8201, 32), (120, 66001, 66001, 1),
+                                          (2, 70001, 70003, 32), (3, 16385, 16386, 7)])
+@pytest.mark.parametrize("kind", ["normal", "few values", "mostly -inf"])
+def test_topm_many_rows_and_overflowing_lists(N, V, stride, m, kind):
+    """Rows in registers, streamed rows (alignments of all kinds, the stretch's ends, several stages) and, with many
+    equal values, the exact route of both."""
+    rng = np.random.default_rng(V + N)
+    x = rng.standard_normal((N, stride)).astype(np.float32)
+    if kind == "few values":
+        x = np.round(x * 2)
+    elif kind == "mostly -inf":
+        x[rng.random(x.shape) < 0.999] = -np.inf
+    rv, ri = oracle.topm(x, m, vocab=V)
+    for _ in range(2):
+        gv, gi, _ = H.run_topm(x, m, vocab=V)
+        np.testing.assert_array_equal(gi, ri)
+        np.testing.assert_array_equal(gv, rv)
+
+
 def test_topm_ties_nan_inf_and_argmax_agreement():
     rng = np.random.default_rng(77)
     x = rng.standard_normal((6, 9000)).astype(np.float32)
