@@ -33,7 +33,8 @@ struct falcon_ctx {
   // three variants (times head dimension and place of the tree's K/V for the limit).
   bool attn_attr_set[13] = {};
   bool lm_attr_set = false;    // the same for the LM-head kernel
-  bool topm_attr_set = false;  // and for the streaming top-m kernel
+  bool topm_attr_set = false;  // and for the kernels that stream logits
+  bool sample_attr_set = false;
   int attn_resident[4][9] = {};
 };
 
@@ -67,6 +68,12 @@ void tree_attn_tc_release(falcon_ctx* ctx);
 
 #ifdef __CUDACC__
 constexpr float kLog2e = 1.4426950408889634f;
+
+// The number of the thread's warp, by way of a shuffle: the compiler then knows that it is the same in all
+// lanes and that branches on it are taken by whole warps.  With threadIdx.x / 32 it does not, and every
+// warp-wide operation inside such a branch first gathers the lanes, which takes about 200 cycles (a
+// five-step warp reduction 1000 instead of 150).
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x) >> 5, 0); }
 
 __device__ __forceinline__ void dev_status_or(int32_t* status, int b, int bits) {
   if (status != nullptr) atomicOr(&status[b], bits);

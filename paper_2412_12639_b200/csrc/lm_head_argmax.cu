@@ -101,7 +101,7 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_con
   volatile int* s_last = reinterpret_cast<volatile int*>(small + 8 * kLmNumBars + 8);
   auto bar = [&](int i) { return bars + 8u * static_cast<uint32_t>(i); };
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
   const int cta = blockIdx.x, n_cta = gridDim.x;
   const int S = p.n_stages;
   const int v_lo = cta * p.span, v_hi = min(p.vocab, v_lo + p.span);

@@ -5,7 +5,7 @@
 #include <cfloat>
 #include <climits>
 
-#include "common.cuh"
+#include "row_stream.cuh"
 
 namespace falcon {
 namespace {
@@ -31,8 +31,7 @@ struct AcceptParams {
   // non-greedy only
   float inv_t_log2e;       // log2(e) / temperature
   const float* uniforms;   // [N]
-  float* part_sum;         // [N, chunks] sum of exp((x - chunk max) / temperature)
-  int* row_tickets;        // [N]
+  int32_t slices;          // per CTA: see tree_sample_kernel
 };
 
 struct Best {
@@ -53,21 +52,40 @@ __device__ __forceinline__ void take(Best& s, float x, int i) {
   }
 }
 
+// A node's parent and drafted token, for the thread that has it in the search below: loaded early, where the
+// trip to L2 is hidden.
+struct NodeOf {
+  int parent, token;
+};
+__device__ __forceinline__ NodeOf load_node(const AcceptParams& p, int base, int T_real) {
+  NodeOf n{0, 0};
+  if (static_cast<int>(threadIdx.x) < min(T_real, FALCON_T_MAX)) {
+    n.parent = p.parent[base + threadIdx.x];
+    n.token = p.token[base + threadIdx.x];
+  }
+  return n;
+}
+
 // The longest accepted path of sequence b from the nodes' argmax tokens: thread tid < T brings
-// g = the argmax of node tid; every thread of the CTA calls this.
-__device__ __forceinline__ void search_tree(const AcceptParams& p, int b, int base, int T_real, int g, int* s_par, int* s_tok,
-                                            int* s_g, int* s_key) {
+// g = the argmax of node tid and the node itself; every (working) thread of the CTA calls this.
+__device__ __forceinline__ void search_tree(const AcceptParams& p, int b, int base, int T_real, int g, NodeOf node, int* s_par,
+                                            int* s_tok, int* s_g, int* s_key) {
   const int tid = threadIdx.x;
   const int T = min(T_real, FALCON_T_MAX);
   bool bad = (T_real > FALCON_T_MAX);
   if (tid < T) {
     s_g[tid] = g;
-    const int pr = p.parent[base + tid];
+    const int pr = node.parent;
     s_par[tid] = pr;
-    s_tok[tid] = p.token[base + tid];
+    s_tok[tid] = node.token;
     bad = bad || ((tid == 0) ? (pr != -1) : (pr < 0 || pr >= tid));
   }
-  const int any_bad = __syncthreads_or(bad ? 1 : 0);
+  // (barriers of the 256 working threads: one of the kernels has a warp more, which has left)
+  int any_bad;
+  asm volatile("{ .reg .pred p, q; setp.ne.s32 p, %1, 0; barrier.cta.red.or.pred q, 1, %2, p; selp.s32 %0, 1, 0, q; }"
+               : "=r"(any_bad)
+               : "r"(bad ? 1 : 0), "n"(kAcceptThreads)
+               : "memory");
 
   // alive(c): every non-root node on the chain root..c carries the argmax of its parent
   int key = -1;
@@ -86,7 +104,7 @@ __device__ __forceinline__ void search_tree(const AcceptParams& p, int b, int ba
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) key = max(key, __shfl_xor_sync(0xffffffffu, key, o));
   if ((tid & 31) == 0) s_key[tid >> 5] = key;
-  __syncthreads();
+  asm volatile("bar.sync 1, %0;" ::"n"(kAcceptThreads) : "memory");
   key = s_key[0];
 #pragma unroll
   for (int w = 1; w < kAcceptThreads / 32; ++w) key = max(key, s_key[w]);
@@ -154,6 +172,7 @@ __global__ void __launch_bounds__(kAcceptThreads) tree_accept_kernel(const Accep
     const int t0 = b0 + 4 * nvec;
     if (tid < c1 - t0) take(mine, __ldcs(rowp + t0 + tid), t0 + tid);
   }
+  const NodeOf node = load_node(p, base, T_real);  // (used by the last CTA only; on the way during the reduction)
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     Best other{__shfl_xor_sync(0xffffffffu, mine.v, o), __shfl_xor_sync(0xffffffffu, mine.i, o)};
@@ -196,7 +215,7 @@ __global__ void __launch_bounds__(kAcceptThreads) tree_accept_kernel(const Accep
     g = (r.i == kNone) ? 0 : r.i;
     p.argmax_out[base + tid] = g;
   }
-  search_tree(p, b, base, T_real, g, s_par, s_tok, s_g, s_key);
+  search_tree(p, b, base, T_real, g, node, s_par, s_tok, s_g, s_key);
   if (tid == 0) p.tickets[b] = 0;  // ready for the next call
 }
 
@@ -210,237 +229,247 @@ __global__ void __launch_bounds__(kAcceptThreads) tree_search_kernel(const Accep
   const int base = p.node_off[b];
   const int T_real = p.node_off[b + 1] - base;
   const int g = tid < min(T_real, FALCON_T_MAX) ? p.argmax_out[base + tid] : 0;
-  search_tree(p, b, base, T_real, g, s_par, s_tok, s_g, s_key);
+  search_tree(p, b, base, T_real, g, load_node(p, base, T_real), s_par, s_tok, s_g, s_key);
 }
 
 // ---------------------------------------------------------------------------------------------
 // Non-greedy acceptance: g[i] is the target's own draw from softmax(logits[i] / temperature)
 // (Section 3.1: the next token is sampled from the LM head's distribution) by the inverse-CDF rule
 // with the caller's uniform u[i]: the lowest v whose partial sum of weights exceeds u[i] times the
-// total.  One launch.  Every CTA takes one chunk (at most 4096 entries, in registers) of one row:
-// chunk maximum, then the chunk's sum of weights relative to it.  The last CTA of a row to finish
-// (counter) rescales the chunks' sums to the row maximum, finds the chunk in which the partial sums
-// pass the target, loads that chunk again (L2) and finds the position: warp by warp, then row of
-// 32 by row, then by a scan over the lanes.  The last row of a sequence (second counter) runs the
-// same path search as the greedy call.  fp32 sums: a draw within rounding of a boundary between
-// two tokens may fall on either side.
-constexpr int kSamplePerLane = 16;
-constexpr int kSampleChunkMax = (kAcceptThreads / 32) * 32 * kSamplePerLane;  // 4096
+// total.  One launch, one cluster of up to eight CTAs per row; bound by reading the logits once (4 N V
+// bytes; 411 rows of 32000: 25 us with a round trip to scratch memory per row and the logits in
+// registers, 13 us streamed).  The row goes through shared memory in stages; a warp takes a slice of
+// 1024 entries of each and leaves the slice's maximum and its sum of weights relative to it in every CTA
+// of the row.  Each CTA rescales the slices' sums to the row maximum and finds the slice in which the
+// partial sums pass the target; the CTA it belongs to, which mostly still has it in shared memory, finds
+// the position: lane by lane, then entry by entry.  The last row of a sequence (counter) runs the same path search as the greedy call.  fp32 sums: a draw
+// within rounding of a boundary between two tokens may fall on either side.
+constexpr int kSlice = 32 * kStreamLane;                 // 1024: one warp's share of a stage
+constexpr int kMaxSlices = 320;                          // of a row (262144 entries, plus two edges per CTA)
+constexpr int kSampleMaxCluster = 8;
+constexpr int kMaxSampleVocab = 262144;
 
 __device__ __forceinline__ float warp_add(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
+__device__ __forceinline__ float warp_max(float v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+  return v;
+}
+__device__ __forceinline__ float warp_scan(float v, int lane) {
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const float t = __shfl_up_sync(0xffffffffu, v, o);
+    if (lane >= o) v += t;
+  }
+  return v;
+}
+// weight of logit x relative to a finite maximum m (NaN and -inf: 0)
+__device__ __forceinline__ float weight(float x, float m, float kq) { return tc::ex2((fmaxf(x, -INFINITY) - m) * kq); }
 
-__global__ void __launch_bounds__(kAcceptThreads) tree_sample_kernel(const AcceptParams p) {
-  constexpr int kWarps = kAcceptThreads / 32;
-  __shared__ Best warp_best[kWarps];
-  __shared__ float s_wsum[kWarps];
-  __shared__ float s_scaled[64];
-  __shared__ float s_bcast[4];
-  __shared__ int s_ibcast[4];
+__global__ void __launch_bounds__(kStreamThreads + 32, 3) tree_sample_kernel(const AcceptParams p) {
+  extern __shared__ __align__(128) unsigned char stream_buf[];
+  __shared__ __align__(8) StreamBars bars;
+  __shared__ float2 s_slice[kMaxSlices];  // (maximum, sum) of every slice of the row
+  __shared__ __align__(16) float s_w[kStreamLane + 4];
   __shared__ int s_flag;
   __shared__ int s_par[FALCON_T_MAX], s_tok[FALCON_T_MAX], s_g[FALCON_T_MAX];
-  __shared__ int s_key[kWarps];
+  __shared__ int s_key[kAcceptThreads / 32];
+  static_assert(kStreamThreads == kAcceptThreads, "the path search counts on 256 working threads");
 
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  const int row = blockIdx.y, chunk = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const float* rowp = p.logits + static_cast<int64_t>(row) * p.logits_stride;
-  int lo = 0, hi = p.batch;
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (p.node_off[mid] <= row) lo = mid; else hi = mid;
-  }
-  const int b = lo;
-  const int base = p.node_off[b];
-  const int T_real = p.node_off[b + 1] - base;
+  const int row = blockIdx.y, rank = blockIdx.x, n_ctas = gridDim.x;
+  const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
   const float kq = p.inv_t_log2e;
+  const float* rowp = p.logits + static_cast<int64_t>(row) * p.logits_stride;
+  auto stretch = [&](int r) { return max(0, min(p.vocab, (r + 1) * p.chunk_len) - r * p.chunk_len); };
+  const RowStream rs(rowp + rank * p.chunk_len, stretch(rank), stream_buf, &bars);
+  if (tid == kStreamThreads) RowStream::init(&bars);
+  __syncthreads();
+  if (n_ctas > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");  // "this CTA runs"
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (warp == kStreamWarps) {  // (gone by the time of the next barrier: all copies have landed then)
+    if (lane == 0) rs.produce(0, rs.stages());
+    return;
+  }
+  // sequence that owns this row (its loads overlap the scan below)
+  int b = 0;
+  for (int hi = p.batch; hi - b > 1;) {
+    const int mid = (b + hi) >> 1;
+    if (p.node_off[mid] <= row) b = mid; else hi = mid;
+  }
+  const int base = p.node_off[b], T_real = p.node_off[b + 1] - base;
+  auto worker_sync = [] { asm volatile("bar.sync 1, %0;" ::"n"(kStreamThreads) : "memory"); };
 
-  // entry k of lane l of warp w is element w * 512 + k * 32 + l of the chunk (coalesced rows of 32)
-  auto load_chunk = [&](int ch, float (&x)[kSamplePerLane], bool streaming) {
-    const int c0 = ch * p.chunk_len;
-    const int n = min(p.vocab, c0 + p.chunk_len) - c0;
-#pragma unroll
-    for (int k = 0; k < kSamplePerLane; ++k) {
-      const int j = warp * (32 * kSamplePerLane) + k * 32 + lane;
-      x[k] = j < n ? (streaming ? __ldcs(rowp + c0 + j) : __ldcg(rowp + c0 + j)) : __int_as_float(0x7fc00000);  // NaN = no entry
+  // ---- every CTA: its slices' maxima and sums; slice 0 is the entries before the copies, the last one those after ----
+  const int n_st = rs.stages();
+  const uint32_t table = tc::smem_u32(s_slice) + rank * p.slices * 8;
+  auto put = [&](int slice, float m, float sum) {  // (every lane has the values: lane r stores them in CTA r)
+    if (lane < n_ctas) {
+      uint32_t to = table + slice * 8;
+      if (n_ctas > 1) asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(to) : "r"(to), "r"(lane));
+      asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(to), "f"(m), "f"(sum) : "memory");
     }
-    return c0;
   };
-
-  // ---- every CTA: the chunk's maximum (and where it first occurs) and its sum of weights ----
-  {
-    float x[kSamplePerLane];
-    const int c0 = load_chunk(chunk, x, true);
-    Best mine{-INFINITY, kNone};
-#pragma unroll
-    for (int k = 0; k < kSamplePerLane; ++k) take(mine, x[k], c0 + warp * (32 * kSamplePerLane) + k * 32 + lane);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      Best other{__shfl_xor_sync(0xffffffffu, mine.v, o), __shfl_xor_sync(0xffffffffu, mine.i, o)};
-      mine = merge(mine, other);
+  const NodeOf node = load_node(p, base, T_real);
+  const float uniform = p.uniforms[row];
+  if (n_ctas > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  if (warp == 0) {
+#pragma unroll 1
+    for (int side = 0; side < 2; ++side) {
+      const int n_e = side ? rs.tail : rs.head;
+      float m = -INFINITY, sum = 0.f;
+      if (n_e > 0) {
+        const float x = lane < n_e ? rs.base[(side ? rs.body : -rs.head) + lane] : -INFINITY;
+        m = warp_max(x);
+        sum = warp_add(m > -INFINITY && m < INFINITY ? weight(x, m, kq) : 0.f);
+      }
+      put(side ? p.slices - 1 : 0, m, sum);
     }
-    if (lane == 0) warp_best[warp] = mine;
-    __syncthreads();
-    Best r = warp_best[0];
+  }
+  for (int st = 0; st < p.slices / kStreamWarps; ++st) {
+    float m = -INFINITY, sum = 0.f;
+    if (st < n_st) {
+      float x[kStreamLane];
+      if (rs.take(st, x)) {
+        if (st + kStreamStages < n_st) rs.give_back(st);
 #pragma unroll
-    for (int w = 1; w < kWarps; ++w) r = merge(r, warp_best[w]);
-    float s = 0.f;
-    if (r.v > -INFINITY && r.v < INFINITY) {
+        for (int k = 0; k < kStreamLane; ++k) m = fmaxf(m, x[k]);
+        m = warp_max(m);
+        if (m > -INFINITY && m < INFINITY) {
 #pragma unroll
-      for (int k = 0; k < kSamplePerLane; ++k)
-        if (x[k] == x[k]) s += exp2f((x[k] - r.v) * kq);
+          for (int k = 0; k < kStreamLane; ++k) sum += weight(x[k], m, kq);
+        }
+        sum = warp_add(sum);
+      } else if (lane == 0) {
+        dev_status_or(p.status, b, FALCON_DEV_TIMEOUT);
+      }
     }
-    s = warp_add(s);
-    if (lane == 0) s_wsum[warp] = s;
-    __syncthreads();
-    if (tid == 0) {
-      float tot = 0.f;
-#pragma unroll
-      for (int w = 0; w < kWarps; ++w) tot += s_wsum[w];
-      const int64_t o = static_cast<int64_t>(row) * p.chunks + chunk;
-      p.part_val[o] = r.v;
-      p.part_sum[o] = tot;
-      p.part_idx[o] = r.i;
-      __threadfence();
-      s_flag = (atomicAdd(&p.row_tickets[row], 1) == p.chunks - 1);
-    }
-    __syncthreads();
-    if (!s_flag) return;
-    __threadfence();
+    put(1 + st * kStreamWarps + warp, m, sum);
+  }
+  if (n_ctas > 1) {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  } else {
+    worker_sync();
   }
 
-  // ---- last CTA of the row: the chunk in which the partial sums pass u * total ----
-  if (tid == 0) {
-    const int64_t o = static_cast<int64_t>(row) * p.chunks;
+  // ---- the slice in which the partial sums pass u * total (every CTA, the same arithmetic), then the position in
+  // it (the CTA that has it) ----
+  if (tid == 0) s_flag = 0;
+  if (warp == 0) {
+    // Serial work of one warp: every step is a scan or a ballot over the lanes, nothing walks through
+    // entries one by one (a lane that did took 70 cycles an entry).
+    const int n_sl = n_ctas * p.slices;
     float M = -INFINITY;
-    for (int c = 0; c < p.chunks; ++c) M = fmaxf(M, __ldcg(p.part_val + o + c));
-    int direct = -1, cstar = 0;
-    float resid = 0.f;
-    if (!(M > -INFINITY)) {
-      direct = 0;  // nothing to draw from
-    } else if (!(M < INFINITY)) {
-      for (int c = 0; c < p.chunks && direct < 0; ++c)  // a +inf logit takes everything: its first position
-        if (__ldcg(p.part_val + o + c) == M) direct = __ldcg(p.part_idx + o + c);
-    } else {
-      float total = 0.f;
-      for (int c = 0; c < p.chunks; ++c) {
-        const float mc = __ldcg(p.part_val + o + c);
-        const float sc = mc > -INFINITY ? __ldcg(p.part_sum + o + c) * exp2f((mc - M) * kq) : 0.f;
-        s_scaled[c] = sc;
-        total += sc;
-      }
-      const float target = p.uniforms[row] * total;
-      float run = 0.f;
-      int last = 0;
-      cstar = -1;
-      for (int c = 0; c < p.chunks; ++c) {
-        const float sc = s_scaled[c];
-        if (sc > 0.f) last = c;
-        if (run + sc > target) {
-          cstar = c;
+    for (int i0 = 0; i0 < n_sl; i0 += 32)
+      if (i0 + lane < n_sl) M = fmaxf(M, s_slice[i0 + lane].x);
+    M = warp_max(M);
+    const bool inf = M == INFINITY;  // a +inf logit takes everything: its first position
+    // (maximum, sum) -> (partial sum up to and with the slice, its weight)
+    float total = 0.f;
+    for (int i0 = 0; i0 < n_sl; i0 += 32) {
+      const float2 v = i0 + lane < n_sl ? s_slice[i0 + lane] : make_float2(-INFINITY, 0.f);
+      const float w = v.x > -INFINITY ? (inf ? (v.x == M ? 1.f : 0.f) : v.y * tc::ex2((v.x - M) * kq)) : 0.f;
+      const float upto = total + warp_scan(w, lane);
+      if (i0 + lane < n_sl) s_slice[i0 + lane] = make_float2(upto, w);
+      total = __shfl_sync(0xffffffffu, upto, 31);
+    }
+    // (with rounding the target may reach the total: the last slice that has weight then)
+    const float target = inf ? 0.f : fminf(uniform * total, total);
+    int g = 0, owner = 0;
+    if (M > -INFINITY) {
+      int slice = 0;
+      for (int i0 = 0; i0 < n_sl; i0 += 32) {
+        const float2 v = i0 + lane < n_sl ? s_slice[i0 + lane] : make_float2(0.f, 0.f);
+        const unsigned pass = __ballot_sync(0xffffffffu, v.y > 0.f && v.x > target), any = __ballot_sync(0xffffffffu, v.y > 0.f);
+        if (any) slice = i0 + 31 - __clz(static_cast<int>(any));
+        if (pass) {
+          slice = i0 + __ffs(static_cast<int>(pass)) - 1;
           break;
         }
-        run += sc;
       }
-      if (cstar < 0) {  // rounding left the target at or past the total: the end of the last chunk that has weight
-        cstar = last;
-        run -= s_scaled[last];
-      }
-      resid = target - run;
-    }
-    s_ibcast[0] = direct;
-    s_ibcast[1] = cstar;
-    s_bcast[0] = resid;
-    s_bcast[1] = M;
-    p.row_tickets[row] = 0;  // ready for the next call
-  }
-  __syncthreads();
-  int g = s_ibcast[0];
-  if (g < 0) {
-    // ---- the position inside that chunk: warp, then row of 32, then lane ----
-    const int cstar = s_ibcast[1];
-    const float M = s_bcast[1];
-    float x[kSamplePerLane], w[kSamplePerLane];
-    const int c0 = load_chunk(cstar, x, false);
-    float ws = 0.f;
+      const float before = slice > 0 ? s_slice[slice - 1].x : 0.f;
+      owner = slice / p.slices;
+      if (owner == rank) {
+        // its entries, 32 in a row for each lane (the edges have at most three)
+        const int k = slice - owner * p.slices, st = (k - 1) / kStreamWarps;
+        const bool edge = k == 0 || k == p.slices - 1;
+        const int first = rank * p.chunk_len + (k == 0 ? 0 : k == p.slices - 1 ? rs.head + rs.body : rs.head + (k - 1) * kSlice);
+        const int count = k == 0 ? rs.head : k == p.slices - 1 ? rs.tail : min(kSlice, rs.body - (k - 1) * kSlice);
+        const int at = lane * kStreamLane;
+        float x[kStreamLane];
 #pragma unroll
-    for (int k = 0; k < kSamplePerLane; ++k) {
-      w[k] = (x[k] == x[k]) ? exp2f((x[k] - M) * kq) : 0.f;
-      ws += w[k];
-    }
-    ws = warp_add(ws);
-    if (lane == 0) s_wsum[warp] = ws;
-    __syncthreads();
-    // every thread: which warp (the sums are the same in all of them)
-    float resid = s_bcast[0], tot = 0.f;
+        for (int e = 0; e < kStreamLane; ++e) x[e] = -INFINITY;
+        if (edge) {
 #pragma unroll
-    for (int i = 0; i < kWarps; ++i) tot += s_wsum[i];
-    resid = fminf(resid, tot * 0.99999f);  // recomputed with the row maximum the chunk may sum to a hair less
-    int wstar = -1, wlast = 0;
-    float run = 0.f;
+          for (int e = 0; e < 3; ++e)
+            if (at + e < count) x[e] = __ldcg(rowp + first + at + e);
+        } else {
+          const bool here = st + kStreamStages >= n_st;  // among the last stages, which are still in shared memory
+          const float4* have = reinterpret_cast<const float4*>(stream_buf) + (st % kStreamStages) * (kStreamStage / 4) +
+                               ((k - 1) % kStreamWarps) * (kSlice / 4) + lane * (kStreamLane / 4);
+          const float4* far = reinterpret_cast<const float4*>(rowp + first + at);
+          float4 v[kStreamLane / 4];
+          if (here) {
 #pragma unroll
-    for (int i = 0; i < kWarps; ++i) {
-      const float v = s_wsum[i];
-      if (v > 0.f) wlast = i;
-      if (wstar < 0) {
-        if (run + v > resid) wstar = i; else run += v;
-      }
-    }
-    if (wstar < 0) {
-      wstar = wlast;
-      run -= s_wsum[wlast];
-    }
-    if (warp == wstar) {
-      float rw = fminf(resid - run, s_wsum[wstar] * 0.99999f);
-      int kstar = -1, klast = 0;
-      float wk = 0.f, before = 0.f, acc = 0.f;
-#pragma unroll
-      for (int k = 0; k < kSamplePerLane; ++k) {
-        const float rs = warp_add(w[k]);
-        if (rs > 0.f) klast = k;
-        if (kstar < 0) {
-          if (acc + rs > rw) {
-            kstar = k;
-            before = acc;
+            for (int j = 0; j < kStreamLane / 4; ++j) v[j] = have[j];
           } else {
-            acc += rs;
+#pragma unroll
+            for (int j = 0; j < kStreamLane / 4; ++j)
+              if (at + 4 * j < count) v[j] = __ldcg(far + j);
           }
+#pragma unroll
+          for (int j = 0; j < kStreamLane / 4; ++j)
+            if (at + 4 * j < count) {
+              x[4 * j] = v[j].x;
+              x[4 * j + 1] = v[j].y;
+              x[4 * j + 2] = v[j].z;
+              x[4 * j + 3] = v[j].w;
+            }
         }
-      }
-      if (kstar < 0) kstar = klast;
+        float w0 = 0.f, w1 = 0.f, w2 = 0.f, w3 = 0.f;
 #pragma unroll
-      for (int k = 0; k < kSamplePerLane; ++k)
-        if (k == kstar) wk = w[k];
-      const float rsel = warp_add(wk);  // (if no row passed the target, `before` is 0 and the clamp below ends the search
-                                        // at the last entry of the last row that has weight)
-      float incl = wk;
+        for (int e = 0; e < kStreamLane; ++e) x[e] = tc::ex2(inf ? (x[e] == M ? 0.f : -INFINITY) : (fmaxf(x[e], -INFINITY) - M) * kq);
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const float t = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += t;
+        for (int e = 0; e < kStreamLane; e += 4) {
+          w0 += x[e];
+          w1 += x[e + 1];
+          w2 += x[e + 2];
+          w3 += x[e + 3];
+        }
+        const float ws = (w0 + w1) + (w2 + w3);
+        const float in = warp_scan(ws, lane), tot = __shfl_sync(0xffffffffu, in, 31);
+        const float resid = fminf(target - before, tot * 0.99999f);  // (summed another way the slice may come to a hair less)
+        const unsigned pl = __ballot_sync(0xffffffffu, ws > 0.f && in > resid), al = __ballot_sync(0xffffffffu, ws > 0.f);
+        const int wl = pl ? __ffs(static_cast<int>(pl)) - 1 : (al ? 31 - __clz(static_cast<int>(al)) : 0);
+        // that lane's 32 weights dealt out over the lanes
+        if (lane == wl) {
+#pragma unroll
+          for (int e = 0; e < kStreamLane; e += 4) *reinterpret_cast<float4*>(s_w + e) = make_float4(x[e], x[e + 1], x[e + 2], x[e + 3]);
+          s_w[kStreamLane] = in - ws;
+        }
+        __syncwarp();
+        const float we = s_w[lane], acc = s_w[kStreamLane] + warp_scan(we, lane);
+        const unsigned pe = __ballot_sync(0xffffffffu, we > 0.f && acc > resid), ae = __ballot_sync(0xffffffffu, we > 0.f);
+        const int found = pe ? __ffs(static_cast<int>(pe)) - 1 : (ae ? 31 - __clz(static_cast<int>(ae)) : 0);
+        g = first + wl * kStreamLane + found;
       }
-      const float rl = fminf(rw - before, rsel * 0.99999f);
-      const unsigned pass = __ballot_sync(0xffffffffu, wk > 0.f && incl > rl);
-      const unsigned any = __ballot_sync(0xffffffffu, wk > 0.f);
-      const int lstar = pass ? __ffs(static_cast<int>(pass)) - 1 : (any ? 31 - __clz(static_cast<int>(any)) : 0);
-      if (lane == 0) s_ibcast[2] = c0 + wstar * (32 * kSamplePerLane) + kstar * 32 + lstar;
     }
-    __syncthreads();
-    g = s_ibcast[2];
+    if (owner == rank && lane == 0) {
+      p.argmax_out[row] = g;
+      __threadfence();
+      s_flag = (atomicAdd(&p.tickets[b], 1) == T_real - 1);
+    }
   }
-  if (tid == 0) {
-    p.argmax_out[row] = g;
-    __threadfence();
-    s_flag = (atomicAdd(&p.tickets[b], 1) == T_real - 1);
-  }
-  __syncthreads();
+  worker_sync();
   if (!s_flag) return;
   __threadfence();
   // ---- last row of sequence b: the path search on the drawn tokens ----
   const int gt = tid < min(T_real, FALCON_T_MAX) ? __ldcg(p.argmax_out + base + tid) : 0;
-  search_tree(p, b, base, T_real, gt, s_par, s_tok, s_g, s_key);
+  search_tree(p, b, base, T_real, gt, node, s_par, s_tok, s_g, s_key);
   if (tid == 0) p.tickets[b] = 0;  // ready for the next call
 }
 
@@ -485,8 +514,7 @@ AcceptParams accept_params(const falcon_accept_args& a, int chunks, int chunk_le
   p.tickets = tickets;
   p.inv_t_log2e = 0.f;
   p.uniforms = nullptr;
-  p.part_sum = nullptr;
-  p.row_tickets = nullptr;
+  p.slices = 0;
   return p;
 }
 
@@ -523,34 +551,38 @@ int launch_tree_accept(falcon_ctx* ctx, const falcon_accept_args& a, cudaStream_
 int launch_tree_sample(falcon_ctx* ctx, const falcon_accept_args& a, cudaStream_t s) {
   const int N = a.tree.total_nodes, B = a.tree.batch;
   if (N > 65535) return FALCON_ERR_CAPACITY;
-  int chunks, chunk_len;
-  accept_plan(ctx->sm_count, N, a.vocab, &chunks, &chunk_len);
-  const int min_chunks = (a.vocab + kSampleChunkMax - 1) / kSampleChunkMax;  // a chunk is held in registers
-  if (chunks < min_chunks) chunks = min_chunks;
-  if (chunks > kAcceptMaxChunks) return FALCON_ERR_CAPACITY;
-  chunk_len = ((a.vocab + chunks - 1) / chunks + 3) & ~3;
-  chunks = (a.vocab + chunk_len - 1) / chunk_len;
-
-  const size_t part = static_cast<size_t>(N) * chunks;
-  int rc = ensure_workspace(ctx, part * 12 + 256);
+  if (a.vocab > kMaxSampleVocab) return FALCON_ERR_CAPACITY;
+  // CTAs per row: as many as are resident at once (three per SM) while each has a few slices of its own
+  int ctas = 1;
+  while (ctas < kSampleMaxCluster && static_cast<int64_t>(N) * 2 * ctas <= 3 * ctx->sm_count && a.vocab > 2 * ctas * kSlice) ctas *= 2;
+  const int chunk_len = ((a.vocab + ctas - 1) / ctas + 3) & ~3;
+  int rc = ensure_tickets(ctx, static_cast<size_t>(B), s);
   if (rc) return rc;
-  rc = ensure_tickets(ctx, static_cast<size_t>(B) + N, s);
-  if (rc) return rc;
-  AcceptParams p = accept_params(a, chunks, chunk_len, ctx->ws, ctx->tickets);
-  p.part_sum = reinterpret_cast<float*>(p.part_idx + part);
-  p.row_tickets = ctx->tickets + B;
+  AcceptParams p = accept_params(a, 1, chunk_len, nullptr, ctx->tickets);
+  p.slices = kStreamWarps * ((chunk_len + kStreamStage - 1) / kStreamStage) + 2;
   p.uniforms = a.uniforms;
   p.inv_t_log2e = kLog2e / a.temperature;
+  if (ctas * p.slices > kMaxSlices) return FALCON_ERR_CAPACITY;  // (not reached: 8 x 34 and 258 at most)
 
+  if (!ctx->sample_attr_set) {
+    const cudaError_t e = cudaFuncSetAttribute(tree_sample_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kStreamBytes));
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute(tree_sample_kernel)");
+    ctx->sample_attr_set = true;
+  }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(chunks, N);
-  cfg.blockDim = dim3(kAcceptThreads);
+  cfg.gridDim = dim3(ctas, N);
+  cfg.blockDim = dim3(kStreamThreads + 32);
+  cfg.dynamicSmemBytes = kStreamBytes;
   cfg.stream = s;
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = ctas;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = ctas > 1 ? 2 : 1;
   cudaError_t e = cudaLaunchKernelEx(&cfg, tree_sample_kernel, p);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "tree_sample_kernel launch");
   return FALCON_OK;

@@ -147,7 +147,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem_gen + C::kOffMisc + 4);
   auto bar = [&](int i) { return smem_base + C::kOffBars + 8u * static_cast<uint32_t>(i); };
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
   FALCON_TRACE(tid == 0, 0);
   const int n_splits = gridDim.x, split = blockIdx.x;  // cluster = all CTAs of a row of the grid
   const int kvh = blockIdx.y % p.Hkv, unit = blockIdx.y / p.Hkv;

@@ -295,7 +295,7 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
   const uint32_t tmem_cols = (kVar == 0 || p.n_rows <= 64) ? 256u : 512u, col_stride = tmem_cols / 4;  // S^T(0), S^T(1), O^T
   auto bar = [&](int i) { return bars + 8u * static_cast<uint32_t>(i); };
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
   const int n_splits = gridDim.x, split = blockIdx.x;  // cluster = all CTAs of a row of the grid
   const int kvh = blockIdx.y % p.Hkv, mtile = blockIdx.y / p.Hkv;
   const int b = p.have_host ? p.h_order[blockIdx.z] : static_cast<int>(blockIdx.z);

@@ -60,7 +60,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerCta) tree_attn_warp_kernel(const
   // Under programmatic dependent launch the grid may start while the previous kernel of the stream
   // drains: nothing is read or written before that kernel has completed.
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
   const int h = blockIdx.x, node = blockIdx.y, b = blockIdx.z;
   // With the caller's host copies of the per-sequence scalars nothing has to be fetched before the
   // addresses are known, and the query row, the tree's parent array and every thread's first key are

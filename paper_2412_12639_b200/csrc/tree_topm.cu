@@ -288,7 +288,7 @@ __device__ __forceinline__ void find_tau(TopmShared& sh, int m, int warp, int la
 // The CTA's list thinned in place by a threshold of its own (64 groups of its entries, dealt out evenly):
 // at least m of them stay.  Every thread of the CTA calls this.  Returns the threshold.
 __device__ __forceinline__ uint32_t thin_list(TopmShared& sh, int m, int tid) {
-  const int warp = tid >> 5, lane = tid & 31, n = sh.cnt;
+  const int warp = warp_index(), lane = tid & 31, n = sh.cnt;
   const uint64_t e0 = tid < n ? sh.list[tid] : 0ull, e1 = tid + kTopmThreads < n ? sh.list[tid + kTopmThreads] : 0ull;
   if (tid < kTopmGroups) sh.max[tid] = 0u;
   if (tid == 0) sh.tau = 0xffffffffu;
@@ -312,7 +312,7 @@ __device__ __forceinline__ uint32_t thin_list(TopmShared& sh, int m, int tid) {
 // each).  Every thread of the cluster calls this, with CTA 0's shared memory still there.
 template <int kRows>
 __device__ __noinline__ void exact_entries(const TopmParams& p, TopmShared& sh, const float* rowp, int n, int c0, int rank) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, m = p.m;
+  const int warp = warp_index(), lane = threadIdx.x & 31, m = p.m;
   auto from_list = [&](const uint32_t* lk, const int* li, int fill, uint32_t (&key)[kTopmPerLane], int (&id)[kTopmPerLane]) {
 #pragma unroll
     for (int k = 0; k < kTopmPerLane; ++k) {
@@ -459,7 +459,7 @@ template <int kRows>
 __global__ void __launch_bounds__(kTopmThreads, kRows <= 8 ? 6 : (kRows <= 16 ? 4 : 3)) tree_topm_kernel(const __grid_constant__ TopmParams p) {
   __shared__ __align__(16) TopmShared sh;
   const int row = blockIdx.y, rank = blockIdx.x, n_ctas = gridDim.x;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
   const int c0 = rank * p.chunk_len;
   const int n = max(0, min(p.vocab, c0 + p.chunk_len) - c0);
   const float* rowp = p.logits + static_cast<int64_t>(row) * p.logits_stride + c0;
@@ -499,7 +499,7 @@ __global__ void __launch_bounds__(kStreamThreads + 32, 3) tree_topm_stream_kerne
   __shared__ __align__(8) StreamBars bars;
   static_assert(kStreamThreads == kTopmThreads, "the list passes count on 256 working threads");
   const int row = blockIdx.y, rank = blockIdx.x, n_ctas = gridDim.x;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
   const int m = p.m, c0 = rank * p.chunk_len;
   const int n = max(0, min(p.vocab, c0 + p.chunk_len) - c0);
   const float* rowp = p.logits + static_cast<int64_t>(row) * p.logits_stride + c0;
