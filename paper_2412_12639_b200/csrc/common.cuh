@@ -32,9 +32,6 @@ struct falcon_ctx {
   // (0 = not asked yet, -1 = none).  Index 0: rows-on-lanes kernel; from 1: the keys-on-lanes kernel's
   // three variants (times head dimension and place of the tree's K/V for the limit).
   bool attn_attr_set[13] = {};
-  bool lm_attr_set = false;    // the same for the LM-head kernel
-  bool topm_attr_set = false;  // and for the kernels that stream logits
-  bool sample_attr_set = false;
   int attn_resident[4][9] = {};
 };
 
@@ -43,6 +40,19 @@ namespace falcon {
 int ensure_workspace(falcon_ctx* ctx, size_t bytes);
 int ensure_tickets(falcon_ctx* ctx, size_t count, cudaStream_t stream);
 int cuda_fail(falcon_ctx* ctx, cudaError_t e, const char* where);
+// Every kernel of the library asks for the largest shared-memory share of an SM, whatever it uses itself: an SM
+// that goes from a kernel with another share to one of the attention kernels has to drain first.
+template <class Kernel>
+cudaError_t prefer_shared(Kernel kernel) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+}
+// Kernel attributes of one file, set when a context is created (its device is current).
+cudaError_t set_up_accept();
+cudaError_t set_up_compact();
+cudaError_t set_up_topm();
+cudaError_t set_up_lm_head();
+cudaError_t set_up_attn_warp();
+cudaError_t set_up_attn_simt();
 int check_tree_desc(const falcon_tree_desc& t, bool need_token);
 
 // launchers (one per kernel file)

@@ -69,6 +69,8 @@ int falcon_create(falcon_ctx** out, int device) {
   e = cudaGetDeviceProperties(&prop, device);
   if (e != cudaSuccess) return FALCON_ERR_CUDA;
   if (prop.major != 10) return FALCON_ERR_UNSUPPORTED;  // built for sm_100a only
+  for (auto set_up : {set_up_accept, set_up_compact, set_up_topm, set_up_lm_head, set_up_attn_warp, set_up_attn_simt})
+    if (set_up() != cudaSuccess) return FALCON_ERR_CUDA;
   falcon_ctx* ctx = new (std::nothrow) falcon_ctx();
   if (!ctx) return FALCON_ERR_INVALID_ARG;
   ctx->device = device;

@@ -64,6 +64,7 @@ __global__ void __launch_bounds__(kCompactThreads) kv_compact_kernel(const Compa
   // Under programmatic dependent launch the grid may start while the previous kernel of the stream
   // drains: nothing is read or written before that kernel has completed.
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int h = blockIdx.x, b = blockIdx.y;
   const bool gather_slice = p.features != nullptr && static_cast<int>(blockIdx.z) == p.gather_z;
   const int layer = gather_slice ? 0 : (kBoth ? blockIdx.z : (blockIdx.z >> 1));
@@ -158,6 +159,7 @@ __global__ void __launch_bounds__(kCompactThreads) feature_gather_kernel(const C
   __shared__ int s_path[FALCON_T_MAX];
   __shared__ int s_bad;
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int b = blockIdx.y, tid = threadIdx.x;
   const int base = p.node_off[b];
   const int T = p.node_off[b + 1] - base;
@@ -192,6 +194,14 @@ void set_gather(CompactParams& p, const falcon_gather_args& g, const int32_t* to
 }
 
 }  // namespace
+
+cudaError_t set_up_compact() {
+  cudaError_t e = prefer_shared(kv_compact_kernel<kSmallChunksPerThread, true>);
+  if (e == cudaSuccess) e = prefer_shared(kv_compact_kernel<kMidChunksPerThread, true>);
+  if (e == cudaSuccess) e = prefer_shared(kv_compact_kernel<kMaxChunksPerThread, false>);
+  if (e == cudaSuccess) e = prefer_shared(feature_gather_kernel);
+  return e;
+}
 
 int check_gather_args(const falcon_gather_args& g, int max_tree) {
   if (!g.features || !g.features_out || !g.tokens_out) return FALCON_ERR_INVALID_ARG;

@@ -304,6 +304,10 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_con
 
 }  // namespace
 
+cudaError_t set_up_lm_head() {
+  return cudaFuncSetAttribute(lm_head_argmax_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kLmSmemMax));
+}
+
 int launch_lm_head_argmax(falcon_ctx* ctx, const falcon_lm_argmax_args& a, cudaStream_t s) {
   const int N = a.n_rows, V = a.vocab, H = a.hidden;
   const int n_mt = (N + 127) / 128;
@@ -326,13 +330,6 @@ int launch_lm_head_argmax(falcon_ctx* ctx, const falcon_lm_argmax_args& a, cudaS
   if (n_stages < 2) return FALCON_ERR_CAPACITY;
   const uint32_t smem_bytes = static_cast<uint32_t>(n_stages) * stage_bytes + kLmSmallBytes;
 
-
-  if (!ctx->lm_attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(lm_head_argmax_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(kLmSmemMax));
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute(lm_head_argmax_kernel)");
-    ctx->lm_attr_set = true;
-  }
   // scratch that is zero between calls: the arrival counter and one 64-bit word per node
   int rc = ensure_tickets(ctx, 2 + 2 * N, s);
   if (rc) return rc;

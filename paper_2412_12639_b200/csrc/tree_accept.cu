@@ -135,6 +135,7 @@ __global__ void __launch_bounds__(kAcceptThreads) tree_accept_kernel(const Accep
   // Under programmatic dependent launch the grid may start while the previous kernel of the stream
   // drains: nothing is read or written before that kernel has completed.
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int row = blockIdx.y, chunk = blockIdx.x, tid = threadIdx.x;
   const int c0 = chunk * p.chunk_len;
   const int c1 = min(p.vocab, c0 + p.chunk_len);
@@ -225,6 +226,7 @@ __global__ void __launch_bounds__(kAcceptThreads) tree_search_kernel(const Accep
   __shared__ int s_par[FALCON_T_MAX], s_tok[FALCON_T_MAX], s_g[FALCON_T_MAX];
   __shared__ int s_key[kAcceptThreads / 32];
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int b = blockIdx.x, tid = threadIdx.x;
   const int base = p.node_off[b];
   const int T_real = p.node_off[b + 1] - base;
@@ -520,6 +522,14 @@ AcceptParams accept_params(const falcon_accept_args& a, int chunks, int chunk_le
 
 }  // namespace
 
+cudaError_t set_up_accept() {
+  cudaError_t e = prefer_shared(tree_accept_kernel);
+  if (e == cudaSuccess) e = prefer_shared(tree_search_kernel);
+  if (e == cudaSuccess) e = prefer_shared(tree_sample_kernel);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(tree_sample_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kStreamBytes));
+  return e;
+}
+
 int launch_tree_accept(falcon_ctx* ctx, const falcon_accept_args& a, cudaStream_t s) {
   const int N = a.tree.total_nodes;
   if (N > 65535) return FALCON_ERR_CAPACITY;
@@ -564,11 +574,6 @@ int launch_tree_sample(falcon_ctx* ctx, const falcon_accept_args& a, cudaStream_
   p.inv_t_log2e = kLog2e / a.temperature;
   if (ctas * p.slices > kMaxSlices) return FALCON_ERR_CAPACITY;  // (not reached: 8 x 34 and 258 at most)
 
-  if (!ctx->sample_attr_set) {
-    const cudaError_t e = cudaFuncSetAttribute(tree_sample_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kStreamBytes));
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute(tree_sample_kernel)");
-    ctx->sample_attr_set = true;
-  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(ctas, N);
   cfg.blockDim = dim3(kStreamThreads + 32);

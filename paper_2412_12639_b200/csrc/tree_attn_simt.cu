@@ -333,6 +333,12 @@ constexpr size_t simt_smem_bytes() {
 
 }  // namespace
 
+cudaError_t set_up_attn_simt() {
+  cudaError_t e = cudaFuncSetAttribute(tree_attn_simt_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(simt_smem_bytes<128>()));
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(tree_attn_simt_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(simt_smem_bytes<64>()));
+  return e;
+}
+
 int launch_tree_attn_simt(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s) {
   const int B = a.tree.batch, Hq = a.n_q_heads;
   if (B > 65535 || Hq > 65535) return FALCON_ERR_CAPACITY;
@@ -389,13 +395,9 @@ int launch_tree_attn_simt(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream
   cudaError_t e;
   if (a.head_dim == 128) {
     constexpr size_t smem = simt_smem_bytes<128>();
-    e = cudaFuncSetAttribute(tree_attn_simt_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute(simt<128>)");
     tree_attn_simt_kernel<128><<<grid, kThreads, smem, s>>>(p);
   } else {
     constexpr size_t smem = simt_smem_bytes<64>();
-    e = cudaFuncSetAttribute(tree_attn_simt_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute(simt<64>)");
     tree_attn_simt_kernel<64><<<grid, kThreads, smem, s>>>(p);
   }
   e = cudaGetLastError();

@@ -60,6 +60,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerCta) tree_attn_warp_kernel(const
   // Under programmatic dependent launch the grid may start while the previous kernel of the stream
   // drains: nothing is read or written before that kernel has completed.
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
   const int h = blockIdx.x, node = blockIdx.y, b = blockIdx.z;
   // With the caller's host copies of the per-sequence scalars nothing has to be fetched before the
@@ -227,6 +228,11 @@ __global__ void __launch_bounds__(32 * kWarpsPerCta) tree_attn_warp_kernel(const
 }
 
 }  // namespace
+
+cudaError_t set_up_attn_warp() {
+  const cudaError_t e = prefer_shared(tree_attn_warp_kernel<64>);
+  return e == cudaSuccess ? prefer_shared(tree_attn_warp_kernel<128>) : e;
+}
 
 bool tree_attn_warp_supports(const falcon_ctx* ctx, const falcon_attn_args& a) {
   (void)ctx;

@@ -584,6 +584,15 @@ __global__ void __launch_bounds__(kStreamThreads + 32, 3) tree_topm_stream_kerne
 
 }  // namespace
 
+cudaError_t set_up_topm() {
+  cudaError_t e = prefer_shared(tree_topm_kernel<8>);
+  if (e == cudaSuccess) e = prefer_shared(tree_topm_kernel<16>);
+  if (e == cudaSuccess) e = prefer_shared(tree_topm_kernel<kTopmRowsMax>);
+  if (e == cudaSuccess) e = prefer_shared(tree_topm_stream_kernel);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(tree_topm_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kStreamBytes));
+  return e;
+}
+
 int launch_tree_topm(falcon_ctx* ctx, const falcon_topm_args& a, cudaStream_t s) {
   const int N = a.n_rows;
   if (N > 65535) return FALCON_ERR_CAPACITY;
@@ -641,11 +650,6 @@ int launch_tree_topm(falcon_ctx* ctx, const falcon_topm_args& a, cudaStream_t s)
         : per_lane <= 16 ? cudaLaunchKernelEx(&cfg, tree_topm_kernel<16>, p)
                          : cudaLaunchKernelEx(&cfg, tree_topm_kernel<kTopmRowsMax>, p);
   } else {
-    if (!ctx->topm_attr_set) {
-      e = cudaFuncSetAttribute(tree_topm_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kStreamBytes));
-      if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute(tree_topm_stream_kernel)");
-      ctx->topm_attr_set = true;
-    }
     p.steps = (chunk + kTopmThreads * kStreamLane - 1) / (kTopmThreads * kStreamLane);
     cfg.blockDim = dim3(kStreamThreads + 32);
     cfg.dynamicSmemBytes = kStreamBytes;
