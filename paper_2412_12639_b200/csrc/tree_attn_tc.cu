@@ -721,7 +721,9 @@ struct Plan {
 // A CTA costs a fixed part (launch, Q, merge: 4 us, 5 with splits) and its tiles, 64 keys each: 0.92 us
 // with two row blocks (0.75 for 64-wide heads: softmax and MMA issue), with one block 0.73 (0.38)
 // where the K/V stream comes from HBM, at the 45 GB/s that one SM draws, and 0.5 (0.38) where other
-// row blocks' CTAs bring the same tiles into L2.  Units beyond the resident clusters wait for a slot.
+// row blocks' CTAs bring the same tiles into L2.  Units beyond the resident clusters wait for a slot, and a cluster for
+// all of its SMs at once: 4 us more for each (16 sequences of 350-3850 keys, 8 KV heads of 4 query heads: two
+// splits of 256-row units 52 us, no split 64; no split of 128-row units 47, which is what this finds).
 // One sequence's tile height is chosen so that its tiles divide evenly over the splits.
 Plan make_plan(falcon_ctx* ctx, const falcon_attn_args& a) {
   const int B = a.tree.batch, G = a.n_q_heads / a.n_kv_heads;
@@ -751,7 +753,7 @@ Plan make_plan(falcon_ctx* ctx, const falcon_attn_args& a) {
         const bool two = std::min(T, q_nodes) * G > 128;
         const double tile_us = two ? (wide ? 0.92 : 0.75) : wide ? (u > 1 ? 0.5 : 0.73) : 0.38;
         const double t = (s > 1 ? 5.0 : 4.0) + mine * tile_us;
-        total += t * u * a.n_kv_heads * (host ? 1 : B);
+        total += (t + (s > 1 ? 4.0 : 0.0)) * u * a.n_kv_heads * (host ? 1 : B);
         units += static_cast<double>(u) * a.n_kv_heads * (host ? 1 : B);
         longest = std::max(longest, t);
       }
