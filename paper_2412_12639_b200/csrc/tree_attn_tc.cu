@@ -4,6 +4,8 @@
 // Row r of a KV head is (tree node r / G, query head r % G), so grouped-query heads share the K/V
 // stream.  A unit is (sequence, KV head, block of at most 256 query rows); one thread-block cluster per
 // unit, whose CTAs split the key range (prefix + tree) into runs of whole tiles of up to 128 keys.
+// Where there are many units of few tiles, the grid is one CTA per SM instead, which works on one unit after the
+// other (kLoop): the next one's K, V and Q are on their way while the rows of the one before are delivered.
 //
 // Inside a CTA (576 threads) two streams of 128 TMEM lanes each work on tiles in turn, so that one
 // stream's softmax runs under the other's MMAs:
@@ -55,8 +57,10 @@ constexpr int kWarpMma = 1;
 constexpr int kWarpSm0 = 2;
 constexpr int kMaxSplits = 8;
 constexpr int kHostSeqs = 32;
+constexpr int kLoopTiles = 8;      // see launch_impl
 constexpr float kLMin = 7.8886090522101181e-31f;  // 2^-100
 constexpr float kLMax = 1.2676506002282294e+30f;  // 2^100
+constexpr uint32_t kPollLimit = 1u << 24;
 constexpr int kEarlyItems = 2;    // ring slots requested before the grid dependency wait (one K and one V tile)
 
 // Shared memory: the Q block (two 64-column halves for 128-wide heads), the ring, small arrays.
@@ -72,7 +76,8 @@ struct Cfg {
   static constexpr uint32_t kOffPar = kOffRescue + kRowsMax;          // [128] int8: the tree's parent array
   static constexpr uint32_t kOffBars = kOffPar + FALCON_T_MAX;
   static constexpr int kBarKVFull = 0, kBarKVEmpty = kSlots, kBarQ = 2 * kSlots, kBarSFull = kBarQ + 1,
-                       kBarPFull = kBarSFull + 4, kBarODone = kBarPFull + 4, kNumBars = kBarODone + 1;
+                       kBarPFull = kBarSFull + 4, kBarODone = kBarPFull + 4, kBarQFree = kBarODone + 1, kBarOFree = kBarQFree + 1,
+                       kNumBars = kBarOFree + 1;
   static constexpr uint32_t kOffMisc = kOffBars + 8 * kNumBars;       // tmem base, abort flag
   static constexpr uint32_t kSmemBytes = kOffMisc + 16;
   static_assert(kSmemBytes <= 232448, "shared memory");
@@ -85,6 +90,8 @@ constexpr uint32_t kTmemS = 0, kTmemO = 256;
 struct TcParams {
   int32_t Hq, Hkv, G, g_shift, s_cap;
   int32_t unit_rows;     // query rows per unit (whole nodes), at most kRowsMax
+  int32_t n_units;       // units per KV head and sequence
+  int32_t n_total;       // (kLoop) all units
   int32_t tile_keys;     // keys per tile, a multiple of 16, at most kBKMax
   uint32_t q_half_bytes; // between the two 64-column halves of the Q block in shared memory
   uint32_t q_box_bytes;  // bytes the Q load brings in
@@ -131,7 +138,8 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
   return *reinterpret_cast<const uint32_t*>(&h);
 }
 
-template <int kHD>
+// kLoop: the grid is one CTA per SM, each working on several units one after the other.
+template <int kHD, bool kLoop>
 __global__ void __launch_bounds__(kTcThreads, 1)
 tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                     const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_tk,
@@ -149,9 +157,9 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
 
   const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
   FALCON_TRACE(tid == 0, 0);
-  const int n_splits = gridDim.x, split = blockIdx.x;  // cluster = all CTAs of a row of the grid
-  const int kvh = blockIdx.y % p.Hkv, unit = blockIdx.y / p.Hkv;
-  const int b = p.have_host ? p.h_order[blockIdx.z] : static_cast<int>(blockIdx.z);
+  const int n_splits = kLoop ? 1 : gridDim.x, split = kLoop ? 0 : blockIdx.x;  // cluster = all CTAs of a row of the grid
+  int kvh = blockIdx.y % p.Hkv, unit = blockIdx.y / p.Hkv;
+  int b = p.have_host ? p.h_order[blockIdx.z] : static_cast<int>(blockIdx.z);
   const int G = p.G, BK = p.tile_keys, R = p.unit_rows;
   const uint32_t half_tile = static_cast<uint32_t>(BK) * 128u, tile_bytes = half_tile * kHalves;
 
@@ -165,7 +173,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       prefetch_tmap(&tm_v);
     }
     for (int i = lane; i < C::kNumBars; i += 32)
-      mbar_init(bar(i), i >= C::kBarPFull && i < C::kBarPFull + 4 ? 4 : 1);
+      mbar_init(bar(i), i >= C::kBarPFull && i < C::kBarPFull + 4 ? 4 : (i == C::kBarOFree ? kSmThreads / 32 : 1));
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     __syncwarp();
   } else if (warp == kWarpMma) {
@@ -209,11 +217,45 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     row0 = split * rows_per;
     rows_mine = max(0, min(n_valid, row0 + rows_per) - row0);
   };
+  auto host_scalars = [&]() {
+    node_base = p.h_node_off[b];
+    T_real = p.h_node_off[b + 1] - node_base;
+    L_raw = p.h_prefix[b];
+    geometry();
+  };
   auto device_scalars = [&]() {
     node_base = p.node_off[b];
     T_real = p.node_off[b + 1] - node_base;
     L_raw = p.prefix_len[b];
     geometry();
+  };
+  // kLoop: this CTA's next unit that has rows; every role walks through them by itself.  The units lie in order of
+  // falling length, and the CTAs take them forwards and backwards in turn: the longest is paired with the shortest.
+  int step = -1, nth = -1, ring0 = 0;  // place in the CTA's list, units worked on before this one, ring items before it
+  auto unit_at = [&]() -> bool {       // false past the last one
+    const int n = gridDim.x, at = step * n + ((step & 1) ? n - 1 - static_cast<int>(blockIdx.x) : static_cast<int>(blockIdx.x));
+    if (at >= p.n_total) return false;
+    const int per_seq = p.Hkv * p.n_units, z = at / per_seq, y = at - z * per_seq;
+    unit = y / p.Hkv;
+    kvh = y - unit * p.Hkv;
+    b = p.have_host ? p.h_order[z] : z;
+    return true;
+  };
+  auto next_unit = [&]() -> bool {
+    if constexpr (kLoop) {
+      ring0 += 2 * n_my;
+      for (;;) {
+        ++step;
+        if (step * static_cast<int>(gridDim.x) >= p.n_total) return false;
+        if (!unit_at()) continue;
+        if (p.have_host) host_scalars();
+        else device_scalars();
+        if (n_valid > 0) break;
+      }
+      ++nth;
+      return true;
+    }
+    return false;
   };
   // tile j of this CTA: its first key (prefix keys 0 .. Lc-1, then the tree's) and how many keys it holds
   auto tile_key0 = [&](int j) {
@@ -226,8 +268,8 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
   };
   // ring item i: K (even) or V (odd) tile i / 2
   auto load_item = [&](int i) {
-    const int j = i >> 1, slot = i % kSlots;
-    if (j == 0 && p.stall_first) return;
+    const int j = i >> 1, slot = (ring0 + i) % kSlots;
+    if (ring0 + i < 2 && p.stall_first) return;
     const uint32_t dst = smem_base + C::kOffKV + slot * C::kSlotBytes;
     mbar_expect_tx(bar(C::kBarKVFull + slot), tile_bytes);
     if (p.separate && tile_begin + j >= n_pre)
@@ -236,12 +278,17 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       tma_load_5d(dst, (i & 1) ? &tm_v : &tm_k, bar(C::kBarKVFull + slot), 0, tile_key0(j), 0, kvh, b);
   };
 
+  // Wait (within a limit) for what was asked for, so that no copy is in flight when the CTA leaves.
+  auto drain_loads = [&](int n_ring, int n_q) {
+    if (n_q > 0) mbar_wait_drain(bar(C::kBarQ), (n_q - 1) & 1);
+    for (int i = max(0, n_ring - kSlots); i < n_ring; ++i)
+      if (!(i < 2 && p.stall_first)) mbar_wait_drain(bar(C::kBarKVFull + i % kSlots), (i / kSlots) & 1);
+  };
+
   int n_early = 0;  // ring items requested before the wait below
   if (p.have_host) {
-    node_base = p.h_node_off[b];
-    T_real = p.h_node_off[b + 1] - node_base;
-    L_raw = p.h_prefix[b];
-    geometry();
+    if constexpr (kLoop) next_unit();
+    else host_scalars();
     // Prefix rows that the caller declares stable (written before the kernel that precedes this one
     // in the stream started) may be requested while that kernel is still finishing.
     if (warp == kWarpProducer && lane == 0 && p.early_prefix && n_valid > 0)
@@ -257,38 +304,79 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   FALCON_TRACE(tid == 0, 1);
-  if (!p.have_host) device_scalars();
+  if (!p.have_host) {
+    if constexpr (kLoop) next_unit();
+    else device_scalars();
+  }
   if (n_valid <= 0) {  // no query rows here; same decision in every CTA of the cluster
     if (warp == kWarpMma)
       asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols) : "memory");
     return;
   }
 
+  int issued = 0, q_issued = 0;  // (producer) ring items and Q blocks asked for
   if (warp == kWarpProducer) {
     // ================================ TMA producer (ring refills) ================================
     if (lane == 0) {
-      if (n_my > 0) {  // Q first, so that it is not queued behind the K/V tiles
+      auto load_q = [&]() {
         mbar_expect_tx(bar(C::kBarQ), p.q_box_bytes);
         tma_load_5d(smem_base, &tm_q, bar(C::kBarQ), 0, 0, kvh, node_base + unit * (R >> p.g_shift), 0);
-      }
-      int issued = min(2 * n_my, kSlots);
+        ++q_issued;
+      };
+      auto capacity = [&]() {
+        if (split == 0 && unit == 0 && kvh == 0 && (L + (p.separate ? 0 : T) > p.s_cap || T_real > FALCON_T_MAX))
+          dev_status_or(p.status, b, FALCON_DEV_CAPACITY);
+      };
+      // Q first, so that it is not queued behind the K/V tiles
+      if (n_my > 0) load_q();
+      issued = min(2 * n_my, kSlots);
       for (int i = n_early; i < issued; ++i) load_item(i);
       FALCON_TRACE(true, 2);
-      if (split == 0 && unit == 0 && kvh == 0 && (L + (p.separate ? 0 : T) > p.s_cap || T_real > FALCON_T_MAX))
-        dev_status_or(p.status, b, FALCON_DEV_CAPACITY);
+      capacity();
+      bool ok = true;
       for (int i = kSlots; i < 2 * n_my; ++i) {
-        if (!mbar_wait(bar(C::kBarKVEmpty + i % kSlots), (i / kSlots - 1) & 1, abort_flag)) break;
+        ok = mbar_wait(bar(C::kBarKVEmpty + i % kSlots), (i / kSlots - 1) & 1, abort_flag);
+        if (!ok) break;
         load_item(i);
         issued = i + 1;
       }
-      // If some wait gives up, what was asked for still arrives: stay until it has, so that no copy is
-      // in flight into this CTA's shared memory when it leaves.  (Waiting for the last MMAs here
-      // means that whatever went wrong is known by now.)
-      if (n_my > 0) mbar_wait(bar(C::kBarODone), 0, abort_flag);
-      if (*abort_flag) {
-        if (n_my > 0) mbar_wait_drain(bar(C::kBarQ), 0);
-        for (int i = max(0, issued - kSlots); i < issued; ++i)
-          if (!(i < 2 && p.stall_first)) mbar_wait_drain(bar(C::kBarKVFull + i % kSlots), (i / kSlots) & 1);
+      if constexpr (kLoop) {
+        while (ok && next_unit()) {
+          // A later unit's Q comes when the MMAs have read the one before; its K and V tiles do not wait for that.
+          bool q_due = true;
+          capacity();
+          for (int i = 0; ok && i < 2 * n_my; ++i) {
+            const int ri = ring0 + i;
+            if (ri >= kSlots) {
+              const uint32_t empty = bar(C::kBarKVEmpty + ri % kSlots), parity = (ri / kSlots - 1) & 1;
+              for (uint32_t it = 0; q_due; ++it) {
+                if (mbar_test(bar(C::kBarQFree), (nth - 1) & 1)) {
+                  load_q();
+                  q_due = false;
+                } else if (mbar_test(empty, parity)) {
+                  break;
+                } else if (*abort_flag || it >= kPollLimit) {
+                  *abort_flag = 1;
+                  break;
+                }
+              }
+              ok = mbar_wait(empty, parity, abort_flag);
+              if (!ok) break;
+            }
+            load_item(i);
+            issued = ri + 1;
+          }
+          if (ok && q_due) {
+            ok = mbar_wait(bar(C::kBarQFree), (nth - 1) & 1, abort_flag);
+            if (ok) load_q();
+          }
+        }
+      } else {
+        // If some wait gives up, what was asked for still arrives: stay until it has, so that no copy is
+        // in flight into this CTA's shared memory when it leaves.  (Waiting for the last MMAs here
+        // means that whatever went wrong is known by now.)
+        if (n_my > 0) mbar_wait(bar(C::kBarODone), 0, abort_flag);
+        if (*abort_flag) drain_loads(issued, q_issued);
       }
     }
     __syncwarp();
@@ -297,14 +385,20 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     // The whole warp runs this loop and one elected lane issues.  What an MMA's operands are made of must be
     // the same in every lane as far as the compiler can see (loop counters, parameters, constants), or each
     // MMA costs about 100 cycles of register traffic instead of 30: hence one loop per arrangement.
-    if (n_my > 0) {
-      uint32_t elected;
-      asm volatile("{ .reg .pred p; elect.sync _|p, 0xffffffff; selp.u32 %0, 1, 0, p; }" : "=r"(elected));
+    uint32_t elected;
+    asm volatile("{ .reg .pred p; elect.sync _|p, 0xffffffff; selp.u32 %0, 1, 0, p; }" : "=r"(elected));
+    uint32_t pbase = 0;  // (kLoop) parities of the four P barriers at the start of a unit, as bits
+    do {
+      if (n_my <= 0) break;
       // The tiles that are not full: the last one, and (separate buffers) the one the prefix ends in.
       const int j_a = n_pre - 1 - tile_begin, j_b = n_my - 1;
       const int nk_full = BK >> 4, nk_a = p.separate && j_a >= 0 && j_a < n_my ? (tile_keys_in(j_a, tile_key0(j_a)) + 15) >> 4 : nk_full,
                 nk_b = (tile_keys_in(j_b, tile_key0(j_b)) + 15) >> 4;
-      const bool ok = mbar_wait(bar(C::kBarQ), 0, abort_flag);
+      // (the shuffles: the same in every lane, and known to be)
+      const int slot0 = kLoop ? __shfl_sync(0xffffffffu, ring0 % kSlots, 0) : 0;
+      const uint32_t phase0 = kLoop ? __shfl_sync(0xffffffffu, (ring0 / kSlots) & 1, 0) : 0u;
+      bool ok = mbar_wait(bar(C::kBarQ), kLoop ? nth & 1 : 0, abort_flag);
+      if constexpr (kLoop) ok = __all_sync(0xffffffffu, ok);
       FALCON_TRACE(elected, 5);
       // Every lane walks through the loop and looks at the barriers by itself (no votes: this warp shares its
       // scheduler with four softmax warps, and each instruction here is one the tensor core waits for).
@@ -318,7 +412,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         const uint32_t q_lo = desc_lo(smem_base, 16), q_step = p.q_half_bytes >> 4, k_step = half_tile >> 4;
         const uint32_t k_lo = desc_lo(smem_base + C::kOffKV, 16), v_lo = desc_lo(smem_base + C::kOffKV, half_tile);
         constexpr uint32_t kSlotStep = C::kSlotBytes >> 4;
-        auto issue_qk = [&](int s, int buf, int slot) {
+        auto issue_qk = [&](int s, int buf, int slot, bool last) {
           const uint32_t q = q_lo + s * (128 * 128 >> 4), k = k_lo + slot * kSlotStep;
           if (elected) {
 #pragma unroll
@@ -328,6 +422,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                 umma_bf16_ss(tmem_base + kTmemS + buf * 64, desc_of(q + h * q_step + kk * 2), desc_of(k + h * k_step + kk * 2),
                              p.idesc_qk, (h | kk) ? 1u : 0u);
             umma_commit(bar(C::kBarSFull) + 8u * buf);
+            if (kLoop && last) umma_commit(bar(C::kBarQFree));
           }
         };
         auto issue_pv = [&](int s, int buf, int slot, int j, bool last_block) {
@@ -346,8 +441,8 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         // Four items' scores are in flight: 4 / kBlocks tiles.  P(i) lies over S(i), so the scores of item
         // i + 4 are issued behind P(i).V (the MMAs of a CTA run in the order of issue).
         constexpr int kAhead = 4 / kBlocks;
-        int kslot = 0, vslot = 1;           // ring slots of the next K and V tile
-        uint32_t kphase = 0, pphase = 0;
+        int kslot = slot0, vslot = slot0 + 1;  // ring slots of the next K and V tile
+        uint32_t kphase = phase0, pphase = 0;
         auto k_wait = [&]() { return mbar_wait(bar(C::kBarKVFull) + 8u * kslot, kphase, abort_flag); };
         auto k_next = [&]() {
           kslot += 2;
@@ -360,7 +455,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         for (int j = 0; j < min(kAhead, n_my); ++j) {
           if (!k_wait()) return;
 #pragma unroll
-          for (int s = 0; s < kBlocks; ++s) issue_qk(s, (j * kBlocks + s) & 3, kslot);
+          for (int s = 0; s < kBlocks; ++s) issue_qk(s, (j * kBlocks + s) & 3, kslot, s == kBlocks - 1 && j == n_my - 1);
           k_next();
         }
         for (int j = 0; j < n_my; ++j) {
@@ -368,13 +463,15 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
 #pragma unroll
           for (int s = 0; s < kBlocks; ++s) {
             const int buf = (j * kBlocks + s) & 3;
-            if (!mbar_wait(bar(C::kBarPFull) + 8u * buf, pphase, abort_flag)) return;
+            if (!mbar_wait(bar(C::kBarPFull) + 8u * buf, kLoop ? ((pbase >> buf) ^ pphase) & 1u : pphase, abort_flag)) return;
+            // (the accumulators are free again: the unit before has been read out)
+            if (kLoop && j == 0 && s == 0 && nth > 0 && !mbar_wait(bar(C::kBarOFree), (nth - 1) & 1, abort_flag)) return;
             tc_fence_after();
             FALCON_TRACE(elected && j * kBlocks + s < 8, 42 + j * kBlocks + s);
             issue_pv(s, buf, vslot, j, s == kBlocks - 1);
             if (more) {
               if (s == 0 && !k_wait()) return;
-              issue_qk(s, buf, kslot);
+              issue_qk(s, buf, kslot, s == kBlocks - 1 && j + kAhead == n_my - 1);
             }
             FALCON_TRACE(elected && j * kBlocks + s < 8, 50 + j * kBlocks + s);
           }
@@ -390,12 +487,21 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       __syncwarp();
       if (elected) umma_commit(bar(C::kBarODone));  // fires once every MMA issued so far has finished
       __syncwarp();
-    }
+      if constexpr (kLoop) {
+#pragma unroll
+        for (int g = 0; g < 4; ++g) pbase ^= static_cast<uint32_t>(((n_items + 3 - g) >> 2) & 1) << g;
+        // (after a wait that gave up, MMAs may still be running)
+        if (*abort_flag && lane == 0) mbar_wait_drain(bar(C::kBarODone), nth & 1);
+        __syncwarp();
+      }
+    } while (kLoop && next_unit());
   } else {
     // ================================ softmax warps ================================
     // Four groups of four warps (one per TMEM lane quadrant); group g takes the items i = g mod 4, each in score
     // buffer g, so a group's waits and loads run under the other three groups' exponentials.
     const int q4 = warp & 3, grp = (warp - kWarpSm0) >> 2;
+    uint32_t sphase = 0;                           // parity of this group's score barrier
+    do {
     const int blk = two_blocks ? grp & 1 : 0;      // row block
     const int lane_row = q4 * 32 + lane;           // TMEM lane
     const int row = blk * 128 + lane_row;          // query row of the unit
@@ -450,7 +556,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         else asm volatile("bar.arrive %0, 128;" ::"r"(1 + q4) : "memory");
       }
     };
-    if (grp == 0 || (two_blocks && grp == 1)) s_rescue[row] = 0;
+    if (!kLoop && (grp == 0 || (two_blocks && grp == 1))) s_rescue[row] = 0;
     bool published = !source || n_items == 0;  // (source groups have item `grp`: n_items >= n_src or 0)
     if (!source && n_items > 0) {
       ref_barrier(true);
@@ -460,11 +566,12 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     for (int i = grp; i < n_items; i += 4) {
       const int j = two_blocks ? i >> 1 : i;
       const int k0 = tile_key0(j), nv = tile_keys_in(j, k0);
-      if (!mbar_wait_warp(bar(C::kBarSFull + grp), (i >> 2) & 1, abort_flag)) break;
+      if (!mbar_wait_warp(bar(C::kBarSFull + grp), sphase, abort_flag)) break;
+      sphase ^= 1;
       FALCON_TRACE(q4 == 2 && lane == 0 && i < 8, 10 + 2 * i);
       tc_fence_after();
       // the scores are there, so the K tile is no longer needed (two blocks: the second's come last)
-      if (q4 == 0 && lane == 0 && (!two_blocks || blk == 1)) mbar_arrive(bar(C::kBarKVEmpty + (2 * j) % kSlots));
+      if (q4 == 0 && lane == 0 && (!two_blocks || blk == 1)) mbar_arrive(bar(C::kBarKVEmpty + (ring0 + 2 * j) % kSlots));
       if (warp_valid) {
         const bool full = k0 + BK <= Lc;  // every key lies in the prefix: visible to every row
         auto load32 = [&](int c, uint32_t (&sr)[32]) {
@@ -512,8 +619,8 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       // The MMA warp takes P's barrier for V's as well: one warp of the group waits for the tile to have landed.
       const bool clear_v = (nv & 15) && blk == 0;
       if (q4 == 0 || clear_v) {
-        const int slot = (2 * j + 1) % kSlots;
-        if (!mbar_wait_warp(bar(C::kBarKVFull + slot), ((2 * j + 1) / kSlots) & 1, abort_flag)) break;
+        const int item = ring0 + 2 * j + 1, slot = item % kSlots;
+        if (!mbar_wait_warp(bar(C::kBarKVFull + slot), (item / kSlots) & 1, abort_flag)) break;
         if (clear_v) {
           // The last MMA step over this tile's keys reads V rows past the last key, which may hold anything
           // (0 x NaN = NaN): clear them.
@@ -551,7 +658,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       }
     }
     bool have = n_my > 0 && !*abort_flag;
-    if (have) have = mbar_wait_warp(bar(C::kBarODone), 0, abort_flag);
+    if (have) have = mbar_wait_warp(bar(C::kBarODone), kLoop ? nth & 1 : 0, abort_flag);
     FALCON_TRACE(tid == 64, 58);
     tc_fence_after();
     if (l_row == 0.f) m_ref = -INFINITY;  // no key of this row here: the merge leaves this part out
@@ -561,9 +668,11 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     const int mg = unit * R + row;
     __nv_bfloat16* dst = p.out + (static_cast<int64_t>(node_base + (mg >> p.g_shift)) * p.Hq + kvh * G + (mg & (G - 1))) * kHD;
     float inv = 1.f;
+    bool inexact = false;  // the row needs the exact path (kLoop: or a wait gave up)
     if (n_splits == 1) {
       const bool fine = l_row >= kLMin && l_row <= kLMax;
-      if (valid && have && !fine && first_cols) s_rescue[row] = 1;
+      inexact = valid && first_cols && (kLoop ? !(have && fine) : have && !fine);
+      if (!kLoop && inexact) s_rescue[row] = 1;
       inv = have && fine ? 1.f / l_row : 0.f;
     }
     unsigned char* part = p.part + static_cast<int64_t>((blockIdx.z * gridDim.y + blockIdx.y) * n_splits + split) * part_bytes(kHD, R);
@@ -600,11 +709,34 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       }
     }
     FALCON_TRACE(tid == 64, 59);
+    if constexpr (kLoop) {
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar(C::kBarOFree));
+      // One barrier for all: the small arrays are free for the next unit, and whether any row needs the exact path.
+      int exact;
+      asm volatile("{ .reg .pred p, q; setp.ne.s32 p, %1, 0; bar.red.or.pred q, 13, %2, p; selp.b32 %0, 1, 0, q; }"
+                   : "=r"(exact)
+                   : "r"(inexact ? 1 : 0), "n"(kSmThreads)
+                   : "memory");
+      if (exact) {
+        if (first_cols) s_rescue[row] = inexact;
+        asm volatile("bar.sync 13, %0;" ::"n"(kSmThreads) : "memory");
+        if (*abort_flag) {  // (the unit's rows read as zero)
+          if (st_id == 0) dev_status_or(p.status, b, FALCON_DEV_TIMEOUT);
+        } else {
+          for (int rr = warp - kWarpSm0; rr < n_valid; rr += kSmThreads / 32)
+            if (s_rescue[rr]) rescue_row<kHD>(p, b, kvh, node_base, T, Lc, S_valid, unit * R + rr, lane);
+        }
+        asm volatile("bar.sync 13, %0;" ::"n"(kSmThreads) : "memory");
+      }
+    }
+    } while (kLoop && next_unit());
   }
 
   tc_fence_before();
-  bool rescue = true;
-  if (n_splits > 1) {
+  bool rescue = !kLoop;
+  if (!kLoop && n_splits > 1) {
     // ================================ merge ================================
     cluster_sync_release();  // every split's partial rows are visible (it is this CTA's barrier as well)
     FALCON_TRACE(tid == 0, 60);
@@ -664,6 +796,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
   } else {
     __syncthreads();
     if (*abort_flag) rescue = false;  // the rows read as zero
+    if (kLoop && *abort_flag && tid == 0) drain_loads(issued, q_issued);
   }
   if (*abort_flag && tid == 0) dev_status_or(p.status, b, FALCON_DEV_TIMEOUT);
   FALCON_TRACE(tid == 0, 62);
@@ -673,7 +806,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       if (s_rescue[r]) rescue_row<kHD>(p, b, kvh, node_base, T, Lc, S_valid, unit * R + r, lane);
   if (warp == kWarpMma) {
     // (after a wait that gave up, MMAs may still be running: the last commit covers them all)
-    if (n_my > 0 && *abort_flag && lane == 0) mbar_wait_drain(bar(C::kBarODone), 0);
+    if (!kLoop && n_my > 0 && *abort_flag && lane == 0) mbar_wait_drain(bar(C::kBarODone), 0);
     __syncwarp();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols) : "memory");
   }
@@ -698,7 +831,7 @@ int resident_clusters(falcon_ctx* ctx, int s) {
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, tree_attn_tc_kernel<128>, &cfg) != cudaSuccess) n = -1;
+    if (cudaOccupancyMaxActiveClusters(&n, tree_attn_tc_kernel<128, false>, &cfg) != cudaSuccess) n = -1;
     resident[s] = n > 0 ? n : -1;
     cudaGetLastError();
   }
@@ -768,22 +901,43 @@ Plan make_plan(falcon_ctx* ctx, const falcon_attn_args& a) {
   return best;
 }
 
+// Tiles of a sequence, on average (of the longest one where the lengths are on the device only).
+int mean_tiles(const falcon_attn_args& a) {
+  int64_t keys = a.tree.max_tree + a.tree.max_prefix_len;
+  if (a.tree.prefix_len_host && a.tree.node_off_host) {
+    keys = a.tree.total_nodes;
+    for (int i = 0; i < a.tree.batch; ++i) keys += a.tree.prefix_len_host[i];
+    keys = (keys + a.tree.batch - 1) / a.tree.batch;
+  }
+  return static_cast<int>((keys + kBKMax - 1) / kBKMax);
+}
+
 template <int kHD>
 int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s) {
   using C = Cfg<kHD>;
   const int B = a.tree.batch, Hq = a.n_q_heads, Hkv = a.n_kv_heads, G = Hq / Hkv;
   bool& attr_set = ctx->attn_attr_set[0];
   if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(tree_attn_tc_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(Cfg<128>::kSmemBytes));
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(tree_attn_tc_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               static_cast<int>(Cfg<64>::kSmemBytes));
+    cudaError_t e = cudaSuccess;
+    auto set = [&](auto* kernel, uint32_t bytes) {
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
+    };
+    set(tree_attn_tc_kernel<128, false>, Cfg<128>::kSmemBytes);
+    set(tree_attn_tc_kernel<64, false>, Cfg<64>::kSmemBytes);
+    set(tree_attn_tc_kernel<128, true>, Cfg<128>::kSmemBytes);
+    set(tree_attn_tc_kernel<64, true>, Cfg<64>::kSmemBytes);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute(tree_attn_tc_kernel)");
     attr_set = true;
   }
   const Plan plan = make_plan(ctx, a);
   const int q_nodes = plan.q_nodes, n_units = plan.n_units, splits = plan.splits, tile_keys = plan.tile;
+  // More units than SMs, of few tiles each: one CTA per SM works on several (see kLoop).  What a unit costs beside its
+  // tiles is about 2 us then and 4.5 us as a CTA of its own, but the hardware gives out CTAs as SMs become free
+  // and the loop's shares are fixed: units of 3 to 7 tiles 29.7 -> 24.1 and 35.7 -> 29.3 us a launch (16 and 15
+  // sequences, 40 heads of 64), of 5 tiles on average (13 sequences, 8 KV heads of 128) 14.0 both ways, of 19 tiles
+  // 40 -> 42, of 34 tiles 47 -> 54.
+  const int64_t n_total = static_cast<int64_t>(Hkv) * n_units * B;
+  const bool loop = splits == 1 && n_total > ctx->sm_count && n_total < (1 << 30) && mean_tiles(a) <= kLoopTiles;
   if (static_cast<int64_t>(Hkv) * n_units > 65535) return FALCON_ERR_CAPACITY;
 
 
@@ -832,6 +986,8 @@ int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s) {
   while ((1 << p.g_shift) < G) ++p.g_shift;
   p.s_cap = a.s_cap;
   p.unit_rows = q_nodes * G;
+  p.n_units = n_units;
+  p.n_total = loop ? static_cast<int32_t>(n_total) : 0;
   p.tile_keys = tile_keys;
   p.q_half_bytes = static_cast<uint32_t>(q_nodes) * G * 128u;
   p.q_box_bytes = p.q_half_bytes * C::kHalves;
@@ -868,7 +1024,7 @@ int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s) {
   FALCON_TRACE_LAUNCH(p)
 
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(splits, Hkv * n_units, B);
+  cfg.gridDim = loop ? dim3(ctx->sm_count) : dim3(splits, Hkv * n_units, B);
   cfg.blockDim = dim3(kTcThreads);
   cfg.dynamicSmemBytes = C::kSmemBytes;
   cfg.stream = s;
@@ -883,7 +1039,7 @@ int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s) {
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, tree_attn_tc_kernel<kHD>, mq, mk, mv, mtk, mtv, p);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, loop ? tree_attn_tc_kernel<kHD, true> : tree_attn_tc_kernel<kHD, false>, mq, mk, mv, mtk, mtv, p);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "tree_attn_tc_kernel launch");
   return FALCON_OK;
 }

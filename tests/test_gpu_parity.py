@@ -536,6 +536,37 @@ def test_attn_tc_head_sizes_and_separate_tree_buffers(T, G, L, splits, separate,
         assert not dt.status.cpu().numpy().any()
 
 
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("separate", [False, True])
+@pytest.mark.parametrize("sizes,prefs,Hkv,G", [
+    ([3, 20, 1, 17, 9, 12, 5, 30], [40, 700, 0, 64, 127, 300, 1, 65], 38, 1),  # 304 units: two or three a CTA, one row block
+    ([40, 20, 64, 33, 7], [130, 64, 0, 400, 63], 40, 4),                        # two row blocks and one, in turn
+    ([2] * 38, [16] * 38, 16, 2),                                               # more sequences than the call's own tables hold
+])
+def test_attn_tc_more_units_than_sms(sizes, prefs, Hkv, G, separate, D):
+    """Rows-on-lanes kernel, several units per CTA: the rings, barriers and accumulators go from one unit to the next."""
+    rng = np.random.default_rng(len(sizes) * 100 + Hkv + G + D)
+    tb, q, k, v = random_case(rng, sizes, prefs, Hkv * G, Hkv, D, slack=1)
+    ref = oracle_attn(tb, Hkv * G, Hkv, D, q, k, v)
+    kw = {}
+    if separate:
+        kt = np.empty((tb.total_nodes, Hkv, D), np.uint16)
+        vt = np.empty_like(kt)
+        for b, (Tb, Lb) in enumerate(zip(sizes, prefs)):
+            o = tb.node_off[b]
+            kt[o:o + Tb] = k[b, :, Lb:Lb + Tb].transpose(1, 0, 2)
+            vt[o:o + Tb] = v[b, :, Lb:Lb + Tb].transpose(1, 0, 2)
+            k[b, :, Lb:] = 0x7FC0
+            v[b, :, Lb:] = 0x7FC0
+        kw = dict(k_tree=kt, v_tree=vt)
+    for hc in (False, True):
+        for flags in (0, binding.ATTN_PREFIX_STABLE):
+            dt = H.DevTrees(tb)
+            out, rc = H.run_attn(dt, Hkv * G, Hkv, D, q, k, v, kernel=binding.ATTN_TC, n_splits=1, host_copies=hc, flags=flags, **kw)
+            H.assert_attn_close(out, ref, tb.node_off)
+            assert not dt.status.cpu().numpy().any()
+
+
 @pytest.mark.parametrize("tck", TC_KERNELS)
 @pytest.mark.parametrize("T,G,L,splits", [(60, 1, 1024, 0), (60, 1, 700, 4), (80, 1, 500, 3), (16, 8, 1000, 5),
                                            (20, 1, 10, 2), (33, 2, 0, 1)])
