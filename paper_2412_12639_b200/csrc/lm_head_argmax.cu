@@ -4,20 +4,26 @@
 // largest logit).  logit[i, v] = sum_k feat[i, k] * head[v, k] is a dense bf16 contraction whose
 // [N, V] fp32 result is never written: the argmax is taken where the accumulator is read.
 //
-// The head (V x hidden bf16, 262 MB at 32000 x 4096) is read once and dominates: the kernel is
+// Up to 128 nodes: the head (V x hidden bf16, 262 MB at 32000 x 4096) is read once and dominates: the kernel is
 // bound by HBM, the tensor core is about a third busy.  Every CTA owns a run of vocabulary rows
 // (V split evenly over the SMs, in steps of 16, so one launch is one wave) and streams it through a
 // TMA ring in chunks of 64 hidden columns together with the matching chunk of the features (L2
-// hits after the first CTA).  tcgen05.mma with the nodes on the M side (128 per tile; up to two
-// tiles resident, so up to 256 nodes read the head once) and the CTA's vocabulary rows on the N
+// hits after the first CTA).  tcgen05.mma with the nodes on the M side and the CTA's vocabulary rows on the N
 // side (up to 256 per instruction) accumulates in TMEM; four warps then read one accumulator row
 // (= one node) each, 32 columns at a time, and keep the first maximum.  A CTA's result for a node
 // is one 64-bit atomicMax on a word ordered by (logit, then lower index), so ties go to the lowest
 // index whatever the timing; the last CTA to arrive unpacks the words.
 //
+// More nodes: pairs of CTAs (kPair, cta_group::2).  What bounds then is what an SM can draw from L2, about 33 bytes per
+// cycle, and a pair's MMA of 256 nodes x up to 256 vocabulary rows takes half of each operand from either CTA's shared
+// memory: 47 KB per 64 hidden columns and CTA for 512 nodes x 224 rows, where single CTAs drew 61 KB for 256 x 224.
+// All of TMEM holds accumulators: two node tiles (up to 512 nodes read the head once) or, up to 256
+// nodes, two vocabulary tiles (the features are read once for both).  32000 x 5120: 512 nodes 157 -> 133 us (2.5 times
+// the MMAs' time), 300 nodes 147 -> 123, 256 nodes 78 -> 72, 130 nodes 73 -> 68; 600 nodes (two groups) 229 -> 223.
+//
 // Warp roles: 0 = TMA producer (one thread), 1 = MMA issuer (one elected thread) and TMEM owner,
-// 2-5 = accumulator readers.  Every wait is bounded; a wait that gives up sets FALCON_DEV_TIMEOUT
-// in the caller's status word and the kernel still leaves in order (loads drained, MMAs finished,
+// 2-5 = accumulator readers; of a pair, the first CTA's warp 1 issues for both, and each CTA loads its own halves.
+// Every wait is bounded; a wait that gives up sets FALCON_DEV_TIMEOUT in the caller's status word and the kernel still leaves in order (loads drained, MMAs finished,
 // TMEM freed).
 
 #include <climits>
@@ -53,10 +59,11 @@ struct LmParams {
   int32_t f_rows;     // rows of a feature tile as loaded: 128, or with a single tile the number of nodes rounded up
                       // to 8 (64 at least); the MMA still reads 128 rows, and what follows the tile gives
                       // accumulator rows that nobody looks at
-  int32_t n_mt;       // 128-node tiles
-  int32_t m_res;      // node tiles resident in TMEM at once (1 or 2)
+  int32_t n_mt;       // node tiles: of 128 rows, of a pair's 256
+  int32_t m_res;      // node tiles resident in TMEM at once (1; a pair: 1 or 2)
+  int32_t v_res;      // vocabulary tiles resident at once (1; a pair with one node tile: 2)
   int32_t tile_n;     // vocabulary rows per MMA (multiple of 16)
-  int32_t span;       // vocabulary rows per CTA (multiple of 16)
+  int32_t span;       // vocabulary rows per CTA or pair (multiple of 16)
   int32_t n_stages;
   int32_t stall_first;  // test hook: the features of ring stage 0 are never requested (a bounded wait then runs out)
   uint32_t stage_bytes, idesc;
@@ -90,6 +97,36 @@ __device__ __forceinline__ bool lm_wait_drain(uint32_t bar, uint32_t parity) {
   return false;
 }
 
+// The pair's forms of what tc_util.cuh has for one CTA.  A load may signal the other CTA's barrier (`bar`: a
+// shared::cluster address); a commit arrives at the same barrier of both CTAs.
+__device__ __forceinline__ void tma_load_pair(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1) {
+  asm volatile(
+      "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes.cta_group::2 [%0], [%1, {%3, %4, %5, %5, %5}], "
+      "[%2];" ::"r"(dst),
+      "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(0)
+      : "memory");
+}
+__device__ __forceinline__ void umma_pair_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{ .reg .pred p; setp.ne.b32 p, %4, 0; tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p; }" ::"r"(d_tmem),
+      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+__device__ __forceinline__ void umma_pair_commit(uint32_t bar) {
+  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
+               "h"(static_cast<uint16_t>(3))
+               : "memory");
+}
+__device__ __forceinline__ uint32_t map_to_leader(uint32_t addr) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(addr));
+  return r;
+}
+__device__ __forceinline__ void arrive_remote(uint32_t bar) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+
+template <bool kPair>
 __global__ void __launch_bounds__(kLmThreads, 1)
 lm_head_argmax_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_f, const LmParams p) {
   extern __shared__ __align__(1024) unsigned char smem_gen[];
@@ -102,36 +139,60 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_con
   auto bar = [&](int i) { return bars + 8u * static_cast<uint32_t>(i); };
 
   const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
-  const int cta = blockIdx.x, n_cta = gridDim.x;
+  const int n_cta = gridDim.x;
+  const int rank = kPair ? blockIdx.x & 1 : 0, cta = kPair ? blockIdx.x >> 1 : blockIdx.x;  // place in the pair; pair or CTA
+  const bool leader = rank == 0;
   const int S = p.n_stages;
   const int v_lo = cta * p.span, v_hi = min(p.vocab, v_lo + p.span);
   const int n_vt = (v_hi - v_lo + p.tile_n - 1) / p.tile_n;  // >= 1 by construction of the grid
-  const int n_groups = (p.n_mt + p.m_res - 1) / p.m_res;
-  const uint32_t tmem_cols = static_cast<uint32_t>(p.m_res) * 256u;
-  const uint32_t w_bytes = static_cast<uint32_t>(p.tile_n) * (kLmKC * 2u);   // one chunk of the head tile
+  const int m_res = kPair ? p.m_res : 1, v_res = kPair ? p.v_res : 1;
+  const int n_vp = (n_vt + v_res - 1) / v_res;                               // passes over the hidden dimension per group
+  const uint32_t tmem_cols = kPair ? 512u : 256u;
+  const int w_rows = kPair ? p.tile_n >> 1 : p.tile_n;                       // of a head tile in this CTA's shared memory
+  const uint32_t w_bytes = static_cast<uint32_t>(w_rows) * (kLmKC * 2u);     // one chunk of it
   const uint32_t f_bytes = static_cast<uint32_t>(p.f_rows) * (kLmKC * 2u);   // one chunk of one feature tile
+  const int n_groups = (p.n_mt + m_res - 1) / m_res;
   const int n_ks = (p.n_kc + p.kch - 1) / p.kch;                             // ring stages per accumulator tile
-  const int n_iter = n_groups * n_vt * n_ks;                                 // ring stages this CTA goes through
+  const int n_iter = n_groups * n_vp * n_ks;                                 // ring stages this CTA goes through
   const int n_pre = min(S, n_iter);
   // CTAs start at different places of the hidden dimension (a sum does not care where it starts), so that at
   // any moment they read different column ranges of their rows instead of all the same one.
   const int rot = static_cast<int>((static_cast<unsigned>(cta) * 11u) % static_cast<unsigned>(n_ks));
   // Ring stage `it` = (node-tile group, vocabulary tile, K step), K fastest.  Its chunks are asked for back to
   // back; a chunk past the hidden size reads as zeros, and so does a node tile past the last one.
+  // (a pair: both CTAs' loads signal the first one's barrier, which it arms for both)
+  auto full_bar = [&](int st) { return kPair ? map_to_leader(bar(kLmBarFull + st)) : bar(kLmBarFull + st); };
+  auto tiles_of = [&](int g) { return kPair ? min(m_res, p.n_mt - g * m_res) : 1; };  // node tiles of a group
+  auto arm = [&](int it) {
+    if (!leader) return;
+    const uint32_t absent = kPair ? static_cast<uint32_t>(p.kch * (m_res - tiles_of(it / (n_ks * n_vp)))) * f_bytes : 0u;
+    mbar_expect_tx(bar(kLmBarFull + it % S), (kPair ? 2 : 1) * (p.stage_bytes - absent));
+  };
   auto issue_head = [&](int it) {
-    const int st = it % S, kq = (it % n_ks + rot) % n_ks, vt = (it / n_ks) % n_vt;
+    const int st = it % S, kq = (it % n_ks + rot) % n_ks, vp = (it / n_ks) % n_vp;
     const uint32_t dst = smem_base + static_cast<uint32_t>(st) * p.stage_bytes;
-    for (int c = 0; c < p.kch; ++c)
-      tma_load_5d(dst + c * w_bytes, &tm_w, bar(kLmBarFull + st), (kq * p.kch + c) * kLmKC, v_lo + vt * p.tile_n, 0, 0, 0);
+    for (int c = 0; c < p.kch; ++c) {
+      if constexpr (kPair) {
+        for (int u = 0; u < v_res; ++u)
+          tma_load_pair(dst + (c * v_res + u) * w_bytes, &tm_w, full_bar(st), (kq * p.kch + c) * kLmKC,
+                        v_lo + (vp * v_res + u) * p.tile_n + rank * w_rows);
+      } else {
+        tma_load_5d(dst + c * w_bytes, &tm_w, full_bar(st), (kq * p.kch + c) * kLmKC, v_lo + vp * p.tile_n, 0, 0, 0);
+      }
+    }
   };
   auto issue_feat = [&](int it) {
     if (it == 0 && p.stall_first) return;
-    const int st = it % S, kq = (it % n_ks + rot) % n_ks, g = it / (n_ks * n_vt);
-    const uint32_t fdst = smem_base + static_cast<uint32_t>(st) * p.stage_bytes + static_cast<uint32_t>(p.kch) * w_bytes;
-    for (int c = 0; c < p.kch; ++c)
-      for (int j = 0; j < p.m_res; ++j)
-        tma_load_5d(fdst + (c * p.m_res + j) * f_bytes, &tm_f, bar(kLmBarFull + st), (kq * p.kch + c) * kLmKC,
-                    (g * p.m_res + j) * 128, 0, 0, 0);
+    const int st = it % S, kq = (it % n_ks + rot) % n_ks, g = it / (n_ks * n_vp);
+    const uint32_t fdst = smem_base + static_cast<uint32_t>(st) * p.stage_bytes + static_cast<uint32_t>(p.kch * v_res) * w_bytes;
+    for (int c = 0; c < p.kch; ++c) {
+      if constexpr (kPair) {
+        for (int j = 0; j < tiles_of(g); ++j)
+          tma_load_pair(fdst + (c * m_res + j) * f_bytes, &tm_f, full_bar(st), (kq * p.kch + c) * kLmKC, (g * m_res + j) * 256 + rank * 128);
+      } else {
+        tma_load_5d(fdst + c * f_bytes, &tm_f, full_bar(st), (kq * p.kch + c) * kLmKC, g * 128, 0, 0, 0);
+      }
+    }
   };
 
   if (warp == 0) {
@@ -140,22 +201,29 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_con
       *s_last = 0;
       prefetch_tmap(&tm_w);
       prefetch_tmap(&tm_f);
-      for (int i = 0; i < kLmNumBars; ++i) mbar_init(bar(i), i == kLmBarAccEmpty ? kLmReaders / 32 : 1);
+      for (int i = 0; i < kLmNumBars; ++i) mbar_init(bar(i), i == kLmBarAccEmpty ? (kPair ? 2 : 1) * kLmReaders / 32 : 1);
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-      // The head is a constant of the model: its first ring fill is asked for before the wait below, while
-      // the previous kernel of the stream is still finishing.  The features are that kernel's to write.
-      if (!*abort_flag)
-        for (int it = 0; it < n_pre; ++it) {
-          mbar_expect_tx(bar(kLmBarFull + it), p.stage_bytes);
-          issue_head(it);
-        }
     }
     __syncwarp();
   } else if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(s_tmem_base)), "r"(tmem_cols)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    if constexpr (kPair) {
+      asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(s_tmem_base)), "r"(tmem_cols)
+                   : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    } else {
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(s_tmem_base)), "r"(tmem_cols)
+                   : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
   }
+  if constexpr (kPair) cluster_sync_release();  // both CTAs' barriers exist
+  // The head is a constant of the model: its first ring fill is asked for before the wait below, while
+  // the previous kernel of the stream is still finishing.  The features are that kernel's to write.
+  if (warp == 0 && lane == 0 && !*abort_flag)
+    for (int it = 0; it < n_pre; ++it) {
+      arm(it);
+      issue_head(it);
+    }
   // Under programmatic dependent launch the grid may start while the previous kernel of the stream
   // drains: the features (and the scratch) are that kernel's business until it has completed.
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -176,24 +244,28 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_con
         const int st = it % S;
         ok = mbar_wait(bar(kLmBarEmpty + st), (it / S - 1) & 1, abort_flag);
         if (!ok) break;
-        mbar_expect_tx(bar(kLmBarFull + st), p.stage_bytes);
+        arm(it);
         issue_head(it);
         issue_feat(it);
       }
       if (!ok || *abort_flag) {
         // Some wait gave up.  The tiles asked for still arrive: stay until they have, so that no copy
         // is in flight into this CTA's shared memory when it leaves.
-        for (int j = max(0, it - S); j < it; ++j) lm_wait_drain(bar(kLmBarFull + j % S), (j / S) & 1);
+        if (leader)
+          for (int j = max(0, it - S); j < it; ++j) lm_wait_drain(bar(kLmBarFull + j % S), (j / S) & 1);
+        else  // (they signal the other CTA's barriers: leave them a millisecond)
+          for (int j = 0; j < 1000; ++j) __nanosleep(1000);
       }
     }
+    __syncwarp();
   } else if (warp == 1) {
     // ================================ MMA issuer ================================
     uint32_t elected;
     asm volatile("{ .reg .pred p; elect.sync _|p, 0xffffffff; selp.u32 %0, 1, 0, p; }" : "=r"(elected));
     int it = 0, tile = 0;
-    bool ok = !*abort_flag;
+    bool ok = leader && !*abort_flag;
     for (int g = 0; ok && g < n_groups; ++g) {
-      for (int vt = 0; ok && vt < n_vt; ++vt, ++tile) {
+      for (int vp = 0; ok && vp < n_vp; ++vp, ++tile) {
         if (tile > 0) ok = mbar_wait_warp(bar(kLmBarAccEmpty), (tile - 1) & 1, abort_flag);  // the readers are done with TMEM
         if (!ok) break;
         tc_fence_after();
@@ -204,29 +276,39 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_con
           tc_fence_after();
           if (elected) {
             const uint32_t wbase = smem_base + static_cast<uint32_t>(st) * p.stage_bytes;
-            const uint32_t fbase = wbase + static_cast<uint32_t>(p.kch) * w_bytes;
+            const uint32_t fbase = wbase + static_cast<uint32_t>(p.kch * v_res) * w_bytes;
             for (int c = 0; c < p.kch; ++c) {
-              for (int j = 0; j < p.m_res; ++j) {
+              for (int j = 0; j < (v_res > 1 ? 2 : tiles_of(g)); ++j) {  // accumulators: node tiles or vocabulary tiles
+                const uint32_t fj = fbase + (c * m_res + (m_res > 1 ? j : 0)) * f_bytes, wj = wbase + (c * v_res + (v_res > 1 ? j : 0)) * w_bytes;
 #pragma unroll
                 for (int kk = 0; kk < kLmKC / 16; ++kk) {
                   // features (A) and head rows (B): both K-major, 16 hidden columns = 32 bytes inside the 128-byte swizzle row
-                  const uint64_t ad = smem_desc(fbase + (c * p.m_res + j) * f_bytes + kk * 32, 16, 1024);
-                  const uint64_t bd = smem_desc(wbase + c * w_bytes + kk * 32, 16, 1024);
-                  umma_bf16_ss(tmem_base + static_cast<uint32_t>(j) * 256u, ad, bd, p.idesc, (ks > 0 || c > 0 || kk > 0) ? 1u : 0u);
+                  const uint64_t ad = smem_desc(fj + kk * 32, 16, 1024), bd = smem_desc(wj + kk * 32, 16, 1024);
+                  const uint32_t acc = tmem_base + static_cast<uint32_t>(j) * 256u, more = (ks > 0 || c > 0 || kk > 0) ? 1u : 0u;
+                  if constexpr (kPair) umma_pair_ss(acc, ad, bd, p.idesc, more);
+                  else umma_bf16_ss(acc, ad, bd, p.idesc, more);
                 }
               }
             }
-            umma_commit(bar(kLmBarEmpty + st));
+            if constexpr (kPair) umma_pair_commit(bar(kLmBarEmpty + st));
+            else umma_commit(bar(kLmBarEmpty + st));
           }
           __syncwarp();
         }
-        if (ok && elected) umma_commit(bar(kLmBarAccFull));
+        if (ok && elected) {
+          if constexpr (kPair) umma_pair_commit(bar(kLmBarAccFull));
+          else umma_commit(bar(kLmBarAccFull));
+        }
         __syncwarp();
       }
     }
     // every MMA issued so far has finished before TMEM is given back
     if (elected) {
-      umma_commit(bar(kLmBarDone));
+      if constexpr (kPair) {
+        if (leader) umma_pair_commit(bar(kLmBarDone));
+      } else {
+        umma_commit(bar(kLmBarDone));
+      }
       lm_wait_drain(bar(kLmBarDone), 0);
     }
     __syncwarp();
@@ -241,15 +323,17 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_con
     for (int g = 0; g < n_groups; ++g) {
       float best[2] = {-INFINITY, -INFINITY};
       int idx[2] = {INT_MAX, INT_MAX};
-      for (int vt = 0; ok && vt < n_vt; ++vt, ++tile) {
+      for (int vp = 0; ok && vp < n_vp; ++vp, ++tile) {
         ok = mbar_wait_warp(bar(kLmBarAccFull), tile & 1, abort_flag);
         if (!ok) break;
         tc_fence_after();
-        const int v0 = v_lo + vt * p.tile_n;
-        const int ncols = min(p.tile_n, v_hi - v0);
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          if (j >= p.m_res) break;
+        for (int j = 0; j < (kPair ? 2 : 1); ++j) {
+          const int v0 = v_lo + (v_res > 1 ? vp * 2 + j : vp) * p.tile_n;
+          const int ncols = v_res > 1 || j < tiles_of(g) ? min(p.tile_n, v_hi - v0) : 0;
+          // (vocabulary tiles follow one another: one maximum per row; node tiles are different rows)
+          float m = v_res > 1 ? best[0] : best[j];
+          int mi = v_res > 1 ? idx[0] : idx[j];
           for (int c0 = 0; c0 < ncols; c0 += 32) {
             uint32_t x[32];
             FALCON_TMEM_LD32(tmem_lane + static_cast<uint32_t>(j) * 256u + static_cast<uint32_t>(c0), x);
@@ -257,22 +341,32 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_con
 #pragma unroll
             for (int c = 0; c < 32; ++c) {
               const float f = __uint_as_float(x[c]);
-              if (c0 + c < ncols && f > best[j]) {  // strict: columns ascend, so the first maximum stays; NaN never wins
-                best[j] = f;
-                idx[j] = v0 + c0 + c;
+              if (c0 + c < ncols && f > m) {  // strict: columns ascend, so the first maximum stays; NaN never wins
+                m = f;
+                mi = v0 + c0 + c;
               }
             }
+          }
+          if (v_res > 1) {
+            best[0] = m;
+            idx[0] = mi;
+          } else {
+            best[j] = m;
+            idx[j] = mi;
           }
         }
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(bar(kLmBarAccEmpty));
+        if (lane == 0) {
+          if constexpr (kPair) arrive_remote(map_to_leader(bar(kLmBarAccEmpty)));
+          else mbar_arrive(bar(kLmBarAccEmpty));
+        }
       }
 #pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        const int node = (g * p.m_res + j) * 128 + r;
+      for (int j = 0; j < (kPair ? 2 : 1); ++j) {
+        const int node = kPair ? (g * m_res + j) * 256 + rank * 128 + r : g * 128 + r;
         // one atomic per node and CTA: the order of arrival does not matter, the word's order decides
-        if (j < p.m_res && node < p.n_rows && ok && idx[j] != INT_MAX) atomicMax(p.best + node, lm_pack(best[j], idx[j]));
+        if (j < m_res && node < p.n_rows && ok && idx[j] != INT_MAX) atomicMax(p.best + node, lm_pack(best[j], idx[j]));
       }
     }
     // the last CTA to arrive folds the CTAs' results in vocabulary order
@@ -295,33 +389,47 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_con
     }
   }
   tc_fence_before();
-  __syncthreads();
+  if constexpr (kPair) cluster_sync_release();  // (and neither CTA leaves while the other may still signal it)
+  else __syncthreads();
   if (warp == 1) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(tmem_cols) : "memory");
+    if constexpr (kPair)
+      asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(tmem_cols) : "memory");
+    else
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(tmem_cols) : "memory");
   }
 }
 
 }  // namespace
 
 cudaError_t set_up_lm_head() {
-  return cudaFuncSetAttribute(lm_head_argmax_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kLmSmemMax));
+  const cudaError_t e = cudaFuncSetAttribute(lm_head_argmax_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kLmSmemMax));
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(lm_head_argmax_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kLmSmemMax));
 }
 
 int launch_lm_head_argmax(falcon_ctx* ctx, const falcon_lm_argmax_args& a, cudaStream_t s) {
   const int N = a.n_rows, V = a.vocab, H = a.hidden;
-  const int n_mt = (N + 127) / 128;
-  const int m_res = n_mt >= 2 ? 2 : 1;
-  // One wave: the vocabulary split evenly over the SMs in steps of 16 rows.
-  int span = ((V + ctx->sm_count - 1) / ctx->sm_count + 15) & ~15;
-  const int n_cta = (V + span - 1) / span;
-  const int tile_n = span < kLmTileMax ? span : kLmTileMax;
-  const int f_rows = n_mt > 1 ? 128 : (N <= 64 ? 64 : ((N + 7) & ~7));
+  const bool pair = N > 128;  // (a single tile has nothing to share: the head's rows bound it)
+  const int n_mt = pair ? (N + 255) / 256 : 1;
+  const int m_res = n_mt >= 2 ? 2 : 1, v_res = pair && m_res == 1 ? 2 : 1;
+  // One wave: the vocabulary split evenly over the SMs or pairs of them, in tiles of the same multiple of 16 rows.
+  const int workers = pair ? ctx->sm_count / 2 : ctx->sm_count;
+  const int share = (V + workers - 1) / workers, n_vt = (share + kLmTileMax - 1) / kLmTileMax;
+  int tile_n = ((share + n_vt - 1) / n_vt + 15) & ~15;
+  int span = tile_n * n_vt;
+  if (!pair) {
+    span = (share + 15) & ~15;
+    tile_n = span < kLmTileMax ? span : kLmTileMax;
+  }
+  const int n_cta = (V + span - 1) / span * (pair ? 2 : 1);
+  const int f_rows = pair ? 128 : (N <= 64 ? 64 : ((N + 7) & ~7));
+  const int w_rows = pair ? tile_n / 2 : tile_n;
   const int n_kc = (H + kLmKC - 1) / kLmKC;
   // Chunks per stage: two where two such stages fit.  Fewer, larger stages mean fewer trips round the ring
   // (32000 x 4096, 60 nodes: 43 us with two chunks in three stages against 53 with one in five and 46 with
-  // three in two; a head stored chunk by chunk so that a tile is contiguous made no difference).
-  const uint32_t chunk_bytes = (static_cast<uint32_t>(tile_n) + static_cast<uint32_t>(m_res * f_rows)) * (kLmKC * 2u);
+  // three in two; in pairs, 512 nodes of 5120: 133 with two chunks in two stages, 158 with one in four; a head stored chunk by chunk so that a tile is contiguous made no difference).
+  const uint32_t chunk_bytes = static_cast<uint32_t>(v_res * w_rows + m_res * f_rows) * (kLmKC * 2u);
   int kch = (2 * 2 * chunk_bytes <= kLmSmemMax - kLmSmallBytes) ? 2 : 1;
   if (kch > n_kc) kch = n_kc;
   const uint32_t stage_bytes = static_cast<uint32_t>(kch) * chunk_bytes;
@@ -341,7 +449,7 @@ int launch_lm_head_argmax(falcon_ctx* ctx, const falcon_lm_argmax_args& a, cudaS
     const uint64_t hs = static_cast<uint64_t>(a.head_stride) * 2, fs = static_cast<uint64_t>(a.feat_stride) * 2;
     const uint64_t w_dims[5] = {static_cast<uint64_t>(H), static_cast<uint64_t>(V), 1, 1, 1};
     const uint64_t w_strides[4] = {hs, hs * V, hs * V, hs * V};
-    const uint32_t w_box[5] = {kLmKC, static_cast<uint32_t>(tile_n), 1, 1, 1};
+    const uint32_t w_box[5] = {kLmKC, static_cast<uint32_t>(w_rows), 1, 1, 1};
     const uint64_t f_dims[5] = {static_cast<uint64_t>(H), static_cast<uint64_t>(N), 1, 1, 1};
     const uint64_t f_strides[4] = {fs, fs * N, fs * N, fs * N};
     const uint32_t f_box[5] = {kLmKC, static_cast<uint32_t>(f_rows), 1, 1, 1};
@@ -359,12 +467,13 @@ int launch_lm_head_argmax(falcon_ctx* ctx, const falcon_lm_argmax_args& a, cudaS
   p.f_rows = f_rows;
   p.n_mt = n_mt;
   p.m_res = m_res;
+  p.v_res = v_res;
   p.tile_n = tile_n;
   p.span = span;
   p.n_stages = n_stages;
   p.stall_first = (a.flags & FALCON_LM_TEST_STALL) ? 1 : 0;
   p.stage_bytes = stage_bytes;
-  p.idesc = make_idesc(128, static_cast<uint32_t>(tile_n), false, false);
+  p.idesc = make_idesc(pair ? 256 : 128, static_cast<uint32_t>(tile_n), false, false);
   p.argmax_out = a.argmax_out;
   p.max_out = a.max_out;
   p.status = a.status;
@@ -376,12 +485,16 @@ int launch_lm_head_argmax(falcon_ctx* ctx, const falcon_lm_argmax_args& a, cudaS
   cfg.blockDim = dim3(kLmThreads);
   cfg.dynamicSmemBytes = smem_bytes;
   cfg.stream = s;
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, lm_head_argmax_kernel, mw, mf, p);
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = 2;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = pair ? 2 : 1;
+  cudaError_t e = cudaLaunchKernelEx(&cfg, pair ? lm_head_argmax_kernel<true> : lm_head_argmax_kernel<false>, mw, mf, p);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "lm_head_argmax_kernel launch");
   return FALCON_OK;
 }

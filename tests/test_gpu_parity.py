@@ -961,6 +961,14 @@ def test_lm_head_argmax_integer_data_is_bit_exact(N, Hd, V):
         np.testing.assert_array_equal(mx.astype(np.float64), best_ref)
 
 
+@pytest.mark.parametrize("N,Hd,V", [(129, 64, 1), (256, 72, 2369), (256, 128, 45000), (257, 8, 33), (385, 192, 20000), (512, 320, 2368),
+                                    (513, 136, 40001)])
+def test_lm_head_argmax_pairs_of_ctas(N, Hd, V):
+    # more than 128 nodes: a pair of CTAs shares the work; edges of its 256-node tiles, one and several vocabulary
+    # tiles, a second group of node tiles, and a pair's last vocabulary tile cut short or empty
+    test_lm_head_argmax_integer_data_is_bit_exact(N, Hd, V)
+
+
 @pytest.mark.parametrize("N,Hd,V,pad", [(60, 512, 5000, 0), (130, 320, 3001, 8), (15, 72, 1000, 24), (257, 256, 4096, 0)])
 def test_lm_head_argmax_random_data(N, Hd, V, pad):
     # hidden sizes that are not multiples of the 64-column stage, padded row pitches, ragged tails
@@ -1055,6 +1063,23 @@ def test_lm_head_argmax_bounded_wait_runs_out_and_the_context_stays_usable():
     c.falcon_lm_head_argmax(binding.lm_argmax_args(N, Hd, V, fd, Hd, wd, Hd, g, None, st))
     torch.cuda.synchronize()
     assert int(st.item()) == 0
+    np.testing.assert_array_equal(g.cpu().numpy(), oracle.lm_head_argmax(f, w)[0])
+
+
+def test_lm_head_argmax_pairs_bounded_wait():
+    # the same with pairs of CTAs, both of which have to leave in order
+    N, Hd, V = 200, 256, 3000
+    rng = np.random.default_rng(13)
+    f = synth.f32_to_bf16_bits(rng.integers(-3, 4, size=(N, Hd)).astype(np.float32))
+    w = synth.f32_to_bf16_bits(rng.integers(-3, 4, size=(V, Hd)).astype(np.float32))
+    fd, wd = H.dev_bf16(f), H.dev_bf16(w)
+    g = torch.zeros(N, dtype=torch.int32, device="cuda")
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    for flags in (binding.LM_TEST_STALL, 0):
+        st.zero_()
+        H.ctx().falcon_lm_head_argmax(binding.lm_argmax_args(N, Hd, V, fd, Hd, wd, Hd, g, None, st, flags=flags))
+        torch.cuda.synchronize()
+        assert int(st.item()) == (binding.DEV_TIMEOUT if flags else 0)
     np.testing.assert_array_equal(g.cpu().numpy(), oracle.lm_head_argmax(f, w)[0])
 
 
