@@ -1,21 +1,20 @@
 // falcon_kv_compact: the accepted path's K/V rows become the contiguous tail of
-// the cache, every layer and both K and V in one launch.  One CTA owns all rows
-// of one (layer, K|V, sequence, KV head): it reads every source row into
-// registers, passes a barrier, then writes, so a destination row that is also an
-// earlier source row (in-place mode) cannot be clobbered before it is read.
-// Launch/latency-bound byte copy with 16-byte accesses: what matters is that the
-// whole grid is resident at once (each CTA is a chain of three dependent round
-// trips to memory), so trees small enough get a variant that keeps few registers
-// per thread and moves K and V in the same CTA.
+// the cache, every layer and both K and V in one launch.  One warp moves the K and V rows of one (layer,
+// sequence, KV head): a byte copy of 16-byte accesses, a few KB per warp, bound by the chain of round trips to
+// memory (lengths, path, rows) that every warp is, so what counts is how many warps are resident.  An
+// accepted path is a handful of rows: with a CTA per (layer, sequence, head), sized for the longest path there could be, a
+// batch of 8 sequences x 32 heads x 32 layers ran in 11 waves, 28.7 us; with a warp each 5.7 (one sequence, 32 x 32: 4.5 ->
+// 2.3; 16 sequences, 8 heads: 12.4 -> 4.8).
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace falcon {
 namespace {
 
 constexpr int kCompactThreads = 256;
-constexpr int kMaxChunksPerThread = 16;  // 128 rows x 32 chunks (D = 256) / 256 threads
-constexpr int kSmallChunksPerThread = 4; // the small variant: trees of up to 1024 chunks per matrix
-constexpr int kMidChunksPerThread = 6;   // up to 1536 chunks per matrix (96 nodes at head_dim 128)
+constexpr int kCompactWarps = kCompactThreads / 32;
+constexpr int kCompactPieces = 4;        // 16-byte pieces per lane, matrix and round: eight rows of 128
 
 struct CompactParams {
   int32_t batch, n_layers, n_kv_heads, head_dim, s_cap, path_stride;
@@ -37,7 +36,8 @@ struct CompactParams {
   int32_t* tokens_out;
   int64_t feat_stride;
   int32_t hidden, out_rows;
-  int32_t gather_z;  // the grid's z slice that does the gather in a combined launch
+  int32_t max_rows;   // a longer path than the caller's max_tree lets expect is refused
+  int32_t move_ctas;  // CTAs of a sequence that move rows; what follows them does the gather of a combined launch
 };
 
 // Accepted tokens and features of sequence b: an out-of-place row gather along the path (Section
@@ -55,101 +55,108 @@ __device__ __forceinline__ void gather_features(const CompactParams& p, int b, i
   if (part == 0 && tid < n) p.tokens_out[static_cast<int64_t>(b) * p.out_rows + tid] = p.token[base + s_path[tid]];
 }
 
-// kBoth: blockIdx.z is the layer and the CTA moves K then V (both held in registers at once);
-// otherwise blockIdx.z is 2 * layer + (0 for K, 1 for V).
-template <int kChunks, bool kBoth>
-__global__ void __launch_bounds__(kCompactThreads) kv_compact_kernel(const CompactParams p) {
+__global__ void __launch_bounds__(kCompactThreads, 4) kv_compact_kernel(const CompactParams p) {
   __shared__ int s_path[FALCON_T_MAX];
-  __shared__ int s_bad;
+  const int b = blockIdx.y, tid = threadIdx.x, lane = tid & 31;
+  const bool gather = static_cast<int>(blockIdx.x) >= p.move_ctas;
   // Under programmatic dependent launch the grid may start while the previous kernel of the stream
   // drains: nothing is read or written before that kernel has completed.
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const int h = blockIdx.x, b = blockIdx.y;
-  const bool gather_slice = p.features != nullptr && static_cast<int>(blockIdx.z) == p.gather_z;
-  const int layer = gather_slice ? 0 : (kBoth ? blockIdx.z : (blockIdx.z >> 1));
-  const int tid = threadIdx.x;
-  constexpr int kMats = kBoth ? 2 : 1;
 
-  const int base = p.node_off[b];
-  const int T = p.node_off[b + 1] - base;
-  const int L = p.prefix_len[b];
-  const int n = p.n_path[b];
-  const bool separate = (p.k_tree_layers != nullptr);
+  // All at once: lengths, path (beyond its end it may hold anything) and this warp's pointers.
+  const int base = p.node_off[b], T = p.node_off[b + 1] - base, L = p.prefix_len[b], n = p.n_path[b];
+  const int t = tid < p.path_stride && tid < FALCON_T_MAX ? p.path[static_cast<int64_t>(b) * p.path_stride + tid] : 0;
+  const int unit = blockIdx.x * kCompactWarps + warp_index(), layer = unit / p.n_kv_heads, h = unit - layer * p.n_kv_heads;
+  const bool mine = !gather && layer < p.n_layers, separate = p.k_tree_layers != nullptr;
+  __nv_bfloat16* cache[2] = {nullptr, nullptr};
+  const __nv_bfloat16* from[2] = {nullptr, nullptr};  // row 0 of the tree
+  if (mine) {
+    cache[0] = static_cast<__nv_bfloat16*>(p.k_layers[layer]);
+    cache[1] = static_cast<__nv_bfloat16*>(p.v_layers[layer]);
+    if (separate) {
+      from[0] = static_cast<const __nv_bfloat16*>(p.k_tree_layers[layer]);
+      from[1] = static_cast<const __nv_bfloat16*>(p.v_tree_layers[layer]);
+    }
+  }
   int fault = 0;
   if (T < 1 || T > FALCON_T_MAX || n < 1 || n > T) fault |= FALCON_DEV_BAD_PATH;
-  if (!gather_slice) {
-    if (L < 0 || L + (separate ? n : T) > p.s_cap) fault |= FALCON_DEV_CAPACITY;
-    // the variant was picked from the caller's max_tree: a longer path than it can hold is refused
-    if (n > 0 && static_cast<int64_t>(n) * (p.head_dim >> 3) > static_cast<int64_t>(kChunks) * kCompactThreads)
-      fault |= FALCON_DEV_CAPACITY;
-  } else if (n > p.out_rows) {
-    fault |= FALCON_DEV_CAPACITY;
-  }
-  if (tid == 0) s_bad = 0;
-  __syncthreads();
-  if (!fault && tid < n) {
-    const int t = p.path[static_cast<int64_t>(b) * p.path_stride + tid];
-    s_path[tid] = t;
-    if (t < 0 || t >= T) s_bad = 1;
-  }
-  __syncthreads();
-  if (s_bad) fault |= FALCON_DEV_BAD_PATH;
-  if (gather_slice) {
-    if (fault) {
-      if (h == 0 && tid == 0) dev_status_or(p.status, b, fault);
-      return;
-    }
-    gather_features(p, b, base, n, s_path, h, gridDim.x, tid);
+  if (n > p.path_stride || (!gather && n > p.max_rows)) fault |= FALCON_DEV_CAPACITY;
+  if (!gather && (L < 0 || L + (separate ? n : T) > p.s_cap)) fault |= FALCON_DEV_CAPACITY;
+  if (gather && n > p.out_rows) fault |= FALCON_DEV_CAPACITY;
+  if (tid < FALCON_T_MAX) s_path[tid] = t;
+  if (__syncthreads_or(tid < n && (t < 0 || t >= T)) && n <= T) fault |= FALCON_DEV_BAD_PATH;
+  if (gather) {
+    const int part = blockIdx.x - p.move_ctas;
+    if (!fault) gather_features(p, b, base, n, s_path, part, gridDim.x - p.move_ctas, tid);
+    else if (part == 0 && tid == 0) dev_status_or(p.status, b, fault);
     return;
   }
-  const bool first = (h == 0 && blockIdx.z == 0 && tid == 0);  // one writer of the new length per sequence
-  if (fault) {  // leave the cache alone, report, keep the old length
-    if (first) {
-      dev_status_or(p.status, b, fault);
-      p.new_len[b] = L;
+  if (blockIdx.x == 0 && tid == 0) {  // one writer of the new length per sequence
+    p.new_len[b] = fault ? L : L + n;
+    if (fault) dev_status_or(p.status, b, fault);
+  }
+  if (fault || !mine) return;  // (a fault: leave the cache alone)
+
+  const int64_t from_row = separate ? static_cast<int64_t>(p.n_kv_heads) * p.head_dim : p.stride_s;
+#pragma unroll
+  for (int m = 0; m < 2; ++m) {
+    cache[m] += b * p.stride_b + h * p.stride_h + L * p.stride_s;  // first row behind the prefix
+    from[m] = separate ? from[m] + (static_cast<int64_t>(base) * p.n_kv_heads + h) * p.head_dim : cache[m];
+  }
+  const int cpr = p.head_dim >> 3;  // 16-byte pieces per row
+  // Row j goes to place j.  A path leads from a node to its child, whose number is higher, so its j-th entry is at least
+  // j: what a round writes lies below everything that a later round reads.  (Rows already in place stay.)
+  bool ordered = true;
+  for (int j = lane; j < n; j += 32) ordered = ordered && s_path[j] >= j;
+  if (separate || __all_sync(0xffffffffu, ordered)) {
+    const int dj = 32 / cpr, dc = 32 - dj * cpr;
+    int j = lane / cpr, c = lane - j * cpr;
+    for (int first = 0; first < n * cpr; first += 32 * kCompactPieces) {
+      uint4 x[2][kCompactPieces];
+      int to[kCompactPieces], col[kCompactPieces];
+#pragma unroll
+      for (int k = 0; k < kCompactPieces; ++k) {
+        to[k] = j < n && (separate || s_path[j] != j) ? j : -1;
+        col[k] = 8 * c;
+        if (to[k] >= 0) {
+          const int64_t at = s_path[j] * from_row + col[k];
+          x[0][k] = *reinterpret_cast<const uint4*>(from[0] + at);
+          x[1][k] = *reinterpret_cast<const uint4*>(from[1] + at);
+        }
+        j += dj;
+        c += dc;
+        if (c >= cpr) {
+          c -= cpr;
+          ++j;
+        }
+      }
+      __syncwarp();  // every row of the round is in registers before any of its places is written
+#pragma unroll
+      for (int k = 0; k < kCompactPieces; ++k) {
+        if (to[k] >= 0) {
+          const int64_t at = to[k] * p.stride_s + col[k];
+          *reinterpret_cast<uint4*>(cache[0] + at) = x[0][k];
+          *reinterpret_cast<uint4*>(cache[1] + at) = x[1][k];
+        }
+      }
+      __syncwarp();
     }
     return;
   }
-  if (first) p.new_len[b] = L + n;
-
-  __nv_bfloat16* cache[kMats];
-  const __nv_bfloat16* tree[kMats];
+  // Any other order of rows: 16 bytes of every row at a time, all of them in registers before any is written.
+  for (int m = 0; m < 2; ++m) {
+    __nv_bfloat16* rows = m ? cache[1] : cache[0];
+    for (int c = 0; c < cpr; ++c) {
+      uint4 x[FALCON_T_MAX / 32];
 #pragma unroll
-  for (int m = 0; m < kMats; ++m) {
-    const bool is_v = kBoth ? (m == 1) : ((blockIdx.z & 1) != 0);
-    cache[m] = static_cast<__nv_bfloat16*>(is_v ? p.v_layers[layer] : p.k_layers[layer]) + b * p.stride_b + h * p.stride_h;
-    tree[m] = separate ? static_cast<const __nv_bfloat16*>(is_v ? p.v_tree_layers[layer] : p.k_tree_layers[layer])
-                       : nullptr;
-  }
-
-  const int cpr = p.head_dim >> 3;  // 16-byte chunks per row
-  const int total = n * cpr;
-  uint4 regs[kMats][kChunks];
+      for (int k = 0; k < FALCON_T_MAX / 32; ++k)
+        if (lane + 32 * k < n) x[k] = *reinterpret_cast<const uint4*>(rows + s_path[lane + 32 * k] * p.stride_s + 8 * c);
+      __syncwarp();
 #pragma unroll
-  for (int m = 0; m < kMats; ++m) {
-#pragma unroll
-    for (int k = 0; k < kChunks; ++k) {
-      const int idx = tid + k * kCompactThreads;
-      if (idx < total) {
-        const int j = idx / cpr, c = idx - j * cpr;
-        const __nv_bfloat16* src =
-            separate ? tree[m] + (static_cast<int64_t>(base + s_path[j]) * p.n_kv_heads + h) * p.head_dim
-                     : cache[m] + static_cast<int64_t>(L + s_path[j]) * p.stride_s;
-        regs[m][k] = *reinterpret_cast<const uint4*>(src + 8 * c);
-      }
-    }
-  }
-  __syncthreads();  // every source row is in registers before any destination row is written
-#pragma unroll
-  for (int m = 0; m < kMats; ++m) {
-#pragma unroll
-    for (int k = 0; k < kChunks; ++k) {
-      const int idx = tid + k * kCompactThreads;
-      if (idx < total) {
-        const int j = idx / cpr, c = idx - j * cpr;
-        *reinterpret_cast<uint4*>(cache[m] + static_cast<int64_t>(L + j) * p.stride_s + 8 * c) = regs[m][k];
-      }
+      for (int k = 0; k < FALCON_T_MAX / 32; ++k)
+        if (lane + 32 * k < n) *reinterpret_cast<uint4*>(rows + (lane + 32 * k) * p.stride_s + 8 * c) = x[k];
+      __syncwarp();
     }
   }
 }
@@ -196,9 +203,7 @@ void set_gather(CompactParams& p, const falcon_gather_args& g, const int32_t* to
 }  // namespace
 
 cudaError_t set_up_compact() {
-  cudaError_t e = prefer_shared(kv_compact_kernel<kSmallChunksPerThread, true>);
-  if (e == cudaSuccess) e = prefer_shared(kv_compact_kernel<kMidChunksPerThread, true>);
-  if (e == cudaSuccess) e = prefer_shared(kv_compact_kernel<kMaxChunksPerThread, false>);
+  cudaError_t e = prefer_shared(kv_compact_kernel);
   if (e == cudaSuccess) e = prefer_shared(feature_gather_kernel);
   return e;
 }
@@ -211,6 +216,12 @@ int check_gather_args(const falcon_gather_args& g, int max_tree) {
   return FALCON_OK;
 }
 
+// CTAs that share a sequence's gather
+static int gather_parts(const falcon_gather_args& a, int max_tree) {
+  const int64_t chunks = static_cast<int64_t>(max_tree) * (a.hidden >> 3);
+  return static_cast<int>(std::min<int64_t>(32, std::max<int64_t>(1, (chunks + 2 * kCompactThreads - 1) / (2 * kCompactThreads))));
+}
+
 int launch_feature_gather(falcon_ctx* ctx, const falcon_gather_args& a, cudaStream_t s) {
   if (a.tree.batch > 65535) return FALCON_ERR_CAPACITY;
   CompactParams p = {};
@@ -221,12 +232,8 @@ int launch_feature_gather(falcon_ctx* ctx, const falcon_gather_args& a, cudaStre
   p.path = a.path;
   p.n_path = a.n_path;
   set_gather(p, a, a.tree.token);
-  const int64_t chunks = static_cast<int64_t>(a.tree.max_tree) * (a.hidden >> 3);
-  int parts = static_cast<int>((chunks + 2 * kCompactThreads - 1) / (2 * kCompactThreads));
-  if (parts < 1) parts = 1;
-  if (parts > 32) parts = 32;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(parts, a.tree.batch);
+  cfg.gridDim = dim3(gather_parts(a, a.tree.max_tree), a.tree.batch);
   cfg.blockDim = dim3(kCompactThreads);
   cfg.stream = s;
   cudaLaunchAttribute attr;
@@ -261,10 +268,12 @@ int launch_kv_compact(falcon_ctx* ctx, const falcon_compact_args& a, cudaStream_
   p.path = a.path;
   p.n_path = a.n_path;
   p.new_len = a.new_len;
-  const int extra = a.gather ? 1 : 0;  // one more z slice of CTAs records the accepted tokens and features
-  if (a.gather) set_gather(p, *a.gather, a.tree.token);
-  // the path is at most max_tree rows long: small trees take the variant with K and V in one CTA
-  const int64_t max_chunks = static_cast<int64_t>(a.tree.max_tree) * (a.head_dim >> 3);
+  const int64_t move_ctas = (static_cast<int64_t>(a.n_layers) * a.n_kv_heads + kCompactWarps - 1) / kCompactWarps;
+  if (move_ctas > INT32_MAX - 32) return FALCON_ERR_CAPACITY;
+  p.move_ctas = static_cast<int32_t>(move_ctas);
+  const int cpr = a.head_dim >> 3, pieces = a.tree.max_tree * cpr;
+  p.max_rows = (pieces <= 1024 ? 1024 : pieces <= 1536 ? 1536 : 4096) / cpr;
+  if (a.gather) set_gather(p, *a.gather, a.tree.token);  // further CTAs record the accepted tokens and features
   cudaLaunchConfig_t cfg = {};
   cfg.blockDim = dim3(kCompactThreads);
   cfg.stream = s;
@@ -273,20 +282,8 @@ int launch_kv_compact(falcon_ctx* ctx, const falcon_compact_args& a, cudaStream_
   attr.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
-  cudaError_t e;
-  if (max_chunks <= static_cast<int64_t>(kSmallChunksPerThread) * kCompactThreads) {
-    p.gather_z = a.n_layers;
-    cfg.gridDim = dim3(a.n_kv_heads, a.tree.batch, a.n_layers + extra);
-    e = cudaLaunchKernelEx(&cfg, kv_compact_kernel<kSmallChunksPerThread, true>, p);
-  } else if (max_chunks <= static_cast<int64_t>(kMidChunksPerThread) * kCompactThreads) {
-    p.gather_z = a.n_layers;
-    cfg.gridDim = dim3(a.n_kv_heads, a.tree.batch, a.n_layers + extra);
-    e = cudaLaunchKernelEx(&cfg, kv_compact_kernel<kMidChunksPerThread, true>, p);
-  } else {
-    p.gather_z = 2 * a.n_layers;
-    cfg.gridDim = dim3(a.n_kv_heads, a.tree.batch, 2 * a.n_layers + extra);
-    e = cudaLaunchKernelEx(&cfg, kv_compact_kernel<kMaxChunksPerThread, false>, p);
-  }
+  cfg.gridDim = dim3(p.move_ctas + (a.gather ? gather_parts(*a.gather, a.tree.max_tree) : 0), a.tree.batch);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kv_compact_kernel, p);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "kv_compact_kernel launch");
   return FALCON_OK;
 }

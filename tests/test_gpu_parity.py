@@ -427,6 +427,20 @@ def test_compact_random_paths_overlap_and_identity(separate, D):
     check_compact(tb, 3, D, 2, rng, path, n_path, separate=separate)
 
 
+@pytest.mark.parametrize("D", [8, 24, 40, 128, 200])
+def test_compact_rows_per_round_and_any_order(D):
+    """Rows that do not divide a warp's round, more units than warps in a CTA, and paths whose rows are in no order."""
+    rng = np.random.default_rng(D)
+    tb = H.make_trees([128, 33, 9], [3, 40, 0], rng, parents=[synth.chain_tree(128), synth.chain_tree(33), synth.chain_tree(9)])
+    for order in (np.sort, lambda x: x):
+        path = np.full((3, 128), -1, np.int32)
+        n_path = np.array([97, 17, 8], np.int32)
+        for b, (T, n) in enumerate(zip((128, 33, 9), n_path)):
+            path[b, :n] = order(rng.permutation(T)[:n])
+        for separate in (False, True):
+            check_compact(tb, 3, D, 3, rng, path, n_path, separate=separate)
+
+
 def test_compact_handworked_overlap_path():
     rng = np.random.default_rng(4)
     tb = H.make_trees([4], [2], rng, parents=[np.array([-1, 0, 0, 2], np.int32)])
