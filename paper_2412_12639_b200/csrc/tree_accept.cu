@@ -1,7 +1,9 @@
 // falcon_tree_accept: per-node vocabulary argmax and the longest accepted path,
-// one launch.  Every CTA scans one chunk of one logits row with 16-byte loads;
-// the last CTA to finish a sequence (arrival counter) folds the chunk partials
-// into g[] and searches the tree.  HBM-bound: the N*V fp32 logits are read once.
+// one launch.  Every CTA scans one chunk of one logits row; the last CTA to finish a sequence
+// (arrival counter) folds the chunk partials into g[] and searches the tree.  HBM-bound: the N*V fp32
+// logits are read once.  Rows of more than 4096 entries are streamed through shared memory by bulk copies
+// (kStream: row_stream.cuh says why); with 16-byte loads into registers instead, us per call: 60 rows of 32000 6.9
+// (streamed 5.9), 456 rows 17.3 (14.7, 4 TB/s), 300 rows of 100001 38.2 (24.2, 5 TB/s).
 #include <cfloat>
 #include <climits>
 
@@ -126,20 +128,35 @@ __device__ __forceinline__ void search_tree(const AcceptParams& p, int b, int ba
 }
 
 
-__global__ void __launch_bounds__(kAcceptThreads) tree_accept_kernel(const AcceptParams p) {
+template <bool kStream>
+__global__ void __launch_bounds__(kAcceptThreads + (kStream ? 32 : 0)) tree_accept_kernel(const AcceptParams p) {
+  extern __shared__ __align__(128) unsigned char stream_buf[];  // kStream
+  __shared__ __align__(8) StreamBars bars;
   __shared__ Best warp_best[kAcceptThreads / 32];
   __shared__ int s_flag;
   __shared__ int s_par[FALCON_T_MAX], s_tok[FALCON_T_MAX], s_g[FALCON_T_MAX];
   __shared__ int s_key[kAcceptThreads / 32];
 
-  // Under programmatic dependent launch the grid may start while the previous kernel of the stream
-  // drains: nothing is read or written before that kernel has completed.
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int row = blockIdx.y, chunk = blockIdx.x, tid = threadIdx.x;
   const int c0 = chunk * p.chunk_len;
   const int c1 = min(p.vocab, c0 + p.chunk_len);
   const float* rowp = p.logits + static_cast<int64_t>(row) * p.logits_stride;
+  const RowStream rs(rowp + c0, max(0, c1 - c0), stream_buf, &bars);
+  if constexpr (kStream) {
+    if (tid == kStreamThreads) RowStream::init(&bars);
+    __syncthreads();
+  }
+  // Under programmatic dependent launch the grid may start while the previous kernel of the stream
+  // drains: nothing is read or written before that kernel has completed.
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if constexpr (kStream) {
+    if (warp_index() == kStreamWarps) {
+      if ((tid & 31) == 0) rs.produce(0, rs.stages());
+      return;
+    }
+  }
+  auto worker_sync = [] { asm volatile("bar.sync 1, %0;" ::"n"(kAcceptThreads) : "memory"); };
 
   // sequence that owns this row (looked up first: its loads overlap the scan below)
   int lo = 0, hi = p.batch;
@@ -153,7 +170,20 @@ __global__ void __launch_bounds__(kAcceptThreads) tree_accept_kernel(const Accep
   const int T = min(T_real, FALCON_T_MAX);
 
   Best mine{-INFINITY, kNone};
-  if (c0 < c1) {
+  if constexpr (kStream) {
+    if (tid < rs.head) take(mine, __ldcs(rowp + c0 + tid), c0 + tid);
+    for (int st = 0; st < rs.stages(); ++st) {
+      float x[kStreamLane];
+      if (!rs.take(st, x)) {
+        if ((tid & 31) == 0) dev_status_or(p.status, b, FALCON_DEV_TIMEOUT);
+        break;
+      }
+      if (st + kStreamStages < rs.stages()) rs.give_back(st);
+#pragma unroll
+      for (int k = 0; k < kStreamLane; ++k) take(mine, x[k], c0 + rs.head + rs.index(st, k >> 2, k & 3));
+    }
+    if (tid < rs.tail) take(mine, __ldcs(rs.base + rs.body + tid), c0 + rs.head + rs.body + tid);
+  } else if (c0 < c1) {
     // scalar head up to the first 16-byte boundary, float4 body, scalar tail
     const int mis = static_cast<int>((reinterpret_cast<uintptr_t>(rowp + c0) >> 2) & 3);
     const int head = min(c1 - c0, (4 - mis) & 3);
@@ -180,7 +210,7 @@ __global__ void __launch_bounds__(kAcceptThreads) tree_accept_kernel(const Accep
     mine = merge(mine, other);
   }
   if ((tid & 31) == 0) warp_best[tid >> 5] = mine;
-  __syncthreads();
+  worker_sync();
 
   if (tid == 0) {
     Best r = warp_best[0];
@@ -192,7 +222,7 @@ __global__ void __launch_bounds__(kAcceptThreads) tree_accept_kernel(const Accep
     const int arrived = atomicAdd(&p.tickets[b], 1);
     s_flag = (arrived == T_real * p.chunks - 1);
   }
-  __syncthreads();
+  worker_sync();
   if (!s_flag) return;
   __threadfence();
 
@@ -475,20 +505,23 @@ __global__ void __launch_bounds__(kStreamThreads + 32, 3) tree_sample_kernel(con
   if (tid == 0) p.tickets[b] = 0;  // ready for the next call
 }
 
-constexpr int kAcceptMaxChunks = 64;  // vocabulary chunks per row at most (the static scratch is sized by it)
+constexpr int kAcceptMaxChunks = 8;  // vocabulary chunks per row at most (the static scratch is sized by it)
 
-// How a launch splits the vocabulary: enough CTAs for a few waves, chunks of at least 2048 elements
-// and a multiple of 4.  Shared by the two entry points so that they cannot drift apart.
-void accept_plan(int sm_count, int n_nodes, int vocab, int* chunks_out, int* chunk_len_out) {
-  int chunks = (4 * sm_count + n_nodes - 1) / n_nodes;
-  const int max_chunks = (vocab + 2047) / 2048;
-  if (chunks > max_chunks) chunks = max_chunks;
-  if (chunks > kAcceptMaxChunks) chunks = kAcceptMaxChunks;
-  if (chunks < 1) chunks = 1;
+// How a launch splits the vocabulary, and whether its rows are streamed.  Shared by the two entry points so that
+// they cannot drift apart.  Streamed: up to about one and a half CTAs per SM in all, chunks of no less than most of a stage, so that a
+// large batch has a CTA per row (measured, us, with 1 / 2 / 4 / 8 chunks of 32000: 20 rows 5.3 / 4.6 / 4.4 / 4.7, 60 rows 6.6 / 5.9 /
+// 6.3 / 8.1, 100 rows 7.2 / 6.9 / 6.8 / 9.6, 300 rows 11.2 / 12.1 / 13.6 / 20.6; 16 rows of 128000: 11.8 / 8.3 / 6.7 / 6.1).
+// Short rows fit the registers of one pass, and the ring's set-up would only add to it (15 rows of 1000: 4.1 against 4.4).
+bool accept_plan(int sm_count, int n_nodes, int vocab, int* chunks_out, int* chunk_len_out) {
+  const bool streamed = vocab > 4096;
+  const int ctas = streamed ? 3 * sm_count / 2 : 4 * sm_count, shortest = streamed ? kStreamStage * 3 / 4 : 2048;
+  int chunks = 1;  // (doubled: 3 chunks of 32000 fill their last stage by a third, 6.6 us where 2 take 5.9)
+  while (chunks < kAcceptMaxChunks && static_cast<int64_t>(n_nodes) * 2 * chunks <= ctas && vocab / (2 * chunks) >= shortest) chunks *= 2;
   int chunk_len = (vocab + chunks - 1) / chunks;
   chunk_len = (chunk_len + 3) & ~3;
   *chunks_out = (vocab + chunk_len - 1) / chunk_len;
   *chunk_len_out = chunk_len;
+  return streamed;
 }
 
 // Kernel parameters from the caller's arguments, the plan and the scratch: `part` holds
@@ -523,7 +556,9 @@ AcceptParams accept_params(const falcon_accept_args& a, int chunks, int chunk_le
 }  // namespace
 
 cudaError_t set_up_accept() {
-  cudaError_t e = prefer_shared(tree_accept_kernel);
+  cudaError_t e = prefer_shared(tree_accept_kernel<false>);
+  if (e == cudaSuccess) e = prefer_shared(tree_accept_kernel<true>);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(tree_accept_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kStreamBytes));
   if (e == cudaSuccess) e = prefer_shared(tree_search_kernel);
   if (e == cudaSuccess) e = prefer_shared(tree_sample_kernel);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(tree_sample_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kStreamBytes));
@@ -534,7 +569,7 @@ int launch_tree_accept(falcon_ctx* ctx, const falcon_accept_args& a, cudaStream_
   const int N = a.tree.total_nodes;
   if (N > 65535) return FALCON_ERR_CAPACITY;
   int chunks, chunk_len;
-  accept_plan(ctx->sm_count, N, a.vocab, &chunks, &chunk_len);
+  const bool streamed = accept_plan(ctx->sm_count, N, a.vocab, &chunks, &chunk_len);
 
   const size_t part = static_cast<size_t>(N) * chunks;
   int rc = ensure_workspace(ctx, part * 8 + 256);
@@ -545,14 +580,15 @@ int launch_tree_accept(falcon_ctx* ctx, const falcon_accept_args& a, cudaStream_
 
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(chunks, N);
-  cfg.blockDim = dim3(kAcceptThreads);
+  cfg.blockDim = dim3(kAcceptThreads + (streamed ? 32 : 0));
+  cfg.dynamicSmemBytes = streamed ? kStreamBytes : 0;
   cfg.stream = s;
   cudaLaunchAttribute attr;
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, tree_accept_kernel, p);
+  cudaError_t e = cudaLaunchKernelEx(&cfg, streamed ? tree_accept_kernel<true> : tree_accept_kernel<false>, p);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "tree_accept_kernel launch");
   return FALCON_OK;
 }
@@ -657,6 +693,9 @@ int static_scratch(int device, StaticSlot* out) {
     int sms = 0;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
     if (e != cudaSuccess || sms < 1) return FALCON_ERR_CUDA;
+    // (there may be no context that has raised the limit on this device)
+    e = cudaFuncSetAttribute(tree_accept_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kStreamBytes));
+    if (e != cudaSuccess) return FALCON_ERR_CUDA;
     slot.sm_count = sms;
     slot.ptr = ptr;
   }
@@ -688,7 +727,7 @@ extern "C" int falcon_tree_accept_static(const falcon_accept_args* a, void* stre
 
   const int N = a->tree.total_nodes;
   int chunks, chunk_len;
-  accept_plan(slot.sm_count, N, a->vocab, &chunks, &chunk_len);
+  const bool streamed = accept_plan(slot.sm_count, N, a->vocab, &chunks, &chunk_len);
 
   unsigned char* base = static_cast<unsigned char*>(slot.ptr);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -698,7 +737,11 @@ extern "C" int falcon_tree_accept_static(const falcon_accept_args* a, void* stre
   if (e != cudaSuccess) return FALCON_ERR_CUDA;
   const AcceptParams p = accept_params(*a, chunks, chunk_len, base, reinterpret_cast<int*>(base + kStaticPartBytes));
   dim3 grid(chunks, N);
-  tree_accept_kernel<<<grid, kAcceptThreads, 0, s>>>(p);
+  if (streamed) {
+    tree_accept_kernel<true><<<grid, kAcceptThreads + 32, kStreamBytes, s>>>(p);
+  } else {
+    tree_accept_kernel<false><<<grid, kAcceptThreads, 0, s>>>(p);
+  }
   e = cudaGetLastError();
   return e == cudaSuccess ? FALCON_OK : FALCON_ERR_CUDA;
 }
