@@ -79,7 +79,7 @@ constexpr int kWarpProducer = 0;
 constexpr int kWarpMma = 1;
 constexpr int kWarpSm0 = 2;
 constexpr int kMaxSplits = 8;
-constexpr int kHostSeqs = 8;
+constexpr int kHostSeqs = 32;
 constexpr uint32_t kSmemMax = 232448;           // dynamic shared memory a CTA may ask for
 constexpr float kLMin = 7.8886090522101181e-31f;  // 2^-100
 constexpr float kLMax = 1.2676506002282294e+30f;  // 2^100
@@ -160,10 +160,14 @@ struct TckParams {
   int32_t early_prefix;
   int32_t stall_first;     // test hook: tile 0 is never requested (a bounded wait then runs out)
   int32_t prefetch_next;   // tm_nk / tm_nv describe the caches of the next call: bring their prefix tiles into L2
-  int32_t h_node_off[kHostSeqs + 1];
-  int32_t h_prefix[kHostSeqs];
-  int32_t h_order[kHostSeqs];  // grid z -> sequence, longest first (CTAs are handed out in grid order: with more
-                               // CTAs than SMs the long sequences must not be the ones that start last)
+  // What the caller knows of the sequence at grid z, longest first (CTAs are handed out in grid order: with more
+  // CTAs than SMs the long sequences must not be the ones that start last; with more than two waves they even out by
+  // themselves, and CTAs of one length at a time only wait together: 20 sequences of 32 heads 54.9 us as they come,
+  // 60.3 sorted).  One 16-byte piece, so that a CTA touches one line of the parameters for it.  From the
+  // device's arrays, in the caller's order, against this: 14 sequences of 4 heads 15.2 and 14.5 us, 32 of 4 17.7 and 16.9.
+  struct alignas(16) HostSeq {
+    int32_t seq, node_base, nodes, prefix;
+  } h_seq[kHostSeqs];
   FALCON_TRACE_PARAMS
 };
 
@@ -298,7 +302,7 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
   const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
   const int n_splits = gridDim.x, split = blockIdx.x;  // cluster = all CTAs of a row of the grid
   const int kvh = blockIdx.y % p.Hkv, mtile = blockIdx.y / p.Hkv;
-  const int b = p.have_host ? p.h_order[blockIdx.z] : static_cast<int>(blockIdx.z);
+  const int b = p.have_host ? p.h_seq[blockIdx.z].seq : static_cast<int>(blockIdx.z);
   constexpr int kCW = VT::kCW, kPer = VT::kPer;
   const int G = p.G, N = p.n_rows, n_chunks = N / kCW;
   const uint32_t q_half_bytes = static_cast<uint32_t>(N) * 128u;  // between the two 64-column halves of Q
@@ -320,8 +324,7 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
     // the latency overlaps the previous kernel, instead of where its values are needed.
     const uint32_t warm = static_cast<uint32_t>(p.Hq) ^ static_cast<uint32_t>(reinterpret_cast<uintptr_t>(p.tree_mask)) ^
                           static_cast<uint32_t>(reinterpret_cast<uintptr_t>(p.q)) ^ static_cast<uint32_t>(p.kv_stride_s) ^
-                          static_cast<uint32_t>(reinterpret_cast<uintptr_t>(p.out)) ^ static_cast<uint32_t>(p.h_node_off[2]) ^
-                          static_cast<uint32_t>(p.h_prefix[kHostSeqs - 1]);
+                          static_cast<uint32_t>(reinterpret_cast<uintptr_t>(p.out)) ^ static_cast<uint32_t>(p.prefetch_next);
     asm volatile("" ::"r"(warm));
   }
   FALCON_TRACE(tid == 0, 20);
@@ -386,9 +389,9 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
     return p.q + (static_cast<int64_t>(node_base + (mg >> p.g_shift)) * p.Hq + kvh * G + (mg & (G - 1))) * kHD + q_part * (kHD / 8);
   };
   if (p.have_host) {  // the caller's host copies of the per-sequence scalars: no round trip to global memory
-    node_base = p.h_node_off[b];
-    T_real = p.h_node_off[b + 1] - node_base;
-    L_raw = p.h_prefix[b];
+    node_base = p.h_seq[blockIdx.z].node_base;
+    T_real = p.h_seq[blockIdx.z].nodes;
+    L_raw = p.h_seq[blockIdx.z].prefix;
     geometry();
   }
   FALCON_TRACE(tid == 0, 22);
@@ -1078,12 +1081,10 @@ int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s, int 
   p.stall_first = (a.flags & FALCON_ATTN_TEST_STALL) ? 1 : 0;
   if (a.tree.prefix_len_host && a.tree.node_off_host && B <= kHostSeqs) {
     p.have_host = 1;
-    for (int i = 0; i <= B; ++i) p.h_node_off[i] = a.tree.node_off_host[i];
-    for (int i = 0; i < B; ++i) p.h_prefix[i] = a.tree.prefix_len_host[i];
-    for (int i = 0; i < B; ++i) p.h_order[i] = i;
-    std::stable_sort(p.h_order, p.h_order + B, [&](int x, int y) {
-      return p.h_prefix[x] + (p.h_node_off[x + 1] - p.h_node_off[x]) > p.h_prefix[y] + (p.h_node_off[y + 1] - p.h_node_off[y]);
-    });
+    const int32_t* off = a.tree.node_off_host;
+    for (int i = 0; i < B; ++i) p.h_seq[i] = {i, off[i], off[i + 1] - off[i], a.tree.prefix_len_host[i]};
+    if (static_cast<int64_t>(Hkv) * n_units * B <= 2 * ctx->sm_count)
+      std::stable_sort(p.h_seq, p.h_seq + B, [](const auto& x, const auto& y) { return x.prefix + x.nodes > y.prefix + y.nodes; });
   }
 
   FALCON_TRACE_LAUNCH(p)
@@ -1138,11 +1139,13 @@ int nodes_per_unit(const falcon_attn_args& a) {
 // it won everywhere (65-128 rows 4 to 50 % faster, more rows up to 2.5 times).  Up to 16 rows from
 // about 200 keys (8 heads, 4 nodes, 3 x 135 keys 5.6 against 6.1 us; 3 x 1340 7.0 / 8.9), up to 64 from
 // about 640 (32 heads, 60 nodes, 1084 keys 8.8 / 9.8; 16 heads, 24 nodes, 2 x 509 keys 7.1 / 6.7): with
-// fewer keys its output, which one or two CTAs then transpose and store, costs more.
+// fewer keys its output, which one or two CTAs then transpose and store, costs more.  Batches that fill the SMs
+// without a split are the other kernel's from 33 rows on (60 nodes, 32 heads: 10 sequences 47.9 us here and 38.6 there,
+// 16 75.2 / 69.4; 12 sequences of 16 64-wide heads 33.8 / 32.3; but 12 with 30 nodes 51.4 / 53.5, 20 with 8 56.5 / 61.9).
 bool tree_attn_tck_preferred(const falcon_ctx* ctx, const falcon_attn_args& a) {
-  (void)ctx;
   const int rows = a.tree.max_tree * (a.n_q_heads / a.n_kv_heads);
   const int keys = a.tree.max_prefix_len + a.tree.max_tree;
+  if (rows > 32 && static_cast<int64_t>(a.tree.batch) * a.n_kv_heads > ctx->sm_count) return false;
   return rows <= 64 && keys >= (rows <= 16 ? 200 : 640);
 }
 

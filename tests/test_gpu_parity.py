@@ -581,6 +581,22 @@ def test_attn_tc_more_units_than_sms(sizes, prefs, Hkv, G, separate, D):
             assert not dt.status.cpu().numpy().any()
 
 
+@pytest.mark.parametrize("B,Hkv", [(9, 2), (32, 1), (33, 1), (20, 16)])
+def test_attn_tck_batches_with_and_without_host_copies(B, Hkv):
+    """Keys-on-lanes kernel: batches whose sequences travel with the call (up to 32, longest first up to two waves)
+    and longer ones give what the device's own arrays give."""
+    rng = np.random.default_rng(B + Hkv)
+    sizes = rng.integers(1, 12, size=B).tolist()
+    prefs = rng.integers(0, 300, size=B).tolist()
+    tb, q, k, v = random_case(rng, sizes, prefs, Hkv, Hkv, 128, slack=1)
+    ref = oracle_attn(tb, Hkv, Hkv, 128, q, k, v)
+    for hc in (False, True):
+        dt = H.DevTrees(tb)
+        out, rc = H.run_attn(dt, Hkv, Hkv, 128, q, k, v, kernel=binding.ATTN_TCK, host_copies=hc)
+        H.assert_attn_close(out, ref, tb.node_off)
+        assert not dt.status.cpu().numpy().any()
+
+
 @pytest.mark.parametrize("tck", TC_KERNELS)
 @pytest.mark.parametrize("T,G,L,splits", [(60, 1, 1024, 0), (60, 1, 700, 4), (80, 1, 500, 3), (16, 8, 1000, 5),
                                            (20, 1, 10, 2), (33, 2, 0, 1)])
