@@ -1281,6 +1281,24 @@ def test_attn_bounded_wait_runs_out_and_the_context_stays_usable(tck, T):
         assert rc == binding.ERR_INVALID_ARG
 
 
+def test_attn_bounded_wait_with_several_units_per_cta():
+    """The same where a CTA works on several units: none of them waits for good, and all rows read as zero."""
+    rng = np.random.default_rng(77)
+    Hkv = 100
+    tb, q, k, v = random_case(rng, [9, 5, 12, 7], [100, 40, 150, 64], Hkv, Hkv, 64)
+    ref = oracle_attn(tb, Hkv, Hkv, 64, q, k, v)
+    dt = H.DevTrees(tb)
+    for flags in (binding.ATTN_TEST_STALL, 0):
+        dt.status.zero_()
+        out, _ = H.run_attn(dt, Hkv, Hkv, 64, q, k, v, kernel=binding.ATTN_TC, n_splits=1, host_copies=True, flags=flags)
+        if flags:
+            assert (dt.status.cpu().numpy() & binding.DEV_TIMEOUT).any()
+            assert not synth.bf16_bits_to_f32(out).any()
+        else:
+            H.assert_attn_close(out, ref, tb.node_off)
+            assert not dt.status.cpu().numpy().any()
+
+
 # ------------------------------------------------- accepted tokens and features
 def _gather_case(rng, sizes, hidden, stride_pad=0):
     tb = H.make_trees(sizes, [0] * len(sizes), rng, vocab=32000)
