@@ -21,8 +21,9 @@
 //
 // Softmax with a fixed reference: m is the row's score against the first key of this CTA's run, not its
 // maximum: fp32 and bf16 carry exponents to 2^127, so nothing is rescaled while the row's scores
-// stay within about 2^100 of it.  A row whose normaliser leaves [2^-100, 2^100] or is not finite is
-// recomputed exactly from global memory.
+// stay within about 2^100 of it.  A row is recomputed exactly from global memory when its sum over any
+// CTA's run, or over all of them, leaves [2^-100, 2^100] or is not finite, or when the references of two
+// runs are more than 100 apart (in log2 units): all the factors of the merge are then ordinary numbers.
 // The weights are cut to bf16 and the row sums take the same cut values (a row that one key dominates
 // is then exact whatever that key's weight is).
 //
@@ -60,6 +61,7 @@ constexpr int kHostSeqs = 32;
 constexpr int kLoopTiles = 8;      // see launch_impl
 constexpr float kLMin = 7.8886090522101181e-31f;  // 2^-100
 constexpr float kLMax = 1.2676506002282294e+30f;  // 2^100
+constexpr float kRefSpread = 100.f;  // between the references of a row's parts, in log2 units
 constexpr uint32_t kPollLimit = 1u << 24;
 constexpr int kEarlyItems = 2;    // ring slots requested before the grid dependency wait (one K and one V tile)
 
@@ -540,6 +542,15 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       }
       if (bad && split == 0 && kvh == 0) dev_status_or(p.status, b, FALCON_DEV_BAD_TREE);
     }
+    // whether any key of this CTA's run is visible to the row
+    auto row_sees = [&]() {
+      if (n_my <= 0) return false;
+      const int first = tile_key0(0), last = tile_key0(n_my - 1), end = last + tile_keys_in(n_my - 1, last);
+      if (first < Lc) return true;
+      const int n = end - first;  // all of them the tree's
+      const uint64_t w0 = window64(anc_lo, anc_hi, first - Lc), w1 = window64(anc_lo, anc_hi, first - Lc + 64);
+      return ((n >= 64 ? w0 : w0 & ((1ull << n) - 1ull)) | (n <= 64 ? 0ull : n >= 128 ? w1 : w1 & ((1ull << (n - 64)) - 1ull))) != 0ull;
+    };
     // A row's reference: its score against the first key of this CTA's run (0 if it does not see that key),
     // taken by the group that has that item and passed to the others through shared memory.
     const int n_src = two_blocks ? 2 : 1;
@@ -661,7 +672,6 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     if (have) have = mbar_wait_warp(bar(C::kBarODone), kLoop ? nth & 1 : 0, abort_flag);
     FALCON_TRACE(tid == 64, 58);
     tc_fence_after();
-    if (l_row == 0.f) m_ref = -INFINITY;  // no key of this row here: the merge leaves this part out
     const int n_cols = two_blocks ? kHD / 2 : kHD / 4, col0 = (two_blocks ? grp >> 1 : grp) * n_cols;
     const bool first_cols = col0 == 0;
     const uint32_t acc0 = tmem_lane + kTmemO + blk * 128;
@@ -701,11 +711,14 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
           for (int u = 0; u < kC / 8; ++u) put16((c0 >> 3) + u, h[4 * u], h[4 * u + 1], h[4 * u + 2], h[4 * u + 3]);
         }
       }
-      // reference and sum; a split that gave up sends NaN, so that the owner recomputes the row
+      // Reference and sum.  The merge weighs the parts by their references, so each has to be in range by itself: one
+      // that is not, or whose keys' weights all vanish, or that gave up, sends NaN, and the owner recomputes the row.
+      // Only a part without a key of this row is left out.
       if (n_splits > 1 && valid && first_cols) {
-        const bool lost = n_my > 0 && !have;
+        const bool none = l_row == 0.f && !row_sees();
+        const bool fine = n_my > 0 && have && l_row >= kLMin && l_row <= kLMax;
         *reinterpret_cast<float2*>(part + static_cast<uint32_t>(R) * (kHD * 2) + row * 8) =
-            make_float2(lost ? 0.f : m_ref, lost ? __uint_as_float(0x7fc00000u) : l_row);
+            none ? make_float2(-INFINITY, 0.f) : make_float2(fine ? m_ref : 0.f, fine ? l_row : __uint_as_float(0x7fc00000u));
       }
     }
     FALCON_TRACE(tid == 64, 59);
@@ -760,9 +773,12 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             x[s] = __ldcg(reinterpret_cast<const uint4*>(src) + piece * R + rr);
           }
         }
-        float gm = -INFINITY;
+        float gm = -INFINITY, least = INFINITY;  // largest and smallest reference of the parts that count
 #pragma unroll
-        for (int s = 0; s < kM; ++s) gm = fmaxf(gm, ml[s].x);
+        for (int s = 0; s < kM; ++s) {
+          gm = fmaxf(gm, ml[s].x);
+          least = ml[s].x == -INFINITY ? least : fminf(least, ml[s].x);
+        }
         float lsum = 0.f, acc[8];
 #pragma unroll
         for (int c = 0; c < 8; ++c) acc[c] = 0.f;
@@ -779,7 +795,8 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             }
           }
         }
-        if (!(lsum >= kLMin && lsum <= kLMax)) {
+        // (references further apart: the weight of a part could vanish that holds the larger share)
+        if (!(lsum >= kLMin && lsum <= kLMax && gm - least <= kRefSpread)) {
           if (piece == 0) s_rescue[rr] = 1;
           continue;
         }

@@ -157,6 +157,37 @@ def test_attn_large_scores_do_not_overflow(kernel):
     H.assert_attn_close(out, ref, tb.node_off)
 
 
+@pytest.mark.parametrize("kernel", TC_KERNELS)
+@pytest.mark.parametrize("G", [1, 4])
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("prefix, tree, own, root_seen", [
+    # log2 scores (first key, other keys) of the prefix, (root, node itself) of the tree, and whether a node sees the root
+    ((0.0, -30.0), -100.0, 26.5, True),      # a weight of 2^126.5 in the second part, which the merge would scale down
+    ((0.0, -30.0), -127.0, 0.0, True),       # the second part's weight 2^-127 is no normal number
+    ((-130.0, -50.0), 8.0, -60.0, False),    # reference 0 for want of a visible first key: the other part has the weight
+    ((-300.0, -300.0), 8.0, -200.0, False),  # every weight of the second part vanishes, and yet it has the row's key
+])
+def test_attn_parts_far_apart_are_recomputed(prefix, tree, own, root_seen, D, G, kernel):
+    """Two splits of 64 keys (the prefix, the tree) whose scores lie far apart, while the row's sum over both is ordinary."""
+    rng = np.random.default_rng(31)
+    T = L = 64
+    tb = H.make_trees([T], [L], rng, parents=[synth.star_tree(T)])
+    q = np.zeros((T, G, D), np.float32)
+    q[:, :, 0] = 1.0
+    k = np.zeros((1, 1, L + T, D), np.float32)
+    k[0, 0, 0, 0], k[0, 0, 1:L, 0], k[0, 0, L, 0], k[0, 0, L + 1:, 0] = prefix[0], prefix[1], tree, own
+    v = rng.choice([-5.0, -4.0, 4.0, 5.0], size=(1, 1, L + T, D)).astype(np.float32)
+    q, k, v = (synth.f32_to_bf16_bits(x) for x in (q, k, v))
+    rows = None
+    if not root_seen:
+        rows = np.array([[1 << i, 0] for i in range(T)], np.uint64)
+    ref = oracle_attn(tb, G, 1, D, q, k, v, scale=math.log(2.0), tree_mask=rows)
+    out, rc = H.run_attn(H.DevTrees(tb), G, 1, D, q, k, v, scale=math.log(2.0), tree_mask=rows, kernel=kernel, n_splits=2,
+                         check=False)
+    assert rc == binding.OK
+    H.assert_attn_close(out, ref, tb.node_off)
+
+
 @pytest.mark.parametrize("kernel", KERNELS)
 def test_attn_separate_tree_buffers(kernel):
     rng = np.random.default_rng(9)
