@@ -210,6 +210,19 @@ __device__ __forceinline__ bool mbar_wait_drain(uint32_t bar, uint32_t parity) {
 }
 __device__ __forceinline__ float bf16lo(uint32_t x) { return __uint_as_float(x << 16); }
 __device__ __forceinline__ float bf16hi(uint32_t x) { return __uint_as_float(x & 0xffff0000u); }
+__device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
+  const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+  return *reinterpret_cast<const uint32_t*>(&h);
+}
+
+// Where the tensor-core kernels give a weight to the MMA as the sum of two bf16 numbers (the weight rounded to nearest, and
+// its remainder) and keep partial results in fp32.  64-wide heads and trees in buffers of their own ran on CUDA
+// cores with fp32 weights before these kernels took them, and keep that precision: the two parts hold 17 bits of the
+// weight, and what is left of the error is that of the output's own rounding to bf16 (32 cases against float64: 1.000000 to
+// 1.000002 of it, as with fp32 weights; with one bf16 number per weight and bf16 partial results 1.39 to 1.77).  It
+// costs a second P.V MMA, P's stores and twice the merge: a drafter's pass over 1084 keys x 32 heads of 128 15.2 -> 16.8
+// us (123 on CUDA cores), 4 sequences x 16 heads of 64 23.9 -> 25.6 (161), 143 keys x 4 heads of 64 11.5 -> 11.7 for a whole step.
+__host__ __device__ constexpr bool fine_weights(int head_dim, bool separate_tree) { return head_dim == 64 || separate_tree; }
 
 // One query row recomputed exactly by a warp from global memory (running maximum in fp32): the
 // fallback for rows whose scores lie too far from the reference for the fast path.

@@ -25,10 +25,11 @@
 // CTA's run, or over all of them, leaves [2^-100, 2^100] or is not finite, or when the references of two
 // runs are more than 100 apart (in log2 units): all the factors of the merge are then ordinary numbers.
 // The weights are cut to bf16 and the row sums take the same cut values (a row that one key dominates
-// is then exact whatever that key's weight is).
+// is then exact whatever that key's weight is).  64-wide heads and trees in buffers of their own get two bf16
+// numbers per weight and fp32 partial rows instead (kFine: fine_weights in tc_util.cuh).
 //
-// Merge: CTA `rank` owns rows [rank * rows_per, ...) of the unit.  Every CTA writes its partial rows (bf16
-// columns relative to its m, fp32 m and sum) to scratch memory, which stays in L2; one cluster barrier; each
+// Merge: CTA `rank` owns rows [rank * rows_per, ...) of the unit.  Every CTA writes its partial rows (bf16 or, with
+// kFine, fp32 columns relative to its m, fp32 m and sum) to scratch memory, which stays in L2; one cluster barrier; each
 // owner reads its rows of all the splits.  (Through distributed shared memory, which moves about 11 bytes
 // per cycle and SM, the 64 KB of a 256-row unit took 6400 cycles to send and 3200 to merge.)
 // Every wait is bounded; one that runs out sets FALCON_DEV_TIMEOUT, what is in flight is drained, the
@@ -124,7 +125,7 @@ struct TcParams {
 
 // A CTA's partial rows in scratch: 16-byte pieces [piece][row], so that a warp's 32 rows are contiguous for
 // the writer (a thread per row) and the reader alike, then (m, sum) [row].
-__host__ __device__ constexpr uint32_t part_bytes(int hd, int rows) { return static_cast<uint32_t>(rows) * (hd * 2 + 8); }
+__host__ __device__ constexpr uint32_t part_bytes(int hd, int rows, bool fine) { return static_cast<uint32_t>(rows) * (hd * (fine ? 4 : 2) + 8); }
 
 // Shared-memory matrix descriptors of the ring and the Q block (128-byte swizzle, 1 KB between 8-row
 // groups): only the low word, address and leading byte offset, differs.
@@ -135,13 +136,10 @@ __device__ __forceinline__ uint64_t desc_of(uint32_t lo) {
   constexpr uint32_t hi = (1024u >> 4) | (1u << 14) | (2u << 29);
   return (static_cast<uint64_t>(hi) << 32) | lo;
 }
-__device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
-  const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-  return *reinterpret_cast<const uint32_t*>(&h);
-}
 
 // kLoop: the grid is one CTA per SM, each working on several units one after the other.
-template <int kHD, bool kLoop>
+// kFine: a weight is the sum of two bf16 numbers, and partial rows are fp32 (see fine_weights).
+template <int kHD, bool kLoop, bool kFine>
 __global__ void __launch_bounds__(kTcThreads, 1)
 tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                     const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_tk,
@@ -436,7 +434,12 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             // P: 16 keys = 8 packed columns; V: MN-major, 16 keys = 2 KB, the 64-column halves half_tile apart
 #pragma unroll
             for (int kk = 0; kk < kBKMax / 16; ++kk)
-              if (kk < nk) umma_bf16_ts(acc, pbase + kk * 8, desc_of(v + kk * 128), idesc_pv, (j > 0 || kk > 0) ? 1u : 0u);
+              if (kk < nk) {
+                // (kFine: 32 keys' upper parts, then their lower parts)
+                const uint32_t pk = pbase + (kFine ? (kk >> 1) * 32 + (kk & 1) * 8 : kk * 8);
+                umma_bf16_ts(acc, pk, desc_of(v + kk * 128), idesc_pv, (j > 0 || kk > 0) ? 1u : 0u);
+                if constexpr (kFine) umma_bf16_ts(acc, pk + 16, desc_of(v + kk * 128), idesc_pv, 1u);
+              }
             if (last_block) umma_commit(bar(C::kBarKVEmpty) + 8u * slot);
           }
         };
@@ -599,7 +602,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
 #pragma unroll
         for (int c = 0; c < kBKMax; c += 32) {
           if (c < BK) {
-            uint32_t sr[32], pk[16];
+            uint32_t sr[32], pk[16], rest[kFine ? 16 : 1];
             load32(c, sr);
             if (c == 0 && !published) {
               const float s0 = __uint_as_float(sr[0]);
@@ -613,14 +616,27 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             for (int e = 0; e < 32; e += 2) {
               float e0, e1;
               fma2(__uint_as_float(sr[e]), __uint_as_float(sr[e + 1]), scale, scale, neg, neg, e0, e1);
-              const uint32_t b0 = __float_as_uint(ex2(e0)), b1 = __float_as_uint(ex2(e1));
-              pk[e >> 1] = __byte_perm(b0, b1, 0x7632);
+              const float p0 = ex2(e0), p1 = ex2(e1);
+              float t0 = p0, t1 = p1;  // what the row sum takes: the values that the MMA is fed
+              if constexpr (kFine) {
+                pk[e >> 1] = pack_bf16(p0, p1);
+                rest[e >> 1] = pack_bf16(p0 - bf16lo(pk[e >> 1]), p1 - bf16hi(pk[e >> 1]));  // (the differences are exact)
+              } else {
+                pk[e >> 1] = __byte_perm(__float_as_uint(p0), __float_as_uint(p1), 0x7632);
+                t0 = bf16lo(pk[e >> 1]), t1 = bf16hi(pk[e >> 1]);
+              }
               if (e & 2)
-                add2(l2, l3, __uint_as_float(b0 & 0xffff0000u), __uint_as_float(b1 & 0xffff0000u));
+                add2(l2, l3, t0, t1);
               else
-                add2(l0, l1, __uint_as_float(b0 & 0xffff0000u), __uint_as_float(b1 & 0xffff0000u));
+                add2(l0, l1, t0, t1);
             }
-            FALCON_TMEM_ST16(tmem_s + (c >> 1), pk);  // over scores this thread has read already
+            // over scores this thread has read already
+            if constexpr (kFine) {
+              FALCON_TMEM_ST16(tmem_s + c, pk);
+              FALCON_TMEM_ST16(tmem_s + c + 16, rest);
+            } else {
+              FALCON_TMEM_ST16(tmem_s + (c >> 1), pk);
+            }
           }
         }
       } else if (!published) {
@@ -685,7 +701,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       if (!kLoop && inexact) s_rescue[row] = 1;
       inv = have && fine ? 1.f / l_row : 0.f;
     }
-    unsigned char* part = p.part + static_cast<int64_t>((blockIdx.z * gridDim.y + blockIdx.y) * n_splits + split) * part_bytes(kHD, R);
+    unsigned char* part = p.part + static_cast<int64_t>((blockIdx.z * gridDim.y + blockIdx.y) * n_splits + split) * part_bytes(kHD, R, kFine);
     auto put16 = [&](int piece, uint32_t a, uint32_t bq, uint32_t c, uint32_t d) {
       *reinterpret_cast<uint4*>(n_splits == 1 ? reinterpret_cast<unsigned char*>(dst) + piece * 16 : part + (piece * R + row) * 16) =
           make_uint4(a, bq, c, d);
@@ -703,7 +719,12 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
 #pragma unroll
           for (int c = 0; c < kC; ++c) o[c] = 0u;
         }
-        if (valid) {
+        if (kFine && n_splits > 1) {
+          if (valid) {
+#pragma unroll
+            for (int u = 0; u < kC / 4; ++u) put16((c0 >> 2) + u, o[4 * u], o[4 * u + 1], o[4 * u + 2], o[4 * u + 3]);
+          }
+        } else if (valid) {
           uint32_t h[kC / 2];
 #pragma unroll
           for (int c = 0; c < kC / 2; ++c) h[c] = pack_bf16(__uint_as_float(o[2 * c]) * inv, __uint_as_float(o[2 * c + 1]) * inv);
@@ -717,7 +738,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       if (n_splits > 1 && valid && first_cols) {
         const bool none = l_row == 0.f && !row_sees();
         const bool fine = n_my > 0 && have && l_row >= kLMin && l_row <= kLMax;
-        *reinterpret_cast<float2*>(part + static_cast<uint32_t>(R) * (kHD * 2) + row * 8) =
+        *reinterpret_cast<float2*>(part + static_cast<uint32_t>(R) * (kHD * (kFine ? 4 : 2)) + row * 8) =
             none ? make_float2(-INFINITY, 0.f) : make_float2(fine ? m_ref : 0.f, fine ? l_row : __uint_as_float(0x7fc00000u));
       }
     }
@@ -753,10 +774,11 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     // ================================ merge ================================
     cluster_sync_release();  // every split's partial rows are visible (it is this CTA's barrier as well)
     FALCON_TRACE(tid == 0, 60);
-    // An item is one piece (8 columns) of one row; a warp's items are consecutive rows.  All its loads are
+    // An item is one piece (16 bytes of columns) of one row; a warp's items are consecutive rows.  All its loads are
     // issued before any is used: one round trip to L2.
-    constexpr int kPieces = kHD / 8;
-    const unsigned char* parts = p.part + static_cast<int64_t>((blockIdx.z * gridDim.y + blockIdx.y) * n_splits) * part_bytes(kHD, R);
+    constexpr int kCols = kFine ? 4 : 8, kPieces = kHD / kCols;
+    constexpr uint32_t kRowBytes = kHD * (kFine ? 4 : 2);
+    const unsigned char* parts = p.part + static_cast<int64_t>((blockIdx.z * gridDim.y + blockIdx.y) * n_splits) * part_bytes(kHD, R, kFine);
     auto merge = [&](auto most) {
       constexpr int kM = decltype(most)::value;
       for (int item = tid; item < rows_mine * kPieces; item += kTcThreads) {
@@ -768,8 +790,8 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
           ml[s] = make_float2(-INFINITY, 0.f);
           x[s] = make_uint4(0u, 0u, 0u, 0u);
           if (s < n_splits) {
-            const unsigned char* src = parts + s * part_bytes(kHD, R);
-            ml[s] = __ldcg(reinterpret_cast<const float2*>(src + static_cast<uint32_t>(R) * (kHD * 2) + rr * 8));
+            const unsigned char* src = parts + s * part_bytes(kHD, R, kFine);
+            ml[s] = __ldcg(reinterpret_cast<const float2*>(src + static_cast<uint32_t>(R) * kRowBytes + rr * 8));
             x[s] = __ldcg(reinterpret_cast<const uint4*>(src) + piece * R + rr);
           }
         }
@@ -779,9 +801,9 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
           gm = fmaxf(gm, ml[s].x);
           least = ml[s].x == -INFINITY ? least : fminf(least, ml[s].x);
         }
-        float lsum = 0.f, acc[8];
+        float lsum = 0.f, acc[kCols];
 #pragma unroll
-        for (int c = 0; c < 8; ++c) acc[c] = 0.f;
+        for (int c = 0; c < kCols; ++c) acc[c] = 0.f;
 #pragma unroll
         for (int s = 0; s < kM; ++s) {
           if (ml[s].x != -INFINITY) {  // (a split that saw no key of this row has no valid columns)
@@ -790,8 +812,12 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             const uint32_t xs[4] = {x[s].x, x[s].y, x[s].z, x[s].w};
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
-              acc[2 * c] = fmaf(bf16lo(xs[c]), w, acc[2 * c]);
-              acc[2 * c + 1] = fmaf(bf16hi(xs[c]), w, acc[2 * c + 1]);
+              if constexpr (kFine) {
+                acc[c] = fmaf(__uint_as_float(xs[c]), w, acc[c]);
+              } else {
+                acc[2 * c] = fmaf(bf16lo(xs[c]), w, acc[2 * c]);
+                acc[2 * c + 1] = fmaf(bf16hi(xs[c]), w, acc[2 * c + 1]);
+              }
             }
           }
         }
@@ -802,9 +828,12 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         }
         const float inv = 1.f / lsum;
         const int mg = unit * R + rr;
-        *reinterpret_cast<uint4*>(p.out + (static_cast<int64_t>(node_base + (mg >> p.g_shift)) * p.Hq + kvh * G + (mg & (G - 1))) * kHD + piece * 8) =
-            make_uint4(pack_bf16(acc[0] * inv, acc[1] * inv), pack_bf16(acc[2] * inv, acc[3] * inv),
-                       pack_bf16(acc[4] * inv, acc[5] * inv), pack_bf16(acc[6] * inv, acc[7] * inv));
+        __nv_bfloat16* dst = p.out + (static_cast<int64_t>(node_base + (mg >> p.g_shift)) * p.Hq + kvh * G + (mg & (G - 1))) * kHD + piece * kCols;
+        if constexpr (kFine)
+          *reinterpret_cast<uint2*>(dst) = make_uint2(pack_bf16(acc[0] * inv, acc[1] * inv), pack_bf16(acc[2] * inv, acc[3] * inv));
+        else
+          *reinterpret_cast<uint4*>(dst) = make_uint4(pack_bf16(acc[0] * inv, acc[1] * inv), pack_bf16(acc[2] * inv, acc[3] * inv),
+                                                      pack_bf16(acc[4] * inv, acc[5] * inv), pack_bf16(acc[6] * inv, acc[7] * inv));
       }
     };
     if (n_splits <= 4) merge(std::integral_constant<int, 4>{});
@@ -848,7 +877,7 @@ int resident_clusters(falcon_ctx* ctx, int s) {
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, tree_attn_tc_kernel<128, false>, &cfg) != cudaSuccess) n = -1;
+    if (cudaOccupancyMaxActiveClusters(&n, tree_attn_tc_kernel<128, false, false>, &cfg) != cudaSuccess) n = -1;
     resident[s] = n > 0 ? n : -1;
     cudaGetLastError();
   }
@@ -929,7 +958,7 @@ int mean_tiles(const falcon_attn_args& a) {
   return static_cast<int>((keys + kBKMax - 1) / kBKMax);
 }
 
-template <int kHD>
+template <int kHD, bool kFine>
 int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s) {
   using C = Cfg<kHD>;
   const int B = a.tree.batch, Hq = a.n_q_heads, Hkv = a.n_kv_heads, G = Hq / Hkv;
@@ -939,10 +968,12 @@ int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s) {
     auto set = [&](auto* kernel, uint32_t bytes) {
       if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
     };
-    set(tree_attn_tc_kernel<128, false>, Cfg<128>::kSmemBytes);
-    set(tree_attn_tc_kernel<64, false>, Cfg<64>::kSmemBytes);
-    set(tree_attn_tc_kernel<128, true>, Cfg<128>::kSmemBytes);
-    set(tree_attn_tc_kernel<64, true>, Cfg<64>::kSmemBytes);
+    set(tree_attn_tc_kernel<128, false, false>, Cfg<128>::kSmemBytes);
+    set(tree_attn_tc_kernel<128, true, false>, Cfg<128>::kSmemBytes);
+    set(tree_attn_tc_kernel<128, false, true>, Cfg<128>::kSmemBytes);
+    set(tree_attn_tc_kernel<128, true, true>, Cfg<128>::kSmemBytes);
+    set(tree_attn_tc_kernel<64, false, true>, Cfg<64>::kSmemBytes);
+    set(tree_attn_tc_kernel<64, true, true>, Cfg<64>::kSmemBytes);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute(tree_attn_tc_kernel)");
     attr_set = true;
   }
@@ -992,7 +1023,7 @@ int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s) {
   TcParams p;
   p.part = nullptr;
   if (splits > 1) {
-    const int rc = ensure_workspace(ctx, static_cast<size_t>(splits) * Hkv * n_units * B * part_bytes(kHD, q_nodes * G) + 256);
+    const int rc = ensure_workspace(ctx, static_cast<size_t>(splits) * Hkv * n_units * B * part_bytes(kHD, q_nodes * G, kFine) + 256);
     if (rc) return rc;
     p.part = static_cast<unsigned char*>(ctx->ws);
   }
@@ -1056,7 +1087,7 @@ int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s) {
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, loop ? tree_attn_tc_kernel<kHD, true> : tree_attn_tc_kernel<kHD, false>, mq, mk, mv, mtk, mtv, p);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, loop ? tree_attn_tc_kernel<kHD, true, kFine> : tree_attn_tc_kernel<kHD, false, kFine>, mq, mk, mv, mtk, mtv, p);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "tree_attn_tc_kernel launch");
   return FALCON_OK;
 }
@@ -1075,7 +1106,8 @@ bool tree_attn_tc_supports(const falcon_ctx* ctx, const falcon_attn_args& a) {
 }
 
 int launch_tree_attn_tc(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s) {
-  return a.head_dim == 128 ? launch_impl<128>(ctx, a, s) : launch_impl<64>(ctx, a, s);
+  if (a.head_dim == 64) return launch_impl<64, fine_weights(64, false)>(ctx, a, s);
+  return a.k_tree ? launch_impl<128, fine_weights(128, true)>(ctx, a, s) : launch_impl<128, fine_weights(128, false)>(ctx, a, s);
 }
 
 void tree_attn_tc_release(falcon_ctx* ctx) { release_tmaps(ctx); }

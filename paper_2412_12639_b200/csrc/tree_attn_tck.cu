@@ -12,7 +12,7 @@
 // Work decomposition: one thread-block cluster per (sequence, KV head, block of query rows); row r
 // of a KV head is (tree node r / G, query head r % G).  The cluster's CTAs split the key range
 // (prefix + tree) into runs of whole tiles.  Each CTA owns a share of the 128 head-dim rows of the
-// block's result: every CTA sends the other CTAs' shares of its partial O^T (bf16) and its row
+// block's result: every CTA sends the other CTAs' shares of its partial O^T (bf16; with fine weights fp32) and its row
 // sums (fp32) straight from registers into their shared memory (st.async, counted on the owner's
 // mbarrier), and every owner adds what it received, normalises and stores.  No partial result
 // touches global memory, and there is no cluster barrier after the first.
@@ -34,7 +34,8 @@
 //              quadrant w % 4 (32 keys) and on the column chunks (w - 2) / 4, + 4, ... of the query
 //              rows: tcgen05.ld, p = 2^(s.scale - ref), tree mask from the key's descendant bit set,
 //              this key's share of the row sums in registers, P^T as bf16 into the shared memory of
-//              the K tile it was computed from (free once S^T exists).
+//              the K tile it was computed from (free once S^T exists).  64-wide heads and trees in buffers of
+//              their own get two bf16 numbers per weight (kFine: fine_weights in tc_util.cuh).
 // All three falcon kernels are launched programmatically dependent; set-up that touches no global
 // memory, and one prefix tile when the caller declared the prefix stable, come before
 // griddepcontrol.wait.  Every mbarrier wait is bounded; a wait that runs out sets FALCON_DEV_TIMEOUT,
@@ -118,22 +119,27 @@ struct Cfg {
 };
 
 // The K/V ring's stage for a head dimension and a block of at most n_max query rows.  A tile's matrix is
-// kHalves blocks of 64 head-dim columns; P^T (64 query rows a block) lies over the K tile, which
-// for 64-wide heads and more than 64 rows is given the room of two blocks.  The P.V MMA always has
+// kHalves blocks of 64 head-dim columns; P^T (64 query rows a block) lies over the K tile, with
+// fine weights twice (upper and lower parts): where it is larger than the tile, K is given its room.  The P.V MMA always has
 // 128 output lanes: with 64-wide heads its A operand's upper 64 rows are whatever follows the V
 // tile, so there the V tile comes first and K / P^T (always inside the stage) after it; the lanes
 // 64-127 of that accumulator are never read.
-template <int kHD>
+template <int kHD, bool kFine>
 struct Stage {
   static constexpr uint32_t kHalves = kHD / 64;
-  static __host__ __device__ constexpr uint32_t k_halves(int n_max) { return kHD == 128 || n_max > 64 ? 2u : 1u; }
+  static __host__ __device__ constexpr uint32_t p_halves(int n_max) { return n_max > 64 ? 2u : 1u; }
+  static __host__ __device__ constexpr uint32_t k_halves(int n_max) {
+    return p_halves(n_max) * (kFine ? 2u : 1u) > kHalves ? p_halves(n_max) * (kFine ? 2u : 1u) : kHalves;
+  }
   static __host__ __device__ constexpr uint32_t halves(int n_max) { return k_halves(n_max) + kHalves; }
   static __host__ __device__ constexpr uint32_t k_first(void) { return kHD == 128; }
 };
 
 // bytes between the rows of a partial result of n query columns: an odd number of 16-byte units, so
 // that 16-byte accesses of consecutive rows fall into different banks
-__host__ __device__ constexpr uint32_t part_pitch(int n) { return static_cast<uint32_t>(n) * 2u + 16u; }
+__host__ __device__ constexpr uint32_t part_pitch(int n, bool fine) { return static_cast<uint32_t>(n) * (fine ? 4u : 2u) + 16u; }
+// rows of a slot that the row sums (fp32) take
+__host__ __device__ constexpr uint32_t sum_rows(bool fine) { return fine ? 1u : 2u; }
 
 struct TckParams {
   int32_t Hq, Hkv, G, g_shift, s_cap;
@@ -266,16 +272,17 @@ __device__ __forceinline__ int col_of_lane(int lane) {
   return (kW == 16 ? ((lane >> 4) & 1) * 8 : 0) + ((lane >> 3) & 1) * 4 + ((lane >> 2) & 1) * 2 + ((lane >> 1) & 1);
 }
 
-// kFull: the ring is three stages of 128-key tiles (then the geometry is known at compile time).
+// kTile: the ring is three stages of tiles of this many keys, known at compile time (0: not known).
 // kSep: the tree's K/V rows are in buffers of their own; its keys then start a tile of their own
 // (the prefix's last tile is cut at the prefix length) and tm_nk / tm_nv describe those buffers.
-template <int kVar, bool kFull, int kHD, bool kSep>
+template <int kVar, int kTile, int kHD, bool kSep>
 __global__ void __launch_bounds__(Var<kVar>::kThreads, 1)
 tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                      const __grid_constant__ CUtensorMap tm_nk, const __grid_constant__ CUtensorMap tm_nv,
                      const TckParams p) {
   using VT = Var<kVar>;
   using C = Cfg<VT::kCfg>;
+  constexpr bool kFine = fine_weights(kHD, kSep);
   constexpr int kColGroups = VT::kGroups, kSmWarps = VT::kSmWarps, kSmThreads = VT::kSmThreads, kThreads = VT::kThreads;
   extern __shared__ __align__(1024) unsigned char smem_gen[];
   const uint32_t smem_base = smem_u32(smem_gen);
@@ -288,13 +295,14 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
   volatile int* abort_flag = reinterpret_cast<volatile int*>(small + C::kOffMisc + 4);
   const uint32_t bars = smem_base + p.off_small + C::kOffBars;
   // K/V ring geometry
-  const int BK = kFull ? kBKMax : p.tile_keys, kStages = kFull ? 3 : p.n_stages;
+  const int BK = kTile ? kTile : p.tile_keys, kStages = kTile ? 3 : p.n_stages;
   const uint32_t kHalfTile = static_cast<uint32_t>(BK) * 128u;   // one 64-column half of a K or V tile
-  using SG = Stage<kHD>;
+  using SG = Stage<kHD, kFine>;
   constexpr uint32_t kHalves = SG::kHalves;
   const uint32_t kStageBytes = SG::halves(VT::kNMax) * kHalfTile;
   const uint32_t kOffK = SG::k_first() ? 0u : kHalves * kHalfTile;               // within a stage
   const uint32_t kOffV = SG::k_first() ? SG::k_halves(VT::kNMax) * kHalfTile : 0u;
+  const uint32_t kOffRest = SG::p_halves(VT::kNMax) * kHalfTile;                 // kFine: from P^T's upper parts to the lower ones
   const uint32_t off_q = 0, off_kv = static_cast<uint32_t>(p.n_rows) * (2u * kHD), off_mrg = p.off_mrg, off_stage = 0;
   const uint32_t tmem_cols = (kVar == 0 || p.n_rows <= 64) ? 256u : 512u, col_stride = tmem_cols / 4;  // S^T(0), S^T(1), O^T
   auto bar = [&](int i) { return bars + 8u * static_cast<uint32_t>(i); };
@@ -471,15 +479,16 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
   const bool need_tree = has_tree_keys || (split == 0 && kvh == 0);  // the latter reports malformed trees
 
   // merge geometry: CTA `rank` owns head-dim rows [rank * d_per, ...) of the unit's result
-  const uint32_t pitch = part_pitch(N);
+  constexpr uint32_t kElt = kFine ? 4u : 2u, kSumRows = sum_rows(kFine);
+  const uint32_t pitch = part_pitch(N, kFine);
   const int d_per = (kHD + n_splits - 1) / n_splits;
   const int d0 = split * d_per;
   const int d_mine = max(0, min(kHD, d0 + d_per) - d0);
-  const uint32_t slot_bytes = static_cast<uint32_t>(d_per + 2) * pitch;
+  const uint32_t slot_bytes = (d_per + kSumRows) * pitch;
 
   if (warp == kWarpProducer && lane == 0) {
     // every split (this one included) delivers its share of this CTA's head-dim rows and the row sums
-    mbar_expect_tx(bar(kBarMrg), static_cast<uint32_t>(n_splits * (d_mine + 2) * N * 2));
+    mbar_expect_tx(bar(kBarMrg), n_splits * (d_mine + kSumRows) * N * kElt);
     for (int j = n_early; j < min(n_my, kStages); ++j) load_tile(j);
     if (split == 0 && mtile == 0 && kvh == 0 && (L + (kSep ? 0 : T) > p.s_cap || T_real > FALCON_T_MAX))
       dev_status_or(p.status, b, FALCON_DEV_CAPACITY);
@@ -566,6 +575,8 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
             const uint64_t ad = smem_desc(vbase + kk * 2048, kHalfTile, 1024);
             const uint64_t bd = smem_desc(pbase + kk * 2048, kHalfTile, 1024);
             umma_bf16_ss(tmem_base + 2 * col_stride, ad, bd, p.idesc_pv, (t > 0 || kk > 0) ? 1u : 0u);
+            if constexpr (kFine)
+              umma_bf16_ss(tmem_base + 2 * col_stride, ad, smem_desc(pbase + kOffRest + kk * 2048, kHalfTile, 1024), p.idesc_pv, 1u);
           }
           umma_commit(bar(kBarKVEmpty + st));
         }
@@ -752,7 +763,7 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
             }
             tmem_wait_ld();
           }
-          uint32_t pk[kCW / 2];
+          uint32_t pk[kCW / 2], rest[kFine ? kCW / 2 : 1];
 #pragma unroll
           for (int c = 0; c < kCW; c += 2) {
             // two columns at a time: one packed fma for the exponents, one packed add for the row sums
@@ -767,9 +778,16 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
             // The weights are cut to bf16 by dropping the low half (they are positive, and the row
             // sums take the same cut values as the accumulator, so the common bias cancels and a row
             // that one key dominates is exact whatever that key's weight is).
-            const uint32_t b0 = __float_as_uint(p0), b1 = __float_as_uint(p1);
-            pk[c >> 1] = __byte_perm(b0, b1, 0x7632);
-            add2(l_acc[ci][c], l_acc[ci][c + 1], __uint_as_float(b0 & 0xffff0000u), __uint_as_float(b1 & 0xffff0000u));
+            // kFine: rounded to nearest, and the remainder goes to the MMA as a second bf16 number.
+            if constexpr (kFine) {
+              pk[c >> 1] = pack_bf16(p0, p1);
+              rest[c >> 1] = pack_bf16(p0 - bf16lo(pk[c >> 1]), p1 - bf16hi(pk[c >> 1]));  // (the differences are exact)
+              add2(l_acc[ci][c], l_acc[ci][c + 1], p0, p1);
+            } else {
+              const uint32_t b0 = __float_as_uint(p0), b1 = __float_as_uint(p1);
+              pk[c >> 1] = __byte_perm(b0, b1, 0x7632);
+              add2(l_acc[ci][c], l_acc[ci][c + 1], __uint_as_float(b0 & 0xffff0000u), __uint_as_float(b1 & 0xffff0000u));
+            }
           }
           // P^T row of this key: the chunk's columns are 16-byte units (8 columns each) of the
           // 64-column block they fall in, swizzled by the row like everything the MMA reads
@@ -777,9 +795,13 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
           const int u0 = ((ch * kCW) >> 3) & 7;
           if (kr < BK) {
 #pragma unroll
-            for (int u = 0; u < kCW / 8; ++u)
-              *reinterpret_cast<uint4*>(prow + (((u0 + u) ^ (kr & 7)) << 4)) =
-                  make_uint4(pk[4 * u], pk[4 * u + 1], pk[4 * u + 2], pk[4 * u + 3]);
+            for (int u = 0; u < kCW / 8; ++u) {
+              uint4* dst = reinterpret_cast<uint4*>(prow + (((u0 + u) ^ (kr & 7)) << 4));
+              *dst = make_uint4(pk[4 * u], pk[4 * u + 1], pk[4 * u + 2], pk[4 * u + 3]);
+              if constexpr (kFine)
+                *reinterpret_cast<uint4*>(reinterpret_cast<unsigned char*>(dst) + kOffRest) =
+                    make_uint4(rest[4 * u], rest[4 * u + 1], rest[4 * u + 2], rest[4 * u + 3]);
+            }
           }
         }
       }
@@ -860,15 +882,18 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
           tmem_ld_chunk<kCW>(tmem_lane + 2 * col_stride + ch * kCW, o);
           tmem_wait_ld();
         }
-        uint32_t h[kCW / 2];
+        if constexpr (kFine) {
 #pragma unroll
-        for (int c = 0; c < kCW; c += 2) {
-          const __nv_bfloat162 hh = __floats2bfloat162_rn(__uint_as_float(o[c]), __uint_as_float(o[c + 1]));
-          h[c >> 1] = *reinterpret_cast<const uint32_t*>(&hh);
+          for (int u = 0; u < kCW / 4; ++u)
+            st_async_v4(row_dst + ch * (kCW * 4) + u * 16, o[4 * u], o[4 * u + 1], o[4 * u + 2], o[4 * u + 3], row_bar);
+        } else {
+          uint32_t h[kCW / 2];
+#pragma unroll
+          for (int c = 0; c < kCW; c += 2) h[c >> 1] = pack_bf16(__uint_as_float(o[c]), __uint_as_float(o[c + 1]));
+#pragma unroll
+          for (int u = 0; u < kCW / 8; ++u)
+            st_async_v4(row_dst + ch * (kCW * 2) + u * 16, h[4 * u], h[4 * u + 1], h[4 * u + 2], h[4 * u + 3], row_bar);
         }
-#pragma unroll
-        for (int u = 0; u < kCW / 8; ++u)
-          st_async_v4(row_dst + ch * (kCW * 2) + u * 16, h[4 * u], h[4 * u + 1], h[4 * u + 2], h[4 * u + 3], row_bar);
       }
     }
     FALCON_TRACE(tid == 64, 45);
@@ -896,12 +921,18 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
     float acc[4] = {0.f, 0.f, 0.f, 0.f}, ls[4] = {0.f, 0.f, 0.f, 0.f};
     for (int s = 0; s < n_splits; ++s) {
       const unsigned char* base = (s == split) ? own : mrg + static_cast<uint32_t>(s < split ? s : s - 1) * slot_bytes;
-      const uint2 x = *reinterpret_cast<const uint2*>(base + static_cast<uint32_t>(dl) * pitch + qc * 8);
+      float4 x;
+      if constexpr (kFine) {
+        x = *reinterpret_cast<const float4*>(base + static_cast<uint32_t>(dl) * pitch + qc * 16);
+      } else {
+        const uint2 h = *reinterpret_cast<const uint2*>(base + static_cast<uint32_t>(dl) * pitch + qc * 8);
+        x = make_float4(bf16lo(h.x), bf16hi(h.x), bf16lo(h.y), bf16hi(h.y));
+      }
       const float4 lv = *reinterpret_cast<const float4*>(base + static_cast<uint32_t>(d_per) * pitch + qc * 16);
-      acc[0] += bf16lo(x.x);
-      acc[1] += bf16hi(x.x);
-      acc[2] += bf16lo(x.y);
-      acc[3] += bf16hi(x.y);
+      acc[0] += x.x;
+      acc[1] += x.y;
+      acc[2] += x.z;
+      acc[3] += x.w;
       ls[0] += lv.x;
       ls[1] += lv.y;
       ls[2] += lv.z;
@@ -957,7 +988,7 @@ int pick_splits(falcon_ctx* ctx, int units, int max_tiles) {
       cfg.attrs = &attr;
       cfg.numAttrs = 1;
       int n = 0;
-      if (cudaOccupancyMaxActiveClusters(&n, tree_attn_tck_kernel<kVar, true, 128, false>, &cfg) != cudaSuccess) n = -1;
+      if (cudaOccupancyMaxActiveClusters(&n, tree_attn_tck_kernel<kVar, kBKMax, 128, false>, &cfg) != cudaSuccess) n = -1;
       resident[s] = n > 0 ? n : -1;
       cudaGetLastError();
     }
@@ -974,18 +1005,23 @@ int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s, int 
   const int n_units = (a.tree.max_tree + q_nodes - 1) / q_nodes;
   if (static_cast<int64_t>(Hkv) * n_units > 65535) return FALCON_ERR_CAPACITY;
 
-  // 64-wide heads: three stages of 128 keys always fit
-  constexpr bool kMayBeLow = kHD == 128;
+  constexpr bool kFine = fine_weights(kHD, kSep);
+  using SG = Stage<kHD, kFine>;
+  // 64-wide heads and at most 64 rows: three stages of 128 keys always fit
+  constexpr int kLowTile = kHD == 128 || kVar > 0 ? 0 : kBKMax;
+  // fp32 partial rows of 49-64 query rows leave room for tiles of 112 keys: 32 heads of 128, 60 rows, 1084 keys 11.9 us with
+  // the geometry known at run time only, 11.3 with this.
+  constexpr int kMidTile = kFine && kHD == 128 && kVar == 0 ? 112 : kLowTile;
   bool& attr_set = ctx->attn_attr_set[1 + 4 * kVar + 2 * (kHD == 64) + kSep];
   if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(tree_attn_tck_kernel<kVar, true, kHD, kSep>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSmemMax));
-    if (e == cudaSuccess && !(kHD == 128 && !kSep))  // (the occupancy query below is made with this one)
-      e = cudaFuncSetAttribute(tree_attn_tck_kernel<kVar, true, 128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               static_cast<int>(kSmemMax));
-    if (e == cudaSuccess && kMayBeLow)
-      e = cudaFuncSetAttribute(tree_attn_tck_kernel<kVar, !kMayBeLow, kHD, kSep>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSmemMax));
+    cudaError_t e = cudaSuccess;
+    auto set = [&](auto* kernel) {
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSmemMax));
+    };
+    set(tree_attn_tck_kernel<kVar, kBKMax, 128, false>);  // (the occupancy query below is made with this one)
+    set(tree_attn_tck_kernel<kVar, kBKMax, kHD, kSep>);
+    set(tree_attn_tck_kernel<kVar, kLowTile, kHD, kSep>);
+    set(tree_attn_tck_kernel<kVar, kMidTile, kHD, kSep>);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute(tree_attn_tck_kernel)");
     attr_set = true;
   }
@@ -999,9 +1035,9 @@ int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s, int 
   // of the highest tile that fits (two if three would be lower than 64 keys).  A split count whose
   // merge area would leave less than two 64-key stages is reduced.
   const uint32_t q_bytes = static_cast<uint32_t>(N) * 2u * kHD;
-  const int row_bytes = static_cast<int>(Stage<kHD>::halves(Var<kVar>::kNMax)) * 128;  // of the ring, per key
+  const int row_bytes = static_cast<int>(SG::halves(Var<kVar>::kNMax)) * 128;  // of the ring, per key
   auto merge_bytes = [&](int ns) {
-    return ns > 1 ? static_cast<uint32_t>(ns - 1) * ((kHD + ns - 1) / ns + 2) * part_pitch(N) : 0u;
+    return ns > 1 ? static_cast<uint32_t>(ns - 1) * ((kHD + ns - 1) / ns + sum_rows(kFine)) * part_pitch(N, kFine) : 0u;
   };
   auto ring_room = [&](int ns) { return static_cast<int>(kSmemMax) - static_cast<int>(q_bytes + merge_bytes(ns) + C::kSmallBytes); };
   while (splits > 1 && ring_room(splits) < 2 * 64 * row_bytes) --splits;
@@ -1018,12 +1054,12 @@ int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s, int 
 
   // Tensor maps.  The head dimension is split into (64 columns, 2 halves) so that one box covers both
   // 128-byte-swizzled half tiles.  K/V cache: [64, s_cap, 2, Hkv, B], box 64 x tile_keys x 2.
-  uint64_t kv_dims[5] = {64, static_cast<uint64_t>(a.s_cap), Stage<kHD>::kHalves, static_cast<uint64_t>(Hkv), static_cast<uint64_t>(B)};
+  uint64_t kv_dims[5] = {64, static_cast<uint64_t>(a.s_cap), SG::kHalves, static_cast<uint64_t>(Hkv), static_cast<uint64_t>(B)};
   uint64_t kv_strides[4] = {static_cast<uint64_t>(a.kv_stride_s) * 2, 128, static_cast<uint64_t>(a.kv_stride_h) * 2,
                             static_cast<uint64_t>(a.kv_stride_b) * 2};
   if (Hkv == 1 && kv_strides[2] == 0) kv_strides[2] = kv_strides[0] * a.s_cap;  // a size-1 dimension never strides
   if (B == 1 && kv_strides[3] == 0) kv_strides[3] = kv_strides[2] * Hkv;
-  const uint32_t kv_box[5] = {64, static_cast<uint32_t>(tile_keys), Stage<kHD>::kHalves, 1, 1};
+  const uint32_t kv_box[5] = {64, static_cast<uint32_t>(tile_keys), SG::kHalves, 1, 1};
   CUtensorMap mk, mv;
   if (!get_tmap(ctx, a.k_cache, kv_dims, kv_strides, kv_box, &mk) || !get_tmap(ctx, a.v_cache, kv_dims, kv_strides, kv_box, &mv)) {
     ctx->last_error = "cuTensorMapEncodeTiled failed";
@@ -1034,7 +1070,7 @@ int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s, int 
   CUtensorMap mnk = mk, mnv = mv;
   if (kSep) {
     const uint64_t n_all = static_cast<uint64_t>(a.tree.total_nodes), row = static_cast<uint64_t>(Hkv) * kHD * 2;
-    const uint64_t t_dims[5] = {64, n_all, Stage<kHD>::kHalves, static_cast<uint64_t>(Hkv), 1};
+    const uint64_t t_dims[5] = {64, n_all, SG::kHalves, static_cast<uint64_t>(Hkv), 1};
     const uint64_t t_strides[4] = {row, 128, static_cast<uint64_t>(kHD) * 2, row * n_all};
     if (!get_tmap(ctx, a.k_tree, t_dims, t_strides, kv_box, &mnk) || !get_tmap(ctx, a.v_tree, t_dims, t_strides, kv_box, &mnv)) {
       ctx->last_error = "cuTensorMapEncodeTiled failed";
@@ -1103,9 +1139,10 @@ int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s, int 
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  cudaError_t e = (tile_keys == kBKMax && n_stages == 3)
-                      ? cudaLaunchKernelEx(&cfg, tree_attn_tck_kernel<kVar, true, kHD, kSep>, mk, mv, mnk, mnv, p)
-                      : cudaLaunchKernelEx(&cfg, tree_attn_tck_kernel<kVar, !kMayBeLow, kHD, kSep>, mk, mv, mnk, mnv, p);
+  auto* kernel = tree_attn_tck_kernel<kVar, kLowTile, kHD, kSep>;
+  if (n_stages == 3 && tile_keys == kBKMax) kernel = tree_attn_tck_kernel<kVar, kBKMax, kHD, kSep>;
+  else if (kMidTile && n_stages == 3 && tile_keys == kMidTile) kernel = tree_attn_tck_kernel<kVar, kMidTile, kHD, kSep>;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, mk, mv, mnk, mnv, p);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "tree_attn_tck_kernel launch");
   return FALCON_OK;
 }

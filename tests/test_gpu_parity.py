@@ -208,6 +208,34 @@ def test_attn_separate_tree_buffers(kernel):
     H.assert_attn_close(out, ref, tb.node_off)
 
 
+@pytest.mark.parametrize("kernel", [binding.ATTN_AUTO] + KERNELS)
+@pytest.mark.parametrize("D, separate", [(64, False), (64, True), (128, True)])
+@pytest.mark.parametrize("sizes, prefs, Hkv, G, splits", [
+    ([1], [0], 2, 1, 1), ([6], [3], 2, 1, 1), ([33], [20], 2, 1, 0), ([64], [64], 2, 1, 2), ([80], [30], 2, 1, 2),
+    ([20], [100], 1, 8, 3), ([32], [130], 2, 4, 2), ([64], [64], 1, 4, 2), ([128], [700], 1, 2, 8), ([16] * 40, [5] * 40, 4, 1, 1),
+    ([60, 20], [640, 700], 2, 1, 0)])
+def test_attn_keeps_fp32_weights_where_cuda_cores_did(sizes, prefs, Hkv, G, splits, D, separate, kernel):
+    """64-wide heads and trees in buffers of their own: the output's error is that of its rounding to bf16 (2^-8) and of fp32
+    scores: sums of D products, D 2^-24 sum|q k| <= 128 x 2^-24 x 1.3 x 128 x 0.64 on these inputs, times log2(e) / sqrt(128) and
+    twice ln 2 (weight and row sum): below 2^-12 of sum w|v|.  (bf16 weights alone would give up to 2^-8 of it.)"""
+    rng = np.random.default_rng(77)
+    tb, q, k, v = random_case(rng, sizes, prefs, Hkv * G, Hkv, D)
+    ref = oracle_attn(tb, Hkv * G, Hkv, D, q, k, v)
+    size = oracle_attn(tb, Hkv * G, Hkv, D, q, k, v & np.uint16(0x7FFF))
+    kt = vt = None
+    if separate:
+        kt, vt = (np.empty((tb.total_nodes, Hkv, D), np.uint16) for _ in range(2))
+        for b, (T, L) in enumerate(zip(sizes, prefs)):
+            o = int(tb.node_off[b])
+            kt[o:o + T], vt[o:o + T] = (x[b, :, L:L + T].transpose(1, 0, 2) for x in (k, v))
+    out, rc = H.run_attn(H.DevTrees(tb), Hkv * G, Hkv, D, q, k, v, k_tree=kt, v_tree=vt, kernel=kernel, n_splits=splits, check=False)
+    tc_or_skip(rc)
+    got = synth.bf16_bits_to_f32(out).astype(np.float64)
+    excess = np.abs(got - ref) - 2.0 ** -8 * np.abs(ref)
+    worst = float((excess / size).max())
+    assert worst <= 2.0 ** -12, "error beyond the output's rounding: %.3g of sum w|v|" % worst
+
+
 def relaxed_mask_rows(tb, k_block, drop=()):
     """Mask rows of the drafter's relaxed causal mask (Section 3.4): a node sees its predecessors in the tree and the
     nodes of its own block of k_block consecutive nodes.  `drop` lists (packed node, tree key) bits to clear."""
