@@ -236,6 +236,20 @@ def test_attn_keeps_fp32_weights_where_cuda_cores_did(sizes, prefs, Hkv, G, spli
     assert worst <= 2.0 ** -12, "error beyond the output's rounding: %.3g of sum w|v|" % worst
 
 
+def test_attn_tc_weights_are_rounded_to_nearest():
+    """One bf16 number per weight, rounded: its relative error has rms e = 2^-8 / sqrt(3) x sqrt(E[1/m^2]) (m the significand,
+    its logarithm even over [1, 2): E = 0.541), which independent values carry over to the output; the output's own rounding adds
+    the same once more: e sqrt(2) = 2.346e-3, and 1 % for the sample (960 rows of 128).  (Weights cut off instead have a mean error
+    that depends on m, 0.143 x 2^-8: 2.41e-3.)"""
+    rng = np.random.default_rng(5)
+    tb, q, k, v = random_case(rng, [60, 60], [1500, 900], 8, 8, 128)
+    ref = oracle_attn(tb, 8, 8, 128, q, k, v).astype(np.float64)
+    out, rc = H.run_attn(H.DevTrees(tb), 8, 8, 128, q, k, v, kernel=binding.ATTN_TC, n_splits=1)
+    assert rc == binding.OK
+    rel = np.linalg.norm(synth.bf16_bits_to_f32(out).astype(np.float64) - ref) / np.linalg.norm(ref)
+    assert rel <= 1.01 * math.sqrt(2.0) * 2.0 ** -8 / math.sqrt(3.0) * math.sqrt(0.375 / math.log(2.0)), rel
+
+
 def relaxed_mask_rows(tb, k_block, drop=()):
     """Mask rows of the drafter's relaxed causal mask (Section 3.4): a node sees its predecessors in the tree and the
     nodes of its own block of k_block consecutive nodes.  `drop` lists (packed node, tree key) bits to clear."""
