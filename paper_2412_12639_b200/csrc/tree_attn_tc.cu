@@ -41,13 +41,6 @@
 
 #include "tc_util.cuh"
 
-// Profiling hook, off by default: a build may predefine it to record per-phase time stamps.
-#ifndef FALCON_TRACE
-#define FALCON_TRACE(who, id)
-#define FALCON_TRACE_PARAMS
-#define FALCON_TRACE_LAUNCH(p)
-#endif
-
 namespace falcon {
 namespace {
 using namespace tc;
@@ -122,7 +115,6 @@ struct TcParams {
   int32_t h_node_off[kHostSeqs + 1];
   int32_t h_prefix[kHostSeqs];
   int32_t h_order[kHostSeqs];  // grid z -> sequence, longest first
-  FALCON_TRACE_PARAMS
 };
 
 // A CTA's partial rows in scratch: 16-byte pieces [piece][row], so that a warp's 32 rows are contiguous for
@@ -158,7 +150,6 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
   auto bar = [&](int i) { return smem_base + C::kOffBars + 8u * static_cast<uint32_t>(i); };
 
   const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
-  FALCON_TRACE(tid == 0, 0);
   const int n_splits = kLoop ? 1 : gridDim.x, split = kLoop ? 0 : blockIdx.x;  // cluster = all CTAs of a row of the grid
   int kvh = blockIdx.y % p.Hkv, unit = blockIdx.y / p.Hkv;
   int b = p.have_host ? p.h_order[blockIdx.z] : static_cast<int>(blockIdx.z);
@@ -305,7 +296,6 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
   // CTA-wide barrier from here to the merge: each role starts as soon as what it needs is there.
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  FALCON_TRACE(tid == 0, 1);
   if (!p.have_host) {
     if constexpr (kLoop) next_unit();
     else device_scalars();
@@ -333,7 +323,6 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       if (n_my > 0) load_q();
       issued = min(2 * n_my, kSlots);
       for (int i = n_early; i < issued; ++i) load_item(i);
-      FALCON_TRACE(true, 2);
       capacity();
       bool ok = true;
       for (int i = kSlots; i < 2 * n_my; ++i) {
@@ -401,7 +390,6 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       const uint32_t phase0 = kLoop ? __shfl_sync(0xffffffffu, (ring0 / kSlots) & 1, 0) : 0u;
       bool ok = mbar_wait(bar(C::kBarQ), kLoop ? nth & 1 : 0, abort_flag);
       if constexpr (kLoop) ok = __all_sync(0xffffffffu, ok);
-      FALCON_TRACE(elected, 5);
       // Every lane walks through the loop and looks at the barriers by itself (no votes: this warp shares its
       // scheduler with four softmax warps, and each instruction here is one the tensor core waits for).
       // A satisfied wait, a commit and an address each cost 50-150 cycles then, so a tile's K barrier is
@@ -474,13 +462,11 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             // (the accumulators are free again: the unit before has been read out)
             if (kLoop && j == 0 && s == 0 && nth > 0 && !mbar_wait(bar(C::kBarOFree), (nth - 1) & 1, abort_flag)) return;
             tc_fence_after();
-            FALCON_TRACE(elected && j * kBlocks + s < 8, 42 + j * kBlocks + s);
             issue_pv(s, buf, vslot, j, s == kBlocks - 1);
             if (more) {
               if (s == 0 && !k_wait()) return;
               issue_qk(s, buf, kslot, s == kBlocks - 1 && j + kAhead == n_my - 1);
             }
-            FALCON_TRACE(elected && j * kBlocks + s < 8, 50 + j * kBlocks + s);
           }
           if (((j + 1) & (kAhead - 1)) == 0) pphase ^= 1;
           vslot = vslot + 2 == kSlots + 1 ? 1 : vslot + 2;
@@ -584,7 +570,6 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       const int k0 = tile_key0(j), nv = tile_keys_in(j, k0);
       if (!mbar_wait_warp(bar(C::kBarSFull + grp), sphase, abort_flag)) break;
       sphase ^= 1;
-      FALCON_TRACE(q4 == 2 && lane == 0 && i < 8, 10 + 2 * i);
       tc_fence_after();
       // the scores are there, so the K tile is no longer needed (two blocks: the second's come last)
       if (q4 == 0 && lane == 0 && (!two_blocks || blk == 1)) mbar_arrive(bar(C::kBarKVEmpty + (ring0 + 2 * j) % kSlots));
@@ -660,7 +645,6 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(bar(C::kBarPFull + grp));
-      FALCON_TRACE(q4 == 2 && lane == 0 && i < 8, 11 + 2 * i);
     }
     if (!published) ref_barrier(false);  // (a wait gave up before the first tile)
 
@@ -684,7 +668,6 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     }
     bool have = n_my > 0 && !*abort_flag;
     if (have) have = mbar_wait_warp(bar(C::kBarODone), kLoop ? nth & 1 : 0, abort_flag);
-    FALCON_TRACE(tid == 64, 58);
     tc_fence_after();
     const int n_cols = two_blocks ? kHD / 2 : kHD / 4, col0 = (two_blocks ? grp >> 1 : grp) * n_cols;
     const bool first_cols = col0 == 0;
@@ -740,7 +723,6 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             none ? make_float2(-INFINITY, 0.f) : make_float2(fine ? m_ref : 0.f, fine ? l_row : __uint_as_float(0x7fc00000u));
       }
     }
-    FALCON_TRACE(tid == 64, 59);
     if constexpr (kLoop) {
       tc_fence_before();
       __syncwarp();
@@ -771,7 +753,6 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
   if (!kLoop && n_splits > 1) {
     // ================================ merge ================================
     cluster_sync_release();  // every split's partial rows are visible (it is this CTA's barrier as well)
-    FALCON_TRACE(tid == 0, 60);
     // An item is one piece (16 bytes of columns) of one row; a warp's items are consecutive rows.  All its loads are
     // issued before any is used: one round trip to L2.
     constexpr int kCols = kFine ? 4 : 8, kPieces = kHD / kCols;
@@ -843,7 +824,6 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     if (kLoop && *abort_flag && tid == 0) drain_loads(issued, q_issued);
   }
   if (*abort_flag && tid == 0) dev_status_or(p.status, b, FALCON_DEV_TIMEOUT);
-  FALCON_TRACE(tid == 0, 62);
   // exact path for this CTA's rows that need it
   if (rescue)
     for (int r = row0 + warp; r < row0 + rows_mine; r += kTcThreads / 32)
@@ -854,7 +834,6 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     __syncwarp();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols) : "memory");
   }
-  FALCON_TRACE(tid == 0, 63);
 }
 
 bool is_pow2(int x) { return x > 0 && (x & (x - 1)) == 0; }
@@ -986,7 +965,6 @@ int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s) {
   const bool loop = splits == 1 && n_total > ctx->sm_count && n_total < (1 << 30) && mean_tiles(a) <= kLoopTiles;
   if (static_cast<int64_t>(Hkv) * n_units > 65535) return FALCON_ERR_CAPACITY;
 
-
   // Tensor maps.  The head dimension is split into blocks of 64 columns so that one box covers all the
   // 128-byte-swizzled parts of a tile.  K/V cache: [64, s_cap, halves, Hkv, B].
   const uint64_t halves = C::kHalves;
@@ -1066,8 +1044,6 @@ int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s) {
       return p.h_prefix[x] + (p.h_node_off[x + 1] - p.h_node_off[x]) > p.h_prefix[y] + (p.h_node_off[y + 1] - p.h_node_off[y]);
     });
   }
-
-  FALCON_TRACE_LAUNCH(p)
 
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = loop ? dim3(ctx->sm_count) : dim3(splits, Hkv * n_units, B);

@@ -44,13 +44,6 @@
 
 #include "tc_util.cuh"
 
-// Profiling hooks, empty by default: a private build may predefine them to record time stamps.
-#ifndef FALCON_TRACE
-#define FALCON_TRACE(who, id)
-#define FALCON_TRACE_PARAMS
-#define FALCON_TRACE_LAUNCH(p)
-#endif
-
 namespace falcon {
 namespace {
 using namespace tc;
@@ -174,7 +167,6 @@ struct TckParams {
   struct alignas(16) HostSeq {
     int32_t seq, node_base, nodes, prefix;
   } h_seq[kHostSeqs];
-  FALCON_TRACE_PARAMS
 };
 
 // K/V tiles are read once per call and the caches are far larger than L2: the loads carry an
@@ -314,7 +306,6 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
   constexpr int kCW = VT::kCW, kPer = VT::kPer;
   const int G = p.G, N = p.n_rows, n_chunks = N / kCW;
   const uint32_t q_half_bytes = static_cast<uint32_t>(N) * 128u;  // between the two 64-column halves of Q
-  FALCON_TRACE(tid == 0, 0);
   if (warp == kWarpProducer) {
     // the barriers first: their initialisation (and its fence) runs under the parameter reads below
     if (lane == 0) {
@@ -335,7 +326,6 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
                           static_cast<uint32_t>(reinterpret_cast<uintptr_t>(p.out)) ^ static_cast<uint32_t>(p.prefetch_next);
     asm volatile("" ::"r"(warm));
   }
-  FALCON_TRACE(tid == 0, 20);
 
   // Geometry of this CTA's share, from the sequence's node range and prefix length.
   int node_base = 0, T_real = 0, L_raw = 0;
@@ -402,7 +392,6 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
     L_raw = p.h_seq[blockIdx.z].prefix;
     geometry();
   }
-  FALCON_TRACE(tid == 0, 22);
 
   // Under programmatic dependent launch the kernel starts while the previous kernel of the stream
   // is finishing; griddepcontrol.wait returns once that kernel has completed.  Each warp role waits
@@ -440,7 +429,6 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
     if (st_id < C::kN) s_rescue[st_id] = 0;
   } else if (warp == kWarpProducer) {
     __syncwarp();
-    FALCON_TRACE(tid == 0, 21);
     if (p.have_host && n_valid > 0 && lane == 0 && p.early_prefix) {
       // Prefix rows that the caller declares stable (written before the kernel that precedes this
       // one in the stream started) may be requested while that kernel is still finishing.
@@ -451,10 +439,8 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
         ++n_early;
       }
     }
-    FALCON_TRACE(tid == 0, 1);
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    FALCON_TRACE(tid == 0, 2);
     if (!p.have_host) device_scalars();
   } else {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(s_tmem_base)),
@@ -492,12 +478,10 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
     for (int j = n_early; j < min(n_my, kStages); ++j) load_tile(j);
     if (split == 0 && mtile == 0 && kvh == 0 && (L + (kSep ? 0 : T) > p.s_cap || T_real > FALCON_T_MAX))
       dev_status_or(p.status, b, FALCON_DEV_CAPACITY);
-    FALCON_TRACE(true, 3);
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  FALCON_TRACE(tid == 0, 4);
   const uint32_t tmem_base = *s_tmem_base;
   // Cluster phase 1: "my merge barrier exists".  Arrive now, wait just before the first remote copy.
   if (n_splits > 1) cluster_arrive();
@@ -541,11 +525,9 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
       uint32_t elected;
       asm volatile("{ .reg .pred p; elect.sync _|p, 0xffffffff; selp.u32 %0, 1, 0, p; }" : "=r"(elected));
       bool ok = mbar_wait_warp(bar(kBarQ), 0, abort_flag);
-      FALCON_TRACE(elected, 5);
       auto issue_qk = [&](int j) -> bool {
         const int st = j % kStages, sb = j & 1;
         if (!mbar_wait_warp(bar(kBarKVFull + st), (j / kStages) & 1, abort_flag)) return false;
-        FALCON_TRACE(elected && j < 4, 10 + 4 * j);
         tc_fence_after();
         const uint32_t kbase = smem_base + off_kv + st * kStageBytes + kOffK;
         if (elected) {
@@ -557,7 +539,6 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
             umma_bf16_ss(tmem_base + sb * col_stride, ad, bd, p.idesc_qk, kk > 0 ? 1u : 0u);
           }
           umma_commit(bar(kBarSFull + sb));
-          FALCON_TRACE(j == 0, 28);
         }
         __syncwarp();
         return true;
@@ -588,7 +569,6 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
       if (ok && n_my > 1) ok = issue_qk(1);
       for (int t = 0; ok && t < n_my; ++t) {
         if (!mbar_wait_warp(bar(kBarPFull + (t & 1)), (t >> 1) & 1, abort_flag)) { ok = false; break; }
-        FALCON_TRACE(elected && t < 4, 11 + 4 * t);
         tc_fence_after();
         issue_pv(t);
         if (t + 2 < n_my) ok = issue_qk(t + 2);
@@ -604,9 +584,6 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
     const uint32_t tmem_lane = tmem_base + (static_cast<uint32_t>(q4 * 32) << 16);
     bool live = n_my > 0 && !*abort_flag;
 
-    FALCON_TRACE(tid == 64 && live && qreg[0][0].x != 0x12345u, 6);
-    FALCON_TRACE(tid == 64 && live && kref[0].x != 0x12345u, 7);
-    FALCON_TRACE(tid == 64 && live && par_raw != 0x12345, 8);
     if (live) {
       // (a) Q block into shared memory in the layout the MMA reads (K-major rows of 128 bytes per
       // 64-column half, 16-byte units XOR-swizzled by the row).  The MMA warp is told at once; the
@@ -624,7 +601,6 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
       fence_async_smem();  // the MMA reads Q through the async proxy
       __syncwarp();
       if (lane == 0) mbar_arrive(bar(kBarQ));
-      FALCON_TRACE(tid == 64, 9);
       // the reference of every query row: its scaled score against cache row 0 (8 threads per row)
 #pragma unroll
       for (int pass = 0; pass < VT::kQPasses; ++pass) {
@@ -689,7 +665,6 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
       }
     }
     if (has_tree_keys) asm volatile("bar.sync 1, %0;" ::"n"(kSmThreads) : "memory");
-    FALCON_TRACE(tid == 64, 30);
 
     // The references of this thread's columns stay in registers when it has one chunk; with several
     // chunks they are read from shared memory where they are used (registers go to the row sums).
@@ -710,7 +685,6 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
       const int sb = j & 1, st = j % kStages;
       const int k0 = tile_key0(j), key = k0 + kr, nv = tile_keys_in(j, k0);
       if (!mbar_wait_warp(bar(kBarSFull + sb), (j >> 1) & 1, abort_flag)) { live = false; break; }
-      FALCON_TRACE(tid == 64 && j < 4, 32 + 3 * j);
       tc_fence_after();
       if (q4 * 32 < BK) {  // (a tile lower than 128 keys leaves the last quadrants without keys)
       uint32_t sr[kRefInRegs ? kPer : 1][kCW];
@@ -722,7 +696,6 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
         }
         tmem_wait_ld();
       }
-      FALCON_TRACE(tid == 64 && j < 4, 33 + 3 * j);
 
       // all of this warp's keys lie in the prefix: every one exists and is visible to every row
       const bool full = k0 + BK <= Lc && q4 * 32 + 32 <= BK;
@@ -810,7 +783,6 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(bar(kBarPFull + sb));
-      FALCON_TRACE(tid == 64 && j < 4, 34 + 3 * j);
     }
 
     // ---- this CTA's partial result goes straight into the shared memory of the CTAs that own it ----
@@ -862,7 +834,6 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
     // then recomputes the row on the exact path instead of dividing a short numerator by a full row sum.
     bool have_o = have;
     if (have_o) have_o = mbar_wait_warp(bar(kBarODone), 0, abort_flag);
-    FALCON_TRACE(tid == 64, 44);
     tc_fence_after();
     // The ring and P^T are idle now (all of this CTA's MMAs have finished, all its loads landed).
     if (st_id * 4 < N)
@@ -896,16 +867,13 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
         }
       }
     }
-    FALCON_TRACE(tid == 64, 45);
   } 
   if (warp < kWarpSm0 && n_splits > 1) cluster_wait();  // the producer and MMA warps complete phase 1 too
 
   // ================================ merge ================================
   // Wait until every softmax warp of every split has delivered its share of this CTA's rows.  Every
   // CTA delivers whatever happened to it, so the wait ends; it is bounded all the same.
-  FALCON_TRACE(tid == 0, 50);
   bool got = mbar_wait_cluster_warp(bar(kBarMrg), 0);
-  FALCON_TRACE(tid == 0, 52);
   if (tid == 0 && (*abort_flag || !got)) dev_status_or(p.status, b, FALCON_DEV_TIMEOUT);
   const unsigned char* mrg = smem_gen + off_mrg;
   const unsigned char* own = smem_gen + off_stage;
@@ -915,7 +883,6 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
   // from the reference's scale (or not finite) is left to the exact path below.
   __nv_bfloat16* out_base = p.out + (static_cast<int64_t>(node_base) * p.Hq + kvh * G) * kHD + d0;
   const int n_q4 = (n_valid + 3) >> 2;
-  FALCON_TRACE(tid == 0, 56);
   for (int item = tid; item < d_mine * n_q4; item += kThreads) {
     const int qc = item / d_mine, dl = item - qc * d_mine;
     float acc[4] = {0.f, 0.f, 0.f, 0.f}, ls[4] = {0.f, 0.f, 0.f, 0.f};
@@ -938,7 +905,6 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
       ls[2] += lv.z;
       ls[3] += lv.w;
     }
-    FALCON_TRACE(tid == 0 && acc[0] != 1.2345f, 58);
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
       const int r = qc * 4 + c;
@@ -952,12 +918,10 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
       }
     }
   }
-  FALCON_TRACE(tid == 0, 53);
   __syncthreads();
   // exact path for the rows that need it, shared out over the cluster's CTAs and this CTA's warps
   for (int r = split + n_splits * warp; r < n_valid; r += n_splits * (kThreads / 32))
     if (s_rescue[r]) rescue_row<kHD>(p, b, kvh, node_base, T, Lc, S_valid, mtile * N + r, lane);
-  FALCON_TRACE(tid == 0, 54);
   if (warp == kWarpMma) {
     // (after a wait that gave up, MMAs may still be running: the last commit covers them all)
     if (n_my > 0 && *abort_flag && lane == 0) mbar_wait_drain(bar(kBarODone), 0);
@@ -1122,8 +1086,6 @@ int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s, int 
     if (static_cast<int64_t>(Hkv) * n_units * B <= 2 * ctx->sm_count)
       std::stable_sort(p.h_seq, p.h_seq + B, [](const auto& x, const auto& y) { return x.prefix + x.nodes > y.prefix + y.nodes; });
   }
-
-  FALCON_TRACE_LAUNCH(p)
 
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(splits, Hkv * n_units, B);
