@@ -300,6 +300,14 @@ __device__ __forceinline__ uint64_t window64(uint64_t lo, uint64_t hi, int off) 
 }
 
 // ------------------------------------------------------------------------------------ host side
+// Keys of a sequence, on average (of the longest one where the lengths are on the device only).
+inline int64_t mean_keys(const falcon_attn_args& a) {
+  if (!a.tree.prefix_len_host || !a.tree.node_off_host) return static_cast<int64_t>(a.tree.max_tree) + a.tree.max_prefix_len;
+  int64_t keys = a.tree.total_nodes;
+  for (int i = 0; i < a.tree.batch; ++i) keys += a.tree.prefix_len_host[i];
+  return (keys + a.tree.batch - 1) / a.tree.batch;
+}
+
 using EncodeFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                               const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                               CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);

@@ -924,17 +924,6 @@ Plan make_plan(falcon_ctx* ctx, const falcon_attn_args& a) {
   return best;
 }
 
-// Tiles of a sequence, on average (of the longest one where the lengths are on the device only).
-int mean_tiles(const falcon_attn_args& a) {
-  int64_t keys = a.tree.max_tree + a.tree.max_prefix_len;
-  if (a.tree.prefix_len_host && a.tree.node_off_host) {
-    keys = a.tree.total_nodes;
-    for (int i = 0; i < a.tree.batch; ++i) keys += a.tree.prefix_len_host[i];
-    keys = (keys + a.tree.batch - 1) / a.tree.batch;
-  }
-  return static_cast<int>((keys + kBKMax - 1) / kBKMax);
-}
-
 template <int kHD, bool kFine>
 int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s) {
   using C = Cfg<kHD>;
@@ -962,7 +951,7 @@ int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s) {
   // sequences, 40 heads of 64), of 5 tiles on average (13 sequences, 8 KV heads of 128) 14.0 both ways, of 19 tiles
   // 40 -> 42, of 34 tiles 47 -> 54.
   const int64_t n_total = static_cast<int64_t>(Hkv) * n_units * B;
-  const bool loop = splits == 1 && n_total > ctx->sm_count && n_total < (1 << 30) && mean_tiles(a) <= kLoopTiles;
+  const bool loop = splits == 1 && n_total > ctx->sm_count && n_total < (1 << 30) && (mean_keys(a) + kBKMax - 1) / kBKMax <= kLoopTiles;
   if (static_cast<int64_t>(Hkv) * n_units > 65535) return FALCON_ERR_CAPACITY;
 
   // Tensor maps.  The head dimension is split into blocks of 64 columns so that one box covers all the

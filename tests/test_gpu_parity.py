@@ -654,6 +654,26 @@ def test_attn_tc_more_units_than_sms(sizes, prefs, Hkv, G, separate, D):
             assert not dt.status.cpu().numpy().any()
 
 
+@pytest.mark.parametrize("D, T, prefs, expect", [
+    (128, 60, [1987] * 8, binding.ATTN_TC), (128, 60, [1988] * 8, binding.ATTN_TCK), (128, 60, [300, 3676] * 4, binding.ATTN_TCK),
+    (128, 60, [300, 3674] * 4, binding.ATTN_TC), (128, 32, [700] * 8, binding.ATTN_TCK), (128, 33, [700] * 8, binding.ATTN_TC),
+    (128, 65, [4000] * 8, binding.ATTN_TC), (64, 60, [4000] * 8, binding.ATTN_TC), (128, 60, [700] * 4, binding.ATTN_TCK)])
+def test_attn_choice_for_batches_of_many_units(D, T, prefs, expect):
+    """32 KV heads: which kernel AUTO takes on either side of each line (mean keys 2048, 33 and 65 rows, more units than SMs), and
+    that without the host copies the longest sequence counts."""
+    rng = np.random.default_rng(3)
+    tb = H.make_trees([T] * len(prefs), prefs, rng)
+    dt = H.DevTrees(tb)
+    q = torch.zeros((tb.total_nodes, 32, D), dtype=torch.bfloat16, device="cuda")
+    k = torch.zeros(16, dtype=torch.bfloat16, device="cuda")  # (nothing is launched)
+    cap = max(prefs) + T
+    for host in (True, False):
+        a = binding.attn_args(dt.desc(host_copies=host), 32, 32, D, 0.1, q, q, k, k, (32 * cap * D, cap * D, D), cap)
+        got = H.ctx().falcon_tree_attn_kernel(a)
+        by_longest = D == 128 and 32 < T <= 64 and len(prefs) * 32 > 148 and max(prefs) + T >= 2048
+        assert got == (expect if host or not by_longest else binding.ATTN_TCK)
+
+
 @pytest.mark.parametrize("B,Hkv", [(9, 2), (32, 1), (33, 1), (20, 16)])
 def test_attn_tck_batches_with_and_without_host_copies(B, Hkv):
     """Keys-on-lanes kernel: batches whose sequences travel with the call (up to 32, longest first up to two waves)
