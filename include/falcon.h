@@ -115,7 +115,7 @@ typedef struct {
  *             of sequence b holds tree node t's K/V unless k_tree/v_tree given.
  *             Base 16-byte aligned, strides multiples of 8 elements.
  * k/v_tree    optional bf16 [N, Hkv, D]: tree K/V kept outside the cache.
- * kernel      FALCON_ATTN_AUTO picks (by shape, see DESIGN notes in the sources); the others force
+ * kernel      FALCON_ATTN_AUTO picks (by shape: the rules and their figures stand in the sources); the others force
  *             one kernel: _SIMT CUDA cores (any supported shape), _WARP CUDA cores with one warp
  *             per query row (at most 1024 keys per sequence; the small-problem kernel), _TC tensor
  *             cores with the query rows on the tensor-memory lanes, _TCK tensor cores with the

@@ -117,7 +117,7 @@ int falcon_tree_validate_host(const int32_t* parent, int32_t T) {
 }
 
 // Argument checks of falcon_tree_attn and the kernel it dispatches to; *kernel is one of
-// FALCON_ATTN_SIMT / _TC / _TCK on success.
+// FALCON_ATTN_SIMT / _WARP / _TC / _TCK on success.
 static int attn_plan(falcon_ctx* ctx, const falcon_attn_args* a, int* kernel) {
   if (!ctx || !a) return FALCON_ERR_INVALID_ARG;
   int rc = check_tree_desc(a->tree, false);

@@ -272,6 +272,8 @@ int launch_kv_compact(falcon_ctx* ctx, const falcon_compact_args& a, cudaStream_
   if (move_ctas > INT32_MAX - 32) return FALCON_ERR_CAPACITY;
   p.move_ctas = static_cast<int32_t>(move_ctas);
   const int cpr = a.head_dim >> 3, pieces = a.tree.max_tree * cpr;
+  // A path longer than max_tree says that the caller's bound is wrong.  From these lengths on it is refused (a bound of the
+  // interface; the kernel itself would take any path of the tree).
   p.max_rows = (pieces <= 1024 ? 1024 : pieces <= 1536 ? 1536 : 4096) / cpr;
   if (a.gather) set_gather(p, *a.gather, a.tree.token);  // further CTAs record the accepted tokens and features
   cudaLaunchConfig_t cfg = {};

@@ -3,21 +3,19 @@
 //
 // Row r of a KV head is (tree node r / G, query head r % G), so grouped-query heads share the K/V
 // stream.  A unit is (sequence, KV head, block of at most 256 query rows); one thread-block cluster per
-// unit, whose CTAs split the key range (prefix + tree) into runs of whole tiles of up to 128 keys.
+// unit, whose CTAs split the key range (prefix + tree) into runs of whole tiles of up to 64 keys.
 // Where there are many units of few tiles, the grid is one CTA per SM instead, which works on one unit after the
 // other (kLoop): the next one's K, V and Q are on their way while the rows of the one before are delivered.
 //
-// Inside a CTA (576 threads) two streams of 128 TMEM lanes each work on tiles in turn, so that one
-// stream's softmax runs under the other's MMAs:
-//   more than 128 rows   stream s holds rows 128 s ..: every K/V tile is read once from shared memory's
-//                        ring for both (half the L2-to-SM traffic of 128-row units, which is what
-//                        bounded grouped heads);
-//   at most 128 rows     both streams hold the same rows and take the even and the odd tiles.
+// Inside a CTA (576 threads) an item is (tile, block of 128 rows), and four score buffers in TMEM take the items in
+// turn, so that the softmax of some runs under the MMAs of others:
+//   more than 128 rows   two row blocks share every K/V tile: it is read once from L2 for both;
+//   at most 128 rows     one row block: an item is a tile.
 //   warp 0    TMA producer: Q, then K and V tiles (bf16, 128-byte swizzle) into a ring of 16 KB slots (8 KB for 64-wide heads).
-//   warp 1    one elected lane issues tcgen05.mma: S_s = Q_s.K^T (M 128, N = tile, from shared memory)
-//             and O_s += P_s.V (P from TMEM, where it lies over S_s).
-//   warps 2-17 softmax, one thread per (row, stream, half of the key columns): tree mask from the node's
-//             ancestor bit set, p = 2^(s.scale - m), P back to TMEM as bf16.
+//   warp 1    one elected lane issues tcgen05.mma: S_i = Q.K^T of item i (M 128, N = tile, from shared memory) into
+//             score buffer i mod 4, and O += P_i.V into the row block's accumulator (P from TMEM, where it lies over S_i).
+//   warps 2-17 softmax, four groups of four warps: group g takes whole items, i = g mod 4, a thread one row of each:
+//             tree mask from the node's ancestor bit set, p = 2^(s.scale - m), P back to TMEM as bf16.
 //
 // Softmax with a fixed reference: m is the row's score against the first key of this CTA's run, not its
 // maximum: fp32 and bf16 carry exponents to 2^127, so nothing is rescaled while the row's scores
@@ -45,7 +43,7 @@ namespace falcon {
 namespace {
 using namespace tc;
 
-constexpr int kRowsMax = 256;     // query rows per unit at most: two streams of 128 TMEM lanes
+constexpr int kRowsMax = 256;     // query rows per unit at most: two blocks of 128 TMEM lanes
 constexpr int kBKMax = 64;        // keys per tile at most
 constexpr int kSmThreads = 512;
 constexpr int kTcThreads = 64 + kSmThreads;
@@ -875,12 +873,14 @@ struct Plan {
 };
 // Rows per unit (one block of 128 or two), key splits per unit and tile height: the least estimated time.
 // A CTA costs a fixed part (launch, Q, merge: 4 us, 5 with splits) and its tiles, 64 keys each: 0.92 us
-// with two row blocks (0.75 for 64-wide heads: softmax and MMA issue), with one block 0.73 (0.38)
+// with two row blocks (0.75 for 64-wide heads), with one block 0.73 (0.38)
 // where the K/V stream comes from HBM, at the 45 GB/s that one SM draws, and 0.5 (0.38) where other
 // row blocks' CTAs bring the same tiles into L2.  Units beyond the resident clusters wait for a slot, and a cluster for
 // all of its SMs at once: 4 us more for each (16 sequences of 350-3850 keys, 8 KV heads of 4 query heads: two
 // splits of 256-row units 52 us, no split 64; no split of 128-row units 47, which is what this finds).
 // One sequence's tile height is chosen so that its tiles divide evenly over the splits.
+// With fine weights a tile measures more (0.55 and 0.92 us for 64-wide heads, 0.75 and 1.2 for 128-wide), and so does a merge;
+// with those figures for the tiles alone the choice got worse (1.3 % above the best split count over 58 shapes, 0.8 % as it is).
 Plan make_plan(falcon_ctx* ctx, const falcon_attn_args& a) {
   const int B = a.tree.batch, G = a.n_q_heads / a.n_kv_heads;
   const bool host = a.tree.prefix_len_host && a.tree.node_off_host, wide = a.head_dim == 128;
@@ -947,9 +947,9 @@ int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s) {
   const int q_nodes = plan.q_nodes, n_units = plan.n_units, splits = plan.splits, tile_keys = plan.tile;
   // More units than SMs, of few tiles each: one CTA per SM works on several (see kLoop).  What a unit costs beside its
   // tiles is about 2 us then and 4.5 us as a CTA of its own, but the hardware gives out CTAs as SMs become free
-  // and the loop's shares are fixed: units of 3 to 7 tiles 29.7 -> 24.1 and 35.7 -> 29.3 us a launch (16 and 15
-  // sequences, 40 heads of 64), of 5 tiles on average (13 sequences, 8 KV heads of 128) 14.0 both ways, of 19 tiles
-  // 40 -> 42, of 34 tiles 47 -> 54.
+  // and the loop's shares are fixed: units of 2 to 7 tiles 37.6 -> 32.1 and 33.4 -> 27.1 us a launch (16 and 15
+  // sequences, 40 heads of 64), 38.5 -> 31.2 (15, 40 of 128, tree in its own buffers), of 5 tiles on average (13
+  // sequences, 8 KV heads of 128) 14.0 both ways, of 19 tiles 40 -> 42, of 34 tiles 47 -> 54.
   const int64_t n_total = static_cast<int64_t>(Hkv) * n_units * B;
   const bool loop = splits == 1 && n_total > ctx->sm_count && n_total < (1 << 30) && (mean_keys(a) + kBKMax - 1) / kBKMax <= kLoopTiles;
   if (static_cast<int64_t>(Hkv) * n_units > 65535) return FALCON_ERR_CAPACITY;
@@ -1060,7 +1060,7 @@ int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s) {
 bool tree_attn_tc_supports(const falcon_ctx* ctx, const falcon_attn_args& a) {
   (void)ctx;
   if (a.head_dim != 64 && a.head_dim != 128) return false;
-  if (!(a.sm_scale > 0.f)) return false;  // the kernel takes row maxima on unscaled scores
+  if (!(a.sm_scale > 0.f)) return false;  // a masked score is -inf before it is scaled
   const int G = a.n_q_heads / a.n_kv_heads;
   if (!is_pow2(G) || G > 128) return false;
   if (a.n_splits > kMaxSplits) return false;

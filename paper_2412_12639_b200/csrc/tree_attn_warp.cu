@@ -241,9 +241,10 @@ bool tree_attn_warp_supports(const falcon_ctx* ctx, const falcon_attn_args& a) {
 
 // Where this kernel beats the tensor-core kernels, whose set-up costs 4.2 to 5 us whatever the size: a
 // block's time grows with its keys, and the blocks come in waves of a few hundred rows.  Measured, us per
-// launch against the better tensor-core kernel: 4 heads x 64, 8 nodes, 24 / 72 / 136 keys 3.3 / 4.1 / 5.5
-// against 4.2 / 4.9 / 5.1; 16 heads x 64, 16 nodes, 32 / 80 keys 3.8 / 5.2 against 4.2 / 4.9; 16 heads x
-// 128, 8 nodes, 72 keys 4.8 against 5.3; 32 heads x 128, 16 nodes, 32 keys 7.6 against 4.7.
+// launch against the better tensor-core kernel (64-wide heads with fine weights): 4 heads x 64, 8 nodes, 24 / 72 / 136
+// keys 4.0 / 4.9 / 6.7 against 4.4 / 5.1 / 5.5; 8 x 64, 15 nodes, 60 / 96 keys 4.2 / 5.0 against 5.1 / 5.3; 16 x 64, 16
+// nodes, 32 / 80 keys 4.4 / 5.8 against 4.6 / 5.4; 16 x 128, 8 nodes, 72 keys 5.8 against 5.5; 32 x 128, 16 nodes, 32
+// keys 8.3 against 5.0.
 bool tree_attn_warp_preferred(const falcon_attn_args& a) {
   const int64_t keys = a.tree.max_prefix_len + a.tree.max_tree;
   return keys <= 96 && keys * a.head_dim * a.tree.total_nodes * a.n_q_heads <= 1100000;
