@@ -228,6 +228,7 @@ def test_attn_keeps_fp32_weights_where_cuda_cores_did(sizes, prefs, Hkv, G, spli
         for b, (T, L) in enumerate(zip(sizes, prefs)):
             o = int(tb.node_off[b])
             kt[o:o + T], vt[o:o + T] = (x[b, :, L:L + T].transpose(1, 0, 2) for x in (k, v))
+    H.ctx().falcon_test_poison(0xFFFFFFFF)  # what a kernel reads on chip without having written it is NaN
     out, rc = H.run_attn(H.DevTrees(tb), Hkv * G, Hkv, D, q, k, v, k_tree=kt, v_tree=vt, kernel=kernel, n_splits=splits, check=False)
     tc_or_skip(rc)
     got = synth.bf16_bits_to_f32(out).astype(np.float64)
