@@ -9,8 +9,8 @@
 // (V split evenly over the SMs, in steps of 16, so one launch is one wave) and streams it through a
 // TMA ring in chunks of 64 hidden columns together with the matching chunk of the features (L2
 // hits after the first CTA).  tcgen05.mma with the nodes on the M side and the CTA's vocabulary rows on the N
-// side (up to 256 per instruction) accumulates in TMEM; four warps then read one accumulator row
-// (= one node) each, 32 columns at a time, and keep the first maximum.  A CTA's result for a node
+// side (up to 256 per instruction) accumulates in TMEM; eight warps then read the accumulators, a thread half a row
+// (= half of a node's columns), 32 columns at a time, and keep the first maximum.  A CTA's result for a node
 // is one 64-bit atomicMax on a word ordered by (logit, then lower index), so ties go to the lowest
 // index whatever the timing; the last CTA to arrive unpacks the words.
 //
@@ -34,8 +34,8 @@ namespace falcon {
 namespace {
 using namespace tc;
 
-constexpr int kLmThreads = 192;
-constexpr int kLmReaders = 128;
+constexpr int kLmReaders = 256;
+constexpr int kLmThreads = 64 + kLmReaders;
 constexpr int kLmKC = 64;             // hidden columns per ring stage: one 128-byte swizzle row of bf16
 constexpr int kLmMaxStages = 8;
 constexpr int kLmTileMax = 256;       // vocabulary rows per MMA (the N side) at most
@@ -314,45 +314,64 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_con
     __syncwarp();
   } else {
     // ================================ accumulator readers ================================
+    // Two warps for each TMEM lane quadrant: one for each accumulator of a pair, else one for each half of the columns.
+    // The MMAs wait for them wherever another vocabulary tile follows, and the call waits for the last: one thread per row,
+    // with a single chain of compares through its columns, took 740 cycles for 32 of them; four chains and the next
+    // columns' load under the compares take 150.  (What it gave: see the top of the file.)
     const int q = warp & 3;                 // TMEM lane quadrant this warp can reach
+    const int sub = (warp - 2) >> 2;
     const int r = q * 32 + lane;            // accumulator row = node inside its tile
-    const int rt = tid - 64;                // 0 .. 127
-    const uint32_t tmem_lane = tmem_base + (static_cast<uint32_t>(q * 32) << 16);
+    const int rt = tid - 64;                // 0 .. kLmReaders - 1
+    const uint32_t tmem_lane = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + (kPair ? static_cast<uint32_t>(sub) * 256u : 0u);
     int tile = 0;
     bool ok = !*abort_flag;
     for (int g = 0; g < n_groups; ++g) {
-      float best[2] = {-INFINITY, -INFINITY};
-      int idx[2] = {INT_MAX, INT_MAX};
+      constexpr int kChains = 4;
+      float best[kChains];
+      int idx[kChains];
+#pragma unroll
+      for (int i = 0; i < kChains; ++i) {
+        best[i] = -INFINITY;
+        idx[i] = INT_MAX;
+      }
       for (int vp = 0; ok && vp < n_vp; ++vp, ++tile) {
         ok = mbar_wait_warp(bar(kLmBarAccFull), tile & 1, abort_flag);
         if (!ok) break;
         tc_fence_after();
+        const int v0 = v_lo + (v_res > 1 ? vp * 2 + sub : vp) * p.tile_n;
+        const int all = v_res > 1 || !kPair || sub < tiles_of(g) ? min(p.tile_n, v_hi - v0) : 0;  // columns with logits
+        const int half = kPair ? 0 : ((all >> 1) + 31) & ~31;
+        const int begin = kPair || sub == 0 ? 0 : half, end = kPair || sub == 1 ? all : min(all, half);
+        auto look = [&](uint32_t (&x)[32], int c0) {
+          if (c0 + 32 > end) {  // (columns past the last one hold whatever was there)
 #pragma unroll
-        for (int j = 0; j < (kPair ? 2 : 1); ++j) {
-          const int v0 = v_lo + (v_res > 1 ? vp * 2 + j : vp) * p.tile_n;
-          const int ncols = v_res > 1 || j < tiles_of(g) ? min(p.tile_n, v_hi - v0) : 0;
-          // (vocabulary tiles follow one another: one maximum per row; node tiles are different rows)
-          float m = v_res > 1 ? best[0] : best[j];
-          int mi = v_res > 1 ? idx[0] : idx[j];
-          for (int c0 = 0; c0 < ncols; c0 += 32) {
-            uint32_t x[32];
-            FALCON_TMEM_LD32(tmem_lane + static_cast<uint32_t>(j) * 256u + static_cast<uint32_t>(c0), x);
-            tmem_wait_ld();
+            for (int c = 0; c < 32; ++c)
+              if (c0 + c >= end) x[c] = 0xff800000u;
+          }
 #pragma unroll
-            for (int c = 0; c < 32; ++c) {
-              const float f = __uint_as_float(x[c]);
-              if (c0 + c < ncols && f > m) {  // strict: columns ascend, so the first maximum stays; NaN never wins
-                m = f;
-                mi = v0 + c0 + c;
+          for (int c = 0; c < 32; c += kChains)
+#pragma unroll
+            for (int i = 0; i < kChains; ++i) {
+              const float f = __uint_as_float(x[c + i]);
+              if (f > best[i]) {  // strict: a chain's columns ascend, so its first maximum stays; NaN never wins
+                best[i] = f;
+                idx[i] = v0 + c0 + c + i;
               }
             }
-          }
-          if (v_res > 1) {
-            best[0] = m;
-            idx[0] = mi;
-          } else {
-            best[j] = m;
-            idx[j] = mi;
+        };
+        if (begin < end) {
+          uint32_t x0[32], x1[32];
+          FALCON_TMEM_LD32(tmem_lane + static_cast<uint32_t>(begin), x0);
+          tmem_wait_ld();
+          for (int c0 = begin; c0 < end; c0 += 64) {
+            if (c0 + 32 < end) FALCON_TMEM_LD32(tmem_lane + static_cast<uint32_t>(c0 + 32), x1);
+            look(x0, c0);
+            tmem_wait_ld();
+            if (c0 + 32 < end) {
+              if (c0 + 64 < end) FALCON_TMEM_LD32(tmem_lane + static_cast<uint32_t>(c0 + 64), x0);
+              look(x1, c0 + 32);
+              tmem_wait_ld();
+            }
           }
         }
         tc_fence_before();
@@ -362,12 +381,16 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_con
           else mbar_arrive(bar(kLmBarAccEmpty));
         }
       }
+      // the chains' maxima, ties to the lower index
 #pragma unroll
-      for (int j = 0; j < (kPair ? 2 : 1); ++j) {
-        const int node = kPair ? (g * m_res + j) * 256 + rank * 128 + r : g * 128 + r;
-        // one atomic per node and CTA: the order of arrival does not matter, the word's order decides
-        if (j < m_res && node < p.n_rows && ok && idx[j] != INT_MAX) atomicMax(p.best + node, lm_pack(best[j], idx[j]));
-      }
+      for (int i = 1; i < kChains; ++i)
+        if (best[i] > best[0] || (best[i] == best[0] && idx[i] < idx[0])) {
+          best[0] = best[i];
+          idx[0] = idx[i];
+        }
+      const int node = kPair ? (g * m_res + (m_res > 1 ? sub : 0)) * 256 + rank * 128 + r : g * 128 + r;
+      // one atomic per node, CTA and warp: the order of arrival does not matter, the word's order decides
+      if (node < p.n_rows && ok && idx[0] != INT_MAX) atomicMax(p.best + node, lm_pack(best[0], idx[0]));
     }
     // the last CTA to arrive folds the CTAs' results in vocabulary order
     asm volatile("bar.sync 1, %0;" ::"n"(kLmReaders) : "memory");
