@@ -14,15 +14,19 @@
 // is one 64-bit atomicMax on a word ordered by (logit, then lower index), so ties go to the lowest
 // index whatever the timing; the last CTA to arrive unpacks the words.
 //
-// More nodes: pairs of CTAs (kPair, cta_group::2).  What bounds then is what an SM can draw from L2, about 33 bytes per
-// cycle, and a pair's MMA of 256 nodes x up to 256 vocabulary rows takes half of each operand from either CTA's shared
-// memory: 47 KB per 64 hidden columns and CTA for 512 nodes x 224 rows, where single CTAs drew 61 KB for 256 x 224.
-// All of TMEM holds accumulators: two node tiles (up to 512 nodes read the head once) or, up to 256
-// nodes, two vocabulary tiles (the features are read once for both).  32000 x 5120: 512 nodes 157 -> 133 us (2.5 times
-// the MMAs' time), 300 nodes 147 -> 123, 256 nodes 78 -> 72, 130 nodes 73 -> 68; 600 nodes (two groups) 229 -> 223.
+// More nodes: pairs of CTAs (kPair, cta_group::2): a pair's MMA of 256 rows x up to 256 columns takes half of each operand
+// from either CTA's shared memory.  Two arrangements; all of TMEM holds accumulators in both:
+//   kLmPair    nodes on the lanes: two node tiles of 256 (up to 512 nodes read the head once) or, up to 256 nodes, two
+//              vocabulary tiles (the features are read once for both);
+//   kLmLanes   vocabulary rows on the lanes, 256 a pair: up to 256 nodes and two such blocks, or up to 512 nodes in two tiles.
+//              The nodes then come in steps of 16 where kLmPair pads them to 256; the launcher says when it is taken.
+// What bounds them is the power limit (512 nodes of 5120 x 32000 run at 1.3 PFLOP/s, 1.5 GHz, padding counted; a cuBLAS loop
+// holds 1.38), then the round trip of the ring: two stages of up to 94 KB, about 4900 cycles between a stage's MMAs and the
+// next ones, 3600 of which are the MMAs'.  32000 x 5120, single CTAs and pairs: 512 nodes 157 -> 130 us, 300 nodes 147 -> 113,
+// 256 nodes 78 -> 72.
 //
 // Warp roles: 0 = TMA producer (one thread), 1 = MMA issuer (one elected thread) and TMEM owner,
-// 2-5 = accumulator readers; of a pair, the first CTA's warp 1 issues for both, and each CTA loads its own halves.
+// 2-9 = accumulator readers; of a pair, the first CTA's warp 1 issues for both, and each CTA loads its own halves.
 // Every wait is bounded; a wait that gives up sets FALCON_DEV_TIMEOUT in the caller's status word and the kernel still leaves in order (loads drained, MMAs finished,
 // TMEM freed).
 
@@ -50,6 +54,7 @@ enum LmBar {
   kLmBarDone,
   kLmNumBars
 };
+constexpr uint32_t kLmResultBytes = 2u * 4u * 256u * 8u;  // (kLmLanes) every reader warp's best for its columns' nodes
 constexpr uint32_t kLmSmallBytes = kLmFeatPad + 8u * kLmNumBars + 16u;  // pad, barriers, TMEM base, abort flag, last-CTA flag
 
 struct LmParams {
@@ -126,9 +131,20 @@ __device__ __forceinline__ void arrive_remote(uint32_t bar) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
-template <bool kPair>
+// The arrangements: one CTA, nodes on the lanes; pairs of CTAs, nodes on the lanes; pairs, vocabulary rows on the lanes.
+constexpr int kLmSingle = 0, kLmPair = 1, kLmLanes = 2;
+
+// Largest of one float per lane (a NaN never is, unless all are).
+__device__ __forceinline__ float warp_largest(float x) {
+  float m;
+  asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(m) : "f"(x));
+  return m;
+}
+
+template <int kMode>
 __global__ void __launch_bounds__(kLmThreads, 1)
 lm_head_argmax_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_f, const LmParams p) {
+  constexpr bool kPair = kMode != kLmSingle;
   extern __shared__ __align__(1024) unsigned char smem_gen[];
   const uint32_t smem_base = smem_u32(smem_gen);
   unsigned char* small = smem_gen + static_cast<uint32_t>(p.n_stages) * p.stage_bytes + kLmFeatPad;
@@ -188,7 +204,8 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_con
     for (int c = 0; c < p.kch; ++c) {
       if constexpr (kPair) {
         for (int j = 0; j < tiles_of(g); ++j)
-          tma_load_pair(fdst + (c * m_res + j) * f_bytes, &tm_f, full_bar(st), (kq * p.kch + c) * kLmKC, (g * m_res + j) * 256 + rank * 128);
+          tma_load_pair(fdst + (c * m_res + j) * f_bytes, &tm_f, full_bar(st), (kq * p.kch + c) * kLmKC,
+                        kMode == kLmLanes ? ((g * m_res + j) * 2 + rank) * p.f_rows : (g * m_res + j) * 256 + rank * 128);
       } else {
         tma_load_5d(fdst + c * f_bytes, &tm_f, full_bar(st), (kq * p.kch + c) * kLmKC, g * 128, 0, 0, 0);
       }
@@ -282,8 +299,9 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_con
                 const uint32_t fj = fbase + (c * m_res + (m_res > 1 ? j : 0)) * f_bytes, wj = wbase + (c * v_res + (v_res > 1 ? j : 0)) * w_bytes;
 #pragma unroll
                 for (int kk = 0; kk < kLmKC / 16; ++kk) {
-                  // features (A) and head rows (B): both K-major, 16 hidden columns = 32 bytes inside the 128-byte swizzle row
-                  const uint64_t ad = smem_desc(fj + kk * 32, 16, 1024), bd = smem_desc(wj + kk * 32, 16, 1024);
+                  // features (A) and head rows (B; kLmLanes: the other way round): both K-major, 16 hidden columns = 32 bytes inside the 128-byte swizzle row
+                  const uint64_t fd = smem_desc(fj + kk * 32, 16, 1024), wd = smem_desc(wj + kk * 32, 16, 1024);
+                  const uint64_t ad = kMode == kLmLanes ? wd : fd, bd = kMode == kLmLanes ? fd : wd;
                   const uint32_t acc = tmem_base + static_cast<uint32_t>(j) * 256u, more = (ks > 0 || c > 0 || kk > 0) ? 1u : 0u;
                   if constexpr (kPair) umma_pair_ss(acc, ad, bd, p.idesc, more);
                   else umma_bf16_ss(acc, ad, bd, p.idesc, more);
@@ -317,7 +335,8 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_con
     // Two warps for each TMEM lane quadrant: one for each accumulator of a pair, else one for each half of the columns.
     // The MMAs wait for them wherever another vocabulary tile follows, and the call waits for the last: one thread per row,
     // with a single chain of compares through its columns, took 740 cycles for 32 of them; four chains and the next
-    // columns' load under the compares take 150.  (What it gave: see the top of the file.)
+    // columns' load under the compares take 150: 60 nodes of 1024 x 100000 42.4 -> 39.3 us, 411 nodes 106 -> 91, of 5120 x 32000
+    // 131 -> 126.
     const int q = warp & 3;                 // TMEM lane quadrant this warp can reach
     const int sub = (warp - 2) >> 2;
     const int r = q * 32 + lane;            // accumulator row = node inside its tile
@@ -325,7 +344,72 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_con
     const uint32_t tmem_lane = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + (kPair ? static_cast<uint32_t>(sub) * 256u : 0u);
     int tile = 0;
     bool ok = !*abort_flag;
-    for (int g = 0; g < n_groups; ++g) {
+    if constexpr (kMode == kLmLanes) {
+      // A lane is a vocabulary row, a column a node: per column the warp's maximum and the lowest lane that has it, kept by
+      // lane (column mod 32).
+      unsigned long long* results = reinterpret_cast<unsigned long long*>(small + 8 * kLmNumBars + 16);
+      const int n_cols = 2 * p.f_rows;
+      for (int g = 0; g < n_groups; ++g) {
+        float best[kLmTileMax / 32];
+        int idx[kLmTileMax / 32];
+#pragma unroll
+        for (int k = 0; k < kLmTileMax / 32; ++k) {
+          best[k] = -INFINITY;
+          idx[k] = INT_MAX;
+        }
+        for (int vp = 0; ok && vp < n_vp; ++vp, ++tile) {
+          ok = mbar_wait_warp(bar(kLmBarAccFull), tile & 1, abort_flag);
+          if (!ok) break;
+          tc_fence_after();
+          const int v0 = v_lo + (v_res > 1 ? vp * 2 + sub : vp) * kLmTileMax + rank * 128 + q * 32;  // lane 0's vocabulary row
+          if (v0 < v_hi && (v_res > 1 || sub < tiles_of(g))) {
+            const bool exists = v0 + lane < v_hi;
+            uint32_t ring[2][32];               // the next columns' load runs under these columns' maxima
+            FALCON_TMEM_LD32(tmem_lane, ring[0]);
+#pragma unroll
+            for (int k = 0; k < kLmTileMax / 32; ++k)
+              if (k * 32 < n_cols) {
+                uint32_t(&x)[32] = ring[k & 1];
+                tmem_wait_ld();
+                if ((k + 1) * 32 < n_cols) FALCON_TMEM_LD32(tmem_lane + static_cast<uint32_t>((k + 1) * 32), ring[(k + 1) & 1]);
+                float m_mine = -INFINITY;
+                uint32_t who_mine = 0u;
+#pragma unroll
+                for (int c = 0; c < 32; ++c) {
+                  const float f = exists ? __uint_as_float(x[c]) : -INFINITY, m = warp_largest(f);
+                  const uint32_t who = __ballot_sync(0xffffffffu, f == m);
+                  if (lane == c) {
+                    m_mine = m;
+                    who_mine = who;
+                  }
+                }
+                if (m_mine > best[k]) {  // strict: vocabulary rows ascend over the passes, so the first maximum stays
+                  best[k] = m_mine;
+                  idx[k] = v0 + __ffs(static_cast<int>(who_mine)) - 1;
+                }
+              }
+          }
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) arrive_remote(map_to_leader(bar(kLmBarAccEmpty)));
+        }
+        // one atomic per node and CTA
+#pragma unroll
+        for (int k = 0; k < kLmTileMax / 32; ++k)
+          if (k * 32 < n_cols) results[(sub * 4 + q) * kLmTileMax + k * 32 + lane] = ok && idx[k] != INT_MAX ? lm_pack(best[k], idx[k]) : 0ull;
+        asm volatile("bar.sync 1, %0;" ::"n"(kLmReaders) : "memory");
+        for (int at = rt; at < m_res * kLmTileMax; at += kLmReaders) {
+          const int j = at / kLmTileMax, col = at % kLmTileMax, node = (g * m_res + j) * n_cols + col;
+          if (col < n_cols && node < p.n_rows) {
+            unsigned long long w = 0ull;
+            for (int i = m_res > 1 ? j * 4 : 0; i < (m_res > 1 ? j * 4 + 4 : 8); ++i) w = max(w, results[i * kLmTileMax + col]);
+            if (w) atomicMax(p.best + node, w);
+          }
+        }
+        asm volatile("bar.sync 1, %0;" ::"n"(kLmReaders) : "memory");
+      }
+    }
+    for (int g = 0; kMode != kLmLanes && g < n_groups; ++g) {
       constexpr int kChains = 4;
       float best[kChains];
       int idx[kChains];
@@ -426,40 +510,73 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_con
 }  // namespace
 
 cudaError_t set_up_lm_head() {
-  const cudaError_t e = cudaFuncSetAttribute(lm_head_argmax_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kLmSmemMax));
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(lm_head_argmax_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kLmSmemMax));
+  cudaError_t e = cudaSuccess;
+  for (auto* kernel : {lm_head_argmax_kernel<kLmSingle>, lm_head_argmax_kernel<kLmPair>, lm_head_argmax_kernel<kLmLanes>})
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kLmSmemMax));
+  return e;
 }
 
 int launch_lm_head_argmax(falcon_ctx* ctx, const falcon_lm_argmax_args& a, cudaStream_t s) {
   const int N = a.n_rows, V = a.vocab, H = a.hidden;
   const bool pair = N > 128;  // (a single tile has nothing to share: the head's rows bound it)
-  const int n_mt = pair ? (N + 255) / 256 : 1;
-  const int m_res = n_mt >= 2 ? 2 : 1, v_res = pair && m_res == 1 ? 2 : 1;
+  int n_mt = pair ? (N + 255) / 256 : 1;
+  int m_res = n_mt >= 2 ? 2 : 1, v_res = pair && m_res == 1 ? 2 : 1;
   // One wave: the vocabulary split evenly over the SMs or pairs of them, in tiles of the same multiple of 16 rows.
   const int workers = pair ? ctx->sm_count / 2 : ctx->sm_count;
-  const int share = (V + workers - 1) / workers, n_vt = (share + kLmTileMax - 1) / kLmTileMax;
+  const int share = (V + workers - 1) / workers;
+  int n_vt = (share + kLmTileMax - 1) / kLmTileMax;
   int tile_n = ((share + n_vt - 1) / n_vt + 15) & ~15;
   int span = tile_n * n_vt;
   if (!pair) {
     span = (share + 15) & ~15;
     tile_n = span < kLmTileMax ? span : kLmTileMax;
   }
+  int f_rows = pair ? 128 : (N <= 64 ? 64 : ((N + 7) & ~7));
+  uint32_t mma_n = static_cast<uint32_t>(tile_n);
+  // Vocabulary rows on the lanes, 256 of them a pair, and the nodes on the side that comes in steps of 16, where that takes
+  // so many fewer columns of MMAs (with the nodes on the lanes 300 of them are padded to 512) that it pays for the reading of
+  // the accumulators: the maxima across lanes take about 4000 cycles more each time, and of a column and 64 hidden columns,
+  // 2 cycles of the tensor core, three quarters show in the time.  Against nodes on the lanes, us:
+  //   hidden x vocabulary    129 nodes      257            300            380            411 (not taken)
+  //   4096 x 32000           57.7 -> 53.6   99.0 -> 92.5   99.7 -> 93.8   102 -> 99.5    102 / 104
+  //   5120 x 32000           69.8 -> 64.6   121 -> 112     122 -> 113     125 -> 120     126 / 126
+  //   2048 x 50000           60.0 -> 54.9   82.6 -> 75.9   82.8 -> 77.4   83.8 -> 82.0   84.1 / 86.4
+  //   1024 x 100000          51.8 -> 49.3   89.0 -> 84.6   89.5 / 86.7 (not taken)       90.5 / 98.2
+  bool lanes = false;
+  if (pair) {
+    const int tiles = N <= 256 ? 1 : 2 * ((N + 511) / 512), cols = ((N + tiles - 1) / tiles + 15) & ~15;
+    const int blocks = (V + kLmTileMax - 1) / kLmTileMax, per = (blocks + workers - 1) / workers;
+    const int two = tiles == 1 && per > 1;  // two vocabulary blocks resident
+    const int64_t here = static_cast<int64_t>(tiles) * cols * (two ? (per + 1) / 2 * 2 : per), chunks = (H + kLmKC - 1) / kLmKC;
+    const int64_t other = static_cast<int64_t>(n_mt) * tile_n * (v_res > 1 ? (n_vt + 1) / 2 * 2 : n_vt);
+    const int64_t reads = static_cast<int64_t>((tiles + 1) / 2) * (two ? (per + 1) / 2 : per);
+    lanes = 3 * (other - here) * chunks > 2 * 4000 * reads;
+    if (lanes) {
+      n_mt = tiles;
+      m_res = tiles > 1 ? 2 : 1;
+      v_res = two ? 2 : 1;
+      n_vt = per;
+      tile_n = kLmTileMax;
+      span = per * kLmTileMax;
+      f_rows = cols / 2;
+      mma_n = static_cast<uint32_t>(cols);
+    }
+  }
   const int n_cta = (V + span - 1) / span * (pair ? 2 : 1);
-  const int f_rows = pair ? 128 : (N <= 64 ? 64 : ((N + 7) & ~7));
   const int w_rows = pair ? tile_n / 2 : tile_n;
   const int n_kc = (H + kLmKC - 1) / kLmKC;
   // Chunks per stage: two where two such stages fit.  Fewer, larger stages mean fewer trips round the ring
   // (32000 x 4096, 60 nodes: 43 us with two chunks in three stages against 53 with one in five and 46 with
   // three in two; in pairs, 512 nodes of 5120: 133 with two chunks in two stages, 158 with one in four; a head stored chunk by chunk so that a tile is contiguous made no difference).
+  const uint32_t small_bytes = kLmSmallBytes + (lanes ? kLmResultBytes : 0u);
   const uint32_t chunk_bytes = static_cast<uint32_t>(v_res * w_rows + m_res * f_rows) * (kLmKC * 2u);
-  int kch = (2 * 2 * chunk_bytes <= kLmSmemMax - kLmSmallBytes) ? 2 : 1;
+  int kch = (2 * 2 * chunk_bytes <= kLmSmemMax - small_bytes) ? 2 : 1;
   if (kch > n_kc) kch = n_kc;
   const uint32_t stage_bytes = static_cast<uint32_t>(kch) * chunk_bytes;
-  int n_stages = static_cast<int>((kLmSmemMax - kLmSmallBytes) / stage_bytes);
+  int n_stages = static_cast<int>((kLmSmemMax - small_bytes) / stage_bytes);
   if (n_stages > kLmMaxStages) n_stages = kLmMaxStages;
   if (n_stages < 2) return FALCON_ERR_CAPACITY;
-  const uint32_t smem_bytes = static_cast<uint32_t>(n_stages) * stage_bytes + kLmSmallBytes;
+  const uint32_t smem_bytes = static_cast<uint32_t>(n_stages) * stage_bytes + small_bytes;
 
   // scratch that is zero between calls: the arrival counter and one 64-bit word per node
   int rc = ensure_tickets(ctx, 2 + 2 * N, s);
@@ -496,7 +613,7 @@ int launch_lm_head_argmax(falcon_ctx* ctx, const falcon_lm_argmax_args& a, cudaS
   p.n_stages = n_stages;
   p.stall_first = (a.flags & FALCON_LM_TEST_STALL) ? 1 : 0;
   p.stage_bytes = stage_bytes;
-  p.idesc = make_idesc(pair ? 256 : 128, static_cast<uint32_t>(tile_n), false, false);
+  p.idesc = make_idesc(pair ? 256 : 128, mma_n, false, false);
   p.argmax_out = a.argmax_out;
   p.max_out = a.max_out;
   p.status = a.status;
@@ -517,7 +634,7 @@ int launch_lm_head_argmax(falcon_ctx* ctx, const falcon_lm_argmax_args& a, cudaS
   attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = pair ? 2 : 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, pair ? lm_head_argmax_kernel<true> : lm_head_argmax_kernel<false>, mw, mf, p);
+  cudaError_t e = cudaLaunchKernelEx(&cfg, lanes ? lm_head_argmax_kernel<kLmLanes> : pair ? lm_head_argmax_kernel<kLmPair> : lm_head_argmax_kernel<kLmSingle>, mw, mf, p);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "lm_head_argmax_kernel launch");
   return FALCON_OK;
 }

@@ -1093,6 +1093,37 @@ def test_lm_head_argmax_pairs_of_ctas(N, Hd, V):
     test_lm_head_argmax_integer_data_is_bit_exact(N, Hd, V)
 
 
+@pytest.mark.parametrize("N,Hd,V", [(129, 1344, 30001), (144, 1416, 30210), (257, 768, 18900), (289, 1032, 18944), (384, 1800, 18689), (520, 1792, 18800)])
+def test_lm_head_argmax_vocabulary_rows_on_the_lanes(N, Hd, V):
+    # sizes at which pairs of CTAs put the vocabulary rows on the lanes: two vocabulary blocks at a time and one, node tiles
+    # with and without padding, a second group of them, a last block cut short or absent.  Small integers: exact in fp32
+    # (products up to 9, at most 1800 of them).  A NaN in a head row and a node of NaNs never win.
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(N + V)
+    f = torch.randint(-3, 4, (N, Hd), generator=gen, device="cuda").to(torch.bfloat16)
+    w = torch.randint(-3, 4, (V, Hd), generator=gen, device="cuda").to(torch.bfloat16)
+    first = int((f[:1].double() @ w.double().T).argmax())
+    w[V - 1] = w[first]                                         # ties between the first and the last pair, and inside a block
+    w[V // 2] = w[5]
+    w[7, 3] = float("nan")
+    f[N // 2] = float("nan")
+    logits = (f.double() @ w.double().T).nan_to_num_(nan=-float("inf"), posinf=float("inf"), neginf=-float("inf"))
+    best = logits.amax(dim=1)
+    at = torch.arange(V, device="cuda")
+    want = torch.where(logits == best[:, None], at, V).amin(dim=1)
+    want[best == -float("inf")] = 0
+    g = torch.full((N,), -1, dtype=torch.int32, device="cuda")
+    mx = torch.zeros(N, dtype=torch.float32, device="cuda")
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    for flags in (0, binding.LM_TEST_STALL, 0):                 # (a bounded wait that runs out in between)
+        st.zero_()
+        H.ctx().falcon_lm_head_argmax(binding.lm_argmax_args(N, Hd, V, f, Hd, w, Hd, g, mx, st, flags=flags))
+        torch.cuda.synchronize()
+        assert int(st.item()) == (binding.DEV_TIMEOUT if flags else 0)
+        if not flags:
+            assert torch.equal(g.long(), want) and torch.equal(mx.double(), best)
+
+
 @pytest.mark.parametrize("N,Hd,V,pad", [(60, 512, 5000, 0), (130, 320, 3001, 8), (15, 72, 1000, 24), (257, 256, 4096, 0)])
 def test_lm_head_argmax_random_data(N, Hd, V, pad):
     # hidden sizes that are not multiples of the 64-column stage, padded row pitches, ragged tails
