@@ -535,13 +535,12 @@ int launch_lm_head_argmax(falcon_ctx* ctx, const falcon_lm_argmax_args& a, cudaS
   uint32_t mma_n = static_cast<uint32_t>(tile_n);
   // Vocabulary rows on the lanes, 256 of them a pair, and the nodes on the side that comes in steps of 16, where that takes
   // so many fewer columns of MMAs (with the nodes on the lanes 300 of them are padded to 512) that it pays for the reading of
-  // the accumulators: the maxima across lanes take about 4000 cycles more each time, and of a column and 64 hidden columns,
-  // 2 cycles of the tensor core, three quarters show in the time.  Against nodes on the lanes, us:
-  //   hidden x vocabulary    129 nodes      257            300            380            411 (not taken)
-  //   4096 x 32000           57.7 -> 53.6   99.0 -> 92.5   99.7 -> 93.8   102 -> 99.5    102 / 104
-  //   5120 x 32000           69.8 -> 64.6   121 -> 112     122 -> 113     125 -> 120     126 / 126
-  //   2048 x 50000           60.0 -> 54.9   82.6 -> 75.9   82.8 -> 77.4   83.8 -> 82.0   84.1 / 86.4
-  //   1024 x 100000          51.8 -> 49.3   89.0 -> 84.6   89.5 / 86.7 (not taken)       90.5 / 98.2
+  // the accumulators: the maxima across lanes take up to 4000 cycles more each time, and a column and 64 hidden columns are
+  // 2 cycles of the tensor core.  Against nodes on the lanes, us in bursts (and, under the power limit, in a loop):
+  //   4096 x 32000    129 nodes 57.7 -> 53.6, 257 99.0 -> 92.5, 308 118 -> 105 (116 -> 102)
+  //   5120 x 32000    129 nodes 69.8 -> 64.6, 314 146 -> 129 (144 -> 126), 411 126.4 -> 122.1 (145 -> 140)
+  //   2048 x 50000    129 nodes 60.0 -> 54.9, 300 82.8 -> 77.4, 477 (100 / 103: not taken)
+  //   1024 x 100000   129 nodes 51.8 -> 49.3, 257 89.0 -> 84.6, 425 (99 / 106: not taken)
   bool lanes = false;
   if (pair) {
     const int tiles = N <= 256 ? 1 : 2 * ((N + 511) / 512), cols = ((N + tiles - 1) / tiles + 15) & ~15;
@@ -550,7 +549,7 @@ int launch_lm_head_argmax(falcon_ctx* ctx, const falcon_lm_argmax_args& a, cudaS
     const int64_t here = static_cast<int64_t>(tiles) * cols * (two ? (per + 1) / 2 * 2 : per), chunks = (H + kLmKC - 1) / kLmKC;
     const int64_t other = static_cast<int64_t>(n_mt) * tile_n * (v_res > 1 ? (n_vt + 1) / 2 * 2 : n_vt);
     const int64_t reads = static_cast<int64_t>((tiles + 1) / 2) * (two ? (per + 1) / 2 : per);
-    lanes = 3 * (other - here) * chunks > 2 * 4000 * reads;
+    lanes = 2 * (other - here) * chunks > 4000 * reads;
     if (lanes) {
       n_mt = tiles;
       m_res = tiles > 1 ? 2 : 1;
