@@ -604,9 +604,13 @@ int launch_tree_topm(falcon_ctx* ctx, const falcon_topm_args& a, cudaStream_t s)
   p.top_val = a.top_val;
   p.top_idx = a.top_idx;
 
-  // Rows in registers while the whole grid is resident at once (six CTAs per SM with 8 entries per
-  // lane, four with 16, three with 32): the shortest chain.  As many CTAs per row as leave a lane 8 entries.  Else
-  // streamed, three CTAs per SM: a second wave of the register kernel starts its loads only when a
+  // Rows in registers while the whole grid is resident at once (six CTAs per SM with 8 entries per lane, four with 16,
+  // three with 32): the shortest chain.  A cluster costs more than it shares out wherever one CTA's registers hold the row:
+  // 1.2 us at once, and more with every cluster the GPU has to place.  So as few CTAs per row as the registers allow,
+  // four while there are at most 96 of them, eight below 64 (us with 1 / 2 / 4 / 8: 16 rows of 3000 2.8 / 3.5 / 3.7 /
+  // 11.7, 48 of 8000 3.3 / 4.2 / 4.3 / 4.8, 4 of 16000 - / 3.9 / 3.6 / 3.5, 16 of 16000 - / 4.0 / 3.7 / 4.1, 32 of
+  // 16000 - / 4.1 / 4.2 / 4.4, 4 of 32000 - / - / 3.9 / 3.7, 48 of 32000 - / - / 4.9 / 5.6).
+  // Else streamed, three CTAs per SM: a second wave of the register kernel starts its loads only when a
   // first one has gone through its barriers.
   int ctas = 1, per_lane = 0, chunk = 0;
   auto split = [&](int c) {
@@ -614,18 +618,30 @@ int launch_tree_topm(falcon_ctx* ctx, const falcon_topm_args& a, cudaStream_t s)
     chunk = ((a.vocab + c - 1) / c + 3) & ~3;
     per_lane = (chunk + kTopmThreads - 1) / kTopmThreads;
   };
-  auto fits = [&]() { return static_cast<int64_t>(N) * ctas <= (per_lane <= 8 ? 6 : per_lane <= 16 ? 4 : 3) * ctx->sm_count; };
+  // (clusters: 19/20, 14/15 and 13/15 of that for two, four and eight CTAs, since not every SM that has room has it beside the
+  // others: 103 rows of 20000 in clusters of four 5.6 us, 105 7.8, of 50257 streamed 9.8 and 13.4; in clusters of eight 48
+  // rows of 50257 5.8, 49 8.1)
+  auto room = [&](int64_t n_ctas, int of, int per_sm) { return n_ctas * 60 <= (of == 1 ? 60 : of == 2 ? 57 : of == 4 ? 56 : 52) * per_sm * ctx->sm_count; };
+  auto fits = [&]() { return room(static_cast<int64_t>(N) * ctas, ctas, per_lane <= 8 ? 6 : per_lane <= 16 ? 4 : 3); };
   int c = 1;
-  while (c < kTopmMaxCluster && a.vocab > c * kTopmThreads * 8) c *= 2;
-  bool in_regs = false;
-  for (; c >= 1 && !in_regs; c /= 2) {
-    split(c);
-    if (per_lane > kTopmRowsMax) break;
-    in_regs = fits();
-  }
+  while (c < kTopmMaxCluster && a.vocab > c * kTopmThreads * kTopmRowsMax) c *= 2;
+  if (c > 1 && c < 4 && N * 4 <= 96) c = 4;
+  if (c > 1 && c < 8 && N * 8 < 64) c = 8;
+  // (eight again where four would put two CTAs with most of their registers full on an SM: 60 rows of 32000 5.3 us both alone,
+  // 0.2 less behind an attention launch)
+  if (c == 4 && a.vocab > 4 * 24 * kTopmThreads && N * 4 > 4 * ctx->sm_count / 3 && room(static_cast<int64_t>(N) * 8, 8, 4)) c = 8;
+  // (two stages of one CTA against two CTAs' registers: 48 rows of 16000 4.6 and 4.4 us, 64 of 12000 4.6 and 5.0, 120 5.2 and 6.0)
+  const bool short_stream = a.vocab > kStreamStage && a.vocab <= 2 * kStreamStage && N >= 56;
+  split(c);
+  const bool in_regs = !short_stream && per_lane <= kTopmRowsMax && fits();
   if (!in_regs) {
+    // CTAs of a cluster where the rows alone leave SMs idle (us with 1 / 2 / 4 CTAs): 64 rows of 50257 10.2 / 9.5 / 8.9, 100 of
+    // 40000 9.2 / 10.0 / 9.7, 120 of 50257 10.9 / 12.0 / 16.0, 120 of 128256 19.0 / 17.5 / 23.0.  More rows than SMs: two, which
+    // even out better where the SMs become free one by one (158 of 32000 alone 9.3 and 10.3 or, from L2, 8.0 both; behind an
+    // attention launch 0.8 less with two).
     c = 1;
-    while (c < kTopmMaxCluster && static_cast<int64_t>(N) * 2 * c <= 3 * ctx->sm_count && a.vocab >= 2 * c * kStreamStage) c *= 2;
+    while (c < kTopmMaxCluster && room(static_cast<int64_t>(N) * 2 * c, 2 * c, 3) && a.vocab >= 2 * c * kStreamStage) c *= 2;
+    if ((c == 2 && N <= ctx->sm_count && a.vocab < 14 * kStreamStage) || (c > 2 && a.vocab < 6 * kStreamStage && 3 * N * c > 7 * ctx->sm_count)) c = 1;
     split(c);
   }
   p.chunk_len = chunk;

@@ -788,6 +788,22 @@ def test_topm_bit_exact(N, V, stride, m):
         np.testing.assert_array_equal(gv, rv)
 
 
+@pytest.mark.parametrize("N,V,m", [(1, 8192, 32), (444, 8192, 20), (445, 8192, 20), (7, 8193, 20), (25, 8193, 8), (24, 16384, 8), (55, 16384, 32),
+                                   (56, 16385, 5), (56, 16384, 32), (1, 16384, 1), (103, 20001, 20), (104, 20001, 20), (8, 32768, 20), (48, 40003, 8),
+                                   (49, 40003, 8), (86, 40003, 8), (104, 49152, 3), (104, 114687, 9), (104, 114688, 9), (210, 114690, 2), (211, 114690, 2)])
+def test_topm_on_both_sides_of_every_line_of_the_dispatch(N, V, m):
+    """How many CTAs share a row, and whether it is held in registers or streamed: one CTA's registers, stages of one CTA,
+    clusters as far as they have room.  Values repeat, so that ties cross the borders of lanes, warps and CTAs."""
+    rng = np.random.default_rng(N * V + m)
+    x = (rng.integers(-2000, 2000, size=(N, V)) / 16).astype(np.float32)
+    x[0, V // 2:] = x[0].max() + 1                              # a row whose best are half of its entries
+    x[N - 1, -m:] = x[N - 1].max()                              # and one whose best are the last
+    rv, ri = oracle.topm(x, m, vocab=V)
+    gv, gi, _ = H.run_topm(x, m, vocab=V)
+    np.testing.assert_array_equal(gi, ri)
+    np.testing.assert_array_equal(gv, rv)
+
+
 @pytest.mark.parametrize("N,V,stride,m", [(160, 8191, 8191, 20), (150, 24577, 24580, 8), (450, 8200, 8201, 32), (120, 66001, 66001, 1),
                                           (2, 70001, 70003, 32), (3, 16385, 16386, 7)])
 @pytest.mark.parametrize("kind", ["normal", "few values", "mostly -inf"])
