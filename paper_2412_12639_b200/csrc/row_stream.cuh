@@ -21,6 +21,25 @@ constexpr int kStreamLane = 32;                             // entries a lane ta
 constexpr int kStreamStage = kStreamThreads * kStreamLane;  // 8192 entries, 32 KB
 constexpr int kStreamStages = 2;
 constexpr uint32_t kStreamBytes = kStreamStages * kStreamStage * 4;
+constexpr uint32_t kStreamBytesPair = 78u * 1024u;      // more than a third of an SM's shared memory: two CTAs per SM
+constexpr uint32_t kStreamBytesAlone = 116u * 1024u;    // more than half of it: one
+constexpr uint32_t kStreamBytesMax = kStreamBytesAlone; // (the attribute the kernels are given once)
+
+// Dynamic shared memory of a launch of n CTAs in clusters of `of` that take `len` entries each: so much that no SM takes more
+// of them than an even share.  Behind a kernel whose CTAs end at different times the SMs that become free first would be given
+// three each and the last ones none (us, attention over one sequence and then acceptance: 121 rows of 128256 39.5 and 33.7, 136
+// of 64000 33.8 and 30.8, 136 of 32000 31.1 and 29.6; top-m over 121 rows of 32000 32.9 and 30.8).  With all SMs free at once
+// it is the same either way.  Not for more than one and a half rows' length of work on some SMs and half of it on others (170
+// rows of 128256 from L2: 13 us with three per SM allowed, 18 with two), nor where clusters might not all find their places
+// (sample, 140 rows of 128256 in clusters of two 18.8 and 20.8; top-m behind attention, 60 rows of 64000 in clusters of four
+// 7 % slower).
+inline uint32_t stream_bytes(int64_t n_ctas, int of, int len, int sm_count) {
+  if (of > 2) return kStreamBytes;
+  const int64_t slots = of == 2 ? sm_count * 9 / 10 : sm_count;
+  if (n_ctas <= slots) return kStreamBytesAlone;
+  if (n_ctas <= 2 * slots && (2 * n_ctas > 3 * sm_count || len <= 10 * kStreamStage)) return kStreamBytesPair;
+  return kStreamBytes;
+}
 
 struct StreamBars {
   uint64_t full[kStreamStages], empty[kStreamStages];

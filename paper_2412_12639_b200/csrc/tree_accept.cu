@@ -558,10 +558,10 @@ AcceptParams accept_params(const falcon_accept_args& a, int chunks, int chunk_le
 cudaError_t set_up_accept() {
   cudaError_t e = prefer_shared(tree_accept_kernel<false>);
   if (e == cudaSuccess) e = prefer_shared(tree_accept_kernel<true>);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(tree_accept_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kStreamBytes));
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(tree_accept_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kStreamBytesMax));
   if (e == cudaSuccess) e = prefer_shared(tree_search_kernel);
   if (e == cudaSuccess) e = prefer_shared(tree_sample_kernel);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(tree_sample_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kStreamBytes));
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(tree_sample_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kStreamBytesMax));
   return e;
 }
 
@@ -581,7 +581,7 @@ int launch_tree_accept(falcon_ctx* ctx, const falcon_accept_args& a, cudaStream_
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(chunks, N);
   cfg.blockDim = dim3(kAcceptThreads + (streamed ? 32 : 0));
-  cfg.dynamicSmemBytes = streamed ? kStreamBytes : 0;
+  cfg.dynamicSmemBytes = streamed ? stream_bytes(static_cast<int64_t>(chunks) * N, 1, chunk_len, ctx->sm_count) : 0;
   cfg.stream = s;
   cudaLaunchAttribute attr;
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -613,7 +613,7 @@ int launch_tree_sample(falcon_ctx* ctx, const falcon_accept_args& a, cudaStream_
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(ctas, N);
   cfg.blockDim = dim3(kStreamThreads + 32);
-  cfg.dynamicSmemBytes = kStreamBytes;
+  cfg.dynamicSmemBytes = stream_bytes(static_cast<int64_t>(ctas) * N, ctas, chunk_len, ctx->sm_count);
   cfg.stream = s;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -693,8 +693,8 @@ int static_scratch(int device, StaticSlot* out) {
     int sms = 0;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
     if (e != cudaSuccess || sms < 1) return FALCON_ERR_CUDA;
-    // (there may be no context that has raised the limit on this device)
-    e = cudaFuncSetAttribute(tree_accept_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kStreamBytes));
+    // (there may be no context that has raised the limit on this device; the same value as there, which this must not lower)
+    e = cudaFuncSetAttribute(tree_accept_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kStreamBytesMax));
     if (e != cudaSuccess) return FALCON_ERR_CUDA;
     slot.sm_count = sms;
     slot.ptr = ptr;
@@ -738,7 +738,7 @@ extern "C" int falcon_tree_accept_static(const falcon_accept_args* a, void* stre
   const AcceptParams p = accept_params(*a, chunks, chunk_len, base, reinterpret_cast<int*>(base + kStaticPartBytes));
   dim3 grid(chunks, N);
   if (streamed) {
-    tree_accept_kernel<true><<<grid, kAcceptThreads + 32, kStreamBytes, s>>>(p);
+    tree_accept_kernel<true><<<grid, kAcceptThreads + 32, stream_bytes(static_cast<int64_t>(chunks) * N, 1, chunk_len, slot.sm_count), s>>>(p);
   } else {
     tree_accept_kernel<false><<<grid, kAcceptThreads, 0, s>>>(p);
   }

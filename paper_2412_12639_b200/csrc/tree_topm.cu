@@ -589,7 +589,7 @@ cudaError_t set_up_topm() {
   if (e == cudaSuccess) e = prefer_shared(tree_topm_kernel<16>);
   if (e == cudaSuccess) e = prefer_shared(tree_topm_kernel<kTopmRowsMax>);
   if (e == cudaSuccess) e = prefer_shared(tree_topm_stream_kernel);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(tree_topm_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kStreamBytes));
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(tree_topm_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kStreamBytesMax));
   return e;
 }
 
@@ -668,7 +668,7 @@ int launch_tree_topm(falcon_ctx* ctx, const falcon_topm_args& a, cudaStream_t s)
   } else {
     p.steps = (chunk + kTopmThreads * kStreamLane - 1) / (kTopmThreads * kStreamLane);
     cfg.blockDim = dim3(kStreamThreads + 32);
-    cfg.dynamicSmemBytes = kStreamBytes;
+    cfg.dynamicSmemBytes = stream_bytes(static_cast<int64_t>(N) * ctas, ctas, chunk, ctx->sm_count);
     e = cudaLaunchKernelEx(&cfg, tree_topm_stream_kernel, p);
   }
   if (e != cudaSuccess) return cuda_fail(ctx, e, "tree_topm_kernel launch");

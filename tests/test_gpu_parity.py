@@ -911,6 +911,31 @@ def test_sample_equal_logits_are_bit_exact(V, stride):
     np.testing.assert_array_equal(g, np.floor(u.astype(np.float64) * V).astype(np.int32))
 
 
+@pytest.mark.parametrize("N,V", [(133, 12289), (134, 12289), (148, 4097), (149, 4097), (149, 90112), (222, 90112), (223, 90112), (266, 12289),
+                                 (267, 12289), (296, 8200), (297, 8200), (444, 8200), (445, 8200)])
+def test_streamed_rows_on_both_sides_of_every_share_of_an_sm(N, V):
+    """Greedy and drawn tokens where the number of CTAs passes one, one and a half, two and three per SM, alone and in
+    clusters: how much shared memory a CTA is given, and how many share a row.  Greedy rows repeat values, drawn rows
+    are equal logits, so that both are exact."""
+    rng = np.random.default_rng(N + V)
+    sizes = [N // 4, N // 4, N // 4, N - 3 * (N // 4)]
+    tb = H.make_trees(sizes, [1, 0, 3, 2], rng, vocab=V)
+    dt = H.DevTrees(tb)
+    lg = (rng.integers(-2000, 2000, size=(N, V)) / 16).astype(np.float32)
+    u = (rng.integers(0, 1024, N) / 1024.0).astype(np.float32)
+    for temperature in (0.0, 1.3):
+        if temperature:
+            lg[:] = 1.25
+            want = np.floor(u.astype(np.float64) * V).astype(np.int32)
+            got = H.run_accept(dt, lg, temperature=temperature, uniforms=u)
+        else:
+            want = oracle.argmax(lg)
+            got = H.run_accept(dt, lg)
+        np.testing.assert_array_equal(got[0], want)
+        for x, y in zip(got[1:], oracle.tree_accept(tb.node_off, tb.parent, tb.token, want)):
+            np.testing.assert_array_equal(x, y)
+
+
 def test_sample_edge_sizes_and_the_last_representable_uniform():
     rng = np.random.default_rng(41)
     for sizes, V in (([1], 1), ([1], 5), ([2, 1, 3], 4096), ([5], 4097), ([3], 12289)):
