@@ -25,6 +25,13 @@ constexpr uint32_t kStreamBytesPair = 78u * 1024u;      // more than a third of 
 constexpr uint32_t kStreamBytesAlone = 116u * 1024u;    // more than half of it: one
 constexpr uint32_t kStreamBytesMax = kStreamBytesAlone; // (the attribute the kernels are given once)
 
+// Whether the GPU places n CTAs in clusters of `of` at once where an SM has room for per_sm of them: 19/20, 14/15 and 13/15 of the
+// places for two, four and eight CTAs, since not every SM that has room has it beside the others.  (us, top-m: 103 rows of 20000
+// in clusters of four 5.6, 105 7.8, of 50257 streamed 9.8 and 13.4; in clusters of eight 48 rows of 50257 5.8, 49 8.1.)
+inline bool cluster_room(int64_t n_ctas, int of, int per_sm, int sm_count) {
+  return n_ctas * 60 <= static_cast<int64_t>(of == 1 ? 60 : of == 2 ? 57 : of == 4 ? 56 : 52) * per_sm * sm_count;
+}
+
 // Dynamic shared memory of a launch of n CTAs in clusters of `of` that take `len` entries each: so much that no SM takes more
 // of them than an even share.  Behind a kernel whose CTAs end at different times the SMs that become free first would be given
 // three each and the last ones none (us, attention over one sequence and then acceptance: 121 rows of 128256 39.5 and 33.7, 136

@@ -618,10 +618,7 @@ int launch_tree_topm(falcon_ctx* ctx, const falcon_topm_args& a, cudaStream_t s)
     chunk = ((a.vocab + c - 1) / c + 3) & ~3;
     per_lane = (chunk + kTopmThreads - 1) / kTopmThreads;
   };
-  // (clusters: 19/20, 14/15 and 13/15 of that for two, four and eight CTAs, since not every SM that has room has it beside the
-  // others: 103 rows of 20000 in clusters of four 5.6 us, 105 7.8, of 50257 streamed 9.8 and 13.4; in clusters of eight 48
-  // rows of 50257 5.8, 49 8.1)
-  auto room = [&](int64_t n_ctas, int of, int per_sm) { return n_ctas * 60 <= (of == 1 ? 60 : of == 2 ? 57 : of == 4 ? 56 : 52) * per_sm * ctx->sm_count; };
+  auto room = [&](int64_t n_ctas, int of, int per_sm) { return cluster_room(n_ctas, of, per_sm, ctx->sm_count); };
   auto fits = [&]() { return room(static_cast<int64_t>(N) * ctas, ctas, per_lane <= 8 ? 6 : per_lane <= 16 ? 4 : 3); };
   int c = 1;
   while (c < kTopmMaxCluster && a.vocab > c * kTopmThreads * kTopmRowsMax) c *= 2;

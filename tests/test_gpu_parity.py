@@ -912,7 +912,9 @@ def test_sample_equal_logits_are_bit_exact(V, stride):
 
 
 @pytest.mark.parametrize("N,V", [(133, 12289), (134, 12289), (148, 4097), (149, 4097), (149, 90112), (222, 90112), (223, 90112), (266, 12289),
-                                 (267, 12289), (296, 8200), (297, 8200), (444, 8200), (445, 8200)])
+                                 (267, 12289), (296, 8200), (297, 8200), (444, 8200), (445, 8200),
+                                 (4, 8192), (4, 8193), (6, 16388), (48, 32772), (49, 32772), (103, 16388), (104, 16388), (129, 16384), (130, 16384),
+                                 (130, 49152), (210, 16384), (211, 16384)])
 def test_streamed_rows_on_both_sides_of_every_share_of_an_sm(N, V):
     """Greedy and drawn tokens where the number of CTAs passes one, one and a half, two and three per SM, alone and in
     clusters: how much shared memory a CTA is given, and how many share a row.  Greedy rows repeat values, drawn rows
