@@ -508,15 +508,25 @@ __global__ void __launch_bounds__(kStreamThreads + 32, 3) tree_sample_kernel(con
 constexpr int kAcceptMaxChunks = 8;  // vocabulary chunks per row at most (the static scratch is sized by it)
 
 // How a launch splits the vocabulary, and whether its rows are streamed.  Shared by the two entry points so that
-// they cannot drift apart.  Streamed: up to about one and a half CTAs per SM in all, chunks of no less than most of a stage, so that a
-// large batch has a CTA per row (measured, us, with 1 / 2 / 4 / 8 chunks of 32000: 20 rows 5.3 / 4.6 / 4.4 / 4.7, 60 rows 6.6 / 5.9 /
-// 6.3 / 8.1, 100 rows 7.2 / 6.9 / 6.8 / 9.6, 300 rows 11.2 / 12.1 / 13.6 / 20.6; 16 rows of 128000: 11.8 / 8.3 / 6.7 / 6.1).
-// Short rows fit the registers of one pass, and the ring's set-up would only add to it (15 rows of 1000: 4.1 against 4.4).
+// they cannot drift apart.  Chunks are doubled (3 chunks of 32000 fill their last stage by a third, 6.6 us where 2 take 5.9) as
+// long as they stay worth a CTA, which depends on how many CTAs an SM then has.  Streamed (us with 1 / 2 / 4 / 8 chunks):
+//   two thirds of one per SM, 0.6 of a stage: 16 rows of 12000 5.6 / 5.2 / 5.2 / 5.1, of 20000 6.1 / 5.8 / 5.5 / 5.4;
+//                                 behind attention over a batch 74 of 12000 30.0 / 30.8, 37 of 20000 - / 29.9 / 30.4
+//   up to 1.5, three quarters:    50 of 12000 5.4 / 5.0 / 5.6 / 6.2, 100 of 12000 5.4 / 5.6, 50 of 20000 5.7 / 5.4 / 5.7 / 6.2, 50 of 64000 7.3 / 6.2 / 6.3 / 6.5
+//   up to 2, one and three quarters: behind an attention launch 120 of 64000 21.5 / 20.4, 145 of 64000 22.2 / 21.0, of 128256 31.7 / 30.3,
+//                                 of 32000 19.4 / 19.1, of 20000 18.6 / 18.9; 65 of 128256 25.3 / 21.7 / 20.5
+// Short rows fit the registers of one pass, and the ring's set-up would only add to it (15 rows of 1000: 4.1 against 4.4); a
+// chunk of them is 2048 entries, or 1000 while there are no more CTAs than SMs (30 rows of 4000 5.3 / 5.1 / 4.9; 100 5.4 / 5.4, behind
+// attention 17.9 / 18.4).
 bool accept_plan(int sm_count, int n_nodes, int vocab, int* chunks_out, int* chunk_len_out) {
   const bool streamed = vocab > 4096;
-  const int ctas = streamed ? 3 * sm_count / 2 : 4 * sm_count, shortest = streamed ? kStreamStage * 3 / 4 : 2048;
-  int chunks = 1;  // (doubled: 3 chunks of 32000 fill their last stage by a third, 6.6 us where 2 take 5.9)
-  while (chunks < kAcceptMaxChunks && static_cast<int64_t>(n_nodes) * 2 * chunks <= ctas && vocab / (2 * chunks) >= shortest) chunks *= 2;
+  int chunks = 1;
+  auto worth = [&](int c) {
+    const int64_t ctas = static_cast<int64_t>(n_nodes) * c;
+    if (!streamed) return ctas <= 4 * sm_count && vocab / c >= (ctas <= sm_count ? 1000 : 2048);
+    return ctas <= 2 * sm_count && vocab / c >= (3 * ctas <= 2 * sm_count ? kStreamStage * 3 / 5 : 2 * ctas <= 3 * sm_count ? kStreamStage * 3 / 4 : kStreamStage * 7 / 4);
+  };
+  while (chunks < kAcceptMaxChunks && worth(2 * chunks)) chunks *= 2;
   int chunk_len = (vocab + chunks - 1) / chunks;
   chunk_len = (chunk_len + 3) & ~3;
   *chunks_out = (vocab + chunk_len - 1) / chunk_len;

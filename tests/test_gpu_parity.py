@@ -914,14 +914,15 @@ def test_sample_equal_logits_are_bit_exact(V, stride):
 @pytest.mark.parametrize("N,V", [(133, 12289), (134, 12289), (148, 4097), (149, 4097), (149, 90112), (222, 90112), (223, 90112), (266, 12289),
                                  (267, 12289), (296, 8200), (297, 8200), (444, 8200), (445, 8200),
                                  (4, 8192), (4, 8193), (6, 16388), (48, 32772), (49, 32772), (103, 16388), (104, 16388), (129, 16384), (130, 16384),
-                                 (130, 49152), (210, 16384), (211, 16384)])
+                                 (130, 49152), (210, 16384), (211, 16384), (1, 2000), (74, 2000), (75, 4096), (37, 4095), (38, 4095), (9, 9830),
+                                 (9, 9832), (49, 9832), (50, 9832), (24, 19664), (25, 19664), (148, 28672), (149, 28672), (74, 57344), (75, 57344)])
 def test_streamed_rows_on_both_sides_of_every_share_of_an_sm(N, V):
     """Greedy and drawn tokens where the number of CTAs passes one, one and a half, two and three per SM, alone and in
     clusters: how much shared memory a CTA is given, and how many share a row.  Greedy rows repeat values, drawn rows
     are equal logits, so that both are exact."""
     rng = np.random.default_rng(N + V)
-    sizes = [N // 4, N // 4, N // 4, N - 3 * (N // 4)]
-    tb = H.make_trees(sizes, [1, 0, 3, 2], rng, vocab=V)
+    sizes = [N // 4, N // 4, N // 4, N - 3 * (N // 4)] if N >= 4 else [N]
+    tb = H.make_trees(sizes, [1, 0, 3, 2][:len(sizes)], rng, vocab=V)
     dt = H.DevTrees(tb)
     lg = (rng.integers(-2000, 2000, size=(N, V)) / 16).astype(np.float32)
     u = (rng.integers(0, 1024, N) / 1024.0).astype(np.float32)
