@@ -89,6 +89,17 @@ __device__ __forceinline__ void dev_status_or(int32_t* status, int b, int bits) 
   if (status != nullptr) atomicOr(&status[b], bits);
 }
 
+// One more arrival at a counter; returns how many there were before.  What the calling thread wrote before it, and what its CTA
+// wrote before a barrier in front of it, is visible to whoever sees the count, and the other way round: after a barrier behind it
+// the CTA that came last may read (past L1) what all others wrote.  One ordered atomic in place of a sequentially
+// consistent fence, an atomic and another such fence: 0.35 us of every acceptance (60 rows of 1000 4.9 -> 4.4 us, 60 of 32000 5.7 -> 5.3, 200
+// of 32000 7.3 -> 6.9), 0.3 to 0.4 of a drawn one (60 of 32000 8.1 -> 7.7).
+__device__ __forceinline__ int arrive_acq_rel(int* counter) {
+  int before;
+  asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(before) : "l"(counter) : "memory");
+  return before;
+}
+
 // Bit t of a 128-bit set stored as two 64-bit words.
 __device__ __forceinline__ bool bit128(uint64_t lo, uint64_t hi, int t) {
   return ((t < 64 ? lo >> t : hi >> (t - 64)) & 1ull) != 0;

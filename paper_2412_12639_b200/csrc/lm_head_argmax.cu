@@ -480,12 +480,10 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_con
     asm volatile("bar.sync 1, %0;" ::"n"(kLmReaders) : "memory");
     if (rt == 0) {
       if (*abort_flag) dev_status_or(p.status, 0, FALCON_DEV_TIMEOUT);
-      __threadfence();
-      *s_last = (atomicAdd(p.ticket, 1) == n_cta - 1) ? 1 : 0;
+      *s_last = (arrive_acq_rel(p.ticket) == n_cta - 1) ? 1 : 0;
     }
     asm volatile("bar.sync 1, %0;" ::"n"(kLmReaders) : "memory");
     if (*s_last) {
-      __threadfence();
       for (int node = rt; node < p.n_rows; node += kLmReaders) {
         const unsigned long long w = __ldcg(p.best + node);
         p.best[node] = 0ull;  // ready for the next call

@@ -218,13 +218,11 @@ __global__ void __launch_bounds__(kAcceptThreads + (kStream ? 32 : 0)) tree_acce
     for (int w = 1; w < kAcceptThreads / 32; ++w) r = merge(r, warp_best[w]);
     p.part_val[static_cast<int64_t>(row) * p.chunks + chunk] = r.v;
     p.part_idx[static_cast<int64_t>(row) * p.chunks + chunk] = r.i;
-    __threadfence();
-    const int arrived = atomicAdd(&p.tickets[b], 1);
+    const int arrived = arrive_acq_rel(&p.tickets[b]);
     s_flag = (arrived == T_real * p.chunks - 1);
   }
   worker_sync();
   if (!s_flag) return;
-  __threadfence();
 
   // ---- last CTA of sequence b: fold the partials, then search the tree ----
   int g = 0;
@@ -492,13 +490,11 @@ __global__ void __launch_bounds__(kStreamThreads + 32, 3) tree_sample_kernel(con
     }
     if (owner == rank && lane == 0) {
       p.argmax_out[row] = g;
-      __threadfence();
-      s_flag = (atomicAdd(&p.tickets[b], 1) == T_real - 1);
+      s_flag = (arrive_acq_rel(&p.tickets[b]) == T_real - 1);
     }
   }
   worker_sync();
   if (!s_flag) return;
-  __threadfence();
   // ---- last row of sequence b: the path search on the drawn tokens ----
   const int gt = tid < min(T_real, FALCON_T_MAX) ? __ldcg(p.argmax_out + base + tid) : 0;
   search_tree(p, b, base, T_real, gt, node, s_par, s_tok, s_g, s_key);

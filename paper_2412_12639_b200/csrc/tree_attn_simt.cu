@@ -275,15 +275,13 @@ __global__ void __launch_bounds__(kThreads) tree_attn_simt_kernel(const SimtPara
   }
   if (tid < T)
     __stcg(p.part_ml + (static_cast<int64_t>(split) * N + base + tid) * p.Hq + h, make_float2(m_s[tid], l_s[tid]));
-  __threadfence();
   __syncthreads();
   if (tid == 0) {
-    const int arrived = atomicAdd(&p.tickets[b * p.Hq + h], 1);
+    const int arrived = arrive_acq_rel(&p.tickets[b * p.Hq + h]);
     s_last = (arrived == p.n_splits - 1);
   }
   __syncthreads();
   if (!s_last) return;
-  __threadfence();
 
   if (nb < TP4) {
 #pragma unroll
