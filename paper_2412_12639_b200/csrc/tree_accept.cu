@@ -5,6 +5,7 @@
 // (kStream: row_stream.cuh says why); with 16-byte loads into registers instead, us per call: 60 rows of 32000 6.9
 // (streamed 5.9), 456 rows 17.3 (14.7, 4 TB/s), 300 rows of 100001 38.2 (24.2, 5 TB/s).
 #include <cfloat>
+#include <algorithm>
 #include <climits>
 
 #include "row_stream.cuh"
@@ -578,8 +579,12 @@ int launch_tree_accept(falcon_ctx* ctx, const falcon_accept_args& a, cudaStream_
   int chunks, chunk_len;
   const bool streamed = accept_plan(ctx->sm_count, N, a.vocab, &chunks, &chunk_len);
 
+  // (where the scratch has to grow, to what any launch of no more rows takes, see accept_plan: fewer rows may have more chunks in
+  // all, and a call whose scratch would have to grow cannot be captured)
   const size_t part = static_cast<size_t>(N) * chunks;
-  int rc = ensure_workspace(ctx, part * 8 + 256);
+  size_t bytes = part * 8 + 256;
+  if (bytes > ctx->ws_bytes) bytes = std::max<size_t>(part, 4 * static_cast<size_t>(ctx->sm_count)) * 8 + 256;
+  int rc = ensure_workspace(ctx, bytes);
   if (rc) return rc;
   rc = ensure_tickets(ctx, a.tree.batch, s);
   if (rc) return rc;

@@ -1420,6 +1420,36 @@ def test_captured_graph_survives_a_later_call_that_needs_more_scratch():
     c.close()
 
 
+def test_acceptance_of_fewer_rows_is_captured_after_a_first_call_of_more():
+    """149 rows take one chunk each, 148 two: the scratch that the first call leaves is enough for any launch of no more
+    rows, so that the second can be captured at once."""
+    import paper_2412_12639_b200 as falcon
+    V = 28672
+    rng = np.random.default_rng(79)
+    logits = torch.from_numpy(rng.standard_normal((149, V)).astype(np.float32)).cuda()
+    c = falcon.Context(0)
+    st = torch.cuda.Stream()
+    calls = []
+    for sizes in ([75, 74], [74, 74]):
+        tb = H.make_trees(sizes, [0, 0], rng, vocab=V)
+        dt, out = H.DevTrees(tb), _accept_buffers(tb)
+        calls.append((tb, dt, out, binding.accept_args(dt.desc(), V, logits, V, out[0], out[1], 128, out[2], out[3])))
+    torch.cuda.synchronize()
+    with torch.cuda.stream(st):
+        c.falcon_tree_accept(calls[0][3], stream=st)
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=st):
+            c.falcon_tree_accept(calls[1][3], stream=st)
+        graph.replay()
+    torch.cuda.synchronize()
+    for tb, _, out, _ in calls:
+        want = oracle.argmax(logits[:tb.total_nodes].cpu().numpy())
+        np.testing.assert_array_equal(out[0].cpu().numpy(), want)
+        np.testing.assert_array_equal(out[1].cpu().numpy(), oracle.tree_accept(tb.node_off, tb.parent, tb.token, want)[0])
+    c.close()
+
+
 @pytest.mark.parametrize("tck", TC_KERNELS)
 @pytest.mark.parametrize("T", [60, 80])
 def test_attn_bounded_wait_runs_out_and_the_context_stays_usable(tck, T):
