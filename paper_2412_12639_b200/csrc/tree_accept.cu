@@ -3,9 +3,9 @@
 // (arrival counter) folds the chunk partials into g[] and searches the tree.  HBM-bound: the N*V fp32
 // logits are read once.  Rows of more than 4096 entries are streamed through shared memory by bulk copies
 // (kStream: row_stream.cuh says why); with 16-byte loads into registers instead, us per call: 60 rows of 32000 6.9
-// (streamed 5.9), 456 rows 17.3 (14.7, 4 TB/s), 300 rows of 100001 38.2 (24.2, 5 TB/s).
-#include <cfloat>
+// (streamed 5.9; 5.1 with the present hand-over and reductions), 456 rows 17.3 (14.7, 4 TB/s), 300 rows of 100001 38.2 (24.2, 5 TB/s).
 #include <algorithm>
+#include <cfloat>
 #include <climits>
 
 #include "row_stream.cuh"
