@@ -37,6 +37,9 @@ struct falcon_ctx {
 
 namespace falcon {
 
+// Chunks that a greedy acceptance splits its rows into, over all rows, per SM at most (where it splits them at all).
+constexpr int kAcceptChunksPerSm = 4;
+
 int ensure_workspace(falcon_ctx* ctx, size_t bytes);
 int ensure_tickets(falcon_ctx* ctx, size_t count, cudaStream_t stream);
 int cuda_fail(falcon_ctx* ctx, cudaError_t e, const char* where);

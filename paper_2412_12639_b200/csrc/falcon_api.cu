@@ -1,4 +1,5 @@
 // C-ABI entry points: argument validation, context management, dispatch.
+#include <algorithm>
 #include <cstdio>
 #include <cstring>
 #include <new>
@@ -13,10 +14,12 @@ int cuda_fail(falcon_ctx* ctx, cudaError_t e, const char* where) {
 }
 
 // Scratch only ever grows, and a block that was outgrown is kept until the context is destroyed:
-// a kernel already enqueued, or a captured graph, may still name it.
+// a kernel already enqueued, or a captured graph, may still name it.  No block is smaller than the partials of an acceptance
+// that splits its rows, whichever call asked for it: an acceptance of fewer rows may have more chunks in all than one of
+// more rows, and a call for which the scratch would have to grow cannot be captured.
 int ensure_workspace(falcon_ctx* ctx, size_t bytes) {
   if (bytes <= ctx->ws_bytes) return FALCON_OK;
-  const size_t want = bytes + bytes / 4;
+  const size_t want = std::max(bytes + bytes / 4, static_cast<size_t>(ctx->sm_count) * kAcceptChunksPerSm * 8 + 256);
   void* fresh = nullptr;
   cudaError_t e = cudaMalloc(&fresh, want);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaMalloc(workspace)");

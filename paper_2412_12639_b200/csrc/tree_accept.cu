@@ -4,7 +4,6 @@
 // logits are read once.  Rows of more than 4096 entries are streamed through shared memory by bulk copies
 // (kStream: row_stream.cuh says why); with 16-byte loads into registers instead, us per call: 60 rows of 32000 6.9
 // (streamed 5.9; 5.1 with the present hand-over and reductions), 456 rows 17.3 (14.7, 4 TB/s), 300 rows of 100001 38.2 (24.2, 5 TB/s).
-#include <algorithm>
 #include <cfloat>
 #include <climits>
 
@@ -521,7 +520,8 @@ bool accept_plan(int sm_count, int n_nodes, int vocab, int* chunks_out, int* chu
   int chunks = 1;
   auto worth = [&](int c) {
     const int64_t ctas = static_cast<int64_t>(n_nodes) * c;
-    if (!streamed) return ctas <= 4 * sm_count && vocab / c >= (ctas <= sm_count ? 1000 : 2048);
+    if (!streamed) return ctas <= kAcceptChunksPerSm * sm_count && vocab / c >= (ctas <= sm_count ? 1000 : 2048);
+    static_assert(kAcceptChunksPerSm >= 2, "the scratch is sized by it");
     return ctas <= 2 * sm_count && vocab / c >= (3 * ctas <= 2 * sm_count ? kStreamStage * 3 / 5 : 2 * ctas <= 3 * sm_count ? kStreamStage * 3 / 4 : kStreamStage * 7 / 4);
   };
   while (chunks < kAcceptMaxChunks && worth(2 * chunks)) chunks *= 2;
@@ -579,12 +579,7 @@ int launch_tree_accept(falcon_ctx* ctx, const falcon_accept_args& a, cudaStream_
   int chunks, chunk_len;
   const bool streamed = accept_plan(ctx->sm_count, N, a.vocab, &chunks, &chunk_len);
 
-  // (where the scratch has to grow, to what any launch of no more rows takes, see accept_plan: fewer rows may have more chunks in
-  // all, and a call whose scratch would have to grow cannot be captured)
-  const size_t part = static_cast<size_t>(N) * chunks;
-  size_t bytes = part * 8 + 256;
-  if (bytes > ctx->ws_bytes) bytes = std::max<size_t>(part, 4 * static_cast<size_t>(ctx->sm_count)) * 8 + 256;
-  int rc = ensure_workspace(ctx, bytes);
+  int rc = ensure_workspace(ctx, static_cast<size_t>(N) * chunks * 8 + 256);
   if (rc) return rc;
   rc = ensure_tickets(ctx, a.tree.batch, s);
   if (rc) return rc;

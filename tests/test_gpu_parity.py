@@ -1420,15 +1420,23 @@ def test_captured_graph_survives_a_later_call_that_needs_more_scratch():
     c.close()
 
 
-def test_acceptance_of_fewer_rows_is_captured_after_a_first_call_of_more():
+@pytest.mark.parametrize("attention_first", [False, True])
+def test_acceptance_of_fewer_rows_is_captured_after_a_first_call_of_more(attention_first):
     """149 rows take one chunk each, 148 two: the scratch that the first call leaves is enough for any launch of no more
-    rows, so that the second can be captured at once."""
+    rows, so that the second can be captured at once.  Also where the first acceptance finds a block that a small split attention
+    left, 1640 bytes: enough for itself (1448) but not for the second (2624)."""
     import paper_2412_12639_b200 as falcon
     V = 28672
     rng = np.random.default_rng(79)
     logits = torch.from_numpy(rng.standard_normal((149, V)).astype(np.float32)).cuda()
     c = falcon.Context(0)
     st = torch.cuda.Stream()
+    if attention_first:
+        tb, q, k, v = random_case(rng, [2], [40], 1, 1, 64)
+        dt, qd, kd, vd = H.DevTrees(tb), H.dev_bf16(q), H.dev_bf16(k), H.dev_bf16(v)
+        out = torch.zeros_like(qd)
+        c.falcon_tree_attn(binding.attn_args(dt.desc(), 1, 1, 64, 0.125, qd, out, kd, vd, tuple(int(s) for s in kd.stride()[:3]), kd.shape[2],
+                                             kernel=binding.ATTN_SIMT, n_splits=2), stream=st)
     calls = []
     for sizes in ([75, 74], [74, 74]):
         tb = H.make_trees(sizes, [0, 0], rng, vocab=V)
