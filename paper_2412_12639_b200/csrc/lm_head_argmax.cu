@@ -533,12 +533,23 @@ int launch_lm_head_argmax(falcon_ctx* ctx, const falcon_lm_argmax_args& a, cudaS
   uint32_t mma_n = static_cast<uint32_t>(tile_n);
   // Vocabulary rows on the lanes, 256 of them a pair, and the nodes on the side that comes in steps of 16, where that takes
   // so many fewer columns of MMAs (with the nodes on the lanes 300 of them are padded to 512) that it pays for the reading of
-  // the accumulators: the maxima across lanes take up to 4000 cycles more each time, and a column and 64 hidden columns are
-  // 2 cycles of the tensor core.  Against nodes on the lanes, us in bursts (and, under the power limit, in a loop):
-  //   4096 x 32000    129 nodes 57.7 -> 53.6, 257 99.0 -> 92.5, 308 118 -> 105 (116 -> 102)
-  //   5120 x 32000    129 nodes 69.8 -> 64.6, 314 146 -> 129 (144 -> 126), 411 126.4 -> 122.1 (145 -> 140)
-  //   2048 x 50000    129 nodes 60.0 -> 54.9, 300 82.8 -> 77.4, 477 (100 / 103: not taken)
-  //   1024 x 100000   129 nodes 51.8 -> 49.3, 257 89.0 -> 84.6, 425 (99 / 106: not taken)
+  // the accumulators, whose maxima across lanes take longer each time.  What is saved per reading, x = columns of MMAs times
+  // chunks of 64 hidden columns, decides; one of them is 2 cycles of the tensor core.  Both arrangements were timed at 80
+  // sizes, in bursts of six calls and in loops of half a second (under the power limit, where fewer MMAs count for more).  Bursts
+  // alone turn at x = 2200, loops alone at 1000; 1600 is where the two together do: the product of both ratios is 0.999 or more
+  // at every size with x >= 1664, and above one at 6 of 24 below.  us, nodes on the lanes -> vocabulary rows (in a loop):
+  //   x  768  300 nodes of 1536 x 24000  39.9 -> 42.0 (36.9 -> 39.6)       800 of 512 x 131072    121 -> 142 (134 -> 147)
+  //     1024  370 of 1024 x 32000        32.8 -> 34.5 (30.6 -> 32.1)       385 of 2048 x 32000    56.3 -> 59.1 (63.9 -> 63.2)
+  //     1280  400 of 2560 x 32000        67.6 -> 70.0 (78.0 both)          430 of 2560 x 50257    103 -> 105 (121 -> 122)
+  //     1536  400 of 3072 x 32000        78.8 -> 80.9 (92.8 -> 90.5)       340 of 1024 x 32000    32.6 -> 34.0 (30.1 -> 31.7)
+  //     1664  230 of 512 x 16000         13.6 -> 13.1 (12.0 -> 11.7)
+  //     1792  400 of 3584 x 32000        90.8 -> 91.5 (107 -> 104)         430 of 3584 x 100000   280 -> 276 (330 -> 326)
+  //     1920  280 of 768 x 64000         47.8 -> 48.1 (48.5 -> 45.7)       200 of 512 x 16000     13.5 -> 12.6 (12.0 -> 11.2)
+  //     2048  385 of 4096 x 32000        101 -> 103 (122 -> 118), 416 103 both (123 -> 119), 417 (x = 0) 102 -> 106 (123 both)
+  //           385 of 2048 x 50000        84.0 -> 85.0 (97.6 -> 95.4), 416 84.3 -> 85.3 (98.7 -> 96.5), 432 (1024) 84.3 -> 88.1 (99.2 -> 99.8)
+  //     2560  129 of 1024 x 32000        19.3 -> 19.1 (17.4 -> 17.6)
+  //           385 of 5120 x 32000        125 -> 124 (151 -> 145), 411 127 -> 124 (152 -> 146), 417 (0) 127 -> 128 (153 -> 151)
+  //     4096  411 of 8192 x 32000        201 -> 192 (241 -> 229)           6400: 352 of 5120 x 32000  124 -> 116 (148 -> 133)
   bool lanes = false;
   if (pair) {
     const int tiles = N <= 256 ? 1 : 2 * ((N + 511) / 512), cols = ((N + tiles - 1) / tiles + 15) & ~15;
@@ -547,7 +558,7 @@ int launch_lm_head_argmax(falcon_ctx* ctx, const falcon_lm_argmax_args& a, cudaS
     const int64_t here = static_cast<int64_t>(tiles) * cols * (two ? (per + 1) / 2 * 2 : per), chunks = (H + kLmKC - 1) / kLmKC;
     const int64_t other = static_cast<int64_t>(n_mt) * tile_n * (v_res > 1 ? (n_vt + 1) / 2 * 2 : n_vt);
     const int64_t reads = static_cast<int64_t>((tiles + 1) / 2) * (two ? (per + 1) / 2 : per);
-    lanes = 2 * (other - here) * chunks > 4000 * reads;
+    lanes = (other - here) * chunks > 1600 * reads;
     if (lanes) {
       n_mt = tiles;
       m_res = tiles > 1 ? 2 : 1;

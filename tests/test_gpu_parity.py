@@ -1137,11 +1137,14 @@ def test_lm_head_argmax_pairs_of_ctas(N, Hd, V):
     test_lm_head_argmax_integer_data_is_bit_exact(N, Hd, V)
 
 
-@pytest.mark.parametrize("N,Hd,V", [(129, 1344, 30001), (144, 1416, 30210), (257, 768, 18900), (289, 1032, 18944), (384, 1800, 18689), (520, 1792, 18800)])
+@pytest.mark.parametrize("N,Hd,V", [(129, 1344, 30001), (144, 1416, 30210), (257, 768, 18900), (289, 1032, 18944), (384, 1800, 18689), (520, 1792, 18800),
+                                    (200, 1792, 18900), (129, 768, 50001), (411, 3584, 32000), (400, 3072, 32000), (540, 2560, 31990), (300, 768, 90000)])
 def test_lm_head_argmax_vocabulary_rows_on_the_lanes(N, Hd, V):
     # sizes at which pairs of CTAs put the vocabulary rows on the lanes: two vocabulary blocks at a time and one, node tiles
-    # with and without padding, a second group of them, a last block cut short or absent.  Small integers: exact in fp32
-    # (products up to 9, at most 1800 of them).  A NaN in a head row and a node of NaNs never win.
+    # with and without padding, a second group of them, a last block cut short or absent; then one block and one node tile (half of
+    # the readers idle), and several passes of a pair over its blocks: two with an odd last block, two of one block each (and the
+    # size beyond the line, nodes on the lanes), two in each of two groups, five.  Small integers: exact in fp32
+    # (products up to 9, at most 3584 of them).  A NaN in a head row and a node of NaNs never win.
     gen = torch.Generator(device="cuda")
     gen.manual_seed(N + V)
     f = torch.randint(-3, 4, (N, Hd), generator=gen, device="cuda").to(torch.bfloat16)
@@ -1149,6 +1152,9 @@ def test_lm_head_argmax_vocabulary_rows_on_the_lanes(N, Hd, V):
     first = int((f[:1].double() @ w.double().T).argmax())
     w[V - 1] = w[first]                                         # ties between the first and the last pair, and inside a block
     w[V // 2] = w[5]
+    w[min(first + 256, V - 1)] = w[first]                       # a tie with the next block, which may be the pair's next pass,
+    second = int((f[1:2].double() @ w.double().T).argmax())
+    w[max(second - 256, 0)] = w[second]                         # and one with the block before
     w[7, 3] = float("nan")
     f[N // 2] = float("nan")
     logits = (f.double() @ w.double().T).nan_to_num_(nan=-float("inf"), posinf=float("inf"), neginf=-float("inf"))
