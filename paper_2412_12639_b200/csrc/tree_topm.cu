@@ -624,9 +624,20 @@ int launch_tree_topm(falcon_ctx* ctx, const falcon_topm_args& a, cudaStream_t s)
   while (c < kTopmMaxCluster && a.vocab > c * kTopmThreads * kTopmRowsMax) c *= 2;
   if (c > 1 && c < 4 && N * 4 <= 96) c = 4;
   if (c > 1 && c < 8 && N * 8 < 64) c = 8;
-  // (eight again where four would put two CTAs with most of their registers full on an SM: 60 rows of 32000 5.3 us both alone,
-  // 0.2 less behind an attention launch)
-  if (c == 4 && a.vocab > 4 * 24 * kTopmThreads && N * 4 > 4 * ctx->sm_count / 3 && room(static_cast<int64_t>(N) * 8, 8, 4)) c = 8;
+  // Eight again for the rows at which the SMs would no longer take the clusters of four evenly, as long as the clusters of eight
+  // are placed at once, for any length (us with 4 / 8, alone and behind an attention launch; 16385, 24577 and 32768 entries):
+  //   50 rows  5.4 / 5.9  18.0 / 17.9      5.8 / 6.2  18.6 / 18.1      6.1 / 6.5  18.9 / 18.4
+  //   52       5.4 / 5.9  18.1 / 17.9      5.9 / 6.2  18.6 / 18.1      6.1 / 6.5  18.9 / 18.5
+  //   53       6.0 / 5.9  18.1 / 17.9      6.6 / 6.3  18.7 / 18.2      6.9 / 6.5  19.1 / 18.5
+  //   61       6.3 / 6.1  18.2 / 18.4      6.8 / 6.5  18.8 / 18.6      7.2 / 6.7  19.1 / 18.8
+  //   62       6.3 / 6.2  18.2 / 18.5      6.8 / 6.5  18.8 / 18.9      7.2 / 6.8  19.1 / 19.2
+  //   64       6.3 / 6.8  18.2 / 19.4      6.9 / 6.9  18.8 / 19.7      7.2 / 7.1  19.2 / 20.1
+  // (below 53 rows the two regimes disagree, and four stay)
+  const int64_t rows = N, sm = ctx->sm_count;
+  if (c == 4 && 100 * 4 * rows > 142 * sm && 10 * 8 * rows <= 33 * sm) {
+    split(8);
+    if (fits()) c = 8;
+  }
   // (two stages of one CTA against two CTAs' registers: 48 rows of 16000 4.6 and 4.4 us, 64 of 12000 4.6 and 5.0, 120 5.2 and 6.0)
   const bool short_stream = a.vocab > kStreamStage && a.vocab <= 2 * kStreamStage && N >= 56;
   split(c);

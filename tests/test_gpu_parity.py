@@ -790,7 +790,9 @@ def test_topm_bit_exact(N, V, stride, m):
 
 @pytest.mark.parametrize("N,V,m", [(1, 8192, 32), (444, 8192, 20), (445, 8192, 20), (7, 8193, 20), (25, 8193, 8), (24, 16384, 8), (55, 16384, 32),
                                    (56, 16385, 5), (56, 16384, 32), (1, 16384, 1), (103, 20001, 20), (104, 20001, 20), (8, 32768, 20), (48, 40003, 8),
-                                   (49, 40003, 8), (86, 40003, 8), (104, 49152, 3), (104, 114687, 9), (104, 114688, 9), (210, 114690, 2), (211, 114690, 2)])
+                                   (49, 40003, 8), (86, 40003, 8), (104, 49152, 3), (104, 114687, 9), (104, 114688, 9), (210, 114690, 2), (211, 114690, 2),
+                                   (52, 16386, 20), (53, 16386, 20), (61, 32768, 20), (62, 32768, 20), (61, 24577, 32), (87, 40003, 8), (103, 49151, 8),
+                                   (103, 49152, 8)])
 def test_topm_on_both_sides_of_every_line_of_the_dispatch(N, V, m):
     """How many CTAs share a row, and whether it is held in registers or streamed: one CTA's registers, stages of one CTA,
     clusters as far as they have room.  Values repeat, so that ties cross the borders of lanes, warps and CTAs."""
