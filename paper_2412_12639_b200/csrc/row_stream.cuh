@@ -22,8 +22,7 @@ constexpr int kStreamStage = kStreamThreads * kStreamLane;  // 8192 entries, 32 
 constexpr int kStreamStages = 2;
 constexpr uint32_t kStreamBytes = kStreamStages * kStreamStage * 4;
 constexpr uint32_t kStreamBytesPair = 78u * 1024u;      // more than a third of an SM's shared memory: two CTAs per SM
-constexpr uint32_t kStreamBytesAlone = 116u * 1024u;    // more than half of it: one
-constexpr uint32_t kStreamBytesMax = kStreamBytesAlone; // (the attribute the kernels are given once)
+constexpr uint32_t kStreamBytesMax = kStreamBytesPair;  // (the attribute the kernels are given once)
 
 // Whether the GPU places n CTAs in clusters of `of` at once where an SM has room for per_sm of them: 19/20, 14/15 and 13/15 of the
 // places for two, four and eight CTAs, since not every SM that has room has it beside the others.  (us, top-m: 103 rows of 20000
@@ -32,20 +31,26 @@ inline bool cluster_room(int64_t n_ctas, int of, int per_sm, int sm_count) {
   return n_ctas * 60 <= static_cast<int64_t>(of == 1 ? 60 : of == 2 ? 57 : of == 4 ? 56 : 52) * per_sm * sm_count;
 }
 
-// Dynamic shared memory of a launch of n CTAs in clusters of `of` that take `len` entries each: so much that no SM takes more
-// of them than an even share.  Behind a kernel whose CTAs end at different times the SMs that become free first would be given
-// three each and the last ones none (us, attention over one sequence and then acceptance: 121 rows of 128256 39.5 and 33.7, 136
-// of 64000 33.8 and 30.8, 136 of 32000 31.1 and 29.6; top-m over 121 rows of 32000 32.9 and 30.8).  With all SMs free at once
-// it is the same either way.  Not for more than one and a half rows' length of work on some SMs and half of it on others (170
-// rows of 128256 from L2: 13 us with three per SM allowed, 18 with two), nor where clusters might not all find their places
-// (sample, 140 rows of 128256 in clusters of two 18.8 and 20.8; top-m behind attention, 60 rows of 64000 in clusters of four
-// 7 % slower).
+// Dynamic shared memory of a launch of n CTAs in clusters of `of` that take `len` entries each: so much that an SM takes two
+// of them at most, where that is enough places.  Behind a kernel whose CTAs end at different times the SMs that become free first
+// would be given three each and the last ones none.  Not one per SM, although a launch of no more CTAs than SMs is faster still
+// on one stream: a CTA that waits for its turn keeps an SM from the attention launches of other streams, and with one CTA per SM two
+// streams that decide at the same time share none.  us with three / two / one per SM allowed: behind an attention launch over four
+// sequences on one stream, the same on two streams at once, and two streams with the scans alone:
+//   top-m       120 rows of 32000   41.3 / 39.8 / 38.6   55.6 / 56.5 / 60.3   11.6 / 10.7 / 12.1
+//               140 of 50000        45.7 / 43.6 / 41.9   60.6 / 60.8 / 64.2   15.5 / 14.2 / 18.1
+//   acceptance  100 of 12000        35.5 / 35.0 / 35.0   47.4 / 49.7 / 54.0    6.7 /  6.7 /  6.6
+//               148 of 28000        37.8 / 37.3 / 37.4   53.5 / 54.5 / 60.9   10.3 /  9.8 / 11.8
+//   sample      148 of 40000        42.8 / 41.5 / 41.0   58.3 / 58.9 / 63.7   14.3 / 13.7 / 17.5
+// One stream's scans alone are the same with three and with two.  Not for more than one and a half rows' length of work on some SMs
+// and half of it on others (170 rows of 128256 from L2: 13 us with three per SM allowed, 18 with two), nor where clusters might not
+// all find their places (sample, 140 rows of 128256 in clusters of two 18.8 and 20.8; top-m behind attention, 60 rows of
+// 64000 in clusters of four 7 % slower).
 inline uint32_t stream_bytes(int64_t n_ctas, int of, int len, int sm_count) {
   if (of > 2) return kStreamBytes;
   const int64_t slots = of == 2 ? sm_count * 9 / 10 : sm_count;
-  if (n_ctas <= slots) return kStreamBytesAlone;
-  if (n_ctas <= 2 * slots && (2 * n_ctas > 3 * sm_count || len <= 10 * kStreamStage)) return kStreamBytesPair;
-  return kStreamBytes;
+  const bool even = n_ctas <= slots || (n_ctas <= 2 * slots && (2 * n_ctas > 3 * sm_count || len <= 10 * kStreamStage));
+  return even ? kStreamBytesPair : kStreamBytes;
 }
 
 struct StreamBars {

@@ -1389,6 +1389,49 @@ def test_two_contexts_used_in_turn_keep_their_own_state():
         c.close()
 
 
+def test_two_streams_decide_at_the_same_time():
+    """Two contexts, each on a stream of its own, run the streamed calls side by side, CTAs of both on the same SMs: top-m, greedy
+    and drawn acceptance of about one CTA per SM and of two."""
+    import paper_2412_12639_b200 as falcon
+    rng = np.random.default_rng(80)
+    ctxs, streams, jobs = [falcon.Context(0), falcon.Context(0)], [torch.cuda.Stream(), torch.cuda.Stream()], []
+    for N, V in ((140, 20003), (148, 28000), (100, 60001)):
+        for c, st in zip(ctxs, streams):
+            lg = (rng.integers(-2000, 2000, size=(N, V)) / 16).astype(np.float32)
+            flat = np.full((N, V), 1.25, dtype=np.float32)
+            u = (rng.integers(0, 1024, N) / 1024.0).astype(np.float32)
+            tb = H.make_trees([N // 2, N - N // 2], [1, 0], rng, vocab=V)
+            dt, ld, fd, ud = H.DevTrees(tb), torch.from_numpy(lg).cuda(), torch.from_numpy(flat).cuda(), torch.from_numpy(u).cuda()
+            greedy, drawn = _accept_buffers(tb), _accept_buffers(tb)
+            val, idx = torch.zeros((N, 20), device="cuda"), torch.zeros((N, 20), dtype=torch.int32, device="cuda")
+            calls = (lambda c=c, st=st, a=binding.topm_args(N, V, ld, V, 20, val, idx): c.falcon_topm(a, stream=st),
+                     lambda c=c, st=st, a=binding.accept_args(dt.desc(), V, ld, V, greedy[0], greedy[1], 128, greedy[2], greedy[3]):
+                     c.falcon_tree_accept(a, stream=st),
+                     lambda c=c, st=st, a=binding.accept_args(dt.desc(), V, fd, V, drawn[0], drawn[1], 128, drawn[2], drawn[3], temperature=1.3,
+                                                              uniforms=ud): c.falcon_tree_accept(a, stream=st))
+            jobs.append((calls, tb, lg, u, V, greedy, drawn, val, idx, (dt, ld, fd, ud)))
+    for calls, *_ in jobs:
+        for f in calls:
+            f()                                                # (the first call of a size may allocate)
+    torch.cuda.synchronize()
+    for _ in range(3):
+        for pair in zip(jobs[0::2], jobs[1::2]):
+            for fs in zip(*(j[0] for j in pair)):              # the same call on either stream, one after the other
+                for f in fs:
+                    f()
+    torch.cuda.synchronize()
+    for _, tb, lg, u, V, greedy, drawn, val, idx, _ in jobs:
+        g = oracle.argmax(lg)
+        np.testing.assert_array_equal(greedy[0].cpu().numpy(), g)
+        np.testing.assert_array_equal(greedy[1].cpu().numpy(), oracle.tree_accept(tb.node_off, tb.parent, tb.token, g)[0])
+        np.testing.assert_array_equal(drawn[0].cpu().numpy(), np.floor(u.astype(np.float64) * V).astype(np.int32))
+        rv, ri = oracle.topm(lg, 20)
+        np.testing.assert_array_equal(idx.cpu().numpy(), ri)
+        np.testing.assert_array_equal(val.cpu().numpy(), rv)
+    for c in ctxs:
+        c.close()
+
+
 def test_captured_graph_survives_a_later_call_that_needs_more_scratch():
     """An acceptance call captured into a CUDA graph, then a top-m call on the same context that needs a larger
     scratch block and more arrival counters (on a non-blocking stream), then the graph replayed: the graph still
