@@ -33,6 +33,8 @@ struct falcon_ctx {
   // three variants (times head dimension and place of the tree's K/V for the limit).
   bool attn_attr_set[13] = {};
   int attn_resident[4][9] = {};
+  // The same of the kernels that scan logits rows, for clusters of 1, 2, 4 and 8 (clusters_at_once in row_stream.cuh).
+  int scan_resident[5][4] = {};
 };
 
 namespace falcon {

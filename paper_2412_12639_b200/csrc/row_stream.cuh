@@ -24,11 +24,40 @@ constexpr uint32_t kStreamBytes = kStreamStages * kStreamStage * 4;
 constexpr uint32_t kStreamBytesPair = 78u * 1024u;      // more than a third of an SM's shared memory: two CTAs per SM
 constexpr uint32_t kStreamBytesMax = kStreamBytesPair;  // (the attribute the kernels are given once)
 
-// Whether the GPU places n CTAs in clusters of `of` at once where an SM has room for per_sm of them: 19/20, 14/15 and 13/15 of the
-// places for two, four and eight CTAs, since not every SM that has room has it beside the others.  (us, top-m: 103 rows of 20000
-// in clusters of four 5.6, 105 7.8, of 50257 streamed 9.8 and 13.4; in clusters of eight 48 rows of 50257 5.8, 49 8.1.)
-inline bool cluster_room(int64_t n_ctas, int of, int per_sm, int sm_count) {
-  return n_ctas * 60 <= static_cast<int64_t>(of == 1 ? 60 : of == 2 ? 57 : of == 4 ? 56 : 52) * per_sm * sm_count;
+// The kernels that scan rows in clusters: places in falcon_ctx::scan_resident.
+enum ScanKernel { kScanTopm8, kScanTopm16, kScanTopm32, kScanTopmStream, kScanSample };
+
+// Clusters of `of` CTAs of a kernel that the GPU holds at once (asked once per context; 0 where it cannot say).
+inline int clusters_at_once(falcon_ctx* ctx, ScanKernel which, const void* kernel, int threads, uint32_t smem, int of) {
+  int& n = ctx->scan_resident[which][of == 1 ? 0 : of == 2 ? 1 : of == 4 ? 2 : 3];
+  if (n == 0) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(of, ctx->sm_count);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = of;
+    attr.val.clusterDim.y = 1;
+    attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    int got = 0;
+    if (cudaOccupancyMaxActiveClusters(&got, kernel, &cfg) != cudaSuccess) cudaGetLastError();
+    n = got > 0 ? got : -1;
+  }
+  return n > 0 ? n : 0;
+}
+
+// Whether n clusters of `of` CTAs, of which at_once fit, are placed without some of them waiting for others.  Behind an attention
+// launch, whose SMs become free one by one, clusters of four and eight need a few places more than they take (us with
+// clusters of four, alone and behind one; 104 fit: top-m, 64000 entries, 100 rows 11.3 / 23.9, 101 11.4 / 24.5, 102 11.5 / 25.1, 103 11.7 / 26.6, 105
+// 15.0 / 28.0, against 11.9 / 24.1 with clusters of two all along; sample, 32000, 100 rows 9.1 / 21.8, 102 9.1 / 23.0, 105 11.3 / 24.4,
+// against 9.3 / 21.9.  Clusters of eight, 48 fit: top-m, 65536, 45 rows 8.2 / 20.9, 46 8.3 / 21.7, 48 9.2 / 24.3, 49 11.9 / 24.9, against 8.2 / 21.3
+// with four; sample, 64000, 45 rows 9.2 / 21.9, 46 9.2 / 22.5, 48 9.3 / 24.4, 49 12.1 / 25.0, against 9.6 / 22.5).  Clusters of two fill all
+// their 222 places: top-m, 32000, 222 rows 12.0 / 24.3, 223 15.4 / 28.0; sample 12.1 / 24.6, 224 rows 14.3 / 26.8.
+inline bool cluster_room(int64_t n, int of, int at_once) {
+  return of <= 2 ? n <= at_once : of == 4 ? 26 * n <= 25 * static_cast<int64_t>(at_once) : 16 * n <= 15 * static_cast<int64_t>(at_once);
 }
 
 // Dynamic shared memory of a launch of n CTAs in clusters of `of` that take `len` entries each: so much that an SM takes two

@@ -609,8 +609,11 @@ int launch_tree_sample(falcon_ctx* ctx, const falcon_accept_args& a, cudaStream_
   // A cluster costs 0.3 to 0.5 us per doubling, which less than a stage does not win back: us with 1 / 2 / 4 / 8 CTAs, 16 rows of
   // 4000 6.6 / 6.9 / 7.0 / -, of 8192 6.8 / 7.1 / 7.3 / 7.7, of 12000 7.4 / 7.0 / 7.2 / 7.6, of 32000 9.0 / 8.0 / 7.4 / 7.7, of 64000
   // 12.1 / 9.9 / 8.4 / 7.9; 80 of 8192 6.7 / 7.1 / 7.5 / -; 50 of 64000 11.9 / 9.6 / 9.0 / 11.9 (a second wave of clusters).
+  auto room = [&](int of) {
+    return cluster_room(N, of, clusters_at_once(ctx, kScanSample, reinterpret_cast<const void*>(tree_sample_kernel), kStreamThreads + 32, kStreamBytes, of));
+  };
   int ctas = 1;
-  while (ctas < kSampleMaxCluster && a.vocab > ctas * kStreamStage && cluster_room(static_cast<int64_t>(N) * 2 * ctas, 2 * ctas, 3, ctx->sm_count)) ctas *= 2;
+  while (ctas < kSampleMaxCluster && a.vocab > ctas * kStreamStage && room(2 * ctas)) ctas *= 2;
   // (nearly one row per SM: two CTAs per SM share it no better; 145 rows of 20000 8.2 and 9.1, of 32000 9.2 and 9.5, of 64000 12.4 both)
   if (ctas == 2 && N <= ctx->sm_count && 8 * N > 7 * ctx->sm_count && a.vocab < 6 * kStreamStage) ctas = 1;
   const int chunk_len = ((a.vocab + ctas - 1) / ctas + 3) & ~3;

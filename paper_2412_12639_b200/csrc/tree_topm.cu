@@ -618,8 +618,17 @@ int launch_tree_topm(falcon_ctx* ctx, const falcon_topm_args& a, cudaStream_t s)
     chunk = ((a.vocab + c - 1) / c + 3) & ~3;
     per_lane = (chunk + kTopmThreads - 1) / kTopmThreads;
   };
-  auto room = [&](int64_t n_ctas, int of, int per_sm) { return cluster_room(n_ctas, of, per_sm, ctx->sm_count); };
-  auto fits = [&]() { return room(static_cast<int64_t>(N) * ctas, ctas, per_lane <= 8 ? 6 : per_lane <= 16 ? 4 : 3); };
+  auto room = [&](int of, ScanKernel which, const void* kernel, int threads, uint32_t smem) {
+    return cluster_room(N, of, clusters_at_once(ctx, which, kernel, threads, smem, of));
+  };
+  auto fits = [&]() {
+    return per_lane <= 8    ? room(ctas, kScanTopm8, reinterpret_cast<const void*>(tree_topm_kernel<8>), kTopmThreads, 0)
+           : per_lane <= 16 ? room(ctas, kScanTopm16, reinterpret_cast<const void*>(tree_topm_kernel<16>), kTopmThreads, 0)
+                            : room(ctas, kScanTopm32, reinterpret_cast<const void*>(tree_topm_kernel<kTopmRowsMax>), kTopmThreads, 0);
+  };
+  auto streams = [&](int of) {
+    return room(of, kScanTopmStream, reinterpret_cast<const void*>(tree_topm_stream_kernel), kStreamThreads + 32, kStreamBytes);
+  };
   int c = 1;
   while (c < kTopmMaxCluster && a.vocab > c * kTopmThreads * kTopmRowsMax) c *= 2;
   if (c > 1 && c < 4 && N * 4 <= 96) c = 4;
@@ -648,7 +657,7 @@ int launch_tree_topm(falcon_ctx* ctx, const falcon_topm_args& a, cudaStream_t s)
     // even out better where the SMs become free one by one (158 of 32000 alone 9.3 and 10.3 or, from L2, 8.0 both; behind an
     // attention launch 0.8 less with two).
     c = 1;
-    while (c < kTopmMaxCluster && room(static_cast<int64_t>(N) * 2 * c, 2 * c, 3) && a.vocab >= 2 * c * kStreamStage) c *= 2;
+    while (c < kTopmMaxCluster && streams(2 * c) && a.vocab >= 2 * c * kStreamStage) c *= 2;
     if ((c == 2 && N <= ctx->sm_count && a.vocab < 14 * kStreamStage) || (c > 2 && a.vocab < 6 * kStreamStage && 3 * N * c > 7 * ctx->sm_count)) c = 1;
     split(c);
   }
