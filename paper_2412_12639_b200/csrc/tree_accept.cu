@@ -614,8 +614,11 @@ int launch_tree_sample(falcon_ctx* ctx, const falcon_accept_args& a, cudaStream_
   };
   int ctas = 1;
   while (ctas < kSampleMaxCluster && a.vocab > ctas * kStreamStage && room(2 * ctas)) ctas *= 2;
-  // (nearly one row per SM: two CTAs per SM share it no better; 145 rows of 20000 8.2 and 9.1, of 32000 9.2 and 9.5, of 64000 12.4 both)
-  if (ctas == 2 && N <= ctx->sm_count && 8 * N > 7 * ctx->sm_count && a.vocab < 6 * kStreamStage) ctas = 1;
+  // From nearly one row per SM on, rows of up to six stages share it no better in pairs (us with 1 / 2 CTAs, alone and behind an
+  // attention launch: 126 rows of 32000 9.8 / 9.7  22.3 / 22.0, 130 of 20000 8.7 / 9.0  21.2 / 21.4, of 32000 10.2 / 9.9  22.4 / 22.3, 148 of 32000
+  // 10.4 / 10.8  22.6 / 22.9, of 49152 12.1 / 12.4  24.2 / 24.3, of 90112 16.1 / 16.7  28.7 / 28.3; 170 of 12000 8.3 / 8.3  20.3 / 20.5, of 32000
+  // 11.0 / 11.1  22.8 / 23.5, of 49152 12.9 / 12.7  24.5 / 24.9, of 90112 17.6 / 17.3  32.2 / 29.4; 222 of 20000 9.9 / 10.4  21.9 / 22.5).
+  if (ctas == 2 && 8 * N > 7 * ctx->sm_count && a.vocab <= 6 * kStreamStage) ctas = 1;
   const int chunk_len = ((a.vocab + ctas - 1) / ctas + 3) & ~3;
   int rc = ensure_tickets(ctx, static_cast<size_t>(B), s);
   if (rc) return rc;

@@ -652,13 +652,18 @@ int launch_tree_topm(falcon_ctx* ctx, const falcon_topm_args& a, cudaStream_t s)
   split(c);
   const bool in_regs = !short_stream && per_lane <= kTopmRowsMax && fits();
   if (!in_regs) {
-    // CTAs of a cluster where the rows alone leave SMs idle (us with 1 / 2 / 4 CTAs): 64 rows of 50257 10.2 / 9.5 / 8.9, 100 of
-    // 40000 9.2 / 10.0 / 9.7, 120 of 50257 10.9 / 12.0 / 16.0, 120 of 128256 19.0 / 17.5 / 23.0.  More rows than SMs: two, which
-    // even out better where the SMs become free one by one (158 of 32000 alone 9.3 and 10.3 or, from L2, 8.0 both; behind an
-    // attention launch 0.8 less with two).
+    // CTAs of a cluster where the rows alone leave SMs idle: four and eight wherever they have room (us with 1 / 2 / 4 CTAs, alone
+    // and behind an attention launch: 60 rows of 40000 9.0 / 8.9 / 8.8  22.7 / 21.8 / 20.9, 87 of 32769 8.1 / 9.3 / 8.4  21.4 / 21.6 /
+    // 20.5, 100 of 49151 10.2 / 10.6 / 10.2  24.1 / 22.9 / 22.7).  Two (1 / 2 CTAs):
+    //   up to nine tenths of a row per SM, where the pairs are given two places per SM: rows of more than seven stages
+    //     110 of 32769 8.3 / 9.6  21.5 / 22.0, of 49151 10.3 / 10.9  24.1 / 23.1, 120 of 57344 11.3 / 11.9  25.1 / 24.2, of 64000 12.3 / 12.2
+    //     26.2 / 24.5, of 114688 17.9 / 15.7  32.4 / 28.2
+    //   up to one: 135 of 64000 12.5 / 14.3  26.4 / 26.6, 140 of 90112 15.5 / 17.4  29.8 / 29.5, of 114688 18.3 / 18.7  32.9 / 31.3
+    //   more: 149 of 32768 9.7 / 10.4  21.7 / 22.6, 170 of 64000 14.7 / 15.1  26.7 / 27.2, of 90112 18.2 / 18.0  33.4 / 30.3, of 131072 22.9 / 20.7
+    //     39.2 / 33.2, 222 of 64000 15.2 / 16.5  27.2 / 28.5, of 131072 24.1 / 24.9  40.3 / 36.9
     c = 1;
     while (c < kTopmMaxCluster && streams(2 * c) && a.vocab >= 2 * c * kStreamStage) c *= 2;
-    if ((c == 2 && N <= ctx->sm_count && a.vocab < 14 * kStreamStage) || (c > 2 && a.vocab < 6 * kStreamStage && 3 * N * c > 7 * ctx->sm_count)) c = 1;
+    if (c == 2 && a.vocab <= (10 * rows <= 9 * sm ? 7 : rows <= sm ? 13 : 10) * kStreamStage) c = 1;
     split(c);
   }
   p.chunk_len = chunk;

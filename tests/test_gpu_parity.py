@@ -793,7 +793,8 @@ def test_topm_bit_exact(N, V, stride, m):
                                    (49, 40003, 8), (86, 40003, 8), (104, 49152, 3), (104, 114687, 9), (104, 114688, 9), (210, 114690, 2), (211, 114690, 2),
                                    (52, 16386, 20), (53, 16386, 20), (61, 32768, 20), (62, 32768, 20), (61, 24577, 32), (87, 40003, 8), (103, 49151, 8),
                                    (103, 49152, 8), (100, 32768, 20), (101, 32768, 20), (100, 49160, 8), (101, 49160, 8), (45, 131080, 8), (46, 131080, 8),
-                                   (222, 114690, 2), (223, 114690, 2)])
+                                   (222, 114690, 2), (223, 114690, 2), (133, 57344, 8), (133, 57345, 8), (134, 57345, 8), (148, 106496, 3), (148, 106497, 3),
+                                   (149, 81920, 3), (149, 81921, 3)])
 def test_topm_on_both_sides_of_every_line_of_the_dispatch(N, V, m):
     """How many CTAs share a row, and whether it is held in registers or streamed: one CTA's registers, stages of one CTA,
     clusters as far as they have room.  Values repeat, so that ties cross the borders of lanes, warps and CTAs."""
@@ -919,7 +920,7 @@ def test_sample_equal_logits_are_bit_exact(V, stride):
                                  (4, 8192), (4, 8193), (6, 16388), (48, 32772), (49, 32772), (103, 16388), (104, 16388), (129, 16384), (130, 16384),
                                  (130, 49152), (210, 16384), (211, 16384), (1, 2000), (74, 2000), (75, 4096), (37, 4095), (38, 4095), (9, 9830),
                                  (9, 9832), (49, 9832), (50, 9832), (24, 19664), (25, 19664), (148, 28672), (149, 28672), (74, 57344), (75, 57344),
-                                 (45, 65540), (46, 65540), (100, 32772), (101, 32772), (222, 49152), (223, 49152)])
+                                 (45, 65540), (46, 65540), (100, 32772), (101, 32772), (222, 49152), (222, 49153), (223, 49153)])
 def test_streamed_rows_on_both_sides_of_every_share_of_an_sm(N, V):
     """Greedy and drawn tokens where the number of CTAs passes one, one and a half, two and three per SM, alone and in
     clusters: how much shared memory a CTA is given, and how many share a row.  Greedy rows repeat values, drawn rows
