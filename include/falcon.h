@@ -79,6 +79,11 @@ const char* falcon_last_error(const falcon_ctx* ctx);
  * reads on-chip memory it has not written itself then shows it in its results, instead of
  * working by the luck of what an earlier launch left there.  Harmless: plain stores. */
 int falcon_test_poison(falcon_ctx* ctx, uint32_t pattern, void* stream);
+/* Test hook: the calls on this context that stream logits rows (falcon_topm, falcon_tree_accept) never
+ * ask for the given stage (0, 1, ...; -1: all of them are asked for, as always) of a row's copies, so
+ * that the bounded waits for it run out: falcon_topm reads such a row again and is still right, the
+ * acceptance sets FALCON_DEV_TIMEOUT. */
+int falcon_test_stall_scans(falcon_ctx* ctx, int32_t stage);
 /* Host check of one tree: FALCON_OK iff T in [1, FALCON_T_MAX], parent[0] == -1
  * and 0 <= parent[i] < i.  `parent` is a HOST pointer. */
 int falcon_tree_validate_host(const int32_t* parent, int32_t T);

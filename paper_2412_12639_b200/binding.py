@@ -108,6 +108,8 @@ def load_library():
         fn.restype = C.c_int
     lib.falcon_test_poison.argtypes = [C.c_void_p, C.c_uint32, C.c_void_p]
     lib.falcon_test_poison.restype = C.c_int
+    lib.falcon_test_stall_scans.argtypes = [C.c_void_p, C.c_int32]
+    lib.falcon_test_stall_scans.restype = C.c_int
     lib.falcon_tree_attn_kernel.argtypes = [C.c_void_p, C.POINTER(AttnArgs)]
     lib.falcon_tree_attn_kernel.restype = C.c_int
     lib.falcon_tree_accept_static.argtypes = [C.POINTER(AcceptArgs), C.c_void_p]
@@ -243,6 +245,12 @@ class Context:
         """Test hook: every SM's shared and tensor memory filled with `pattern`."""
         rc = self._lib.falcon_test_poison(self._h, pattern, _stream(stream))
         self._check(rc, "falcon_test_poison")
+        return rc
+
+    def falcon_test_stall_scans(self, stage: int) -> int:
+        """Test hook: streamed calls never ask for this stage of a row (-1: they do again)."""
+        rc = self._lib.falcon_test_stall_scans(self._h, stage)
+        self._check(rc, "falcon_test_stall_scans")
         return rc
 
     def falcon_feature_gather(self, args: GatherArgs, stream=None, check: bool = True) -> int:

@@ -24,6 +24,7 @@ struct falcon_ctx {
   // Scratch blocks that were outgrown.  A launch already enqueued, or captured into a CUDA graph,
   // may still name them, so they live until falcon_destroy.
   std::vector<void*> retired;
+  int test_stall_stage = -1;  // test hook: see falcon_test_stall_scans
   std::string last_error;
   // Cached TMA descriptors (opaque here; owned by tc_util.cuh).
   void* tmap_cache = nullptr;

@@ -181,6 +181,12 @@ int falcon_test_poison(falcon_ctx* ctx, uint32_t pattern, void* stream) {
   return launch_test_poison(ctx, pattern, static_cast<cudaStream_t>(stream));
 }
 
+int falcon_test_stall_scans(falcon_ctx* ctx, int32_t stage) {
+  if (!ctx) return FALCON_ERR_INVALID_ARG;
+  ctx->test_stall_stage = stage;
+  return FALCON_OK;
+}
+
 int falcon_tree_attn_kernel(falcon_ctx* ctx, const falcon_attn_args* a) {
   int kernel = -1;
   return attn_plan(ctx, a, &kernel) == FALCON_OK ? kernel : -1;

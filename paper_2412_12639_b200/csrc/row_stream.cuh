@@ -113,15 +113,17 @@ struct RowStream {
     b->abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  // The copying thread: stages [i0, i1), in order.
-  __device__ __forceinline__ void produce(int i0, int i1) const {
+  // The copying thread: stages [i0, i1), in order, without stage `stall` (a test hook: the waits for that one run out).
+  __device__ __forceinline__ void produce(int i0, int i1, int stall) const {
     for (int i = i0; i < i1; ++i) {
       const int st = i % kStreamStages;
       const uint32_t full = bars + 8u * st;
       if (i >= kStreamStages && !tc::mbar_wait(bars + 8u * (kStreamStages + st), (i / kStreamStages - 1) & 1, abort)) {
-        for (int k = i - kStreamStages; k < i; ++k) tc::mbar_wait_drain(bars + 8u * (k % kStreamStages), (k / kStreamStages) & 1);
+        for (int k = i - kStreamStages; k < i; ++k)
+          if (k != stall) tc::mbar_wait_drain(bars + 8u * (k % kStreamStages), (k / kStreamStages) & 1);
         return;
       }
+      if (i == stall) continue;
       const uint32_t bytes = static_cast<uint32_t>(min(kStreamStage, body - i * kStreamStage)) * 4u;
       tc::mbar_expect_tx(full, bytes);
       asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(buf + st * kStreamStage * 4u),
@@ -130,7 +132,8 @@ struct RowStream {
     }
     // (until the last copies have landed: none may be in flight when the CTA leaves, whatever became of its waits)
     if (i1 == stages())
-      for (int k = max(0, i1 - kStreamStages); k < i1; ++k) tc::mbar_wait_drain(bars + 8u * (k % kStreamStages), (k / kStreamStages) & 1);
+      for (int k = max(0, i1 - kStreamStages); k < i1; ++k)
+        if (k != stall) tc::mbar_wait_drain(bars + 8u * (k % kStreamStages), (k / kStreamStages) & 1);
   }
   // Entry e (0 .. 3) of the lane's j-th 16-byte piece of stage i, counted from `base`.
   __device__ __forceinline__ int index(int i, int j, int e) const {

@@ -30,6 +30,7 @@ struct AcceptParams {
   float* part_val;  // [N, chunks]
   int32_t* part_idx;
   int* tickets;     // [B]
+  int32_t stall;    // test hook: see RowStream::produce
   // non-greedy only
   float inv_t_log2e;       // log2(e) / temperature
   const float* uniforms;   // [N]
@@ -159,7 +160,7 @@ __global__ void __launch_bounds__(kAcceptThreads + (kStream ? 32 : 0)) tree_acce
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if constexpr (kStream) {
     if (warp_index() == kStreamWarps) {
-      if ((tid & 31) == 0) rs.produce(0, rs.stages());
+      if ((tid & 31) == 0) rs.produce(0, rs.stages(), p.stall);
       return;
     }
   }
@@ -321,7 +322,7 @@ __global__ void __launch_bounds__(kStreamThreads + 32, 3) tree_sample_kernel(con
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (warp == kStreamWarps) {  // (gone by the time of the next barrier: all copies have landed then)
-    if (lane == 0) rs.produce(0, rs.stages());
+    if (lane == 0) rs.produce(0, rs.stages(), p.stall);
     return;
   }
   // sequence that owns this row (its loads overlap the scan below)
@@ -555,6 +556,7 @@ AcceptParams accept_params(const falcon_accept_args& a, int chunks, int chunk_le
   p.part_val = static_cast<float*>(part);
   p.part_idx = reinterpret_cast<int32_t*>(part) + static_cast<size_t>(a.tree.total_nodes) * chunks;
   p.tickets = tickets;
+  p.stall = -1;
   p.inv_t_log2e = 0.f;
   p.uniforms = nullptr;
   p.slices = 0;
@@ -583,7 +585,8 @@ int launch_tree_accept(falcon_ctx* ctx, const falcon_accept_args& a, cudaStream_
   if (rc) return rc;
   rc = ensure_tickets(ctx, a.tree.batch, s);
   if (rc) return rc;
-  const AcceptParams p = accept_params(a, chunks, chunk_len, ctx->ws, ctx->tickets);
+  AcceptParams p = accept_params(a, chunks, chunk_len, ctx->ws, ctx->tickets);
+  p.stall = ctx->test_stall_stage;
 
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(chunks, N);
@@ -625,6 +628,7 @@ int launch_tree_sample(falcon_ctx* ctx, const falcon_accept_args& a, cudaStream_
   AcceptParams p = accept_params(a, 1, chunk_len, nullptr, ctx->tickets);
   p.slices = kStreamWarps * ((chunk_len + kStreamStage - 1) / kStreamStage) + 2;
   p.uniforms = a.uniforms;
+  p.stall = ctx->test_stall_stage;
   p.inv_t_log2e = kLog2e / a.temperature;
   if (ctas * p.slices > kMaxSlices) return FALCON_ERR_CAPACITY;  // (not reached: 8 x 34 and 258 at most)
 

@@ -50,6 +50,7 @@ struct TopmParams {
   int32_t vocab, m;
   int32_t chunk_len;   // entries per CTA of the cluster
   int32_t steps;       // in which the exact route takes a CTA's share: of 256 x (entries per lane)
+  int32_t stall;       // test hook: see RowStream::produce
   int64_t logits_stride;
   const float* logits;
   float* top_val;
@@ -517,14 +518,14 @@ __global__ void __launch_bounds__(kStreamThreads + 32, 3) tree_topm_stream_kerne
   if (warp == kStreamWarps) {
     // The cluster barriers of first_tau() count this warp too: it goes through them once the ring is full, and
     // has left before the next one (all stages are issued by the time the last is taken).
-    if (lane == 0) rs.produce(0, min(n_st, kStreamStages));
+    if (lane == 0) rs.produce(0, min(n_st, kStreamStages), p.stall);
     __syncwarp();
     if (n_ctas > 1) {
       row_wait(n_ctas);
       row_arrive(n_ctas);
       row_wait(n_ctas);
     }
-    if (lane == 0) rs.produce(min(n_st, kStreamStages), n_st);
+    if (lane == 0) rs.produce(min(n_st, kStreamStages), n_st, p.stall);
     return;
   }
   {
@@ -543,18 +544,20 @@ __global__ void __launch_bounds__(kStreamThreads + 32, 3) tree_topm_stream_kerne
       const float xe[1] = {in ? __ldcs(rowp + i) : -INFINITY};
       append<1>(sh, xe, tau, in ? 1u : 0u, false, lane, [&](int) { return c0 + i; }, [&](int) { return xe[0]; });
     }
-    for (int st = 0; ok && st < n_st; ++st) {
-      if (st > 0) {
+    // (a warp whose wait gave up takes no further stage but comes to the same barriers as the others)
+    for (int st = 0; st < n_st; ++st) {
+      if (st > 0 && ok) {
         ok = rs.take(st, x);
-        if (!ok) break;
         lm = -INFINITY;
 #pragma unroll
         for (int k = 0; k < kStreamLane; ++k) lm = fmaxf(lm, x[k]);
       }
-      if (tau <= to_key(-INFINITY) || __any_sync(0xffffffffu, to_key(lm) >= tau))
-        append<kStreamLane>(sh, x, tau, rs.live(st), false, lane, [&](int k) { return c0 + rs.head + rs.index(st, k >> 2, k & 3); },
-                            [&](int k) { return rs.value(st, k); });
-      rs.give_back(st);
+      if (ok) {
+        if (tau <= to_key(-INFINITY) || __any_sync(0xffffffffu, to_key(lm) >= tau))
+          append<kStreamLane>(sh, x, tau, rs.live(st), false, lane, [&](int k) { return c0 + rs.head + rs.index(st, k >> 2, k & 3); },
+                              [&](int k) { return rs.value(st, k); });
+        rs.give_back(st);
+      }
       if (((st + 1) & st) == 0 && st > 0 && st + 1 < n_st) {  // 2, 4, 8, ... stages seen
         worker_sync();
         if (sh.cnt <= kList) tau = max(tau, thin_list(sh, m, tid));  // (beyond: the exact route)
@@ -599,6 +602,7 @@ int launch_tree_topm(falcon_ctx* ctx, const falcon_topm_args& a, cudaStream_t s)
   TopmParams p;
   p.vocab = a.vocab;
   p.m = a.m;
+  p.stall = ctx->test_stall_stage;
   p.logits_stride = a.logits_stride;
   p.logits = a.logits;
   p.top_val = a.top_val;

@@ -827,6 +827,50 @@ def test_topm_many_rows_and_overflowing_lists(N, V, stride, m, kind):
         np.testing.assert_array_equal(gv, rv)
 
 
+@pytest.mark.parametrize("N,V,stages", [(150, 60001, (0, 1, 3, 7)), (60, 200003, (0, 2, 5)), (20, 131075, (1,))])
+def test_topm_bounded_wait_runs_out(N, V, stages):
+    """A stage of every row is never asked for (one CTA per row, clusters of four and of eight): the warps that give up still come to
+    the barriers at which the list is thinned, after 2, 4, ... stages, and the row is read again on the exact route."""
+    rng = np.random.default_rng(N)
+    x = (rng.integers(-4000, 4000, size=(N, V)) / 16).astype(np.float32)
+    rv, ri = oracle.topm(x, 20)
+    c = H.ctx()
+    for stage in stages + (-1,):
+        c.falcon_test_stall_scans(stage)
+        try:
+            gv, gi, _ = H.run_topm(x, 20)
+        finally:
+            c.falcon_test_stall_scans(-1)
+        np.testing.assert_array_equal(gi, ri)
+        np.testing.assert_array_equal(gv, rv)
+
+
+@pytest.mark.parametrize("N,V,stage", [(150, 60001, 1), (60, 100003, 0), (150, 60001, 3)])
+def test_acceptance_bounded_wait_runs_out(N, V, stage):
+    """The same for greedy and drawn acceptance: the call returns, says so in the status word, and the next one is right."""
+    rng = np.random.default_rng(N)
+    tb = H.make_trees([N // 2, N - N // 2], [1, 0], rng, vocab=V)
+    dt = H.DevTrees(tb)
+    lg = (rng.integers(-2000, 2000, size=(N, V)) / 16).astype(np.float32)
+    flat = np.full((N, V), 1.25, dtype=np.float32)
+    u = (rng.integers(0, 1024, N) / 1024.0).astype(np.float32)
+    c = H.ctx()
+    for s in (stage, -1):
+        for kw, x in (({}, lg), ({"temperature": 1.3, "uniforms": u}, flat)):
+            dt.status.zero_()
+            c.falcon_test_stall_scans(s)
+            try:
+                g = H.run_accept(dt, x, **kw)[0]
+            finally:
+                c.falcon_test_stall_scans(-1)
+            assert g.min() >= 0 and g.max() < V
+            if s < 0:
+                assert not dt.status.cpu().numpy().any()
+                np.testing.assert_array_equal(g, np.floor(u.astype(np.float64) * V).astype(np.int32) if kw else oracle.argmax(x))
+            else:
+                assert (dt.status.cpu().numpy() & binding.DEV_TIMEOUT).all()
+
+
 def test_topm_ties_nan_inf_and_argmax_agreement():
     rng = np.random.default_rng(77)
     x = rng.standard_normal((6, 9000)).astype(np.float32)
