@@ -473,8 +473,8 @@ __global__ void __launch_bounds__(kStreamThreads + 32, 3) tree_sample_kernel(con
           w3 += x[e + 3];
         }
         const float ws = (w0 + w1) + (w2 + w3);
-        const float in = warp_scan(ws, lane), tot = __shfl_sync(0xffffffffu, in, 31);
-        const float resid = fminf(target - before, tot * 0.99999f);  // (summed another way the slice may come to a hair less)
+        const float in = warp_scan(ws, lane);
+        const float resid = target - before;  // (summed another way the slice may come to a hair less: its last entry with weight then)
         const unsigned pl = __ballot_sync(0xffffffffu, ws > 0.f && in > resid), al = __ballot_sync(0xffffffffu, ws > 0.f);
         const int wl = pl ? __ffs(static_cast<int>(pl)) - 1 : (al ? 31 - __clz(static_cast<int>(al)) : 0);
         // that lane's 32 weights dealt out over the lanes

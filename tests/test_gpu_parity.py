@@ -1002,6 +1002,18 @@ def test_sample_edge_sizes_and_the_last_representable_uniform():
         assert_valid_draws(lg, V, 0.9, u, g)
 
 
+@pytest.mark.parametrize("V,at", [(4096, 0), (4096, 3072), (40000, 1024), (40000, 37048), (200000, 53072)])
+def test_sample_reaches_the_last_light_tokens_of_a_slice(V, at):
+    # weights 1 and 2^-18 in the same 1024 entries of a CTA's share of the row (of 40000: 5000, of 200000: 25000; temperature log2(e): powers of two, every sum exact in fp32) and u = 1 - 2^-20: the
+    # target 1 + 2^-18 - 2^-20 lies in the light token's interval, which is the slice's last 4e-6
+    lg = np.full((3, V), -np.inf, dtype=np.float32)
+    lg[:, at + 100], lg[:, at + 900] = 0.0, -18.0
+    u = np.array([1.0 - 2.0 ** -20, 0.5, 1.0 - 2.0 ** -17], dtype=np.float32)
+    tb = H.make_trees([3], [0], np.random.default_rng(3), vocab=V)
+    g = H.run_accept(H.DevTrees(tb), lg, temperature=float(np.float32(1.4426950408889634)), uniforms=u)[0]
+    assert g.tolist() == [at + 900, at + 100, at + 100]
+
+
 def test_sample_special_values_and_the_greedy_limit():
     rng = np.random.default_rng(31)
     tb = H.make_trees([12, 20], [4, 4], rng, vocab=9000)
