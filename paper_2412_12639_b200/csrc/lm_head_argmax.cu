@@ -364,30 +364,33 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_con
           const int v0 = v_lo + (v_res > 1 ? vp * 2 + sub : vp) * kLmTileMax + rank * 128 + q * 32;  // lane 0's vocabulary row
           if (v0 < v_hi && (v_res > 1 || sub < tiles_of(g))) {
             const bool exists = v0 + lane < v_hi;
-            uint32_t ring[2][32];               // the next columns' load runs under these columns' maxima
+            // The next columns' load runs under these columns' maxima.  It is asked for whether they exist or not: the values of
+            // a load under a condition would be merged with older ones before the wait for it.
+            uint32_t ring[2][32];
             FALCON_TMEM_LD32(tmem_lane, ring[0]);
 #pragma unroll
-            for (int k = 0; k < kLmTileMax / 32; ++k)
-              if (k * 32 < n_cols) {
-                uint32_t(&x)[32] = ring[k & 1];
-                tmem_wait_ld();
-                if ((k + 1) * 32 < n_cols) FALCON_TMEM_LD32(tmem_lane + static_cast<uint32_t>((k + 1) * 32), ring[(k + 1) & 1]);
-                float m_mine = -INFINITY;
-                uint32_t who_mine = 0u;
+            for (int k = 0; k < kLmTileMax / 32; ++k) {
+              uint32_t(&x)[32] = ring[k & 1];
+              tmem_wait_ld(x);
+              FALCON_TMEM_LD32(tmem_lane + static_cast<uint32_t>((k + 1) * 32 < n_cols ? (k + 1) * 32 : 0), ring[(k + 1) & 1]);
+              if (k * 32 >= n_cols) continue;
+              float m_mine = -INFINITY;
+              uint32_t who_mine = 0u;
 #pragma unroll
-                for (int c = 0; c < 32; ++c) {
-                  const float f = exists ? __uint_as_float(x[c]) : -INFINITY, m = warp_largest(f);
-                  const uint32_t who = __ballot_sync(0xffffffffu, f == m);
-                  if (lane == c) {
-                    m_mine = m;
-                    who_mine = who;
-                  }
-                }
-                if (m_mine > best[k]) {  // strict: vocabulary rows ascend over the passes, so the first maximum stays
-                  best[k] = m_mine;
-                  idx[k] = v0 + __ffs(static_cast<int>(who_mine)) - 1;
+              for (int c = 0; c < 32; ++c) {
+                const float f = exists ? __uint_as_float(x[c]) : -INFINITY, m = warp_largest(f);
+                const uint32_t who = __ballot_sync(0xffffffffu, f == m);
+                if (lane == c) {
+                  m_mine = m;
+                  who_mine = who;
                 }
               }
+              if (m_mine > best[k]) {  // strict: vocabulary rows ascend over the passes, so the first maximum stays
+                best[k] = m_mine;
+                idx[k] = v0 + __ffs(static_cast<int>(who_mine)) - 1;
+              }
+            }
+            tmem_wait_ld();
           }
           tc_fence_before();
           __syncwarp();
@@ -444,18 +447,20 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_con
             }
         };
         if (begin < end) {
+          // (as above: the loads are unconditional, and take the last columns again behind the end)
+          const int last = begin + ((end - begin - 1) & ~31);
           uint32_t x0[32], x1[32];
           FALCON_TMEM_LD32(tmem_lane + static_cast<uint32_t>(begin), x0);
-          tmem_wait_ld();
-          for (int c0 = begin; c0 < end; c0 += 64) {
-            if (c0 + 32 < end) FALCON_TMEM_LD32(tmem_lane + static_cast<uint32_t>(c0 + 32), x1);
+          tmem_wait_ld(x0);
+          for (int c0 = begin;; c0 += 64) {
+            FALCON_TMEM_LD32(tmem_lane + static_cast<uint32_t>(min(c0 + 32, last)), x1);
             look(x0, c0);
-            tmem_wait_ld();
-            if (c0 + 32 < end) {
-              if (c0 + 64 < end) FALCON_TMEM_LD32(tmem_lane + static_cast<uint32_t>(c0 + 64), x0);
-              look(x1, c0 + 32);
-              tmem_wait_ld();
-            }
+            tmem_wait_ld(x1);
+            if (c0 + 32 > last) break;
+            FALCON_TMEM_LD32(tmem_lane + static_cast<uint32_t>(min(c0 + 64, last)), x0);
+            look(x1, c0 + 32);
+            tmem_wait_ld(x0);
+            if (c0 + 64 > last) break;
           }
         }
         tc_fence_before();
