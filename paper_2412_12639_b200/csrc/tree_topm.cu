@@ -493,6 +493,17 @@ __global__ void __launch_bounds__(kTopmThreads, kRows <= 8 ? 6 : (kRows <= 16 ? 
   finish_row<kRows>(p, sh, rowp, n, c0, rank, n_ctas, row);
 }
 
+// Whether a CTA's list is thinned behind stage st: when 2, 4, 8, ... stages have been seen and more follow.
+__device__ __forceinline__ bool thins_behind(int st, int n_st) { return ((st + 1) & st) == 0 && st > 0 && st + 1 < n_st; }
+// For a warp whose wait for stage st gave up: it takes no further stage but comes to the same barriers as the others.
+__device__ __noinline__ void thin_with_the_others(TopmShared& sh, int m, int tid, int st, int n_st) {
+  for (; st < n_st; ++st)
+    if (thins_behind(st, n_st)) {
+      worker_sync();
+      if (sh.cnt <= kList) thin_list(sh, m, tid);
+    }
+}
+
 // The row streamed through shared memory, 8192 entries of a CTA at a time.
 __global__ void __launch_bounds__(kStreamThreads + 32, 3) tree_topm_stream_kernel(const __grid_constant__ TopmParams p) {
   extern __shared__ __align__(128) unsigned char stream_buf[];
@@ -544,25 +555,25 @@ __global__ void __launch_bounds__(kStreamThreads + 32, 3) tree_topm_stream_kerne
       const float xe[1] = {in ? __ldcs(rowp + i) : -INFINITY};
       append<1>(sh, xe, tau, in ? 1u : 0u, false, lane, [&](int) { return c0 + i; }, [&](int) { return xe[0]; });
     }
-    // (a warp whose wait gave up takes no further stage but comes to the same barriers as the others)
-    for (int st = 0; st < n_st; ++st) {
-      if (st > 0 && ok) {
+    int st = 0;
+    for (; ok && st < n_st; ++st) {
+      if (st > 0) {
         ok = rs.take(st, x);
+        if (!ok) break;
         lm = -INFINITY;
 #pragma unroll
         for (int k = 0; k < kStreamLane; ++k) lm = fmaxf(lm, x[k]);
       }
-      if (ok) {
-        if (tau <= to_key(-INFINITY) || __any_sync(0xffffffffu, to_key(lm) >= tau))
-          append<kStreamLane>(sh, x, tau, rs.live(st), false, lane, [&](int k) { return c0 + rs.head + rs.index(st, k >> 2, k & 3); },
-                              [&](int k) { return rs.value(st, k); });
-        rs.give_back(st);
-      }
-      if (((st + 1) & st) == 0 && st > 0 && st + 1 < n_st) {  // 2, 4, 8, ... stages seen
+      if (tau <= to_key(-INFINITY) || __any_sync(0xffffffffu, to_key(lm) >= tau))
+        append<kStreamLane>(sh, x, tau, rs.live(st), false, lane, [&](int k) { return c0 + rs.head + rs.index(st, k >> 2, k & 3); },
+                            [&](int k) { return rs.value(st, k); });
+      rs.give_back(st);
+      if (thins_behind(st, n_st)) {
         worker_sync();
         if (sh.cnt <= kList) tau = max(tau, thin_list(sh, m, tid));  // (beyond: the exact route)
       }
     }
+    if (!ok) thin_with_the_others(sh, m, tid, st, n_st);
     if (!ok && lane == 0) atomicAdd(&sh.cnt, kList + 1);  // a wait gave up: the exact route reads the row itself
   }
   worker_sync();
