@@ -617,11 +617,15 @@ int launch_tree_sample(falcon_ctx* ctx, const falcon_accept_args& a, cudaStream_
   };
   int ctas = 1;
   while (ctas < kSampleMaxCluster && a.vocab > ctas * kStreamStage && room(2 * ctas)) ctas *= 2;
-  // From nearly one row per SM on, rows of up to six stages share it no better in pairs (us with 1 / 2 CTAs, alone and behind an
-  // attention launch: 126 rows of 32000 9.8 / 9.7  22.3 / 22.0, 130 of 20000 8.7 / 9.0  21.2 / 21.4, of 32000 10.2 / 9.9  22.4 / 22.3, 148 of 32000
-  // 10.4 / 10.8  22.6 / 22.9, of 49152 12.1 / 12.4  24.2 / 24.3, of 90112 16.1 / 16.7  28.7 / 28.3; 170 of 12000 8.3 / 8.3  20.3 / 20.5, of 32000
-  // 11.0 / 11.1  22.8 / 23.5, of 49152 12.9 / 12.7  24.5 / 24.9, of 90112 17.6 / 17.3  32.2 / 29.4; 222 of 20000 9.9 / 10.4  21.9 / 22.5).
-  if (ctas == 2 && 8 * N > 7 * ctx->sm_count && a.vocab <= 6 * kStreamStage) ctas = 1;
+  // Between nine tenths of a row per SM (the pairs are no longer given two places per SM, see stream_bytes) and one, rows of up to six
+  // stages share it no better in pairs (us with 1 / 2 CTAs: logits in L2, not in L2, and behind an attention launch):
+  //   130 rows of 20000   7.2 / 7.4    7.3 / 7.4   26.0 / 25.5       of 32000  8.1 / 7.7    9.4 / 9.3   27.2 / 26.3
+  //   140         20000   7.2 / 7.9    7.8 / 8.4   26.1 / 26.0          38144  8.8 / 9.4   10.3 / 10.9  28.3 / 27.9
+  //   148         38144   8.9 / 9.4   10.4 / 10.9  28.9 / 28.7          49152  9.4 / 9.6   11.1 / 11.4  29.7 / 29.2
+  //               60000  10.8 / 11.0  12.7 / 13.1  31.5 / 30.5
+  //   160         38144   9.7 / 9.3   11.0 / 11.1  29.2 / 29.1      178 of 38144  9.7 / 9.4  11.3 / 11.4  29.7 / 29.8
+  //   222         20000   7.9 / 8.0    9.4 / 9.9   29.5 / 29.7          49152 11.0 / 9.9   12.8 / 13.3  32.8 / 33.1
+  if (ctas == 2 && 10 * N > 9 * ctx->sm_count && N <= ctx->sm_count && a.vocab <= 6 * kStreamStage) ctas = 1;
   const int chunk_len = ((a.vocab + ctas - 1) / ctas + 3) & ~3;
   int rc = ensure_tickets(ctx, static_cast<size_t>(B), s);
   if (rc) return rc;
