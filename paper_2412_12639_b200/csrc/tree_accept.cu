@@ -507,12 +507,15 @@ constexpr int kAcceptMaxChunks = 8;  // vocabulary chunks per row at most (the s
 
 // How a launch splits the vocabulary, and whether its rows are streamed.  Shared by the two entry points so that
 // they cannot drift apart.  Chunks are doubled (3 chunks of 32000 fill their last stage by a third, 6.6 us where 2 take 5.9) as
-// long as they stay worth a CTA, which depends on how many CTAs an SM then has.  Streamed (us with 1 / 2 / 4 / 8 chunks):
-//   two thirds of one per SM, 0.6 of a stage: 16 rows of 12000 5.6 / 5.2 / 5.2 / 5.1, of 20000 6.1 / 5.8 / 5.5 / 5.4;
-//                                 behind attention over a batch 74 of 12000 30.0 / 30.8, 37 of 20000 - / 29.9 / 30.4
-//   up to 1.5, three quarters:    50 of 12000 5.4 / 5.0 / 5.6 / 6.2, 100 of 12000 5.4 / 5.6, 50 of 20000 5.7 / 5.4 / 5.7 / 6.2, 50 of 64000 7.3 / 6.2 / 6.3 / 6.5
-//   up to 2, one and three quarters: behind an attention launch 120 of 64000 21.5 / 20.4, 145 of 64000 22.2 / 21.0, of 128256 31.7 / 30.3,
-//                                 of 32000 19.4 / 19.1, of 20000 18.6 / 18.9; 65 of 128256 25.3 / 21.7 / 20.5
+// long as they stay worth a CTA.  Streamed: 0.6 of a stage, up to two CTAs per SM (us with 1 / 2 / 4 / 8 chunks, logits in L2 and behind
+// an attention launch over a batch of 300 to 3900 keys):
+//    25 rows of 8192   4.0 / 4.1    23.8 / 24.2         of 12000  4.3 / 4.0 / 4.2   24.4 / 24.3 / 24.3     of 40000  5.4 / 4.7 / 4.6 / 4.7  25.9 / 25.4 / 24.9 / 24.7
+//    50         9832   4.4 / 4.2    37.4 / 37.4            20000  4.7 / 4.6 / 4.6   37.8 / 37.8 / 37.6        40000  5.4 / 4.9 / 5.2 / 5.1  39.4 / 38.8 / 38.6 / 38.7
+//    74         8192   4.0 / 4.2    38.6 / 38.7            20000  4.8 / 4.7 / 4.6   40.0 / 39.6 / 39.2        40000  5.5 / 5.0 / 5.2 / 7.2  41.8 / 41.2 / 41.1 / 43.0
+//    75        12000   4.6 / 4.6    39.4 / 39.1            20000  4.9 / 5.0 / 5.2   40.1 / 39.8 / 39.8        40000  5.6 / 5.6 / 5.9 / 7.1  41.9 / 41.4 / 41.7 / 42.6
+//   110         8192   4.1 / 4.5    41.7 / 41.8            12000  4.7 / 4.6 / 5.0   42.6 / 42.2 / 42.5        20000  5.0 / 5.1 / 5.0        43.7 / 43.4 / 43.3
+//   148         8192   4.1 / 4.6    47.6 / 47.6            12000  4.7 / 4.6 / 7.1   48.9 / 48.4 / 51.0        40000  5.7 / 5.8 / 8.4        51.4 / 50.8 / 53.6
+//   149 rows of 12000 behind one sequence 23.2 / 23.0, 20000 24.4 / 24.6, 64000 28.6 / 28.1; 170 of 12000 24.0 / 23.9, 32000 26.3 / 26.4 (not taken)
 // Short rows fit the registers of one pass, and the ring's set-up would only add to it (15 rows of 1000: 4.1 against 4.4); a
 // chunk of them is 2048 entries, or 1000 while there are no more CTAs than SMs (30 rows of 4000 5.3 / 5.1 / 4.9; 100 5.4 / 5.4, behind
 // attention 17.9 / 18.4).
@@ -523,7 +526,7 @@ bool accept_plan(int sm_count, int n_nodes, int vocab, int* chunks_out, int* chu
     const int64_t ctas = static_cast<int64_t>(n_nodes) * c;
     if (!streamed) return ctas <= kAcceptChunksPerSm * sm_count && vocab / c >= (ctas <= sm_count ? 1000 : 2048);
     static_assert(kAcceptChunksPerSm >= 2, "the scratch is sized by it");
-    return ctas <= 2 * sm_count && vocab / c >= (3 * ctas <= 2 * sm_count ? kStreamStage * 3 / 5 : 2 * ctas <= 3 * sm_count ? kStreamStage * 3 / 4 : kStreamStage * 7 / 4);
+    return ctas <= 2 * sm_count && vocab / c >= kStreamStage * 3 / 5;
   };
   while (chunks < kAcceptMaxChunks && worth(2 * chunks)) chunks *= 2;
   int chunk_len = (vocab + chunks - 1) / chunks;
