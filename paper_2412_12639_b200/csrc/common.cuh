@@ -98,12 +98,21 @@ __device__ __forceinline__ void dev_status_or(int32_t* status, int b, int bits) 
 // One more arrival at a counter; returns how many there were before.  What the calling thread wrote before it, and what its CTA
 // wrote before a barrier in front of it, is visible to whoever sees the count, and the other way round: after a barrier behind it
 // the CTA that came last may read (past L1) what all others wrote.  One ordered atomic in place of a sequentially
-// consistent fence, an atomic and another such fence: 0.35 us of every acceptance (60 rows of 1000 4.9 -> 4.4 us, 60 of 32000 5.7 -> 5.3, 200
-// of 32000 7.3 -> 6.9), 0.3 to 0.4 of a drawn one (60 of 32000 8.1 -> 7.7).
+// consistent fence, an atomic and another such fence: 0.4 to 0.5 us of every acceptance (60 rows of 1000 4.9 -> 4.4 us, 60 of 32000 5.7 -> 5.3,
+// 200 of 32000 7.3 -> 6.9), 0.4 of a drawn one (60 of 32000 8.1 -> 7.7).
 __device__ __forceinline__ int arrive_acq_rel(int* counter) {
   int before;
   asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(before) : "l"(counter) : "memory");
   return before;
+}
+
+// Largest of one float per lane (a NaN never is, unless all are) in one instruction: five shuffles are 0.1 us of every chain they are in (60
+// rows of 1000: acceptance 4.5 -> 4.4 us; drawn acceptance, with four chains for a lane's maximum and sum, 6.3 -> 6.0, 411 rows of 32000
+// 15.3 -> 14.8).
+__device__ __forceinline__ float warp_largest(float x) {
+  float m;
+  asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(m) : "f"(x));
+  return m;
 }
 
 // Bit t of a 128-bit set stored as two 64-bit words.

@@ -21,7 +21,7 @@
 //   kLmLanes   vocabulary rows on the lanes, 256 a pair: up to 256 nodes and two such blocks, or up to 512 nodes in two tiles.
 //              The nodes then come in steps of 16 where kLmPair pads them to 256; the launcher says when it is taken.
 // What bounds them is the power limit (512 nodes of 5120 x 32000 run at 1.3 PFLOP/s, 1.5 GHz, padding counted; a cuBLAS loop
-// holds 1.38), then the round trip of the ring: two stages of up to 94 KB, about 4900 cycles between a stage's MMAs and the
+// holds 1.38), then the round trip of the ring: two stages of up to 96 KB, about 4900 cycles between a stage's MMAs and the
 // next ones, 3600 of which are the MMAs'.  32000 x 5120, single CTAs and pairs: 512 nodes 157 -> 130 us, 300 nodes 147 -> 113,
 // 256 nodes 78 -> 72.
 //
@@ -133,13 +133,6 @@ __device__ __forceinline__ void arrive_remote(uint32_t bar) {
 
 // The arrangements: one CTA, nodes on the lanes; pairs of CTAs, nodes on the lanes; pairs, vocabulary rows on the lanes.
 constexpr int kLmSingle = 0, kLmPair = 1, kLmLanes = 2;
-
-// Largest of one float per lane (a NaN never is, unless all are).
-__device__ __forceinline__ float warp_largest(float x) {
-  float m;
-  asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(m) : "f"(x));
-  return m;
-}
 
 template <int kMode>
 __global__ void __launch_bounds__(kLmThreads, 1)

@@ -55,14 +55,6 @@ __device__ __forceinline__ void take(Best& s, float x, int i) {
   }
 }
 
-// The largest of the lanes' values (none a NaN) in one instruction: five shuffles are 0.1 us of every chain they are in (60 rows of
-// 1000: acceptance 4.5 -> 4.4 us; drawn acceptance, with four chains for a lane's maximum and sum, 6.3 -> 6.0, 411 rows of 32000 15.3 -> 14.8).
-__device__ __forceinline__ float lanes_max(float x) {
-  float m;
-  asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(m) : "f"(x));
-  return m;
-}
-
 // A node's parent and drafted token, for the thread that has it in the search below: loaded early, where the
 // trip to L2 is hidden.
 struct NodeOf {
@@ -212,7 +204,7 @@ __global__ void __launch_bounds__(kAcceptThreads + (kStream ? 32 : 0)) tree_acce
     if (tid < c1 - t0) take(mine, __ldcs(rowp + t0 + tid), t0 + tid);
   }
   const NodeOf node = load_node(p, base, T_real);  // (used by the last CTA only; on the way during the reduction)
-  const float top = lanes_max(mine.v);
+  const float top = warp_largest(mine.v);
   mine = Best{top, __reduce_min_sync(0xffffffffu, mine.v == top ? mine.i : kNone)};
   if ((tid & 31) == 0) warp_best[tid >> 5] = mine;
   worker_sync();
@@ -354,7 +346,7 @@ __global__ void __launch_bounds__(kStreamThreads + 32, 3) tree_sample_kernel(con
       float m = -INFINITY, sum = 0.f;
       if (n_e > 0) {
         const float x = lane < n_e ? rs.base[(side ? rs.body : -rs.head) + lane] : -INFINITY;
-        m = lanes_max(fmaxf(x, -INFINITY));
+        m = warp_largest(fmaxf(x, -INFINITY));
         sum = warp_add(m > -INFINITY && m < INFINITY ? weight(x, m, kq) : 0.f);
       }
       put(side ? p.slices - 1 : 0, m, sum);
@@ -369,7 +361,7 @@ __global__ void __launch_bounds__(kStreamThreads + 32, 3) tree_sample_kernel(con
         float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY}, s4[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
         for (int k = 0; k < kStreamLane; ++k) m4[k & 3] = fmaxf(m4[k & 3], x[k]);
-        m = lanes_max(fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])));
+        m = warp_largest(fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])));
         if (m > -INFINITY && m < INFINITY) {
 #pragma unroll
           for (int k = 0; k < kStreamLane; ++k) s4[k & 3] += weight(x[k], m, kq);
@@ -398,7 +390,7 @@ __global__ void __launch_bounds__(kStreamThreads + 32, 3) tree_sample_kernel(con
     float M = -INFINITY;
     for (int i0 = 0; i0 < n_sl; i0 += 32)
       if (i0 + lane < n_sl) M = fmaxf(M, s_slice[i0 + lane].x);
-    M = lanes_max(M);
+    M = warp_largest(M);
     const bool inf = M == INFINITY;  // a +inf logit takes everything: its first position
     // (maximum, sum) -> (partial sum up to and with the slice, its weight)
     float total = 0.f;
