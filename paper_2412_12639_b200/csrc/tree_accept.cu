@@ -499,15 +499,17 @@ constexpr int kAcceptMaxChunks = 8;  // vocabulary chunks per row at most (the s
 
 // How a launch splits the vocabulary, and whether its rows are streamed.  Shared by the two entry points so that
 // they cannot drift apart.  Chunks are doubled (3 chunks of 32000 fill their last stage by a third, 6.6 us where 2 take 5.9) as
-// long as they stay worth a CTA.  Streamed: 0.6 of a stage, up to two CTAs per SM (us with 1 / 2 / 4 / 8 chunks, logits in L2 and behind
-// an attention launch over a batch of 300 to 3900 keys):
-//    25 rows of 8192   4.0 / 4.1    23.8 / 24.2         of 12000  4.3 / 4.0 / 4.2   24.4 / 24.3 / 24.3     of 40000  5.4 / 4.7 / 4.6 / 4.7  25.9 / 25.4 / 24.9 / 24.7
-//    50         9832   4.4 / 4.2    37.4 / 37.4            20000  4.7 / 4.6 / 4.6   37.8 / 37.8 / 37.6        40000  5.4 / 4.9 / 5.2 / 5.1  39.4 / 38.8 / 38.6 / 38.7
-//    74         8192   4.0 / 4.2    38.6 / 38.7            20000  4.8 / 4.7 / 4.6   40.0 / 39.6 / 39.2        40000  5.5 / 5.0 / 5.2 / 7.2  41.8 / 41.2 / 41.1 / 43.0
-//    75        12000   4.6 / 4.6    39.4 / 39.1            20000  4.9 / 5.0 / 5.2   40.1 / 39.8 / 39.8        40000  5.6 / 5.6 / 5.9 / 7.1  41.9 / 41.4 / 41.7 / 42.6
-//   110         8192   4.1 / 4.5    41.7 / 41.8            12000  4.7 / 4.6 / 5.0   42.6 / 42.2 / 42.5        20000  5.0 / 5.1 / 5.0        43.7 / 43.4 / 43.3
-//   148         8192   4.1 / 4.6    47.6 / 47.6            12000  4.7 / 4.6 / 7.1   48.9 / 48.4 / 51.0        40000  5.7 / 5.8 / 8.4        51.4 / 50.8 / 53.6
-//   149 rows of 12000 behind one sequence 23.2 / 23.0, 20000 24.4 / 24.6, 64000 28.6 / 28.1; 170 of 12000 24.0 / 23.9, 32000 26.3 / 26.4 (not taken)
+// long as they stay worth a CTA, which depends on how many CTAs an SM then has.  Streamed: 0.6 of a stage up to nine tenths of a CTA per SM,
+// three quarters up to one and a half, one and three quarters up to two.  One stream alone would take 0.6 all along, but two that decide at
+// the same time, each behind its attention launches, lose more by the second CTA per SM than one gains (us with 1 / 2 / 4 chunks: one stream
+// alone with the logits in L2, behind attention over a batch of 300 to 3900 keys, and a pass of either of two such streams):
+//    25 rows of 8192   4.0 / 4.1 / 4.1  23.8 / 24.2 / 24.2                         30 rows of 12000  4.4 / 4.0 / 4.0  24.4 / 24.4 / 24.4  27.9 / 27.5 / 29.6
+//    37         20000  4.6 / 4.4 / 4.1  25.4 / 25.2 / 24.9  29.2 / 28.9 / 30.9     37         30000  4.9 / 4.4 / 4.2  25.8 / 25.1 / 25.0  29.9 / 29.0 / 31.1
+//    50         12000  4.4 / 4.1 / 4.6  37.4 / 37.4 / 37.6  43.6 / 43.3 / 43.3     50         20000  4.7 / 4.5 / 4.7  37.7 / 37.8 / 37.6  44.2 / 43.7 / 43.4
+//    60         12000  4.4 / 4.1 / 4.6  38.0 / 37.8 / 37.9  43.8 / 43.4 / 43.6     74         12000  4.4 / 4.2 / 4.6  39.1 / 38.9 / 38.7  44.2 / 47.7 / 49.0
+//    74         30000  5.1 / 4.7 / 4.8  40.5 / 39.6 / 39.3  47.1 / 49.3 / 50.0     100        12000  4.5 / 4.6 / 4.9  41.8 / 41.5 / -     54.4 / 56.4 / -
+//   100         28000  5.1 / 5.2        42.9 / 42.1         58.0 / 58.4            148        12000  4.7 / 4.6 / 7.1  47.6 / 47.0 / -     80.6 / 82.3 / -
+//   148         28000  5.3 / 5.4 / 7.3  49.5 / 49.0 / -     82.7 / 84.2 / -        120        64000  9.9 / 9.0        47.5 / 46.4         63.1 / 63.1
 // Short rows fit the registers of one pass, and the ring's set-up would only add to it (15 rows of 1000: 4.1 against 4.4); a
 // chunk of them is 2048 entries, or 1000 while there are no more CTAs than SMs (30 rows of 4000 5.3 / 5.1 / 4.9; 100 5.4 / 5.4, behind
 // attention 17.9 / 18.4).
@@ -518,7 +520,7 @@ bool accept_plan(int sm_count, int n_nodes, int vocab, int* chunks_out, int* chu
     const int64_t ctas = static_cast<int64_t>(n_nodes) * c;
     if (!streamed) return ctas <= kAcceptChunksPerSm * sm_count && vocab / c >= (ctas <= sm_count ? 1000 : 2048);
     static_assert(kAcceptChunksPerSm >= 2, "the scratch is sized by it");
-    return ctas <= 2 * sm_count && vocab / c >= kStreamStage * 3 / 5;
+    return ctas <= 2 * sm_count && vocab / c >= (10 * ctas <= 9 * sm_count ? kStreamStage * 3 / 5 : 2 * ctas <= 3 * sm_count ? kStreamStage * 3 / 4 : kStreamStage * 7 / 4);
   };
   while (chunks < kAcceptMaxChunks && worth(2 * chunks)) chunks *= 2;
   int chunk_len = (vocab + chunks - 1) / chunks;
