@@ -614,15 +614,14 @@ int launch_tree_sample(falcon_ctx* ctx, const falcon_accept_args& a, cudaStream_
   };
   int ctas = 1;
   while (ctas < kSampleMaxCluster && a.vocab > ctas * kStreamStage && room(2 * ctas)) ctas *= 2;
-  // Between nine tenths of a row per SM (the pairs are no longer given two places per SM, see stream_bytes) and one, rows of up to six
-  // stages share it no better in pairs (us with 1 / 2 CTAs: logits in L2, not in L2, and behind an attention launch):
-  //   130 rows of 20000   7.2 / 7.4    7.3 / 7.4   26.0 / 25.5       of 32000  8.1 / 7.7    9.4 / 9.3   27.2 / 26.3
-  //   140         20000   7.2 / 7.9    7.8 / 8.4   26.1 / 26.0          38144  8.8 / 9.4   10.3 / 10.9  28.3 / 27.9
-  //   148         38144   8.9 / 9.4   10.4 / 10.9  28.9 / 28.7          49152  9.4 / 9.6   11.1 / 11.4  29.7 / 29.2
-  //               60000  10.8 / 11.0  12.7 / 13.1  31.5 / 30.5
-  //   160         38144   9.7 / 9.3   11.0 / 11.1  29.2 / 29.1      178 of 38144  9.7 / 9.4  11.3 / 11.4  29.7 / 29.8
-  //   222         20000   7.9 / 8.0    9.4 / 9.9   29.5 / 29.7          49152 11.0 / 9.9   12.8 / 13.3  32.8 / 33.1
-  if (ctas == 2 && 10 * N > 9 * ctx->sm_count && N <= ctx->sm_count && a.vocab <= 6 * kStreamStage) ctas = 1;
+  // From nearly one row per SM up to one, rows of up to six stages share it no better in pairs (us with 1 / 2 CTAs: logits in L2, not
+  // in L2, behind an attention launch, and either of two such streams):
+  //   126 rows of 20000   7.2 / 7.4    7.3 / 7.5   21.7 / 21.6                   38144   8.8 / 8.4   10.1 / 10.1  23.9 / 23.2
+  //   130         20000   7.2 / 7.4    7.3 / 7.4   26.0 / 25.5  67.1 / 68.4      40000   8.7 / 8.5                49.8 / 48.7  69.4 / 70.1
+  //   148         38144   8.9 / 9.4   10.4 / 10.9  28.9 / 28.7                   60000  10.8 / 11.0  12.7 / 13.1  31.5 / 30.5
+  //   160         38144   9.7 / 9.3   11.0 / 11.1  29.2 / 29.1                   178 of 38144  9.7 / 9.4  11.3 / 11.4  29.7 / 29.8
+  //   180         32000   9.4 / 8.9                54.4 / 54.7  90.7 / 92.3      222 of 49152 11.0 / 9.9  12.8 / 13.3  32.8 / 33.1
+  if (ctas == 2 && 8 * N > 7 * ctx->sm_count && N <= ctx->sm_count && a.vocab <= 6 * kStreamStage) ctas = 1;
   const int chunk_len = ((a.vocab + ctas - 1) / ctas + 3) & ~3;
   int rc = ensure_tickets(ctx, static_cast<size_t>(B), s);
   if (rc) return rc;
