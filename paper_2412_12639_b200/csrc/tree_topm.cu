@@ -667,15 +667,19 @@ int launch_tree_topm(falcon_ctx* ctx, const falcon_topm_args& a, cudaStream_t s)
   split(c);
   const bool in_regs = !short_stream && per_lane <= kTopmRowsMax && fits();
   if (!in_regs) {
-    // CTAs of a cluster where the rows alone leave SMs idle: four and eight wherever they have room (us with 1 / 2 / 4 CTAs, alone
-    // and behind an attention launch: 60 rows of 40000 9.0 / 8.9 / 8.8  22.7 / 21.8 / 20.9, 87 of 32769 8.1 / 9.3 / 8.4  21.4 / 21.6 /
-    // 20.5, 100 of 49151 10.2 / 10.6 / 10.2  24.1 / 22.9 / 22.7).  Two (1 / 2 CTAs):
+    // CTAs of a cluster where the rows alone leave SMs idle: four and eight wherever they have room (us with 1 / 2 / 4 CTAs: logits in L2,
+    // not in L2, and behind an attention launch):
+    //   60 rows of 40000  8.2 / 7.9 / 7.6   8.4 / 8.0 / 7.7   20.2 / 19.0 / 17.8    87 of 40000  8.2 / 8.7 / 7.8   9.1 / 9.8 / 9.1  23.7 / 22.7 / 21.8
+    //   100 of 49152      9.0 / 8.9 / 8.2   9.9 / 10.2 / 10.0  25.3 / 23.8 / 24.7   100 of 131072  19.2 / 16.1 / 14.4  19.4 / 16.2 / 15.4  35.7 / 29.8 / 30.2
+    // Two (1 / 2 CTAs):
     //   up to nine tenths of a row per SM, where the pairs are given two places per SM: rows of more than seven stages
-    //     110 of 32769 8.3 / 9.6  21.5 / 22.0, of 49151 10.3 / 10.9  24.1 / 23.1, 120 of 57344 11.3 / 11.9  25.1 / 24.2, of 64000 12.3 / 12.2
-    //     26.2 / 24.5, of 114688 17.9 / 15.7  32.4 / 28.2
-    //   up to one: 135 of 64000 12.5 / 14.3  26.4 / 26.6, 140 of 90112 15.5 / 17.4  29.8 / 29.5, of 114688 18.3 / 18.7  32.9 / 31.3
-    //   more: 149 of 32768 9.7 / 10.4  21.7 / 22.6, 170 of 64000 14.7 / 15.1  26.7 / 27.2, of 90112 18.2 / 18.0  33.4 / 30.3, of 131072 22.9 / 20.7
-    //     39.2 / 33.2, 222 of 64000 15.2 / 16.5  27.2 / 28.5, of 131072 24.1 / 24.9  40.3 / 36.9
+    //     105 of 32768  6.9 / 7.2   7.8 / 8.2  22.8 / 22.0     120 of 57344  9.8 / 10.0  11.2 / 11.7  26.8 / 25.4
+    //     120 of 64000 10.6 / 10.3 12.1 / 11.9 27.8 / 25.7     133 of 106496 17.4 / 15.7 17.5 / 15.9  37.9 / 34.2
+    //   up to one: more than thirteen
+    //     148 of 64000 10.8 / 12.5 12.5 / 14.4 33.5 / 32.9     148 of 106496 17.7 / 18.6 17.7 / 18.7 39.0 / 37.6     131072 20.4 / 20.1  20.5 / 20.1  42.1 / 38.9
+    //   beyond: more than ten
+    //     149 of 32768  8.4 / 8.2   9.6 / 10.2 28.6 / 28.9     170 of 64000  13.4 / 12.8  14.6 / 15.1  34.1 / 33.8   90112  18.0 / 17.7  18.1 / 17.8  40.5 / 37.0
+    //     222 of 64000 15.0 / 16.7 15.1 / 16.8 36.4 / 37.5     222 of 90112  18.7 / 19.8  18.7 / 20.0  42.9 / 40.7
     c = 1;
     while (c < kTopmMaxCluster && streams(2 * c) && a.vocab >= 2 * c * kStreamStage) c *= 2;
     if (c == 2 && a.vocab <= (10 * rows <= 9 * sm ? 7 : rows <= sm ? 13 : 10) * kStreamStage) c = 1;
