@@ -44,7 +44,6 @@ namespace {
 using namespace tc;
 
 constexpr int kRowsMax = 256;     // query rows per unit at most: two blocks of 128 TMEM lanes
-constexpr int kBKMax = 64;        // keys per tile at most
 constexpr int kSmThreads = 512;
 constexpr int kTcThreads = 64 + kSmThreads;
 constexpr int kWarpProducer = 0;
@@ -57,14 +56,18 @@ constexpr float kLMin = 7.8886090522101181e-31f;  // 2^-100
 constexpr float kLMax = 1.2676506002282294e+30f;  // 2^100
 constexpr float kRefSpread = 100.f;  // between the references of a row's parts, in log2 units
 constexpr uint32_t kPollLimit = 1u << 24;
-constexpr int kEarlyItems = 2;    // ring slots requested before the grid dependency wait (one K and one V tile)
 
 // Shared memory: the Q block (two 64-column halves for 128-wide heads), the ring, small arrays.
-template <int kHD>
+template <int kHD, bool kLong>
 struct Cfg {
   static constexpr int kHalves = kHD / 64;
+  static constexpr int kBKMax = kLong ? 128 : 64;                     // keys per tile at most
   static constexpr uint32_t kSlotBytes = kBKMax * kHD * 2;            // one K or V tile
-  static constexpr int kSlots = kHD == 128 ? 10 : 12;                 // (128: what shared memory leaves room for)
+  static constexpr int kSlots = kHD == 128 ? (kLong ? 5 : 10) : 12;   // (128: what shared memory leaves room for)
+  // Tensor memory columns.  Four score buffers of 64 (P over the first half of each), two accumulators of 128.  kLong: one score
+  // buffer of 128, two of weights, two accumulators.
+  static constexpr uint32_t kTmemCols = 512, kTmemS = 0, kTmemP = 128, kTmemO = 256, kTmemQ = 384;
+  static constexpr int kEarlyItems = kLong ? 1 : 2;                   // slots requested before the grid dependency wait
   static constexpr uint32_t kQBytes = kRowsMax * kHD * 2;
   static constexpr uint32_t kOffKV = kQBytes;
   static constexpr uint32_t kOffMl = kOffKV + kSlots * kSlotBytes;    // [softmax group][128]: references, at the end row sums
@@ -72,16 +75,12 @@ struct Cfg {
   static constexpr uint32_t kOffPar = kOffRescue + kRowsMax;          // [128] int8: the tree's parent array
   static constexpr uint32_t kOffBars = kOffPar + FALCON_T_MAX;
   static constexpr int kBarKVFull = 0, kBarKVEmpty = kSlots, kBarQ = 2 * kSlots, kBarSFull = kBarQ + 1,
-                       kBarPFull = kBarSFull + 4, kBarODone = kBarPFull + 4, kBarQFree = kBarODone + 1, kBarOFree = kBarQFree + 1,
+                       kBarPFull = kBarSFull + 4, kBarSFree = kBarPFull + 4, kBarPFree = kBarSFree + 1, kBarODone = kBarPFree + 2, kBarQFree = kBarODone + 1, kBarOFree = kBarQFree + 1, kBarQCopied = kBarOFree,
                        kNumBars = kBarOFree + 1;
   static constexpr uint32_t kOffMisc = kOffBars + 8 * kNumBars;       // tmem base, abort flag
   static constexpr uint32_t kSmemBytes = kOffMisc + 16;
   static_assert(kSmemBytes <= 232448, "shared memory");
 };
-
-// tensor memory columns: four score buffers of 64 (P over the first half of each), two accumulators of 128
-constexpr uint32_t kTmemCols = 512;
-constexpr uint32_t kTmemS = 0, kTmemO = 256;
 
 struct TcParams {
   int32_t Hq, Hkv, G, g_shift, s_cap;
@@ -130,14 +129,23 @@ __device__ __forceinline__ uint64_t desc_of(uint32_t lo) {
 }
 
 // kLoop: the grid is one CTA per SM, each working on several units one after the other.
+// kLong: long runs of keys (128-wide heads, the tree in the cache).  The other loop is held up by hand-overs: an item's scores stay in the
+// way of the next ones until its weights, which lie over them, have been multiplied, and with tiles of 64 keys an MMA of Q from shared
+// memory moves 6 KB where its arithmetic would have time for 4.  Here tiles have up to 128 keys; two pairs of groups take the items in turn, the warps
+// of a lane quadrant 64 keys each; scores go to registers at once, so that one buffer of 128 columns serves all items, and the weights have
+// buffers of their own: a softmax has the time of two items.  With one row block Q is read from tensor memory from the third tile on, which
+// halves what the score MMAs draw from shared memory (and their power).  Cycles per 128 rows x 128 keys, where K and V come from L2 and the
+// clock is not held down: one row block 1760 -> 1560, two 2080 -> 1620, of 1024 that the MMAs take.  148 units of 128 rows x 12352 keys, four a head
+// 119.7 -> 103.9 us; 32 units of 128 rows x 4160 keys 40.8 -> 32.0.
 // kFine: a weight is the sum of two bf16 numbers, and partial rows are fp32 (see fine_weights).
-template <int kHD, bool kLoop, bool kFine>
+template <int kHD, bool kLoop, bool kFine, bool kLong>
 __global__ void __launch_bounds__(kTcThreads, 1)
 tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                     const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_tk,
                     const __grid_constant__ CUtensorMap tm_tv, const TcParams p) {
-  using C = Cfg<kHD>;
-  constexpr int kSlots = C::kSlots, kHalves = C::kHalves;
+  static_assert(!kLong || (kHD == 128 && !kLoop && !kFine), "not built");
+  using C = Cfg<kHD, kLong>;
+  constexpr int kSlots = C::kSlots, kHalves = C::kHalves, kBKMax = C::kBKMax;
   extern __shared__ __align__(1024) unsigned char smem_gen[];
   const uint32_t smem_base = smem_u32(smem_gen);
   float* s_ml = reinterpret_cast<float*>(smem_gen + C::kOffMl);
@@ -164,12 +172,12 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       prefetch_tmap(&tm_v);
     }
     for (int i = lane; i < C::kNumBars; i += 32)
-      mbar_init(bar(i), i >= C::kBarPFull && i < C::kBarPFull + 4 ? 4 : (i == C::kBarOFree ? kSmThreads / 32 : 1));
+      mbar_init(bar(i), i >= C::kBarPFull && i <= C::kBarSFree ? (kLong ? 8 : 4) : (i == C::kBarOFree ? kSmThreads / 32 : 1));
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     __syncwarp();
   } else if (warp == kWarpMma) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(s_tmem_base)),
-                 "r"(kTmemCols)
+                 "r"(C::kTmemCols)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -257,23 +265,28 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     const int end = p.separate && tile_begin + j < n_pre ? Lc : S_valid;
     return min(BK, end - k0);
   };
-  // ring item i: K (even) or V (odd) tile i / 2
+  // The ring holds K and V tiles in turn.  kLong: in the order in which the MMAs need them, K `lead` tiles ahead of V.
+  auto lead = [&]() { return two_blocks ? 1 : 2; };
+  auto k_item = [&](int j) { return ring0 + (kLong ? j + max(0, j - lead()) : 2 * j); };
+  auto v_item = [&](int j) { return ring0 + (kLong ? j + min(n_my, j + lead() + 1) : 2 * j + 1); };
+  int next_k = 0, next_v = 0;  // (kLong, producer) tiles asked for
   auto load_item = [&](int i) {
-    const int j = i >> 1, slot = (ring0 + i) % kSlots;
-    if (ring0 + i < 2 && p.stall_first) return;
+    const bool is_k = kLong ? next_k < n_my && next_k <= next_v + lead() : !(i & 1);
+    const int j = kLong ? (is_k ? next_k++ : next_v++) : i >> 1, slot = (ring0 + i) % kSlots;
+    if (ring0 + i < (kLong ? 1 : 2) && p.stall_first) return;
     const uint32_t dst = smem_base + C::kOffKV + slot * C::kSlotBytes;
     mbar_expect_tx(bar(C::kBarKVFull + slot), tile_bytes);
     if (p.separate && tile_begin + j >= n_pre)
-      tma_load_5d(dst, (i & 1) ? &tm_tv : &tm_tk, bar(C::kBarKVFull + slot), 0, node_base + (tile_begin + j - n_pre) * BK, 0, kvh, 0);
+      tma_load_5d(dst, is_k ? &tm_tk : &tm_tv, bar(C::kBarKVFull + slot), 0, node_base + (tile_begin + j - n_pre) * BK, 0, kvh, 0);
     else
-      tma_load_5d(dst, (i & 1) ? &tm_v : &tm_k, bar(C::kBarKVFull + slot), 0, tile_key0(j), 0, kvh, b);
+      tma_load_5d(dst, is_k ? &tm_k : &tm_v, bar(C::kBarKVFull + slot), 0, tile_key0(j), 0, kvh, b);
   };
 
   // Wait (within a limit) for what was asked for, so that no copy is in flight when the CTA leaves.
   auto drain_loads = [&](int n_ring, int n_q) {
     if (n_q > 0) mbar_wait_drain(bar(C::kBarQ), (n_q - 1) & 1);
     for (int i = max(0, n_ring - kSlots); i < n_ring; ++i)
-      if (!(i < 2 && p.stall_first)) mbar_wait_drain(bar(C::kBarKVFull + i % kSlots), (i / kSlots) & 1);
+      if (!(i < (kLong ? 1 : 2) && p.stall_first)) mbar_wait_drain(bar(C::kBarKVFull + i % kSlots), (i / kSlots) & 1);
   };
 
   int n_early = 0;  // ring items requested before the wait below
@@ -283,7 +296,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     // Prefix rows that the caller declares stable (written before the kernel that precedes this one
     // in the stream started) may be requested while that kernel is still finishing.
     if (warp == kWarpProducer && lane == 0 && p.early_prefix && n_valid > 0)
-      for (; n_early < min(2 * n_my, kEarlyItems) && tile_key0(n_early >> 1) + BK <= Lc; ++n_early) load_item(n_early);
+      for (; n_early < min(2 * n_my, C::kEarlyItems) && tile_key0(n_early >> 1) + BK <= Lc; ++n_early) load_item(n_early);
   }
   tc_fence_before();
   __syncthreads();
@@ -300,7 +313,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
   }
   if (n_valid <= 0) {  // no query rows here; same decision in every CTA of the cluster
     if (warp == kWarpMma)
-      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols) : "memory");
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(C::kTmemCols) : "memory");
     return;
   }
 
@@ -407,7 +420,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             for (int h = 0; h < kHalves; ++h)
 #pragma unroll
               for (int kk = 0; kk < 4; ++kk)
-                umma_bf16_ss(tmem_base + kTmemS + buf * 64, desc_of(q + h * q_step + kk * 2), desc_of(k + h * k_step + kk * 2),
+                umma_bf16_ss(tmem_base + C::kTmemS + (kLong ? 0 : buf * 64), desc_of(q + h * q_step + kk * 2), desc_of(k + h * k_step + kk * 2),
                              p.idesc_qk, (h | kk) ? 1u : 0u);
             umma_commit(bar(C::kBarSFull) + 8u * buf);
             if (kLoop && last) umma_commit(bar(C::kBarQFree));
@@ -415,7 +428,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
         };
         auto issue_pv = [&](int s, int buf, int slot, int j, bool last_block) {
           constexpr uint32_t idesc_pv = make_idesc(128, kHD, false, true);
-          const uint32_t acc = tmem_base + kTmemO + s * 128, pbase = tmem_base + kTmemS + buf * 64, v = v_lo + slot * kSlotStep;
+          const uint32_t acc = tmem_base + C::kTmemO + s * 128, pbase = tmem_base + (kLong ? C::kTmemP : C::kTmemS) + buf * 64, v = v_lo + slot * kSlotStep;
           // keys of the tile that exist, in MMA steps of 16 (P is zero and V cleared in the last step's rest)
           const int nk = j == j_b ? nk_b : (j == j_a ? nk_a : nk_full);
           if (elected) {
@@ -428,9 +441,67 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
                 umma_bf16_ts(acc, pk, desc_of(v + kk * 128), idesc_pv, (j > 0 || kk > 0) ? 1u : 0u);
                 if constexpr (kFine) umma_bf16_ts(acc, pk + 16, desc_of(v + kk * 128), idesc_pv, 1u);
               }
+            if constexpr (kLong) umma_commit(bar(C::kBarPFree) + 8u * buf);
             if (last_block) umma_commit(bar(C::kBarKVEmpty) + 8u * slot);
           }
         };
+        if constexpr (kLong) {
+          // Item i is (tile i / kBlocks, block i % kBlocks), its softmax is that of warp set i mod 2.  The scores of item i + 1 follow
+          // those of item i as soon as the latter are in registers; P(i).V comes behind the scores of item i + 2.
+          // The tiles are in the ring in that order: K tiles come kLead ahead of V's.
+          constexpr int kLead = kBlocks == 1 ? 2 : 1;
+          int kslot = 0, vslot = min(n_my, kLead + 1);  // ring slots of the next K and V tile
+          uint32_t kphase = 0;
+          int k_done = 0, v_done = 0;
+          // One row block: from the third item on Q comes from tensor memory, where the softmax warps have put it by then.
+          auto scores = [&](int s, int set, auto from_tmem) -> bool {
+            if (s == 0 && !mbar_wait(bar(C::kBarKVFull) + 8u * kslot, kphase, abort_flag)) return false;
+            if constexpr (kBlocks == 1 && decltype(from_tmem)::value) {
+              const uint32_t k = k_lo + kslot * kSlotStep;
+              if (elected) {
+#pragma unroll
+                for (int kk = 0; kk < kHD / 16; ++kk)
+                  umma_bf16_ts(tmem_base + C::kTmemS, tmem_base + C::kTmemQ + kk * 8, desc_of(k + (kk >> 2) * k_step + (kk & 3) * 2), p.idesc_qk,
+                               kk ? 1u : 0u);
+                umma_commit(bar(C::kBarSFull) + 8u * set);
+              }
+            } else {
+              issue_qk(s, set, kslot, false);
+            }
+            if (s == kBlocks - 1) {
+              kslot += ++k_done <= kLead ? 1 : 2;
+              if (kslot >= kSlots) {
+                kslot -= kSlots;
+                kphase ^= 1;
+              }
+            }
+            return true;
+          };
+          auto scores_loaded = [&](int i) {
+            const bool ok = mbar_wait(bar(C::kBarSFree), i & 1u, abort_flag);
+            tc_fence_after();
+            return ok;
+          };
+          if (!scores(0, 0, std::false_type{})) return;
+          if (n_items > 1 && (!scores_loaded(0) || !scores(1 % kBlocks, 1, std::false_type{}))) return;
+          if (kBlocks == 1 && n_items > 2 && !mbar_wait(bar(C::kBarQCopied), 0, abort_flag)) return;
+          for (int i0 = 0; i0 < n_items; i0 += 2) {
+#pragma unroll
+            for (int set = 0; set < 2; ++set) {
+              const int i = i0 + set, s = set % kBlocks;
+              if (i >= n_items) break;
+              if (i + 2 < n_items && (!scores_loaded(i + 1) || !scores(s, set, std::true_type{}))) return;
+              if (!mbar_wait(bar(C::kBarPFull) + 8u * set, (i0 >> 1) & 1u, abort_flag)) return;
+              tc_fence_after();
+              issue_pv(s, set, vslot, kBlocks == 2 ? i0 >> 1 : i, s == kBlocks - 1);
+              if (s == kBlocks - 1) {
+                vslot += ++v_done + kLead < n_my ? 2 : 1;
+                if (vslot >= kSlots) vslot -= kSlots;
+              }
+            }
+          }
+          return;
+        }
         // Four items' scores are in flight: 4 / kBlocks tiles.  P(i) lies over S(i), so the scores of item
         // i + 4 are issued behind P(i).V (the MMAs of a CTA run in the order of issue).
         constexpr int kAhead = 4 / kBlocks;
@@ -444,7 +515,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             kphase ^= 1;
           }
         };
-        static_assert(kSlots % 2 == 0, "K tiles stay in the even slots");
+        static_assert(kLong || kSlots % 2 == 0, "K tiles stay in the even slots");
         for (int j = 0; j < min(kAhead, n_my); ++j) {
           if (!k_wait()) return;
 #pragma unroll
@@ -498,7 +569,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     const int row = blk * 128 + lane_row;          // query row of the unit
     const bool valid = row < n_valid, warp_valid = row - lane < n_valid;
     const uint32_t tmem_lane = tmem_base + (static_cast<uint32_t>(q4 * 32) << 16);
-    const uint32_t tmem_s = tmem_lane + kTmemS + grp * 64;  // P (packed pairs) goes over the first half
+    const uint32_t tmem_s = tmem_lane + C::kTmemS + grp * 64;  // (not kLong) P (packed pairs) goes over the first half
 
     // The tree's parent array into shared memory: from global memory the walks below would be a chain of round
     // trips.  (Not needed, and not waited for, where no key of this CTA belongs to the tree.)
@@ -558,91 +629,227 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     };
     if (!kLoop && (grp == 0 || (two_blocks && grp == 1))) s_rescue[row] = 0;
     bool published = !source || n_items == 0;  // (source groups have item `grp`: n_items >= n_src or 0)
+    if (kLong && !two_blocks && n_items > 2) {
+      // Q into tensor memory: group g has 32 head dimensions of every row (rows that do not exist: zeros).
+      if (mbar_wait_warp(bar(C::kBarQ), 0, abort_flag)) {
+        uint32_t w[16];
+        const unsigned char* qrow = smem_gen + (grp >> 1) * p.q_half_bytes + lane_row * 128;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          uint4 x = make_uint4(0u, 0u, 0u, 0u);
+          if (valid) x = *reinterpret_cast<const uint4*>(qrow + ((((grp & 1) * 4 + u) ^ (lane_row & 7)) << 4));
+          w[4 * u] = x.x;
+          w[4 * u + 1] = x.y;
+          w[4 * u + 2] = x.z;
+          w[4 * u + 3] = x.w;
+        }
+        __syncwarp();
+        FALCON_TMEM_ST16(tmem_lane + C::kTmemQ + grp * 16, w);
+        tmem_wait_st();
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar(C::kBarQCopied));
+    }
     if (!source && n_items > 0) {
       ref_barrier(true);
       m_ref = *ref;
     }
     const float scale = p.scale_log2;
-    for (int i = grp; i < n_items; i += 4) {
-      const int j = two_blocks ? i >> 1 : i;
-      const int k0 = tile_key0(j), nv = tile_keys_in(j, k0);
-      if (!mbar_wait_warp(bar(C::kBarSFull + grp), sphase, abort_flag)) break;
-      sphase ^= 1;
-      tc_fence_after();
-      // the scores are there, so the K tile is no longer needed (two blocks: the second's come last)
-      if (q4 == 0 && lane == 0 && (!two_blocks || blk == 1)) mbar_arrive(bar(C::kBarKVEmpty + (ring0 + 2 * j) % kSlots));
-      if (warp_valid) {
-        const bool full = k0 + BK <= Lc;  // every key lies in the prefix: visible to every row
-        auto load32 = [&](int c, uint32_t (&sr)[32]) {
-          FALCON_TMEM_LD32(tmem_s + c, sr);
-          tmem_wait_ld();
-          if (!full || c + 32 > BK) {
-            uint32_t vis = full ? 0xffffffffu : static_cast<uint32_t>(window64(anc_lo, anc_hi, k0 - Lc + c));
-            if (nv - c < 32) vis &= nv - c <= 0 ? 0u : (1u << (nv - c)) - 1u;
+    if constexpr (kLong) {
+      // Groups 0 and 2 take the even items, 1 and 3 the odd ones: the first of a pair the lower half of the tile's keys, the other
+      // the upper half.
+      constexpr int kC = kBKMax / 2;  // keys of an item to a thread
+      const int set = grp & 1, half = grp >> 1;
+      const uint32_t tmem_sc = tmem_lane + C::kTmemS + half * kC, tmem_p = tmem_lane + C::kTmemP + set * 64 + half * (kC / 2);
+      uint32_t p_uses = 0;            // items this warp has given weights to
+      if (!warp_valid) {  // rows that do not exist: weights of zero, which cost the least power
+        uint32_t zero[32];
 #pragma unroll
-            for (int e = 0; e < 32; ++e)
-              if (!((vis >> e) & 1u)) sr[e] = 0xff800000u;
-          }
+        for (int e = 0; e < 32; ++e) zero[e] = 0u;
+        FALCON_TMEM_ST32(tmem_p, zero);
+      }
+      for (int i = set; i < n_items; i += 2) {
+        const int j = two_blocks ? i >> 1 : i;
+        const int k0 = tile_key0(j), nv = tile_keys_in(j, k0);
+        // The MMA warp takes P's barrier for V's as well: one warp of the item waits for the tile to have landed.  (After the scores: the
+        // slot may be that of this tile's K, which the same warp gives back.)
+        const bool clear_v = (nv & 15) && blk == 0 && half == 0, v_waits = (q4 == 0 && half == 0) || clear_v;
+        const int v_at = v_item(j), v_slot = v_at % kSlots;
+        auto v_landed = [&]() { return mbar_wait_warp(bar(C::kBarKVFull + v_slot), (v_at / kSlots) & 1, abort_flag); };
+        if (!mbar_wait_warp(bar(C::kBarSFull + set), sphase, abort_flag)) break;
+        sphase ^= 1;
+        tc_fence_after();
+        // the scores are there, so the K tile is no longer needed (two blocks: the second's come last)
+        if (q4 == 0 && lane == 0 && half == 0 && (!two_blocks || blk == 1)) mbar_arrive(bar(C::kBarKVEmpty + k_item(j) % kSlots));
+        auto scores_taken = [&]() {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bar(C::kBarSFree));
         };
+        uint32_t pk[kC / 2];
+        const bool work = warp_valid && half * kC < nv;
+        // This set's weights of two items before have been read.  Every warp waits for it, with weights to store or without: one that
+        // ran ahead would arrive twice for one item.
+        auto weights_read = [&]() { return p_uses == 0 || mbar_wait_warp(bar(C::kBarPFree + set), (p_uses - 1) & 1, abort_flag); };
+        bool free_again;
+        if (work) {
+          // The scores go to registers at once and their buffer back to the MMA warp.
+          uint32_t sr[kC / 32][32];
 #pragma unroll
-        for (int c = 0; c < kBKMax; c += 32) {
-          if (c < BK) {
-            uint32_t sr[32], pk[16], rest[kFine ? 16 : 1];
-            load32(c, sr);
-            if (c == 0 && !published) {
-              const float s0 = __uint_as_float(sr[0]);
-              m_ref = s0 == -INFINITY ? 0.f : s0 * scale;
-              *ref = m_ref;
-              published = true;
-              ref_barrier(false);
-            }
-            const float neg = -m_ref;
+          for (int c = 0; c < kC / 32; ++c) FALCON_TMEM_LD32(tmem_sc + 32 * c, sr[c]);
+#pragma unroll
+          for (int c = 0; c < kC / 32; ++c) tmem_wait_ld(sr[c]);
+          scores_taken();
+          // which of 32 keys exist and are visible to the row
+          auto visible = [&](int c) -> uint32_t {
+            const int col = half * kC + c;
+            const uint32_t vis = static_cast<uint32_t>(window64(anc_lo, anc_hi, k0 - Lc + col));
+            return nv - col >= 32 ? vis : nv <= col ? 0u : vis & ((1u << (nv - col)) - 1u);
+          };
+          const bool full = k0 + BK <= Lc && half * kC + kC <= BK;  // all of them
+          if (!published) {
+            m_ref = full || (visible(0) & 1u) ? __uint_as_float(sr[0][0]) * scale : 0.f;
+            if (m_ref == -INFINITY) m_ref = 0.f;
+            *ref = m_ref;
+            published = true;
+            ref_barrier(false);
+          }
+          const float neg = -m_ref;
+#pragma unroll
+          for (int c = 0; c < kC / 32; ++c)
 #pragma unroll
             for (int e = 0; e < 32; e += 2) {
               float e0, e1;
-              fma2(__uint_as_float(sr[e]), __uint_as_float(sr[e + 1]), scale, scale, neg, neg, e0, e1);
-              const float p0 = ex2(e0), p1 = ex2(e1);
-              pk[e >> 1] = pack_bf16(p0, p1);
-              const float h0 = bf16lo(pk[e >> 1]), h1 = bf16hi(pk[e >> 1]);
-              if constexpr (kFine) rest[e >> 1] = pack_bf16(p0 - h0, p1 - h1);  // (the differences are exact)
-              // the row sum takes the values that the MMA is fed
-              if (e & 2)
-                add2(l2, l3, kFine ? p0 : h0, kFine ? p1 : h1);
-              else
-                add2(l0, l1, kFine ? p0 : h0, kFine ? p1 : h1);
+              fma2(__uint_as_float(sr[c][e]), __uint_as_float(sr[c][e + 1]), scale, scale, neg, neg, e0, e1);
+              pk[16 * c + (e >> 1)] = pack_bf16(ex2(e0), ex2(e1));
             }
-            // over scores this thread has read already
-            if constexpr (kFine) {
-              FALCON_TMEM_ST16(tmem_s + c, pk);
-              FALCON_TMEM_ST16(tmem_s + c + 16, rest);
-            } else {
-              FALCON_TMEM_ST16(tmem_s + (c >> 1), pk);
+          free_again = weights_read();
+          if (!full) {
+#pragma unroll
+            for (int c = 0; c < kC / 32; ++c) {
+              const uint32_t vis = visible(32 * c);
+#pragma unroll
+              for (int e = 0; e < 16; ++e)
+                pk[16 * c + e] &= ((vis >> (2 * e)) & 1u ? 0xffffu : 0u) | ((vis >> (2 * e + 1)) & 1u ? 0xffff0000u : 0u);
             }
           }
+          FALCON_TMEM_ST32(tmem_p, pk);
+        } else {
+          scores_taken();
+          free_again = weights_read();
+          if (!published) {
+            published = true;
+            ref_barrier(false);
+          }
         }
-      } else if (!published) {
-        published = true;
-        ref_barrier(false);
-      }
-      // The MMA warp takes P's barrier for V's as well: one warp of the group waits for the tile to have landed.
-      const bool clear_v = (nv & 15) && blk == 0;
-      if (q4 == 0 || clear_v) {
-        const int item = ring0 + 2 * j + 1, slot = item % kSlots;
-        if (!mbar_wait_warp(bar(C::kBarKVFull + slot), (item / kSlots) & 1, abort_flag)) break;
+        ++p_uses;
+        if (v_waits && !v_landed()) break;
+        if (!free_again) break;
         if (clear_v) {
           // The last MMA step over this tile's keys reads V rows past the last key, which may hold anything
           // (0 x NaN = NaN): clear them.
-          unsigned char* vtile = smem_gen + C::kOffKV + slot * C::kSlotBytes;
+          unsigned char* vtile = smem_gen + C::kOffKV + v_slot * C::kSlotBytes;
           const int units = (16 - (nv & 15)) * 8;  // of 16 bytes, per half
           for (int u = lane_row; u < kHalves * units; u += 128)
             *reinterpret_cast<uint4*>(vtile + (u / units) * half_tile + nv * 128 + (u % units) * 16) = make_uint4(0, 0, 0, 0);
           fence_async_smem();
         }
+        tmem_wait_st();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(C::kBarPFull + set));
+        // The row sum takes the values that the MMA is fed, after they have been handed over.
+        if (work) {
+#pragma unroll
+          for (int e = 0; e < kC / 2; e += 2) {
+            add2(l0, l1, bf16lo(pk[e]), bf16hi(pk[e]));
+            add2(l2, l3, bf16lo(pk[e + 1]), bf16hi(pk[e + 1]));
+          }
+        }
       }
-      tmem_wait_st();
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(bar(C::kBarPFull + grp));
+    } else {
+      for (int i = grp; i < n_items; i += 4) {
+        const int j = two_blocks ? i >> 1 : i;
+        const int k0 = tile_key0(j), nv = tile_keys_in(j, k0);
+        if (!mbar_wait_warp(bar(C::kBarSFull + grp), sphase, abort_flag)) break;
+        sphase ^= 1;
+        tc_fence_after();
+        // the scores are there, so the K tile is no longer needed (two blocks: the second's come last)
+        if (q4 == 0 && lane == 0 && (!two_blocks || blk == 1)) mbar_arrive(bar(C::kBarKVEmpty + (ring0 + 2 * j) % kSlots));
+        if (warp_valid) {
+          const bool full = k0 + BK <= Lc;  // every key lies in the prefix: visible to every row
+          auto load32 = [&](int c, uint32_t (&sr)[32]) {
+            FALCON_TMEM_LD32(tmem_s + c, sr);
+            tmem_wait_ld();
+            if (!full || c + 32 > BK) {
+              uint32_t vis = full ? 0xffffffffu : static_cast<uint32_t>(window64(anc_lo, anc_hi, k0 - Lc + c));
+              if (nv - c < 32) vis &= nv - c <= 0 ? 0u : (1u << (nv - c)) - 1u;
+#pragma unroll
+              for (int e = 0; e < 32; ++e)
+                if (!((vis >> e) & 1u)) sr[e] = 0xff800000u;
+            }
+          };
+#pragma unroll
+          for (int c = 0; c < kBKMax; c += 32) {
+            if (c < BK) {
+              uint32_t sr[32], pk[16], rest[kFine ? 16 : 1];
+              load32(c, sr);
+              if (c == 0 && !published) {
+                const float s0 = __uint_as_float(sr[0]);
+                m_ref = s0 == -INFINITY ? 0.f : s0 * scale;
+                *ref = m_ref;
+                published = true;
+                ref_barrier(false);
+              }
+              const float neg = -m_ref;
+#pragma unroll
+              for (int e = 0; e < 32; e += 2) {
+                float e0, e1;
+                fma2(__uint_as_float(sr[e]), __uint_as_float(sr[e + 1]), scale, scale, neg, neg, e0, e1);
+                const float p0 = ex2(e0), p1 = ex2(e1);
+                pk[e >> 1] = pack_bf16(p0, p1);
+                const float h0 = bf16lo(pk[e >> 1]), h1 = bf16hi(pk[e >> 1]);
+                if constexpr (kFine) rest[e >> 1] = pack_bf16(p0 - h0, p1 - h1);  // (the differences are exact)
+                // the row sum takes the values that the MMA is fed
+                if (e & 2)
+                  add2(l2, l3, kFine ? p0 : h0, kFine ? p1 : h1);
+                else
+                  add2(l0, l1, kFine ? p0 : h0, kFine ? p1 : h1);
+              }
+              // over scores this thread has read already
+              if constexpr (kFine) {
+                FALCON_TMEM_ST16(tmem_s + c, pk);
+                FALCON_TMEM_ST16(tmem_s + c + 16, rest);
+              } else {
+                FALCON_TMEM_ST16(tmem_s + (c >> 1), pk);
+              }
+            }
+          }
+        } else if (!published) {
+          published = true;
+          ref_barrier(false);
+        }
+        // The MMA warp takes P's barrier for V's as well: one warp of the group waits for the tile to have landed.
+        const bool clear_v = (nv & 15) && blk == 0;
+        if (q4 == 0 || clear_v) {
+          const int item = ring0 + 2 * j + 1, slot = item % kSlots;
+          if (!mbar_wait_warp(bar(C::kBarKVFull + slot), (item / kSlots) & 1, abort_flag)) break;
+          if (clear_v) {
+            // The last MMA step over this tile's keys reads V rows past the last key, which may hold anything
+            // (0 x NaN = NaN): clear them.
+            unsigned char* vtile = smem_gen + C::kOffKV + slot * C::kSlotBytes;
+            const int units = (16 - (nv & 15)) * 8;  // of 16 bytes, per half
+            for (int u = lane_row; u < kHalves * units; u += 128)
+              *reinterpret_cast<uint4*>(vtile + (u / units) * half_tile + nv * 128 + (u % units) * 16) = make_uint4(0, 0, 0, 0);
+            fence_async_smem();
+          }
+        }
+        tmem_wait_st();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(C::kBarPFull + grp));
+      }
     }
     if (!published) ref_barrier(false);  // (a wait gave up before the first tile)
 
@@ -651,25 +858,19 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     // takes a part of the accumulator's columns below).
     float l_row = (l0 + l1) + (l2 + l3);
     {
+      // (barriers of their own: a warp that only arrived at its reference's barrier may be here before the others are there)
       float* sums = reinterpret_cast<float*>(smem_gen + C::kOffMl) + lane_row;
-      if (two_blocks) {
-        asm volatile("bar.sync %0, 64;" ::"r"(1 + blk * 4 + q4) : "memory");  // (the references have been read)
-        sums[grp * 128] = l_row;
-        asm volatile("bar.sync %0, 64;" ::"r"(1 + blk * 4 + q4) : "memory");
-        l_row = sums[blk * 128] + sums[(blk + 2) * 128];
-      } else {
-        asm volatile("bar.sync %0, 128;" ::"r"(1 + q4) : "memory");
-        sums[grp * 128] = l_row;
-        asm volatile("bar.sync %0, 128;" ::"r"(1 + q4) : "memory");
-        l_row = (sums[0] + sums[128]) + (sums[256] + sums[384]);
-      }
+      asm volatile("bar.sync %0, 128;" ::"r"(9 + q4) : "memory");  // (the references have been read)
+      sums[grp * 128] = l_row;
+      asm volatile("bar.sync %0, 128;" ::"r"(9 + q4) : "memory");
+      l_row = two_blocks ? sums[blk * 128] + sums[(blk + 2) * 128] : (sums[0] + sums[128]) + (sums[256] + sums[384]);
     }
     bool have = n_my > 0 && !*abort_flag;
     if (have) have = mbar_wait_warp(bar(C::kBarODone), kLoop ? nth & 1 : 0, abort_flag);
     tc_fence_after();
     const int n_cols = two_blocks ? kHD / 2 : kHD / 4, col0 = (two_blocks ? grp >> 1 : grp) * n_cols;
     const bool first_cols = col0 == 0;
-    const uint32_t acc0 = tmem_lane + kTmemO + blk * 128;
+    const uint32_t acc0 = tmem_lane + C::kTmemO + blk * 128;
     const int mg = unit * R + row;
     __nv_bfloat16* dst = p.out + (static_cast<int64_t>(node_base + (mg >> p.g_shift)) * p.Hq + kvh * G + (mg & (G - 1))) * kHD;
     float inv = 1.f;
@@ -830,7 +1031,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     // (after a wait that gave up, MMAs may still be running: the last commit covers them all)
     if (!kLoop && n_my > 0 && *abort_flag && lane == 0) mbar_wait_drain(bar(C::kBarODone), 0);
     __syncwarp();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(C::kTmemCols) : "memory");
   }
 }
 
@@ -843,7 +1044,7 @@ int resident_clusters(falcon_ctx* ctx, int s) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(s, ctx->sm_count, 1);
     cfg.blockDim = dim3(kTcThreads);
-    cfg.dynamicSmemBytes = Cfg<128>::kSmemBytes;
+    cfg.dynamicSmemBytes = Cfg<128, false>::kSmemBytes;
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeClusterDimension;
     attr.val.clusterDim.x = s;
@@ -852,7 +1053,7 @@ int resident_clusters(falcon_ctx* ctx, int s) {
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, tree_attn_tc_kernel<128, false, false>, &cfg) != cudaSuccess) n = -1;
+    if (cudaOccupancyMaxActiveClusters(&n, tree_attn_tc_kernel<128, false, false, false>, &cfg) != cudaSuccess) n = -1;
     resident[s] = n > 0 ? n : -1;
     cudaGetLastError();
   }
@@ -868,8 +1069,21 @@ int nodes_per_unit(const falcon_attn_args& a, int rows) {
   return std::min(most, (nodes + gran - 1) / gran * gran);
 }
 
+// Keys that one CTA of a cluster has: of the longest sequence, three times, and of the mean one.
+int keys_per_cta(const falcon_attn_args& a, int splits) {
+  int64_t longest = static_cast<int64_t>(a.tree.max_prefix_len) + a.tree.max_tree;
+  if (a.tree.prefix_len_host && a.tree.node_off_host) {
+    longest = 1;
+    for (int i = 0; i < a.tree.batch; ++i)
+      longest = std::max<int64_t>(longest, static_cast<int64_t>(a.tree.prefix_len_host[i]) + a.tree.node_off_host[i + 1] - a.tree.node_off_host[i]);
+  }
+  return static_cast<int>(((3 * longest + mean_keys(a)) / 4 + splits - 1) / splits);
+}
+
 struct Plan {
   int q_nodes, n_units, splits, tile;
+  double ctas;  // that have rows
+  bool long_runs;
 };
 // Rows per unit (one block of 128 or two), key splits per unit and tile height: the least estimated time.
 // A CTA costs a fixed part (launch, Q, merge: 4 us, 5 with splits) and its tiles, 64 keys each: 0.92 us
@@ -884,7 +1098,8 @@ struct Plan {
 Plan make_plan(falcon_ctx* ctx, const falcon_attn_args& a) {
   const int B = a.tree.batch, G = a.n_q_heads / a.n_kv_heads;
   const bool host = a.tree.prefix_len_host && a.tree.node_off_host, wide = a.head_dim == 128;
-  Plan best = {nodes_per_unit(a, kRowsMax), 1, std::max(1, a.n_splits), kBKMax};
+  constexpr int kBKMax = Cfg<128, false>::kBKMax;
+  Plan best = {nodes_per_unit(a, kRowsMax), 1, std::max(1, a.n_splits), kBKMax, 0., false};
   best.n_units = (a.tree.max_tree + best.q_nodes - 1) / best.q_nodes;
   double best_us = 1e30;
   for (int rows = 128; rows <= kRowsMax; rows += 128) {
@@ -917,8 +1132,22 @@ Plan make_plan(falcon_ctx* ctx, const falcon_attn_args& a) {
       if (units > slots) est = B == 1 ? longest * static_cast<double>(static_cast<int64_t>((units + slots - 1) / slots)) : std::max(longest, total / slots + 0.3 * longest);
       if (est < best_us) {
         best_us = est;
-        best = {q_nodes, n_units, s, tile};
+        best = {q_nodes, n_units, s, tile, units * s, false};
       }
+    }
+  }
+  // Long runs of keys have a loop of their own (kLong).  Against the other one at equal rows and splits it takes 0.6 to 0.9 us more a
+  // CTA (its first tile is twice as high) and 10 to 20 % less for every tile.  2568 random shapes of 128-wide heads, by keys per CTA (the longest
+  // sequence counted three times against the mean), other / this: no more CTAs than SMs and one row block, 600-700 1.00,
+  // 700-800 1.02, 800-1200 1.06, above 1.10 (up to 1.25); more CTAs than SMs, where short ones follow the long ones, 800-1200 0.98, above 1.06; two row
+  // blocks 700-1200 0.98, 1200-1500 1.03, above 1.06.
+  if (wide && !fine_weights(128, a.k_tree != nullptr) &&
+      keys_per_cta(a, best.splits) >= (best.q_nodes * G > 128 || best.ctas > ctx->sm_count ? 1400 : 800)) {
+    best.long_runs = true;
+    best.tile = Cfg<128, true>::kBKMax;
+    if (B == 1) {
+      const int per = keys_per_cta(a, best.splits), nt = (per + best.tile - 1) / best.tile;
+      best.tile = std::min(best.tile, ((per + nt - 1) / nt + 15) / 16 * 16);
     }
   }
   return best;
@@ -926,7 +1155,7 @@ Plan make_plan(falcon_ctx* ctx, const falcon_attn_args& a) {
 
 template <int kHD, bool kFine>
 int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s) {
-  using C = Cfg<kHD>;
+  using C = Cfg<kHD, false>;
   const int B = a.tree.batch, Hq = a.n_q_heads, Hkv = a.n_kv_heads, G = Hq / Hkv;
   bool& attr_set = ctx->attn_attr_set[0];
   if (!attr_set) {
@@ -934,12 +1163,13 @@ int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s) {
     auto set = [&](auto* kernel, uint32_t bytes) {
       if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
     };
-    set(tree_attn_tc_kernel<128, false, false>, Cfg<128>::kSmemBytes);
-    set(tree_attn_tc_kernel<128, true, false>, Cfg<128>::kSmemBytes);
-    set(tree_attn_tc_kernel<128, false, true>, Cfg<128>::kSmemBytes);
-    set(tree_attn_tc_kernel<128, true, true>, Cfg<128>::kSmemBytes);
-    set(tree_attn_tc_kernel<64, false, true>, Cfg<64>::kSmemBytes);
-    set(tree_attn_tc_kernel<64, true, true>, Cfg<64>::kSmemBytes);
+    set(tree_attn_tc_kernel<128, false, false, false>, Cfg<128, false>::kSmemBytes);
+    set(tree_attn_tc_kernel<128, false, false, true>, Cfg<128, true>::kSmemBytes);
+    set(tree_attn_tc_kernel<128, true, false, false>, Cfg<128, false>::kSmemBytes);
+    set(tree_attn_tc_kernel<128, false, true, false>, Cfg<128, false>::kSmemBytes);
+    set(tree_attn_tc_kernel<128, true, true, false>, Cfg<128, false>::kSmemBytes);
+    set(tree_attn_tc_kernel<64, false, true, false>, Cfg<64, false>::kSmemBytes);
+    set(tree_attn_tc_kernel<64, true, true, false>, Cfg<64, false>::kSmemBytes);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute(tree_attn_tc_kernel)");
     attr_set = true;
   }
@@ -951,7 +1181,7 @@ int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s) {
   // sequences, 40 heads of 64), 38.5 -> 31.2 (15, 40 of 128, tree in its own buffers), of 5 tiles on average (13
   // sequences, 8 KV heads of 128) 14.0 both ways, of 19 tiles 40 -> 42, of 34 tiles 47 -> 54.
   const int64_t n_total = static_cast<int64_t>(Hkv) * n_units * B;
-  const bool loop = splits == 1 && n_total > ctx->sm_count && n_total < (1 << 30) && (mean_keys(a) + kBKMax - 1) / kBKMax <= kLoopTiles;
+  const bool loop = splits == 1 && !plan.long_runs && n_total > ctx->sm_count && n_total < (1 << 30) && (mean_keys(a) + C::kBKMax - 1) / C::kBKMax <= kLoopTiles;
   if (static_cast<int64_t>(Hkv) * n_units > 65535) return FALCON_ERR_CAPACITY;
 
   // Tensor maps.  The head dimension is split into blocks of 64 columns so that one box covers all the
@@ -1037,7 +1267,7 @@ int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = loop ? dim3(ctx->sm_count) : dim3(splits, Hkv * n_units, B);
   cfg.blockDim = dim3(kTcThreads);
-  cfg.dynamicSmemBytes = C::kSmemBytes;
+  cfg.dynamicSmemBytes = plan.long_runs ? Cfg<128, true>::kSmemBytes : C::kSmemBytes;
   cfg.stream = s;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -1050,7 +1280,9 @@ int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s) {
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, loop ? tree_attn_tc_kernel<kHD, true, kFine> : tree_attn_tc_kernel<kHD, false, kFine>, mq, mk, mv, mtk, mtv, p);
+  auto* kernel = loop ? tree_attn_tc_kernel<kHD, true, kFine, false> : tree_attn_tc_kernel<kHD, false, kFine, false>;
+  if (plan.long_runs) kernel = tree_attn_tc_kernel<128, false, false, true>;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, mq, mk, mv, mtk, mtv, p);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "tree_attn_tc_kernel launch");
   return FALCON_OK;
 }

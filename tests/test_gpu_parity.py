@@ -624,6 +624,49 @@ def test_attn_tc_head_sizes_and_separate_tree_buffers(T, G, L, splits, separate,
         assert not dt.status.cpu().numpy().any()
 
 
+# From 800 (two row blocks: 1200) keys per CTA on the rows-on-lanes kernel runs its loop for long runs.
+LONG_RUNS = [([60], [1000], 2, 1, 1),                   # the last tile ends inside a step of 16 keys
+             ([1], [1024], 1, 1, 1),                    # one row; the last tile holds one key
+             ([65], [1087], 1, 1, 1),                   # tiles that end on the upper half's first key and inside it
+             ([80, 17, 40], [1500, 30, 120], 2, 1, 1),  # sequences of one and two tiles beside a long one
+             ([64, 30], [3400, 3000], 2, 8, 4),         # several blocks of 128 rows, four splits
+             ([32, 20, 9, 31], [1300, 1281, 1216, 1407], 20, 8, 1)]  # units of up to 256 rows: two row blocks, and one
+
+
+@pytest.mark.parametrize("sizes,prefs,Hkv,G,splits", LONG_RUNS)
+def test_attn_tc_long_runs(sizes, prefs, Hkv, G, splits):
+    rng = np.random.default_rng(sum(prefs) + G)
+    tb, q, k, v = random_case(rng, sizes, prefs, Hkv * G, Hkv, 128, slack=1)
+    ref = oracle_attn(tb, Hkv * G, Hkv, 128, q, k, v)
+    for hc in (True, False):
+        dt = H.DevTrees(tb)
+        out, _ = H.run_attn(dt, Hkv * G, Hkv, 128, q, k, v, kernel=binding.ATTN_TC, n_splits=splits, host_copies=hc)
+        H.assert_attn_close(out, ref, tb.node_off)
+        assert not dt.status.cpu().numpy().any()
+
+
+def test_attn_tc_long_runs_exact_rows_mask_rows_and_bounded_wait():
+    rng = np.random.default_rng(77)
+    T, L = 24, 1100
+    tb, q, k, v = random_case(rng, [T], [L], 4, 2, 128, slack=1)
+    dt = H.DevTrees(tb)
+    rows = relaxed_mask_rows(tb, 3)
+    out, _ = H.run_attn(dt, 4, 2, 128, q, k, v, tree_mask=rows, kernel=binding.ATTN_TC, n_splits=1)
+    H.assert_attn_close(out, oracle_attn(tb, 4, 2, 128, q, k, v, tree_mask=rows), tb.node_off)
+    out, _ = H.run_attn(dt, 4, 2, 128, q, k, v, kernel=binding.ATTN_TC, n_splits=1, flags=binding.ATTN_TEST_STALL)
+    assert dt.status.cpu().numpy()[0] & binding.DEV_TIMEOUT
+    assert not synth.bf16_bits_to_f32(out).any()
+    dt.status.zero_()
+    # scores that run from -256 to 256: the rows are recomputed exactly
+    q = synth.f32_to_bf16_bits(np.ones((T, 1, 128), np.float32))
+    ramp = np.linspace(-2.0, 2.0, L + T, dtype=np.float32)[None, None, :, None]
+    k = synth.f32_to_bf16_bits(np.broadcast_to(ramp, (1, 1, L + T, 128)).copy())
+    v = synth.normal_bf16(rng, (1, 1, L + T, 128))
+    out, _ = H.run_attn(dt, 1, 1, 128, q, k, v, scale=1.0, kernel=binding.ATTN_TC, n_splits=1)
+    H.assert_attn_close(out, oracle_attn(tb, 1, 1, 128, q, k, v, scale=1.0), tb.node_off)
+    assert not dt.status.cpu().numpy().any()
+
+
 @pytest.mark.parametrize("D", [64, 128])
 @pytest.mark.parametrize("separate", [False, True])
 @pytest.mark.parametrize("sizes,prefs,Hkv,G", [
