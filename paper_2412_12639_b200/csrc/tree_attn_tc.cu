@@ -113,6 +113,11 @@ struct TcParams {
   int32_t h_prefix[kHostSeqs];
   int32_t h_order[kHostSeqs];  // grid z -> sequence, longest first
 };
+// kMix: the sequences are split differently, and `mix` says what a CTA does.  (A kernel of its own: the longer parameters cost every launch
+// up to 0.2 us.)
+struct TcMixParams : TcParams {
+  MixTable mix;
+};
 
 // A CTA's partial rows in scratch: 16-byte pieces [piece][row], so that a warp's 32 rows are contiguous for
 // the writer (a thread per row) and the reader alike, then (m, sum) [row].
@@ -138,11 +143,11 @@ __device__ __forceinline__ uint64_t desc_of(uint32_t lo) {
 // clock is not held down: one row block 1760 -> 1560, two 2080 -> 1620, of 1024 that the MMAs take.  148 units of 128 rows x 12352 keys, four a head
 // 119.7 -> 103.9 us; 32 units of 128 rows x 4160 keys 40.8 -> 32.0.
 // kFine: a weight is the sum of two bf16 numbers, and partial rows are fp32 (see fine_weights).
-template <int kHD, bool kLoop, bool kFine, bool kLong>
+template <int kHD, bool kLoop, bool kFine, bool kLong, bool kMix>
 __global__ void __launch_bounds__(kTcThreads, 1)
 tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                     const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_tk,
-                    const __grid_constant__ CUtensorMap tm_tv, const TcParams p) {
+                    const __grid_constant__ CUtensorMap tm_tv, const std::conditional_t<kMix, TcMixParams, TcParams> p) {
   static_assert(!kLong || (kHD == 128 && !kLoop && !kFine), "not built");
   using C = Cfg<kHD, kLong>;
   constexpr int kSlots = C::kSlots, kHalves = C::kHalves, kBKMax = C::kBKMax;
@@ -156,9 +161,16 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
   auto bar = [&](int i) { return smem_base + C::kOffBars + 8u * static_cast<uint32_t>(i); };
 
   const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
-  const int n_splits = kLoop ? 1 : gridDim.x, split = kLoop ? 0 : blockIdx.x;  // cluster = all CTAs of a row of the grid
-  int kvh = blockIdx.y % p.Hkv, unit = blockIdx.y / p.Hkv;
-  int b = p.have_host ? p.h_order[blockIdx.z] : static_cast<int>(blockIdx.z);
+  // cluster = all CTAs of a row of the grid: the splits of one unit, or (mixed) of several units of one or more sequences
+  uint32_t mix = 0u;
+  if constexpr (kMix) {
+    mix = p.mix.cta[blockIdx.y * gridDim.x + blockIdx.x];
+    if (mix == kMixIdle) return;  // (the cluster's barrier does not wait for those that have left)
+  }
+  const int n_splits = kLoop ? 1 : kMix ? (mix >> 18 & 7) + 1 : gridDim.x, split = kLoop ? 0 : kMix ? mix >> 15 & 7 : blockIdx.x;
+  const uint32_t unit_kvh = kMix ? mix >> 5 & 1023 : blockIdx.y, z0 = kMix ? mix & 31 : blockIdx.z;
+  int kvh = unit_kvh % p.Hkv, unit = unit_kvh / p.Hkv;
+  int b = p.have_host ? p.h_order[z0] : static_cast<int>(z0);
   const int G = p.G, BK = p.tile_keys, R = p.unit_rows;
   const uint32_t half_tile = static_cast<uint32_t>(BK) * 128u, tile_bytes = half_tile * kHalves;
 
@@ -881,7 +893,8 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
       if (!kLoop && inexact) s_rescue[row] = 1;
       inv = have && fine ? 1.f / l_row : 0.f;
     }
-    unsigned char* part = p.part + static_cast<int64_t>((blockIdx.z * gridDim.y + blockIdx.y) * n_splits + split) * part_bytes(kHD, R, kFine);
+    const uint32_t part0 = kMix ? blockIdx.y * gridDim.x + (mix >> 21 & 7) : (blockIdx.z * gridDim.y + blockIdx.y) * n_splits;  // of the unit's first split
+    unsigned char* part = p.part + static_cast<int64_t>(part0 + split) * part_bytes(kHD, R, kFine);
     auto put16 = [&](int piece, uint32_t a, uint32_t bq, uint32_t c, uint32_t d) {
       *reinterpret_cast<uint4*>(n_splits == 1 ? reinterpret_cast<unsigned char*>(dst) + piece * 16 : part + (piece * R + row) * 16) =
           make_uint4(a, bq, c, d);
@@ -949,6 +962,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
 
   tc_fence_before();
   bool rescue = !kLoop;
+  if (kMix && n_splits == 1) cluster_sync_release();  // (others of the cluster wait for it)
   if (!kLoop && n_splits > 1) {
     // ================================ merge ================================
     cluster_sync_release();  // every split's partial rows are visible (it is this CTA's barrier as well)
@@ -956,7 +970,8 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
     // issued before any is used: one round trip to L2.
     constexpr int kCols = kFine ? 4 : 8, kPieces = kHD / kCols;
     constexpr uint32_t kRowBytes = kHD * (kFine ? 4 : 2);
-    const unsigned char* parts = p.part + static_cast<int64_t>((blockIdx.z * gridDim.y + blockIdx.y) * n_splits) * part_bytes(kHD, R, kFine);
+    const uint32_t part0 = kMix ? blockIdx.y * gridDim.x + (mix >> 21 & 7) : (blockIdx.z * gridDim.y + blockIdx.y) * n_splits;
+    const unsigned char* parts = p.part + static_cast<int64_t>(part0) * part_bytes(kHD, R, kFine);
     auto merge = [&](auto most) {
       constexpr int kM = decltype(most)::value;
       for (int item = tid; item < rows_mine * kPieces; item += kTcThreads) {
@@ -1053,7 +1068,7 @@ int resident_clusters(falcon_ctx* ctx, int s) {
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, tree_attn_tc_kernel<128, false, false, false>, &cfg) != cudaSuccess) n = -1;
+    if (cudaOccupancyMaxActiveClusters(&n, tree_attn_tc_kernel<128, false, false, false, false>, &cfg) != cudaSuccess) n = -1;
     resident[s] = n > 0 ? n : -1;
     cudaGetLastError();
   }
@@ -1083,6 +1098,8 @@ int keys_per_cta(const falcon_attn_args& a, int splits) {
 struct Plan {
   int q_nodes, n_units, splits, tile;
   double ctas;  // that have rows
+  bool may_mix;
+  int mix_size, mix_clusters;  // clusters of CTAs on units of different numbers of splits (0: all have `splits`)
   bool long_runs;
 };
 // Rows per unit (one block of 128 or two), key splits per unit and tile height: the least estimated time.
@@ -1095,11 +1112,11 @@ struct Plan {
 // One sequence's tile height is chosen so that its tiles divide evenly over the splits.
 // With fine weights a tile measures more (0.55 and 0.92 us for 64-wide heads, 0.75 and 1.2 for 128-wide), and so does a merge;
 // with those figures for the tiles alone the choice got worse (1.3 % above the best split count over 58 shapes, 0.8 % as it is).
-Plan make_plan(falcon_ctx* ctx, const falcon_attn_args& a) {
+Plan make_plan(falcon_ctx* ctx, const falcon_attn_args& a, MixTable* mix) {
   const int B = a.tree.batch, G = a.n_q_heads / a.n_kv_heads;
   const bool host = a.tree.prefix_len_host && a.tree.node_off_host, wide = a.head_dim == 128;
   constexpr int kBKMax = Cfg<128, false>::kBKMax;
-  Plan best = {nodes_per_unit(a, kRowsMax), 1, std::max(1, a.n_splits), kBKMax, 0., false};
+  Plan best = {nodes_per_unit(a, kRowsMax), 1, std::max(1, a.n_splits), kBKMax, 0., false, 0, 0, false};
   best.n_units = (a.tree.max_tree + best.q_nodes - 1) / best.q_nodes;
   double best_us = 1e30;
   for (int rows = 128; rows <= kRowsMax; rows += 128) {
@@ -1132,8 +1149,43 @@ Plan make_plan(falcon_ctx* ctx, const falcon_attn_args& a) {
       if (units > slots) est = B == 1 ? longest * static_cast<double>(static_cast<int64_t>((units + slots - 1) / slots)) : std::max(longest, total / slots + 0.3 * longest);
       if (est < best_us) {
         best_us = est;
-        best = {q_nodes, n_units, s, tile, units * s, false};
+        best = {q_nodes, n_units, s, tile, units * s, false, 0, 0, false};
       }
+    }
+  }
+  int per_cta = keys_per_cta(a, best.splits);
+  // Sequences of very different lengths in one wave get different numbers of splits (mix_plan).  Tiles and merges cost here what random shapes
+  // say; the plan has to promise 8 % (15 % against no split) and 1.2 us.  1633 random batches: taken for 194, 1.15 times as fast there (0.95 to
+  // 1.6).  5 sequences of 300-6565 keys, 8 KV heads of two query heads, 21.3 -> 14.9 us; 3 of 700-3565, 16 heads of 64, 20.3 -> 14.3.
+  if (B > 1 && B <= kHostSeqs && host && a.n_splits == 0 && static_cast<int64_t>(a.n_kv_heads) * best.n_units * B <= ctx->sm_count) {
+    best.may_mix = true;
+    struct Seq {
+      int keys, rows;
+    } seq[kHostSeqs];  // in the order of the kernel's table (h_order)
+    for (int i = 0; i < B; ++i) {
+      const int nodes = a.tree.node_off_host[i + 1] - a.tree.node_off_host[i];
+      seq[i] = {a.tree.prefix_len_host[i] + nodes, std::min(nodes, best.q_nodes) * G};
+    }
+    std::stable_sort(seq, seq + B, [](const Seq& x, const Seq& y) { return x.keys > y.keys; });
+    const bool fine = fine_weights(a.head_dim, a.k_tree != nullptr);
+    auto time_us = [&](int i, int ns) {
+      const int tiles = ((std::max(seq[i].keys, 1) + kBKMax - 1) / kBKMax + ns - 1) / ns;
+      return (ns > 1 ? 1.0 : 0.0) + tiles * (seq[i].rows > 128 ? 0.9 : 0.5) * (fine ? 1.3 : 1.0);
+    };
+    double uniform = 0.;
+    for (int i = 0; i < B; ++i) uniform = std::max(uniform, time_us(i, best.splits));
+    if (mix_plan(B, a.n_kv_heads * best.n_units, uniform * (best.splits > 1 ? 0.92 : 0.85) - 1.2, time_us,
+                 [&](int ns) { return resident_clusters(ctx, ns); }, mix, &best.mix_size, &best.mix_clusters)) {
+      best.splits = 1;
+      per_cta = 0;
+      for (int i = 0; i < best.mix_size * best.mix_clusters; ++i) {
+        if (mix->cta[i] == kMixIdle) continue;
+        const int ns = static_cast<int>((mix->cta[i] >> 18) & 7) + 1;
+        best.splits = std::max(best.splits, ns);
+        per_cta = std::max(per_cta, (seq[mix->cta[i] & 31].keys + ns - 1) / ns);
+      }
+    } else {
+      best.mix_size = 0;
     }
   }
   // Long runs of keys have a loop of their own (kLong).  Against the other one at equal rows and splits it takes 0.6 to 0.9 us more a
@@ -1142,11 +1194,11 @@ Plan make_plan(falcon_ctx* ctx, const falcon_attn_args& a) {
   // 700-800 1.02, 800-1200 1.06, above 1.10 (up to 1.25); more CTAs than SMs, where short ones follow the long ones, 800-1200 0.98, above 1.06; two row
   // blocks 700-1200 0.98, 1200-1500 1.03, above 1.06.
   if (wide && !fine_weights(128, a.k_tree != nullptr) &&
-      keys_per_cta(a, best.splits) >= (best.q_nodes * G > 128 || best.ctas > ctx->sm_count ? 1400 : 800)) {
+      per_cta >= (best.q_nodes * G > 128 || best.ctas > ctx->sm_count ? 1400 : 800)) {
     best.long_runs = true;
     best.tile = Cfg<128, true>::kBKMax;
     if (B == 1) {
-      const int per = keys_per_cta(a, best.splits), nt = (per + best.tile - 1) / best.tile;
+      const int per = per_cta, nt = (per + best.tile - 1) / best.tile;
       best.tile = std::min(best.tile, ((per + nt - 1) / nt + 15) / 16 * 16);
     }
   }
@@ -1163,17 +1215,23 @@ int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s) {
     auto set = [&](auto* kernel, uint32_t bytes) {
       if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
     };
-    set(tree_attn_tc_kernel<128, false, false, false>, Cfg<128, false>::kSmemBytes);
-    set(tree_attn_tc_kernel<128, false, false, true>, Cfg<128, true>::kSmemBytes);
-    set(tree_attn_tc_kernel<128, true, false, false>, Cfg<128, false>::kSmemBytes);
-    set(tree_attn_tc_kernel<128, false, true, false>, Cfg<128, false>::kSmemBytes);
-    set(tree_attn_tc_kernel<128, true, true, false>, Cfg<128, false>::kSmemBytes);
-    set(tree_attn_tc_kernel<64, false, true, false>, Cfg<64, false>::kSmemBytes);
-    set(tree_attn_tc_kernel<64, true, true, false>, Cfg<64, false>::kSmemBytes);
+    set(tree_attn_tc_kernel<128, false, false, false, false>, Cfg<128, false>::kSmemBytes);
+    set(tree_attn_tc_kernel<128, false, false, false, true>, Cfg<128, false>::kSmemBytes);
+    set(tree_attn_tc_kernel<128, false, false, true, false>, Cfg<128, true>::kSmemBytes);
+    set(tree_attn_tc_kernel<128, false, false, true, true>, Cfg<128, true>::kSmemBytes);
+    set(tree_attn_tc_kernel<128, true, false, false, false>, Cfg<128, false>::kSmemBytes);
+    set(tree_attn_tc_kernel<128, false, true, false, false>, Cfg<128, false>::kSmemBytes);
+    set(tree_attn_tc_kernel<128, false, true, false, true>, Cfg<128, false>::kSmemBytes);
+    set(tree_attn_tc_kernel<128, true, true, false, false>, Cfg<128, false>::kSmemBytes);
+    set(tree_attn_tc_kernel<64, false, true, false, false>, Cfg<64, false>::kSmemBytes);
+    set(tree_attn_tc_kernel<64, false, true, false, true>, Cfg<64, false>::kSmemBytes);
+    set(tree_attn_tc_kernel<64, true, true, false, false>, Cfg<64, false>::kSmemBytes);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute(tree_attn_tc_kernel)");
     attr_set = true;
   }
-  const Plan plan = make_plan(ctx, a);
+  TcMixParams p;
+  const Plan plan = make_plan(ctx, a, &p.mix);
+  const bool mixed = plan.mix_size > 0;
   const int q_nodes = plan.q_nodes, n_units = plan.n_units, splits = plan.splits, tile_keys = plan.tile;
   // More units than SMs, of few tiles each: one CTA per SM works on several (see kLoop).  What a unit costs beside its
   // tiles is about 2 us then and 4.5 us as a CTA of its own, but the hardware gives out CTAs as SMs become free
@@ -1215,10 +1273,11 @@ int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s) {
     return FALCON_ERR_CUDA;
   }
 
-  TcParams p;
   p.part = nullptr;
-  if (splits > 1) {
-    const int rc = ensure_workspace(ctx, static_cast<size_t>(splits) * Hkv * n_units * B * part_bytes(kHD, q_nodes * G, kFine) + 256);
+  if (splits > 1 || plan.may_mix) {
+    // (Where the lengths decide between one split and several, scratch for either: it must not have to grow when they do.)
+    const int64_t parts = std::max<int64_t>(mixed ? 0 : static_cast<int64_t>(splits) * Hkv * n_units * B, plan.may_mix ? kMixCtas : 0);
+    const int rc = ensure_workspace(ctx, static_cast<size_t>(parts) * part_bytes(kHD, q_nodes * G, kFine) + 256);
     if (rc) return rc;
     p.part = static_cast<unsigned char*>(ctx->ws);
   }
@@ -1265,13 +1324,13 @@ int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s) {
   }
 
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = loop ? dim3(ctx->sm_count) : dim3(splits, Hkv * n_units, B);
+  cfg.gridDim = mixed ? dim3(plan.mix_size, plan.mix_clusters) : loop ? dim3(ctx->sm_count) : dim3(splits, Hkv * n_units, B);
   cfg.blockDim = dim3(kTcThreads);
   cfg.dynamicSmemBytes = plan.long_runs ? Cfg<128, true>::kSmemBytes : C::kSmemBytes;
   cfg.stream = s;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = splits;
+  attr[0].val.clusterDim.x = loop ? 1 : cfg.gridDim.x;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   // Programmatic dependent launch: this grid may be scheduled while the previous kernel of the stream
@@ -1280,9 +1339,15 @@ int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s) {
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  auto* kernel = loop ? tree_attn_tc_kernel<kHD, true, kFine, false> : tree_attn_tc_kernel<kHD, false, kFine, false>;
-  if (plan.long_runs) kernel = tree_attn_tc_kernel<128, false, false, true>;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, mq, mk, mv, mtk, mtv, p);
+  auto launch = [&](auto mix, const auto& params) {
+    constexpr bool kMix = decltype(mix)::value;
+    auto* kernel = tree_attn_tc_kernel<kHD, false, kFine, false, kMix>;
+    if constexpr (!kMix)
+      if (loop) kernel = tree_attn_tc_kernel<kHD, true, kFine, false, false>;
+    if (plan.long_runs) kernel = tree_attn_tc_kernel<128, false, false, true, kMix>;
+    return cudaLaunchKernelEx(&cfg, kernel, mq, mk, mv, mtk, mtv, params);
+  };
+  const cudaError_t e = mixed ? launch(std::true_type{}, p) : launch(std::false_type{}, static_cast<const TcParams&>(p));
   if (e != cudaSuccess) return cuda_fail(ctx, e, "tree_attn_tc_kernel launch");
   return FALCON_OK;
 }

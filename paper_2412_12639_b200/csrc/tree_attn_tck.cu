@@ -41,6 +41,7 @@
 // griddepcontrol.wait.  Every mbarrier wait is bounded; a wait that runs out sets FALCON_DEV_TIMEOUT,
 // what is in flight is drained, and the rows are still delivered (by the exact path).
 #include <algorithm>
+#include <type_traits>
 
 #include "tc_util.cuh"
 
@@ -168,6 +169,11 @@ struct TckParams {
     int32_t seq, node_base, nodes, prefix;
   } h_seq[kHostSeqs];
 };
+// kMix: the sequences are split differently, and `mix` says what a CTA does.  (A kernel of its own: the longer parameters cost every launch
+// 0.06 to 0.1 us.)
+struct TckMixParams : TckParams {
+  MixTable mix;
+};
 
 // K/V tiles are read once per call and the caches are far larger than L2: the loads carry an
 // evict-first policy, so the stream does not push out what is reused (q, the outputs, the next
@@ -267,11 +273,11 @@ __device__ __forceinline__ int col_of_lane(int lane) {
 // kTile: the ring is three stages of tiles of this many keys, known at compile time (0: not known).
 // kSep: the tree's K/V rows are in buffers of their own; its keys then start a tile of their own
 // (the prefix's last tile is cut at the prefix length) and tm_nk / tm_nv describe those buffers.
-template <int kVar, int kTile, int kHD, bool kSep>
+template <int kVar, int kTile, int kHD, bool kSep, bool kMix>
 __global__ void __launch_bounds__(Var<kVar>::kThreads, 1)
 tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                      const __grid_constant__ CUtensorMap tm_nk, const __grid_constant__ CUtensorMap tm_nv,
-                     const TckParams p) {
+                     const std::conditional_t<kMix, TckMixParams, TckParams> p) {
   using VT = Var<kVar>;
   using C = Cfg<VT::kCfg>;
   constexpr bool kFine = fine_weights(kHD, kSep);
@@ -300,9 +306,16 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
   auto bar = [&](int i) { return bars + 8u * static_cast<uint32_t>(i); };
 
   const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
-  const int n_splits = gridDim.x, split = blockIdx.x;  // cluster = all CTAs of a row of the grid
-  const int kvh = blockIdx.y % p.Hkv, mtile = blockIdx.y / p.Hkv;
-  const int b = p.have_host ? p.h_seq[blockIdx.z].seq : static_cast<int>(blockIdx.z);
+  // cluster = all CTAs of a row of the grid: the splits of one unit, or (mixed) of several units of one or more sequences
+  uint32_t mix = 0u;
+  if constexpr (kMix) {
+    mix = p.mix.cta[blockIdx.y * gridDim.x + blockIdx.x];
+    if (mix == kMixIdle) return;  // (the cluster's barrier does not wait for those that have left)
+  }
+  const int n_splits = kMix ? (mix >> 18 & 7) + 1 : gridDim.x, split = kMix ? mix >> 15 & 7 : blockIdx.x, rank0 = mix >> 21 & 7;
+  const uint32_t unit = kMix ? mix >> 5 & 1023 : blockIdx.y, z = kMix ? mix & 31 : blockIdx.z;
+  const int kvh = unit % p.Hkv, mtile = unit / p.Hkv;
+  const int b = p.have_host ? p.h_seq[z].seq : static_cast<int>(z);
   constexpr int kCW = VT::kCW, kPer = VT::kPer;
   const int G = p.G, N = p.n_rows, n_chunks = N / kCW;
   const uint32_t q_half_bytes = static_cast<uint32_t>(N) * 128u;  // between the two 64-column halves of Q
@@ -387,9 +400,9 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
     return p.q + (static_cast<int64_t>(node_base + (mg >> p.g_shift)) * p.Hq + kvh * G + (mg & (G - 1))) * kHD + q_part * (kHD / 8);
   };
   if (p.have_host) {  // the caller's host copies of the per-sequence scalars: no round trip to global memory
-    node_base = p.h_seq[blockIdx.z].node_base;
-    T_real = p.h_seq[blockIdx.z].nodes;
-    L_raw = p.h_seq[blockIdx.z].prefix;
+    node_base = p.h_seq[z].node_base;
+    T_real = p.h_seq[z].nodes;
+    L_raw = p.h_seq[z].prefix;
     geometry();
   }
 
@@ -484,7 +497,7 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
   tc_fence_after();
   const uint32_t tmem_base = *s_tmem_base;
   // Cluster phase 1: "my merge barrier exists".  Arrive now, wait just before the first remote copy.
-  if (n_splits > 1) cluster_arrive();
+  if (gridDim.x > 1) cluster_arrive();
 
   if (warp == kWarpProducer) {
     // ================================ TMA producer (ring refills) ================================
@@ -792,11 +805,11 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
     auto slot_addr = [&](int owner) -> uint32_t {  // shared::cluster address of this split's slot in `owner`
       const uint32_t local = owner == split ? smem_base + off_stage
                                             : smem_base + off_mrg + static_cast<uint32_t>(split < owner ? split : split - 1) * slot_bytes;
-      return map_to_rank(local, static_cast<uint32_t>(owner));
+      return map_to_rank(local, static_cast<uint32_t>(rank0 + owner));
     };
     const bool have = live && n_my > 0 && !*abort_flag;
     uint32_t own_l[4] = {0u, 0u, 0u, 0u};
-    if (n_splits > 1) cluster_wait();  // phase 1 (arrived long ago): every peer's merge barrier is initialised
+    if (gridDim.x > 1) cluster_wait();  // phase 1 (arrived long ago): every peer's merge barrier is initialised
     // The row sums first: they are complete with the last tile's softmax pass and do not have to wait for the
     // MMAs that are still running.  They go to the other CTAs at once; this CTA's own slot lies over Q and,
     // where it is larger than Q, over the ring's first stage, which the last MMAs may still be reading: its
@@ -824,7 +837,7 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
       for (int i = 0; i < n_splits; ++i)
         if (i != split)
           st_async_v4(slot_addr(i) + static_cast<uint32_t>(d_per) * pitch + st_id * 16, l0, l1, l2, l3,
-                      map_to_rank(bar(kBarMrg), static_cast<uint32_t>(i)));
+                      map_to_rank(bar(kBarMrg), static_cast<uint32_t>(rank0 + i)));
       own_l[0] = l0;
       own_l[1] = l1;
       own_l[2] = l2;
@@ -838,10 +851,10 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
     // The ring and P^T are idle now (all of this CTA's MMAs have finished, all its loads landed).
     if (st_id * 4 < N)
       st_async_v4(slot_addr(split) + static_cast<uint32_t>(d_per) * pitch + st_id * 16, own_l[0], own_l[1], own_l[2], own_l[3],
-                  map_to_rank(bar(kBarMrg), static_cast<uint32_t>(split)));
+                  map_to_rank(bar(kBarMrg), static_cast<uint32_t>(rank0 + split)));
     const bool o_lane = kHD == 128 || kr < kHD;  // this lane holds a head-dim row (whole warps do or do not)
     const uint32_t row_dst = slot_addr(o_lane ? o_me : split) + static_cast<uint32_t>(dl_me) * pitch;
-    const uint32_t row_bar = map_to_rank(bar(kBarMrg), static_cast<uint32_t>(o_lane ? o_me : split));
+    const uint32_t row_bar = map_to_rank(bar(kBarMrg), static_cast<uint32_t>(rank0 + (o_lane ? o_me : split)));
 #pragma unroll
     for (int ci = 0; ci < kPer; ++ci) {
       const int ch = grp + kColGroups * ci;
@@ -868,7 +881,7 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
       }
     }
   } 
-  if (warp < kWarpSm0 && n_splits > 1) cluster_wait();  // the producer and MMA warps complete phase 1 too
+  if (warp < kWarpSm0 && gridDim.x > 1) cluster_wait();  // the producer and MMA warps complete phase 1 too
 
   // ================================ merge ================================
   // Wait until every softmax warp of every split has delivered its share of this CTA's rows.  Every
@@ -932,33 +945,36 @@ tree_attn_tck_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_cons
 
 bool is_pow2(int x) { return x > 0 && (x & (x - 1)) == 0; }
 
-// (every instantiation of a variant has the same footprint: one CTA per SM)
+// Clusters of s CTAs that are resident at once, asked once per context (every instantiation of a variant has the same
+// footprint: one CTA per SM).
+template <int kVar>
+int resident_clusters(falcon_ctx* ctx, int s) {
+  int* resident = ctx->attn_resident[1 + kVar];
+  if (resident[s] == 0) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(s, ctx->sm_count, 1);
+    cfg.blockDim = dim3(Var<kVar>::kThreads);
+    cfg.dynamicSmemBytes = kSmemMax;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = s;
+    attr.val.clusterDim.y = 1;
+    attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, tree_attn_tck_kernel<kVar, kBKMax, 128, false, false>, &cfg) != cudaSuccess) n = -1;
+    resident[s] = n > 0 ? n : -1;
+    cudaGetLastError();
+  }
+  return resident[s];
+}
+
 template <int kVar>
 int pick_splits(falcon_ctx* ctx, int units, int max_tiles) {
-  int* resident = ctx->attn_resident[1 + kVar];
-  int best = 1;
-  for (int s = kMaxSplits; s >= 1; --s) {
-    if (s > max_tiles) continue;
-    if (resident[s] == 0) {
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3(s, ctx->sm_count, 1);
-      cfg.blockDim = dim3(Var<kVar>::kThreads);
-      cfg.dynamicSmemBytes = kSmemMax;
-      cudaLaunchAttribute attr;
-      attr.id = cudaLaunchAttributeClusterDimension;
-      attr.val.clusterDim.x = s;
-      attr.val.clusterDim.y = 1;
-      attr.val.clusterDim.z = 1;
-      cfg.attrs = &attr;
-      cfg.numAttrs = 1;
-      int n = 0;
-      if (cudaOccupancyMaxActiveClusters(&n, tree_attn_tck_kernel<kVar, kBKMax, 128, false>, &cfg) != cudaSuccess) n = -1;
-      resident[s] = n > 0 ? n : -1;
-      cudaGetLastError();
-    }
-    if (resident[s] >= units) { best = s; break; }
-  }
-  return best;
+  for (int s = kMaxSplits; s > 1; --s)
+    if (s <= max_tiles && resident_clusters<kVar>(ctx, s) >= units) return s;
+  return 1;
 }
 
 template <int kVar, int kHD, bool kSep>
@@ -982,10 +998,13 @@ int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s, int 
     auto set = [&](auto* kernel) {
       if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSmemMax));
     };
-    set(tree_attn_tck_kernel<kVar, kBKMax, 128, false>);  // (the occupancy query below is made with this one)
-    set(tree_attn_tck_kernel<kVar, kBKMax, kHD, kSep>);
-    set(tree_attn_tck_kernel<kVar, kLowTile, kHD, kSep>);
-    set(tree_attn_tck_kernel<kVar, kMidTile, kHD, kSep>);
+    set(tree_attn_tck_kernel<kVar, kBKMax, 128, false, false>);  // (the occupancy query below is made with this one)
+    set(tree_attn_tck_kernel<kVar, kBKMax, kHD, kSep, false>);
+    set(tree_attn_tck_kernel<kVar, kBKMax, kHD, kSep, true>);
+    set(tree_attn_tck_kernel<kVar, kLowTile, kHD, kSep, false>);
+    set(tree_attn_tck_kernel<kVar, kLowTile, kHD, kSep, true>);
+    set(tree_attn_tck_kernel<kVar, kMidTile, kHD, kSep, false>);
+    set(tree_attn_tck_kernel<kVar, kMidTile, kHD, kSep, true>);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFuncSetAttribute(tree_attn_tck_kernel)");
     attr_set = true;
   }
@@ -994,6 +1013,35 @@ int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s, int 
   int splits = a.n_splits;
   if (splits == 0) splits = pick_splits<kVar>(ctx, Hkv * n_units * B, max_tiles > 0 ? max_tiles : 1);
   if (splits < 1) splits = 1;
+  // A sequence's share of the caller's host copies, the longest first (see HostSeq).
+  TckMixParams p;
+  p.have_host = 0;
+  if (a.tree.prefix_len_host && a.tree.node_off_host && B <= kHostSeqs) {
+    p.have_host = 1;
+    const int32_t* off = a.tree.node_off_host;
+    for (int i = 0; i < B; ++i) p.h_seq[i] = {i, off[i], off[i + 1] - off[i], a.tree.prefix_len_host[i]};
+    if (static_cast<int64_t>(Hkv) * n_units * B <= 2 * ctx->sm_count)
+      std::stable_sort(p.h_seq, p.h_seq + B, [](const auto& x, const auto& y) { return x.prefix + x.nodes > y.prefix + y.nodes; });
+  }
+  // In one wave the slowest CTA is the launch: sequences of very different lengths get different numbers of splits (mix_plan).  A tile's
+  // time and a merge's are what random shapes say; the plan has to promise 8 % (15 % against no split) and 1.2 us, since clusters that
+  // hold several units start and end together.  1244 random batches: taken for 168, 1.25 times as fast there (0.97 to 1.9).  8 sequences of
+  // 300-6565 keys, 16 heads of 128, 51.2 -> 30.1 us; 5 of 300-6565, 8 KV heads of two query heads, 22.0 -> 15.8.
+  bool mixed_splits = false;
+  int mix_size = 0, mix_clusters = 0;
+  if (a.n_splits == 0 && p.have_host && B > 1 && static_cast<int64_t>(Hkv) * n_units * B <= ctx->sm_count) {
+    auto time_us = [&](int i, int ns) {
+      const int tiles = (std::max(p.h_seq[i].prefix + p.h_seq[i].nodes, 1) + kBKMax - 1) / kBKMax + (kSep ? 1 : 0);
+      return (ns > 1 ? 0.6 : 0.0) + (tiles + ns - 1) / ns * (kFine ? 1.05 : 0.85);
+    };
+    if (mix_plan(B, Hkv * n_units, time_us(0, splits) * (splits > 1 ? 0.92 : 0.85) - 1.2, time_us,
+                 [&](int ns) { return resident_clusters<kVar>(ctx, ns); }, &p.mix, &mix_size, &mix_clusters)) {
+      mixed_splits = true;
+      splits = 1;
+      for (int i = 0; i < mix_size * mix_clusters; ++i)
+        if (p.mix.cta[i] != kMixIdle) splits = std::max(splits, static_cast<int>((p.mix.cta[i] >> 18) & 7) + 1);
+    }
+  }
   // Shared memory: Q, merge area (the other splits' shares of this CTA's head-dim rows and the row
   // sums) and the small arrays are fixed by the shape; the K/V ring takes the rest, as three stages
   // of the highest tile that fits (two if three would be lower than 64 keys).  A split count whose
@@ -1004,7 +1052,7 @@ int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s, int 
     return ns > 1 ? static_cast<uint32_t>(ns - 1) * ((kHD + ns - 1) / ns + sum_rows(kFine)) * part_pitch(N, kFine) : 0u;
   };
   auto ring_room = [&](int ns) { return static_cast<int>(kSmemMax) - static_cast<int>(q_bytes + merge_bytes(ns) + C::kSmallBytes); };
-  while (splits > 1 && ring_room(splits) < 2 * 64 * row_bytes) --splits;
+  while (!mixed_splits && splits > 1 && ring_room(splits) < 2 * 64 * row_bytes) --splits;
   const int room = ring_room(splits);
   int n_stages = 3, tile_keys = room / (3 * row_bytes) / 16 * 16;
   if (tile_keys < 64) {
@@ -1046,7 +1094,6 @@ int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s, int 
                              get_tmap(ctx, a.next_k_cache, kv_dims, kv_strides, kv_box, &mnk) &&
                              get_tmap(ctx, a.next_v_cache, kv_dims, kv_strides, kv_box, &mnv);
 
-  TckParams p;
   p.Hq = Hq;
   p.Hkv = Hkv;
   p.G = G;
@@ -1075,36 +1122,32 @@ int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s, int 
   p.kv_stride_h = a.kv_stride_h;
   p.kv_stride_s = a.kv_stride_s;
   p.out = static_cast<__nv_bfloat16*>(a.out);
-  p.have_host = 0;
   p.early_prefix = (a.flags & FALCON_ATTN_PREFIX_STABLE) ? 1 : 0;
   p.prefetch_next = prefetch_next ? 1 : 0;
   p.stall_first = (a.flags & FALCON_ATTN_TEST_STALL) ? 1 : 0;
-  if (a.tree.prefix_len_host && a.tree.node_off_host && B <= kHostSeqs) {
-    p.have_host = 1;
-    const int32_t* off = a.tree.node_off_host;
-    for (int i = 0; i < B; ++i) p.h_seq[i] = {i, off[i], off[i + 1] - off[i], a.tree.prefix_len_host[i]};
-    if (static_cast<int64_t>(Hkv) * n_units * B <= 2 * ctx->sm_count)
-      std::stable_sort(p.h_seq, p.h_seq + B, [](const auto& x, const auto& y) { return x.prefix + x.nodes > y.prefix + y.nodes; });
-  }
 
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(splits, Hkv * n_units, B);
+  cfg.gridDim = mixed_splits ? dim3(mix_size, mix_clusters) : dim3(splits, Hkv * n_units, B);
   cfg.blockDim = dim3(Var<kVar>::kThreads);
   cfg.dynamicSmemBytes = smem_bytes;
   cfg.stream = s;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = splits;
+  attr[0].val.clusterDim.x = cfg.gridDim.x;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  auto* kernel = tree_attn_tck_kernel<kVar, kLowTile, kHD, kSep>;
-  if (n_stages == 3 && tile_keys == kBKMax) kernel = tree_attn_tck_kernel<kVar, kBKMax, kHD, kSep>;
-  else if (kMidTile && n_stages == 3 && tile_keys == kMidTile) kernel = tree_attn_tck_kernel<kVar, kMidTile, kHD, kSep>;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, mk, mv, mnk, mnv, p);
+  auto launch = [&](auto mix, const auto& params) {
+    constexpr bool kMix = decltype(mix)::value;
+    auto* kernel = tree_attn_tck_kernel<kVar, kLowTile, kHD, kSep, kMix>;
+    if (n_stages == 3 && tile_keys == kBKMax) kernel = tree_attn_tck_kernel<kVar, kBKMax, kHD, kSep, kMix>;
+    else if (kMidTile && n_stages == 3 && tile_keys == kMidTile) kernel = tree_attn_tck_kernel<kVar, kMidTile, kHD, kSep, kMix>;
+    return cudaLaunchKernelEx(&cfg, kernel, mk, mv, mnk, mnv, params);
+  };
+  const cudaError_t e = mixed_splits ? launch(std::true_type{}, p) : launch(std::false_type{}, static_cast<const TckParams&>(p));
   if (e != cudaSuccess) return cuda_fail(ctx, e, "tree_attn_tck_kernel launch");
   return FALCON_OK;
 }

@@ -698,6 +698,37 @@ def test_attn_tc_more_units_than_sms(sizes, prefs, Hkv, G, separate, D):
             assert not dt.status.cpu().numpy().any()
 
 
+@pytest.mark.parametrize("kernel", TC_KERNELS)
+@pytest.mark.parametrize("D,separate", [(128, False), (64, False), (128, True)])
+@pytest.mark.parametrize("sizes,prefs,Hkv,G", [
+    ([31, 9, 30], [4000, 300, 900], 4, 1),                # groups of one to six CTAs, clusters with a place left over
+    ([12, 30, 7, 1, 25], [2500, 61, 640, 0, 1300], 3, 2),  # units of one tile beside long ones
+    ([40, 20], [3300, 100], 2, 4),                        # (rows on lanes) two row blocks and one
+])
+def test_attn_sequences_with_different_numbers_of_splits(sizes, prefs, Hkv, G, D, separate, kernel):
+    """Batches in one wave whose lengths differ so much that the plan splits them differently, against the oracle; and twice, with
+    the same bits (the merge does not depend on which CTA is done first)."""
+    rng = np.random.default_rng(sum(prefs) + Hkv + D)
+    tb, q, k, v = random_case(rng, sizes, prefs, Hkv * G, Hkv, D, slack=1)
+    ref = oracle_attn(tb, Hkv * G, Hkv, D, q, k, v)
+    kw = {}
+    if separate:
+        kt = np.empty((tb.total_nodes, Hkv, D), np.uint16)
+        vt = np.empty_like(kt)
+        for b in range(tb.batch):
+            Lb, Tb, o = prefs[b], sizes[b], tb.node_off[b]
+            kt[o:o + Tb] = k[b, :, Lb:Lb + Tb].transpose(1, 0, 2)
+            vt[o:o + Tb] = v[b, :, Lb:Lb + Tb].transpose(1, 0, 2)
+            k[b, :, Lb:] = 0x7FC0
+            v[b, :, Lb:] = 0x7FC0
+        kw = dict(k_tree=kt, v_tree=vt)
+    dt = H.DevTrees(tb)
+    outs = [H.run_attn(dt, Hkv * G, Hkv, D, q, k, v, kernel=kernel, host_copies=True, **kw)[0] for _ in range(2)]
+    H.assert_attn_close(outs[0], ref, tb.node_off)
+    np.testing.assert_array_equal(outs[0], outs[1])
+    assert not dt.status.cpu().numpy().any()
+
+
 @pytest.mark.parametrize("D, T, prefs, expect", [
     (128, 60, [1987] * 8, binding.ATTN_TC), (128, 60, [1988] * 8, binding.ATTN_TCK), (128, 60, [300, 3676] * 4, binding.ATTN_TCK),
     (128, 60, [300, 3674] * 4, binding.ATTN_TC), (128, 32, [700] * 8, binding.ATTN_TCK), (128, 33, [700] * 8, binding.ATTN_TC),
