@@ -161,28 +161,29 @@ __global__ void __launch_bounds__(kCompactThreads, 4) kv_compact_kernel(const Co
   }
 }
 
-// The gather alone: grid (parts, B).
-__global__ void __launch_bounds__(kCompactThreads) feature_gather_kernel(const CompactParams p) {
+// The gather alone: grid (parts, B).  Everything up to the path is asked for at once.
+__global__ void __launch_bounds__(kCompactThreads) feature_gather_kernel(const CompactParams p, const HostOffsets h) {
   __shared__ int s_path[FALCON_T_MAX];
-  __shared__ int s_bad;
+  const int b = blockIdx.y, tid = threadIdx.x;
+  int base = 0, end = 0;
+  if (h.have) {
+    base = h.off[b];
+    end = h.off[b + 1];
+  }
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const int b = blockIdx.y, tid = threadIdx.x;
-  const int base = p.node_off[b];
-  const int T = p.node_off[b + 1] - base;
-  const int n = p.n_path[b];
+  // (beyond its end the path may hold anything)
+  const int n = p.n_path[b], t = tid < p.path_stride && tid < FALCON_T_MAX ? p.path[static_cast<int64_t>(b) * p.path_stride + tid] : 0;
+  if (!h.have) {
+    base = p.node_off[b];
+    end = p.node_off[b + 1];
+  }
+  const int T = end - base;
   int fault = 0;
   if (T < 1 || T > FALCON_T_MAX || n < 1 || n > T) fault |= FALCON_DEV_BAD_PATH;
   if (n > p.out_rows) fault |= FALCON_DEV_CAPACITY;
-  if (tid == 0) s_bad = 0;
-  __syncthreads();
-  if (!fault && tid < n) {
-    const int t = p.path[static_cast<int64_t>(b) * p.path_stride + tid];
-    s_path[tid] = t;
-    if (t < 0 || t >= T) s_bad = 1;
-  }
-  __syncthreads();
-  if (s_bad) fault |= FALCON_DEV_BAD_PATH;
+  if (tid < FALCON_T_MAX) s_path[tid] = t;
+  if (__syncthreads_or(tid < n && (t < 0 || t >= T)) && !fault) fault |= FALCON_DEV_BAD_PATH;
   if (fault) {
     if (blockIdx.x == 0 && tid == 0) dev_status_or(p.status, b, fault);
     return;
@@ -241,7 +242,7 @@ int launch_feature_gather(falcon_ctx* ctx, const falcon_gather_args& a, cudaStre
   attr.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, feature_gather_kernel, p);
+  cudaError_t e = cudaLaunchKernelEx(&cfg, feature_gather_kernel, p, host_offsets(a.tree));
   if (e != cudaSuccess) return cuda_fail(ctx, e, "feature_gather_kernel launch");
   return FALCON_OK;
 }
