@@ -727,7 +727,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             published = true;
             ref_barrier(false);
           }
-          const float neg = -m_ref;
+          const float neg = valid ? -m_ref : -INFINITY;  // (rows that do not exist: weights of zero, which cost the least power)
 #pragma unroll
           for (int c = 0; c < kC / 32; ++c)
 #pragma unroll
