@@ -3,11 +3,13 @@
 //
 // Row r of a KV head is (tree node r / G, query head r % G), so grouped-query heads share the K/V
 // stream.  A unit is (sequence, KV head, block of at most 256 query rows); one thread-block cluster per
-// unit, whose CTAs split the key range (prefix + tree) into runs of whole tiles of up to 64 keys.
+// unit, whose CTAs split the key range (prefix + tree) into runs of whole tiles of up to 64 keys, or 128 where the runs are long (kLong).
+// Where the sequences of a batch that fits in one wave are of very different lengths, a cluster holds units of several with different
+// numbers of splits (kMix).
 // Where there are many units of few tiles, the grid is one CTA per SM instead, which works on one unit after the
 // other (kLoop): the next one's K, V and Q are on their way while the rows of the one before are delivered.
 //
-// Inside a CTA (576 threads) an item is (tile, block of 128 rows), and four score buffers in TMEM take the items in
+// Inside a CTA (576 threads; kLong differs, see there) an item is (tile, block of 128 rows), and four score buffers in TMEM take the items in
 // turn, so that the softmax of some runs under the MMAs of others:
 //   more than 128 rows   two row blocks share every K/V tile: it is read once from L2 for both;
 //   at most 128 rows     one row block: an item is a tile.
@@ -1098,7 +1100,6 @@ int keys_per_cta(const falcon_attn_args& a, int splits) {
 struct Plan {
   int q_nodes, n_units, splits, tile;
   double ctas;  // that have rows
-  bool may_mix;
   int mix_size, mix_clusters;  // clusters of CTAs on units of different numbers of splits (0: all have `splits`)
   bool long_runs;
 };
@@ -1112,11 +1113,11 @@ struct Plan {
 // One sequence's tile height is chosen so that its tiles divide evenly over the splits.
 // With fine weights a tile measures more (0.55 and 0.92 us for 64-wide heads, 0.75 and 1.2 for 128-wide), and so does a merge;
 // with those figures for the tiles alone the choice got worse (1.3 % above the best split count over 58 shapes, 0.8 % as it is).
-Plan make_plan(falcon_ctx* ctx, const falcon_attn_args& a, MixTable* mix) {
+Plan make_plan(falcon_ctx* ctx, const falcon_attn_args& a, MixTable* mix, bool allow_mix) {
   const int B = a.tree.batch, G = a.n_q_heads / a.n_kv_heads;
   const bool host = a.tree.prefix_len_host && a.tree.node_off_host, wide = a.head_dim == 128;
   constexpr int kBKMax = Cfg<128, false>::kBKMax;
-  Plan best = {nodes_per_unit(a, kRowsMax), 1, std::max(1, a.n_splits), kBKMax, 0., false, 0, 0, false};
+  Plan best = {nodes_per_unit(a, kRowsMax), 1, std::max(1, a.n_splits), kBKMax, 0., 0, 0, false};
   best.n_units = (a.tree.max_tree + best.q_nodes - 1) / best.q_nodes;
   double best_us = 1e30;
   for (int rows = 128; rows <= kRowsMax; rows += 128) {
@@ -1149,16 +1150,15 @@ Plan make_plan(falcon_ctx* ctx, const falcon_attn_args& a, MixTable* mix) {
       if (units > slots) est = B == 1 ? longest * static_cast<double>(static_cast<int64_t>((units + slots - 1) / slots)) : std::max(longest, total / slots + 0.3 * longest);
       if (est < best_us) {
         best_us = est;
-        best = {q_nodes, n_units, s, tile, units * s, false, 0, 0, false};
+        best = {q_nodes, n_units, s, tile, units * s, 0, 0, false};
       }
     }
   }
   int per_cta = keys_per_cta(a, best.splits);
   // Sequences of very different lengths in one wave get different numbers of splits (mix_plan).  Tiles and merges cost here what random shapes
-  // say; the plan has to promise 8 % (15 % against no split) and 1.2 us.  1633 random batches: taken for 194, 1.15 times as fast there (0.95 to
-  // 1.6).  5 sequences of 300-6565 keys, 8 KV heads of two query heads, 21.3 -> 14.9 us; 3 of 700-3565, 16 heads of 64, 20.3 -> 14.3.
-  if (B > 1 && B <= kHostSeqs && host && a.n_splits == 0 && static_cast<int64_t>(a.n_kv_heads) * best.n_units * B <= ctx->sm_count) {
-    best.may_mix = true;
+  // say; the plan has to promise 8 % (15 % against no split) and 1.2 us.  1633 random batches: taken for 166, 1.14 times as fast there (0.95 to
+  // 1.6, two of them below 0.985).  5 sequences of 300-6565 keys, 8 KV heads of two query heads, 21.3 -> 14.9 us; 3 of 700-3565, 16 heads of 64, 20.3 -> 14.3.
+  if (allow_mix && B > 1 && B <= kHostSeqs && host && a.n_splits == 0 && static_cast<int64_t>(a.n_kv_heads) * best.n_units * B <= ctx->sm_count) {
     struct Seq {
       int keys, rows;
     } seq[kHostSeqs];  // in the order of the kernel's table (h_order)
@@ -1170,7 +1170,7 @@ Plan make_plan(falcon_ctx* ctx, const falcon_attn_args& a, MixTable* mix) {
     const bool fine = fine_weights(a.head_dim, a.k_tree != nullptr);
     auto time_us = [&](int i, int ns) {
       const int tiles = ((std::max(seq[i].keys, 1) + kBKMax - 1) / kBKMax + ns - 1) / ns;
-      return (ns > 1 ? 1.0 : 0.0) + tiles * (seq[i].rows > 128 ? 0.9 : 0.5) * (fine ? 1.3 : 1.0);
+      return (ns > 1 ? 0.7 + 0.15 * ns : 0.0) + tiles * (seq[i].rows > 128 ? 0.9 : 0.5) * (!wide ? 1.1 : fine ? 1.3 : 1.0);
     };
     double uniform = 0.;
     for (int i = 0; i < B; ++i) uniform = std::max(uniform, time_us(i, best.splits));
@@ -1230,7 +1230,14 @@ int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s) {
     attr_set = true;
   }
   TcMixParams p;
-  const Plan plan = make_plan(ctx, a, &p.mix);
+  Plan plan = make_plan(ctx, a, &p.mix, true);
+  if (plan.mix_size) {
+    // Scratch cannot grow while the stream is being captured: a call that would not have needed it then keeps the plan without.
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (static_cast<size_t>(kMixCtas) * part_bytes(kHD, plan.q_nodes * G, kFine) + 256 > ctx->ws_bytes &&
+        (cudaStreamIsCapturing(s, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone))
+      plan = make_plan(ctx, a, &p.mix, false);
+  }
   const bool mixed = plan.mix_size > 0;
   const int q_nodes = plan.q_nodes, n_units = plan.n_units, splits = plan.splits, tile_keys = plan.tile;
   // More units than SMs, of few tiles each: one CTA per SM works on several (see kLoop).  What a unit costs beside its
@@ -1274,9 +1281,8 @@ int launch_impl(falcon_ctx* ctx, const falcon_attn_args& a, cudaStream_t s) {
   }
 
   p.part = nullptr;
-  if (splits > 1 || plan.may_mix) {
-    // (Where the lengths decide between one split and several, scratch for either: it must not have to grow when they do.)
-    const int64_t parts = std::max<int64_t>(mixed ? 0 : static_cast<int64_t>(splits) * Hkv * n_units * B, plan.may_mix ? kMixCtas : 0);
+  if (splits > 1) {
+    const int64_t parts = mixed ? kMixCtas : static_cast<int64_t>(splits) * Hkv * n_units * B;
     const int rc = ensure_workspace(ctx, static_cast<size_t>(parts) * part_bytes(kHD, q_nodes * G, kFine) + 256);
     if (rc) return rc;
     p.part = static_cast<unsigned char*>(ctx->ws);

@@ -729,6 +729,33 @@ def test_attn_sequences_with_different_numbers_of_splits(sizes, prefs, Hkv, G, D
     assert not dt.status.cpu().numpy().any()
 
 
+def test_attn_first_call_of_a_batch_that_could_be_mixed_can_be_captured():
+    """Three sequences of which one would get two splits and the others none, on a context without scratch: captured at once, the launch must
+    do with none; the same call outside a capture may take the other plan."""
+    rng = np.random.default_rng(5)
+    sizes, prefs, Hkv, D = [9, 30, 31], [300, 300, 1200], 32, 128
+    tb, q, k, v = random_case(rng, sizes, prefs, Hkv, Hkv, D, slack=1)
+    ref = oracle_attn(tb, Hkv, Hkv, D, q, k, v)
+    dt = H.DevTrees(tb)
+    qd, kd, vd = H.dev_bf16(q), H.dev_bf16(k), H.dev_bf16(v)
+    out = torch.zeros_like(qd)
+    a = binding.attn_args(dt.desc(host_copies=True), Hkv, Hkv, D, 1.0 / math.sqrt(D), qd, out, kd, vd,
+                          tuple(int(s) for s in kd.stride()[:3]), kd.shape[2], kernel=binding.ATTN_TC)
+    ctx = H.falcon.Context(0)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        ctx.falcon_tree_attn(a)
+    g.replay()
+    torch.cuda.synchronize()
+    H.assert_attn_close(H.host_bits(out), ref, tb.node_off)
+    out.zero_()
+    ctx.falcon_tree_attn(a)
+    torch.cuda.synchronize()
+    H.assert_attn_close(H.host_bits(out), ref, tb.node_off)
+    assert not dt.status.cpu().numpy().any()
+
+
 @pytest.mark.parametrize("D, T, prefs, expect", [
     (128, 60, [1987] * 8, binding.ATTN_TC), (128, 60, [1988] * 8, binding.ATTN_TCK), (128, 60, [300, 3676] * 4, binding.ATTN_TCK),
     (128, 60, [300, 3674] * 4, binding.ATTN_TC), (128, 32, [700] * 8, binding.ATTN_TCK), (128, 33, [700] * 8, binding.ATTN_TC),
