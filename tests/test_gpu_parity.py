@@ -624,7 +624,7 @@ def test_attn_tc_head_sizes_and_separate_tree_buffers(T, G, L, splits, separate,
         assert not dt.status.cpu().numpy().any()
 
 
-# From 800 (two row blocks: 1200) keys per CTA on the rows-on-lanes kernel runs its loop for long runs.
+# From 800 (two row blocks: 1400) keys per CTA on the rows-on-lanes kernel runs its loop for long runs.
 LONG_RUNS = [([60], [1000], 2, 1, 1),                   # the last tile ends inside a step of 16 keys
              ([1], [1024], 1, 1, 1),                    # one row; the last tile holds one key
              ([65], [1087], 1, 1, 1),                   # tiles that end on the upper half's first key and inside it
